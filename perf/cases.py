@@ -156,7 +156,7 @@ def _stencil(case, upper=False):
 
 def _powerlaw(n, g):
     """The power-law recipe: lognormal row lengths of mean 12, uniform columns,
-    values in [-1, 1), diagonal twice the row's absolute sum."""
+    values in (-1, 1), diagonal twice the row's absolute sum."""
     mu = math.log(12.0) - 1.5 * 1.5 / 2
     length = torch.empty(n, dtype=torch.float64, device=DEV).log_normal_(mu, 1.5, generator=g)
     length = length.round().clamp(1, max(1, min(20_000, (n - 1) // 2))).long()
@@ -165,7 +165,7 @@ def _powerlaw(n, g):
     cols += cols >= rows
     key = torch.unique(rows * n + cols)
     rows, cols = key // n, key % n
-    vals = _dyadic(g, key.numel(), -1, 1, 20)
+    vals = _dyadic(g, key.numel(), -1, 1, 20) + 2.0 ** -21  # never zero
     total = torch.zeros(n, dtype=torch.float64, device=DEV).index_add_(0, rows, vals.abs())
     at = torch.arange(n, device=DEV)
     key, order = torch.sort(torch.cat([key, at * (n + 1)]))

@@ -38,6 +38,11 @@ constexpr int kRedSlots = 2048;     // max CTAs of a reduction grid
 constexpr int kRedValues = 16;      // max values reduced together by one grid
 constexpr int kScalars = 4096;      // device scalar scratch per plan (doubles)
 
+// Dynamic shared memory of the orthogonalisation kernel: what a CTA has, less
+// its static arrays.
+constexpr int kGsDynMax = 227 * 1024 - 12 * 1024;
+size_t gs_scratch_bytes();          // d_ticket: counters, then the grid exchange
+
 int num_sms();                      // cached cudaDevAttrMultiProcessorCount
 int reduce_grid(int64_t n, int block);  // CTAs for a streaming reduction
 // CTAs of a grid-stride launch of kernel fn: every CTA resident at once (the
@@ -221,7 +226,8 @@ struct xb_plan {
     bool vec_ok = false;                 // val and col 16-byte aligned
     // reduction scratch
     double *d_part = nullptr;            // kRedSlots * kRedValues partials
-    unsigned *d_ticket = nullptr;        // 64 counters (one in use per reduction)
+    unsigned *d_ticket = nullptr;        // 64 counters (one in use per reduction), then
+                                         // the grid exchange of the orthogonalisation
     double *d_scal = nullptr;            // kScalars
     // solver workspace (grown on demand)
     void *d_work = nullptr;

@@ -273,13 +273,14 @@ int xb_lanczos(xb_plan *p, int32_t nev, int32_t m, int32_t m_max, double theta, 
         for (int j = k; j < m; j++) {
             double *vj = V + (size_t)j * ld, *wv = V + (size_t)(j + 1) * ld;
             XB_TRY(xb::spmv_launch(p, variant, block, ipt, 1.0, vj, 0.0, wv, s));
-            XB_TRY(xb::gm_ortho_step<double>(p, st, n, V, ld, wv, j, ortho, s));
+            XB_TRY(xb::gm_ortho_step<double>(p, st, n, V, ld, wv, j, ortho, false, s));
             k_scale_inv<<<sg, 256, 0, s>>>(n, wv, st.H + (size_t)j * (M + 1) + j + 1);
             steps++;
         }
         XB_CUDA(cudaMemcpyAsync(H.data(), st.H, H.size() * sizeof(double), cudaMemcpyDeviceToHost,
                                 s));
         XB_CUDA(cudaStreamSynchronize(s));
+        XB_TRY(xb::gs_check(p));
         for (int j = k; j < m; j++)
             for (int i = 0; i <= j + 1; i++)
                 T[(size_t)i * (M + 1) + j] = H[(size_t)j * (M + 1) + i];
@@ -490,13 +491,14 @@ int xb_arnoldi(xb_plan *p, int32_t nev, int32_t m, int32_t m_max, double theta, 
         for (int j = k; j < m; j++) {
             double *vj = V + (size_t)j * ld, *wv = V + (size_t)(j + 1) * ld;
             XB_TRY(xb::spmv_launch(p, variant, block, ipt, 1.0, vj, 0.0, wv, s));
-            XB_TRY(xb::gm_ortho_step<double>(p, st, n, V, ld, wv, j, ortho, s));
+            XB_TRY(xb::gm_ortho_step<double>(p, st, n, V, ld, wv, j, ortho, false, s));
             k_scale_inv<<<sg, 256, 0, s>>>(n, wv, st.H + (size_t)j * (M + 1) + j + 1);
             steps++;
         }
         XB_CUDA(cudaMemcpyAsync(H.data(), st.H, H.size() * sizeof(double), cudaMemcpyDeviceToHost,
                                 s));
         XB_CUDA(cudaStreamSynchronize(s));
+        XB_TRY(xb::gs_check(p));
         for (int j = k; j < m; j++)
             for (int i = 0; i <= j + 1; i++)
                 T[(size_t)i * (M + 1) + j] = H[(size_t)j * (M + 1) + i];

@@ -1,8 +1,7 @@
 // Krylov vector kernels: deterministic two-stage reductions (per-CTA partials,
 // the last CTA to finish reduces them in a fixed order, so no extra launch and
-// no run-to-run variation), the fused modified Gram-Schmidt step of Arnoldi
-// (Sec. 3.2.2, MGS) with the Givens update folded into its final CTA, and the
-// fused BiCGStab updates.  Scalars never leave the device inside a step.
+// no run-to-run variation), the GMRES cycle's ends and the fused BiCGStab
+// updates (the orthogonalisation is in ortho.cu).  Scalars never leave the device inside a step.
 #include <cstdlib>
 #include "krylov.cuh"
 
@@ -122,43 +121,6 @@ __global__ void k_gm_init(int64_t n, const VB *__restrict__ r0, xb::GmDev st, do
     }
 }
 
-// Givens update of column j after h_{j+1,j} = hn (single thread).
-__device__ void gm_givens(xb::GmDev st, int j, double hn) {
-    double *col = st.H + (size_t)j * (st.M + 1);
-    col[j + 1] = hn;
-    const double len2 = st.misc[xb::GM_LEN2] + hn * hn;
-    for (int i = 0; i < j; i++) {
-        const double a = col[i], b = col[i + 1];
-        col[i] = st.cs[i] * a + st.sn[i] * b;
-        col[i + 1] = -st.sn[i] * a + st.cs[i] * b;
-    }
-    const double a = col[j];
-    const double rr = hypot(a, hn);
-    if (rr == 0.0) {  // A v_j lies in span(v_0..v_{j-1}) with a zero pivot: singular
-        st.misc[xb::GM_STOP] = 2.0;
-        return;
-    }
-    st.cs[j] = a / rr;
-    st.sn[j] = hn / rr;
-    col[j] = rr;
-    col[j + 1] = 0.0;
-    st.g[j + 1] = -st.sn[j] * st.g[j];
-    st.g[j] = st.cs[j] * st.g[j];
-    const double bn = st.misc[xb::GM_BNORM];
-    const double res = fabs(st.g[j + 1]) / bn;
-    st.misc[xb::GM_RES] = res;
-    st.misc[xb::GM_K] = (double)(j + 1);
-    if (hn <= 1e-14 * sqrt(len2)) {  // happy breakdown: the Krylov space is invariant
-        st.misc[xb::GM_STOP] = 1.0;
-        st.sc[j + 1] = 0.0;
-        st.scf[j + 1] = 0.0f;
-        return;
-    }
-    st.sc[j + 1] = 1.0 / hn;
-    st.scf[j + 1] = (float)(1.0 / hn);
-    if (res <= st.misc[xb::GM_TAU]) st.misc[xb::GM_STOP] = 1.0;
-}
-
 template <typename VB>
 struct V16;
 template <>
@@ -186,331 +148,39 @@ struct V16<float> {
     }
 };
 
-// One element of the MGS launch: OP 0 dot(w, vn); OP 1 w -= c vp, dot(w, vn);
-// OP 2 w -= c vp, dot(w, w).
-template <int OP, typename VB>
-__device__ __forceinline__ VB mgs_elem(VB &w, VB vp, VB vn, VB c, VB acc) {
-    if (OP != 0) w = fma(-c, vp, w);
-    return OP == 2 ? fma(w, w, acc) : fma(w, vn, acc);
-}
-
-// 16-byte load with an L2 evict-first policy: v_{i-1} is read for the last time
-// in the sweep, so its lines should make way for w and v_i.
-__device__ __forceinline__ uint64_t l2_evict_first() {
-    uint64_t p;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-    return p;
-}
-__device__ __forceinline__ double2 ld_last_use(const double2 *a, uint64_t pol) {
-    double2 v;
-    asm volatile("ld.global.nc.L2::cache_hint.v2.f64 {%0,%1}, [%2], %3;"
-                 : "=d"(v.x), "=d"(v.y) : "l"(a), "l"(pol));
-    return v;
-}
-__device__ __forceinline__ float4 ld_last_use(const float4 *a, uint64_t pol) {
-    float4 v;
-    asm volatile("ld.global.nc.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(a), "l"(pol));
-    return v;
-}
-
-// One launch of the MGS sweep of Arnoldi step j:
-//   i == 0      : h_0j = (w, v_0)
-//   0 < i <= j  : w -= h_{i-1,j} v_{i-1};  h_ij = (w, v_i)
-//   i == j+1    : w -= h_jj v_j;  h_{j+1,j} = ||w||, then Givens.
-// Basis vectors are stored unnormalised with scales sc (v_i = sc[i]*V_i).
-// Operands move as 16-byte vectors (two grid-wide chunks per thread per
-// iteration) when the three arrays are 16-byte aligned.  flags bit 0: walk the
-// chunks from the end of the vectors (consecutive launches of a sweep alternate
-// direction, so each starts on the w and v_i lines that the previous one
-// touched last and still finds them in L2); bit 1: load v_{i-1} with an L2
-// evict-first policy.
-template <int OP, typename VB>
-__global__ void __launch_bounds__(kVB) k_mgs(int64_t n, VB *__restrict__ w,
-                                             const VB *__restrict__ vprev,
-                                             const VB *__restrict__ vnext, xb::GmDev st, int j,
-                                             int i, double *__restrict__ part,
-                                             unsigned *__restrict__ ticket, int vec, int flags) {
-    if (st.misc[xb::GM_STOP] != 0.0) return;
-    const VB c = (VB)(OP != 0 ? st.misc[xb::GM_COEF] : 0.0);
-    VB acc0 = VB(0), acc1 = VB(0);
-    int64_t done = 0;
-    if (vec) {
-        using T = typename V16<VB>::T;
-        constexpr int N = V16<VB>::N;
-        const int64_t nv = n / N;
-        T *w2 = reinterpret_cast<T *>(w);
-        const T *p2 = reinterpret_cast<const T *>(OP != 0 ? vprev : w);
-        const T *q2 = reinterpret_cast<const T *>(OP != 2 ? vnext : w);
-        const bool rev = flags & 1, hint = flags & 2;
-        const uint64_t pol = l2_evict_first();
-        const int64_t gs = gstride();
-        const int64_t full = nv / gs;            // grid-wide chunks every thread owns
-        const int64_t et = full * gs + gtid();   // this thread's slot in the partial chunk
-        auto one = [&](int64_t e) {
-            T a = w2[e];
-            const T pa = OP != 0 ? (hint ? ld_last_use(p2 + e, pol) : p2[e]) : a;
-            const T qa = OP != 2 ? q2[e] : a;
-#pragma unroll
-            for (int k = 0; k < N; k++) {
-                VB x = V16<VB>::get(a, k);
-                acc0 = mgs_elem<OP>(x, V16<VB>::get(pa, k), V16<VB>::get(qa, k), c, acc0);
-                V16<VB>::set(a, k, x);
-            }
-            if (OP != 0) w2[e] = a;
-        };
-        if (rev && et < nv) one(et);
-        int64_t k = 0;
-        for (; k + 1 < full; k += 2) {
-            const int64_t ka = rev ? full - 1 - k : k;
-            const int64_t e = ka * gs + gtid();
-            const int64_t f = rev ? e - gs : e + gs;
-            T a = w2[e], b = w2[f];
-            const T pa = OP != 0 ? (hint ? ld_last_use(p2 + e, pol) : p2[e]) : a;
-            const T pb = OP != 0 ? (hint ? ld_last_use(p2 + f, pol) : p2[f]) : b;
-            const T qa = OP != 2 ? q2[e] : a, qb = OP != 2 ? q2[f] : b;
-#pragma unroll
-            for (int q = 0; q < N; q++) {
-                VB x = V16<VB>::get(a, q), y = V16<VB>::get(b, q);
-                acc0 = mgs_elem<OP>(x, V16<VB>::get(pa, q), V16<VB>::get(qa, q), c, acc0);
-                acc1 = mgs_elem<OP>(y, V16<VB>::get(pb, q), V16<VB>::get(qb, q), c, acc1);
-                V16<VB>::set(a, q, x);
-                V16<VB>::set(b, q, y);
-            }
-            if (OP != 0) {
-                w2[e] = a;
-                w2[f] = b;
-            }
-        }
-        if (k < full) one((rev ? full - 1 - k : k) * gs + gtid());
-        if (!rev && et < nv) one(et);
-        done = nv * N;
-    }
-    for (int64_t e = done + gtid(); e < n; e += gstride()) {
-        VB x = w[e];
-        acc0 = mgs_elem<OP>(x, OP != 0 ? vprev[e] : x, OP != 2 ? vnext[e] : x, c, acc0);
-        if (OP != 0) w[e] = x;
-    }
-    double v[1] = {(double)acc0 + (double)acc1};
-    double t[1];
-    if (grid_reduce<1>(v, part, ticket, t) && threadIdx.x == 0) {
-        if (OP != 2) {
-            const double h = st.sc[i] * t[0];
-            st.H[(size_t)j * (st.M + 1) + i] = h;
-            st.misc[xb::GM_COEF] = st.sc[i] * h;
-            st.misc[xb::GM_LEN2] = (i == 0 ? 0.0 : st.misc[xb::GM_LEN2]) + h * h;
-        } else if (st.misc[xb::GM_RAW] != 0.0) {
-            st.H[(size_t)j * (st.M + 1) + j + 1] = sqrt(t[0]);
-        } else {
-            gm_givens(st, j, sqrt(t[0]));
-        }
-    }
-}
-
-// ---- block Gram-Schmidt family: CGS, DGKS, BCGS (Sec. 3.2.2) ----------------------
-
-constexpr int kMaxCoef = 520;  // >= M + 1 for every basis capacity M <= 512
-constexpr int kBgsAcc = 1, kBgsFin = 2, kBgsRev = 4;
-
-// Sum cnt <= NV per-thread values over the grid.  Returns true in every thread
-// of the last CTA to finish, with the totals in tot[0..cnt) (shared memory),
-// summed in a fixed order (deterministic).
-template <int NV>
-__device__ bool grid_reduce_n(const double (&v)[NV], int cnt, double *__restrict__ part,
-                              unsigned *__restrict__ ticket, double *tot) {
-    __shared__ double sh[NV][kVB / 32];
-    __shared__ bool last;
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int G = gridDim.x;
-#pragma unroll
-    for (int q = 0; q < NV; q++) {
-        if (q < cnt) {
-            double a = v[q];
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-            if (lane == 0) sh[q][wp] = a;
-        }
-    }
-    __syncthreads();
-    if ((int)threadIdx.x < cnt) {
-        double a = 0.0;
-        for (int k = 0; k < nw; k++) a += sh[threadIdx.x][k];
-        part[(size_t)threadIdx.x * G + blockIdx.x] = a;
-        __threadfence();
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) last = (atomicAdd(ticket, 1u) == (unsigned)G - 1);
-    __syncthreads();
-    if (!last) return false;
-    __threadfence();
-    for (int q = wp; q < cnt; q += nw) {
-        double a = 0.0;
-        for (int i = lane; i < G; i += 32) a += __ldcg(part + (size_t)q * G + i);
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if (lane == 0) tot[q] = a;
-    }
-    if (threadIdx.x == 0) *ticket = 0u;
-    __syncthreads();
-    return true;
-}
-
-// U elements (16-byte vectors at e[0..U)) of one block Gram-Schmidt pass:
-// update by the nu pending vectors (at most KU when KU > 0), store w, then the
-// nd dot products (or the squared norm when fin).  The U elements' loads are
-// issued together.
-template <typename VB, int KD, int KU, int U>
-__device__ __forceinline__ void bgs_elems(int64_t ea, int64_t eb, typename V16<VB>::T *w2,
-                                          const typename V16<VB>::T *V2, int64_t ldv, int u0,
-                                          int nu, int d0, int nd, bool fin, const VB *cf,
-                                          VB (&acc)[KD]) {
-    using T = typename V16<VB>::T;
-    constexpr int N = V16<VB>::N;
-    const int64_t e[2] = {ea, eb};
-    T x[U];
-#pragma unroll
-    for (int u = 0; u < U; u++) x[u] = w2[e[u]];
-    if (nu > 0) {
-        const int cnt = KU > 0 ? KU : nu;
-#pragma unroll 4
-        for (int i = 0; i < cnt; i++) {
-            if (KU > 0 && i >= nu) break;
-            const T *vi = V2 + (size_t)(u0 + i) * ldv;
-            T v[U];
-#pragma unroll
-            for (int u = 0; u < U; u++) v[u] = vi[e[u]];
-            const VB c = cf[i];
-#pragma unroll
-            for (int u = 0; u < U; u++)
-#pragma unroll
-                for (int q = 0; q < N; q++)
-                    V16<VB>::set(x[u], q, fma(-c, V16<VB>::get(v[u], q), V16<VB>::get(x[u], q)));
-        }
-#pragma unroll
-        for (int u = 0; u < U; u++) w2[e[u]] = x[u];
-    }
-    if (fin) {
-#pragma unroll
-        for (int u = 0; u < U; u++)
-#pragma unroll
-            for (int q = 0; q < N; q++)
-                acc[0] = fma(V16<VB>::get(x[u], q), V16<VB>::get(x[u], q), acc[0]);
-        return;
-    }
-#pragma unroll
-    for (int d = 0; d < KD; d++) {
-        if (d < nd) {
-            const T *vd = V2 + (size_t)(d0 + d) * ldv;
-            T v[U];
-#pragma unroll
-            for (int u = 0; u < U; u++) v[u] = vd[e[u]];
-#pragma unroll
-            for (int u = 0; u < U; u++)
-#pragma unroll
-                for (int q = 0; q < N; q++)
-                    acc[d] = fma(V16<VB>::get(x[u], q), V16<VB>::get(v[u], q), acc[d]);
-        }
-    }
-}
-
-// One pass of the block Gram-Schmidt family for Arnoldi step j:
-//   w -= sum_{u0 <= i < u1} coef_i V_i          (the pending update; none if u0 == u1;
-//                                               at most KU vectors when KU > 0)
-//   then either the dots (w, V_i) for d0 <= i < d0 + nd (nd <= KD), or, with
-//   kBgsFin (nd == 0), (w, w).
-// The last CTA turns dots into Hessenberg entries h_i = sc_i (w, V_i) (added to
-// the column with kBgsAcc: the second pass of DGKS) and the coefficients the
-// next pass subtracts, coef_i = sc_i h_i; with kBgsFin it stores
-// h_{j+1,j} = ||w|| and applies the Givens update (or only stores it in raw
-// mode).  kBgsRev walks the grid-wide chunks from the end (alternating passes
-// start on the lines the previous pass touched last).  Operands move as
-// 16-byte vectors, two grid-wide chunks per thread per iteration, when V, w
-// and the row stride allow it.
-template <typename VB, int KD, int KU, int MINB>
-__global__ void __launch_bounds__(kVB, MINB) k_bgs(int64_t n, VB *__restrict__ w,
-                                             const VB *__restrict__ V, int64_t ld, int u0, int u1,
-                                             int d0, int nd, int flags, xb::GmDev st, int j,
-                                             double *__restrict__ part,
-                                             unsigned *__restrict__ ticket, int vec) {
-    if (st.misc[xb::GM_STOP] != 0.0) return;
-    __shared__ VB cf[kMaxCoef];
-    __shared__ double tot[KD];
-    const int nu = u1 - u0;
-    for (int i = threadIdx.x; i < nu; i += blockDim.x) cf[i] = (VB)st.coef[u0 + i];
-    __syncthreads();
-    const bool fin = flags & kBgsFin, rev = flags & kBgsRev;
-    VB acc[KD];
-#pragma unroll
-    for (int q = 0; q < KD; q++) acc[q] = VB(0);
-    int64_t done = 0;
-    if (vec) {
-        using T = typename V16<VB>::T;
-        constexpr int N = V16<VB>::N;
-        const int64_t nv = n / N, ldv = ld / N;
-        T *w2 = reinterpret_cast<T *>(w);
-        const T *V2 = reinterpret_cast<const T *>(V);
-        const int64_t gs = gstride();
-        const int64_t full = nv / gs;           // grid-wide chunks every thread owns
-        const int64_t et = full * gs + gtid();  // this thread's slot in the partial chunk
-        if (rev && et < nv)
-            bgs_elems<VB, KD, KU, 1>(et, et, w2, V2, ldv, u0, nu, d0, nd, fin, cf, acc);
-        int64_t k = 0;
-        for (; k + 1 < full; k += 2) {
-            const int64_t e = (rev ? full - 1 - k : k) * gs + gtid();
-            bgs_elems<VB, KD, KU, 2>(e, rev ? e - gs : e + gs, w2, V2, ldv, u0, nu, d0, nd, fin, cf,
-                                     acc);
-        }
-        if (k < full) {
-            const int64_t e = (rev ? full - 1 - k : k) * gs + gtid();
-            bgs_elems<VB, KD, KU, 1>(e, e, w2, V2, ldv, u0, nu, d0, nd, fin, cf, acc);
-        }
-        if (!rev && et < nv)
-            bgs_elems<VB, KD, KU, 1>(et, et, w2, V2, ldv, u0, nu, d0, nd, fin, cf, acc);
-        done = nv * N;
-    }
-    for (int64_t e = done + gtid(); e < n; e += gstride()) {
-        VB x = w[e];
-        if (nu > 0) {
-            for (int i = 0; i < nu; i++) x = fma(-cf[i], V[(size_t)(u0 + i) * ld + e], x);
-            w[e] = x;
-        }
-        if (fin) {
-            acc[0] = fma(x, x, acc[0]);
-        } else {
-#pragma unroll
-            for (int q = 0; q < KD; q++)
-                if (q < nd) acc[q] = fma(x, V[(size_t)(d0 + q) * ld + e], acc[q]);
-        }
-    }
-    double v[KD];
-#pragma unroll
-    for (int q = 0; q < KD; q++) v[q] = (double)acc[q];
-    if (!grid_reduce_n<KD>(v, fin ? 1 : nd, part, ticket, tot)) return;
-    double *col = st.H + (size_t)j * (st.M + 1);
-    if (!fin) {
-        for (int q = threadIdx.x; q < nd; q += blockDim.x) {
-            const int i = d0 + q;
-            const double h = st.sc[i] * tot[q];
-            col[i] = (flags & kBgsAcc) ? col[i] + h : h;
-            st.coef[i] = st.sc[i] * h;
-        }
-    } else if (threadIdx.x == 0) {
-        double len2 = 0.0;
-        for (int i = 0; i <= j; i++) len2 += col[i] * col[i];
-        st.misc[xb::GM_LEN2] = len2;
-        if (st.misc[xb::GM_RAW] != 0.0) col[j + 1] = sqrt(tot[0]);
-        else gm_givens(st, j, sqrt(tot[0]));
-    }
-}
-
-// Least squares R y = g (upper triangular k x k), then y_i *= sc[i].
-__global__ void k_gm_solve(xb::GmDev st) {
-    if (threadIdx.x != 0) return;
+// Least squares R y = g (upper triangular k x k), then y_i *= sc[i].  One CTA:
+// the triangle comes into shared memory together (k <= kSolveK), then warp 0
+// solves by columns; y_i = s_i / r_ii is a product with the reciprocal taken
+// beforehand and one correction step, as accurate as the division and a third
+// of its latency.
+constexpr int kSolveK = 64;
+__global__ void __launch_bounds__(256) k_gm_solve(xb::GmDev st) {
+    __shared__ double R[kSolveK][kSolveK + 1], s[512], rinv[512];
     const int k = (int)st.misc[xb::GM_K];
-    for (int i = k - 1; i >= 0; i--) {
-        double s = st.g[i];
-        for (int q = i + 1; q < k; q++) s -= st.H[(size_t)q * (st.M + 1) + i] * st.y[q];
-        st.y[i] = s / st.H[(size_t)i * (st.M + 1) + i];
+    const int tid = threadIdx.x;
+    const size_t ldh = st.M + 1;
+    const bool held = k <= kSolveK;
+    if (held)
+        for (int t = tid; t < k * k; t += blockDim.x) {
+            const int c = t / k, r = t % k;
+            if (r <= c) R[c][r] = st.H[c * ldh + r];
+        }
+    for (int i = tid; i < k; i += blockDim.x) {
+        s[i] = st.g[i];
+        rinv[i] = 1.0 / st.H[i * ldh + i];
     }
-    for (int i = 0; i < k; i++) st.y[i] *= st.sc[i];
+    __syncthreads();
+    if (tid >= 32) return;
+    for (int i = k - 1; i >= 0; i--) {
+        const double *col = held ? R[i] : st.H + i * ldh;
+        const double d = col[i], si = s[i];
+        double y = si * rinv[i];
+        if (fabs(d) > 1e-280 && fabs(d) < 1e280) y = fma(fma(-y, d, si), rinv[i], y);
+        else y = si / d;
+        for (int r = tid; r < i; r += 32) s[r] = fma(-col[r], y, s[r]);
+        if (tid == 0) st.y[i] = y * st.sc[i];
+        __syncwarp();
+    }
 }
 
 // x += sum_i y_i V_i (each basis vector read once; 16-byte vectors when the
@@ -776,7 +446,7 @@ GmDev gm_layout(double *base, int M) {
     st.g = q; q += M + 1;
     st.sc = q; q += M + 1;
     st.y = q; q += M;
-    st.coef = q; q += M + 1;
+    st.gram = q; q += 8 * (size_t)(M + 1);
     st.misc = q; q += GM_NMISC;
     st.scf = reinterpret_cast<float *>(q);
     return st;
@@ -835,41 +505,6 @@ int gm_cycle_init_f32(xb_plan *p, GmDev st, int64_t n, const float *r0, double t
     return XB_OK;
 }
 
-// MGS traversal mode (flags of k_mgs: bit 0 alternate direction, bit 1
-// evict-first loads of v_{i-1}); XB_MGS_MODE=0..3 overrides the default.
-int mgs_mode(size_t elem) {
-    static const int env = [] {
-        const char *e = std::getenv("XB_MGS_MODE");
-        return e ? std::atoi(e) & 3 : -1;
-    }();
-    (void)elem;
-    return env >= 0 ? env : 3;
-}
-
-template <typename VB>
-int gm_mgs_step(xb_plan *p, GmDev st, int64_t n, const VB *V, int64_t ld, VB *w, int j,
-                cudaStream_t s) {
-    const int g = rgrid(k_mgs<1, VB>, n);
-    const int vec = (((uintptr_t)V % 16) == 0 && ((uintptr_t)w % 16) == 0 &&
-                     ((ld * sizeof(VB)) % 16) == 0) ? 1 : 0;
-    // With alternation on, pass i walks backwards when i is even (pass 0 then
-    // starts on the tail of w that the SpMV wrote last).
-    const int mode = mgs_mode(sizeof(VB));
-    auto fl = [mode](int i) { return ((mode & 1) && !(i & 1) ? 1 : 0) | (mode & 2); };
-    k_mgs<0, VB><<<g, kVB, 0, s>>>(n, w, nullptr, V, st, j, 0, p->d_part, p->d_ticket, vec, fl(0));
-    for (int i = 1; i <= j; i++)
-        k_mgs<1, VB><<<g, kVB, 0, s>>>(n, w, V + (size_t)(i - 1) * ld, V + (size_t)i * ld, st, j, i,
-                                       p->d_part, p->d_ticket, vec, fl(i));
-    k_mgs<2, VB><<<g, kVB, 0, s>>>(n, w, V + (size_t)j * ld, nullptr, st, j, j + 1, p->d_part,
-                                   p->d_ticket, vec, fl(j + 1));
-    XB_LAUNCHED("k_mgs");
-    return XB_OK;
-}
-template int gm_mgs_step<double>(xb_plan *, GmDev, int64_t, const double *, int64_t, double *,
-                                  int, cudaStream_t);
-template int gm_mgs_step<float>(xb_plan *, GmDev, int64_t, const float *, int64_t, float *, int,
-                                 cudaStream_t);
-
 double ortho_passes(int ortho, int j) {
     const int nb = (j + 1 + 3) / 4;
     switch (ortho) {
@@ -886,56 +521,12 @@ int ortho_choice(int ortho, double tol, bool faulted) {
     return tol <= 1e-10 ? XB_ORTHO_MGS : XB_ORTHO_BCGS;
 }
 
-template <typename VB>
-int gm_ortho_step(xb_plan *p, GmDev st, int64_t n, const VB *V, int64_t ld, VB *w, int j,
-                  int ortho, cudaStream_t s) {
-    if (ortho == XB_ORTHO_MGS) return gm_mgs_step<VB>(p, st, n, V, ld, w, j, s);
-    constexpr int KD = 8;
-    // grids of exactly the resident CTAs (measured 12 % faster than 8 CTAs per SM in waves)
-    const int g4 = rgrid(k_bgs<VB, 4, 4, 4>, n);
-    const int g8 = rgrid(k_bgs<VB, KD, 0, 4>, n);
-    const int vec = (((uintptr_t)V % 16) == 0 && ((uintptr_t)w % 16) == 0 &&
-                     ((ld * sizeof(VB)) % 16) == 0) ? 1 : 0;
-    const bool zig = mgs_mode(sizeof(VB)) & 1;
-    int pass = 0;
-    // the first pass walks backwards (it starts on the tail of w the SpMV wrote last)
-    auto L = [&](int u0, int u1, int d0, int nd, int flags) {
-        if (zig && !(pass & 1)) flags |= kBgsRev;
-        pass++;
-        // 4 resident CTAs per SM (64 registers) measured faster than 2 with no spills
-        if (nd <= 4 && u1 - u0 <= 4)  // BCGS passes, and short CGS/DGKS sweeps
-            k_bgs<VB, 4, 4, 4><<<g4, kVB, 0, s>>>(n, w, V, ld, u0, u1, d0, nd, flags, st, j,
-                                                  p->d_part, p->d_ticket, vec);
-        else
-            k_bgs<VB, KD, 0, 4><<<g8, kVB, 0, s>>>(n, w, V, ld, u0, u1, d0, nd, flags, st, j,
-                                                   p->d_part, p->d_ticket, vec);
-    };
-    const int k = j + 1;  // basis vectors v_0..v_j
-    if (ortho == XB_ORTHO_BCGS) {
-        const int nb = (k + 3) / 4;
-        L(0, 0, 0, std::min(4, k), 0);
-        for (int b = 1; b < nb; b++) L(4 * (b - 1), 4 * b, 4 * b, std::min(4, k - 4 * b), 0);
-        L(4 * (nb - 1), k, 0, 0, kBgsFin);
-    } else {
-        for (int c = 0; c < k; c += KD) L(0, 0, c, std::min(KD, k - c), 0);
-        if (ortho == XB_ORTHO_DGKS)  // second CGS: update by the first, dots added to H
-            for (int c = 0; c < k; c += KD) L(0, c == 0 ? k : 0, c, std::min(KD, k - c), kBgsAcc);
-        L(0, k, 0, 0, kBgsFin);
-    }
-    XB_LAUNCHED("k_bgs");
-    return XB_OK;
-}
-template int gm_ortho_step<double>(xb_plan *, GmDev, int64_t, const double *, int64_t, double *,
-                                   int, int, cudaStream_t);
-template int gm_ortho_step<float>(xb_plan *, GmDev, int64_t, const float *, int64_t, float *,
-                                  int, int, cudaStream_t);
-
 template <typename VB, typename VX>
 int gm_update(xb_plan *p, GmDev st, int64_t n, const VB *V, int64_t ld, int k, VX *x,
               cudaStream_t s) {
     (void)p;
     (void)k;
-    k_gm_solve<<<1, 32, 0, s>>>(st);
+    k_gm_solve<<<1, 256, 0, s>>>(st);
     XB_LAUNCHED("k_gm_solve");
     const int vec = (((uintptr_t)V % 16) == 0 && ((uintptr_t)x % 16) == 0 &&
                      ((ld * sizeof(VB)) % 16) == 0) ? 1 : 0;

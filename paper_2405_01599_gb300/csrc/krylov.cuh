@@ -10,10 +10,11 @@ namespace xb {
 //   sc: 1/||w|| of each stored (unnormalised) basis vector (M+1)
 //   scf: the same scales in FP32 (for the FP32 basis)
 //   y: least-squares solution times the basis scales (M)
-//   coef: pending update coefficients of the block Gram-Schmidt passes (M+1)
+//   gram: inner products of basis row i with the earlier rows of its block of
+//   8, entries 8 i .. 8 i + 7 (the MGS correction terms)
 //   misc: named scalars (below)
 struct GmDev {
-    double *H, *cs, *sn, *g, *sc, *y, *coef, *misc;
+    double *H, *cs, *sn, *g, *sc, *y, *gram, *misc;
     float *scf;
     int M;
 };
@@ -29,7 +30,7 @@ enum GmMisc {
     GM_RAW = 8,     // 1: plain MGS sweep, keep column j unrotated (no Givens)
     GM_NMISC = 9
 };
-inline size_t gm_doubles(int M) { return (size_t)(M + 1) * M + 2 * (size_t)M + 3 * (size_t)(M + 1) + M + GM_NMISC + (M + 2) / 2 + 8; }
+inline size_t gm_doubles(int M) { return (size_t)(M + 1) * M + 2 * (size_t)M + 2 * (size_t)(M + 1) + M + 8 * (size_t)(M + 1) + GM_NMISC + (M + 2) / 2 + 8; }
 GmDev gm_layout(double *base, int M);
 
 // BiCGStab scalars (indices into a device double array).
@@ -37,19 +38,22 @@ enum BiScal {
     BI_RHO = 0, BI_RHO_OLD, BI_ALPHA, BI_OMEGA, BI_SNORM2, BI_RNORM2, BI_FLAG, BI_TAU2, BI_N
 };
 
-// ---- launchers (krylov.cu) ----
+// ---- launchers (krylov.cu, ortho.cu) ----
 int gm_cycle_init(xb_plan *p, GmDev st, int64_t n, const double *r0, double tau, cudaStream_t s);
-// MGS sweep of Arnoldi step j against basis rows V_0..V_j (row stride ld);
-// w holds A v_j on entry and the orthogonalised vector on exit.
-template <typename VB>
-int gm_mgs_step(xb_plan *p, GmDev st, int64_t n, const VB *V, int64_t ld, VB *w, int j,
-                cudaStream_t s);
 // Orthogonalisation of Arnoldi step j with XB_ORTHO_MGS / CGS / DGKS / BCGS
-// (the policy value is resolved by the caller); ends with h_{j+1,j} and the
-// Givens update like gm_mgs_step.
+// (the policy value is resolved by the caller) against basis rows V_0..V_j (row
+// stride ld): w holds A v_j on entry and the orthogonalised vector on exit;
+// ends with h_{j+1,j} and the Givens update, or in raw mode (GM_RAW) with the
+// plain column.  seen: steps 0..j-1 of this cycle went through here with the
+// same basis, so st.gram holds their rows' inner products.
 template <typename VB>
 int gm_ortho_step(xb_plan *p, GmDev st, int64_t n, const VB *V, int64_t ld, VB *w, int j,
-                  int ortho, cudaStream_t s);
+                  int ortho, bool seen, cudaStream_t s);
+// w against the k rows of V (unit scales); h: k coefficients, then ||w||.
+int ortho_sweep(xb_plan *p, int64_t n, int k, const double *V, int64_t ld, double *w, double *h,
+                int ortho, cudaStream_t s);
+// XB_ETIMEOUT if a grid exchange of an earlier, finished launch ran out of time.
+int gs_check(xb_plan *p);
 // Algorithmic vector passes (multiples of n elements read + written) of one
 // orthogonalisation of step j.
 double ortho_passes(int ortho, int j);

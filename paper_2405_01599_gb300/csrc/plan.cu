@@ -793,11 +793,12 @@ namespace xb {
 // Reduction scratch, pinned host mirror and timing events of a plan.
 int plan_scratch(xb_plan *p, cudaStream_t s) {
     cudaError_t e = cudaMalloc(&p->d_part, (size_t)kRedSlots * kRedValues * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&p->d_ticket, 64 * sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMalloc(&p->d_ticket, gs_scratch_bytes());
     if (e == cudaSuccess) e = cudaMalloc(&p->d_scal, (size_t)kScalars * sizeof(double));
-    if (e == cudaSuccess) e = cudaMemsetAsync(p->d_ticket, 0, 64 * sizeof(unsigned), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p->d_ticket, 0, gs_scratch_bytes(), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(p->d_scal, 0, (size_t)kScalars * sizeof(double), s);
     if (e == cudaSuccess) e = cudaMallocHost(&p->h_pin, 64 * sizeof(double));
+    if (e == cudaSuccess) std::memset(p->h_pin, 0, 64 * sizeof(double));
     if (e == cudaSuccess) e = cudaEventCreate(&p->ev[0]);
     if (e == cudaSuccess) e = cudaEventCreate(&p->ev[1]);
     return e == cudaSuccess ? XB_OK : cuda_error(e, "plan_create: scratch");

@@ -30,7 +30,7 @@ double secs_since(clk::time_point t0) {
 int peek(xb_plan *p, const double *dev, int cnt, cudaStream_t s) {
     XB_CUDA(cudaMemcpyAsync(p->h_pin, dev, cnt * sizeof(double), cudaMemcpyDeviceToHost, s));
     XB_CUDA(cudaStreamSynchronize(s));
-    return XB_OK;
+    return xb::gs_check(p);
 }
 
 int64_t ld_of(int64_t n) { return (n + 63) / 64 * 64; }
@@ -187,7 +187,7 @@ int gmres_fp64(xb_plan *p, const double *b, double *x, const xb_options &o, xb_i
             ac.bytes += spmv_b;
             ac.spmv++;
             XB_TRY(xb::gm_ortho_step<double>(p, st, n, V, ld, V + (size_t)(j + 1) * ld, j, ortho,
-                                             s));
+                                             true, s));
             ac.bytes += 8.0 * n * xb::ortho_passes(ortho, j);
             launched++;
             const bool last = (j == m - 1) || (iters + launched >= iter_budget);
@@ -275,7 +275,7 @@ int gmres_f32_inner(xb_plan *p, const float *r32, float *d, float *V, int64_t ld
             ac.bytes += spmv_b;
             ac.spmv++;
             XB_TRY(xb::gm_ortho_step<float>(p, st, n, V, ld, V + (size_t)(j + 1) * ld, j, ortho,
-                                            s));
+                                            true, s));
             ac.bytes += 4.0 * n * xb::ortho_passes(ortho, j);
             launched++;
             const bool last = (j == m - 1) || (*steps + launched >= maxit);

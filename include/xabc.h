@@ -536,19 +536,20 @@ int xb_dense_restart_basis(int32_t n, const double *A, int32_t which, int32_t k,
  * by level); general CRS only (XB_EINVAL for sym_upper plans).  A row without
  * a stored diagonal or a zero pivot gives XB_EBREAKDOWN. */
 int xb_ilu0_setup(xb_plan *plan, void *stream);
-/* z = (L U)^{-1} r: forward then backward substitution, one launch per
- * dependency level.  r and z: DEVICE, n doubles, distinct. */
+/* z = (L U)^{-1} r: forward then backward substitution.  r and z: DEVICE, n
+ * doubles, distinct. */
 int xb_ilu0_apply(xb_plan *plan, const double *r, double *z, void *stream);
-/* Which substitution path the plan's ILU(0) applications take, and the
- * persistent path's barrier poll limit (a control for tests and diagnosis).
- * mode: -1 = automatic (the default; the environment variable XB_ILU_MODE
- * = 0/1 overrides it), 0 = the captured graph of level launches, 1 = one
- * cooperative launch with a grid barrier between levels (used only when the
- * device supports cooperative launches).  barrier_polls: how many times a CTA
- * polls a level barrier before it gives up (0 = default, about 0.5 s of
- * polling); a CTA that gives up sets an error flag and returns, every other
- * CTA returns at its next barrier, and the apply or solve reports
- * XB_ETIMEOUT.  XB_EINVAL for mode outside -1..1 or barrier_polls < 0. */
+/* Which substitution path the plan's ILU(0) applications take, and the flow
+ * path's poll limit (a control for tests and diagnosis).  mode: -1 = automatic
+ * (the default; the environment variable XB_ILU_MODE = 0/1 overrides it), 0 =
+ * the captured graph of level launches (built when first taken), 1 = one
+ * cooperative launch in which every row waits for the values it needs (used
+ * only when the device supports cooperative launches and every pivot and its
+ * reciprocal lie well inside the FP64 range).  barrier_polls: how many times a
+ * warp polls for a value before it gives up (0 = default: 2 s and 2 us per
+ * dependency level); a warp that gives up sets an error flag and leaves, every
+ * other warp leaves at its next look at the flag, and the apply or solve
+ * reports XB_ETIMEOUT.  XB_EINVAL for mode outside -1..1 or barrier_polls < 0. */
 int xb_ilu0_config(xb_plan *plan, int32_t mode, int32_t barrier_polls);
 /* Copy the factors (aligned with the plan's col array: strict lower part = L
  * with unit diagonal not stored, the rest = U) to the DEVICE array lu (nnz). */

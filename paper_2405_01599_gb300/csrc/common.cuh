@@ -159,39 +159,36 @@ struct BssData {
 
 // ILU(0) preconditioner data (built on first use): factors in A's pattern
 // (strict lower part L with unit diagonal, the rest U), the diagonal
-// positions, and the rows grouped by dependency level for the forward (L)
-// and backward (U) substitutions: every row of a level depends only on rows
-// of earlier levels.
+// positions, and the layouts of the two substitution paths (ilu.cu).
 struct IluData {
     bool built = false;
     int status = 0;                  // XB_OK or XB_EBREAKDOWN (zero pivot)
     double *d_lu = nullptr;          // nnz
     int *d_dpos = nullptr;           // n
-    int *d_lrows = nullptr, *d_urows = nullptr;  // n each, ordered by level
-    std::vector<int> loff, uoff;     // level offsets (levels + 1)
-    // Inside a level rows are ordered by tier: short rows (<= 8 entries in the
-    // triangle) first, stored again level by level in ELL form (entry t of
-    // slot s at eoff[l] + t * count + s, padded with zero values) so a thread
-    // loads its row with no dependent index loads; then rows of up to 512
-    // entries (thread or warp per row, CSR); then longer rows (CTA per row).
-    std::vector<int> ln0, ln1, un0, un1;  // per level: ELL-tier and CSR-tier counts
-    std::vector<int> lw, uw;              // per level: ELL width
-    std::vector<long long> leoff, ueoff;  // per level: ELL base offset
-    int *d_lecol = nullptr, *d_uecol = nullptr;
-    double *d_leval = nullptr, *d_ueval = nullptr;
-    int *d_lesrc = nullptr, *d_uesrc = nullptr;  // factor position of each ELL entry (-1: pad)
-    double *d_udiag = nullptr;            // u_ii in backward level order
     int *d_flag = nullptr;           // zero-pivot flag
-    double *d_in = nullptr, *d_out = nullptr;  // fixed operands of the captured solve
-    cudaGraph_t graph = nullptr;     // both substitutions, every level, captured once
+    double *d_in = nullptr;          // n: copy of r when a path needs one
+    // flow path: a CTA per block of consecutive rows (bstart), its rows of each
+    // triangle in level order, cut into items
+    struct Flow {
+        void *d_items = nullptr;
+        int *d_iptr = nullptr, *d_rows = nullptr, *d_ecol = nullptr;
+        long long *d_ebase = nullptr;
+        double *d_eval = nullptr, *d_diag = nullptr, *d_rdiag = nullptr;
+    } fl, fu;
+    int *d_bstart = nullptr;
+    void *d_ty = nullptr, *d_tz = nullptr;  // published values, 16 B a row
+    int *d_stop = nullptr;           // a wait ran out
+    int grid = 0, maxrows = 0, cap = 0;
+    unsigned seq = 0;                // number of the last application
+    unsigned long long limit_ns = 0;
+    // graph path (built when first taken): inside a level rows are ordered by
+    // tier, short rows (<= 8 entries in the triangle) first and stored again
+    // level by level in ELL form, then rows of up to 512 entries (thread or warp
+    // per row, CSR), then longer rows (CTA per row)
+    int *d_lrows = nullptr, *d_urows = nullptr, *d_lecol = nullptr, *d_uecol = nullptr;
+    double *d_leval = nullptr, *d_ueval = nullptr, *d_udiag = nullptr, *d_out = nullptr;
+    cudaGraph_t graph = nullptr;     // both substitutions, every level
     cudaGraphExec_t exec = nullptr;
-    // persistent substitution (one cooperative launch, a bounded grid barrier
-    // between levels): level tables on the device, barrier state, error flag
-    int *d_lmeta = nullptr, *d_umeta = nullptr;        // per level: off, n0, n1, w
-    long long *d_leo = nullptr, *d_ueo = nullptr;      // per level: ELL base offset
-    unsigned *d_bar = nullptr;                          // count, generation
-    int *d_err = nullptr;                               // 1: a barrier wait ran out
-    int pgrid = 0;                                      // CTAs of the persistent launch
 };
 
 }  // namespace xb
@@ -221,8 +218,8 @@ struct xb_plan {
     std::vector<xb::SellPart> sells;     // cache by sigma
     xb::BssData bss;
     xb::IluData ilu;
-    int ilu_mode = -1;                   // substitution path: -1 auto, 0 graph, 1 persistent
-    int ilu_polls = 0;                   // persistent barrier poll limit (0: default)
+    int ilu_mode = -1;                   // substitution path: -1 auto, 0 graph, 1 flow
+    int ilu_polls = 0;                   // polls of one wait of the flow path (0: default)
     bool vec_ok = false;                 // val and col 16-byte aligned
     // reduction scratch
     double *d_part = nullptr;            // kRedSlots * kRedValues partials

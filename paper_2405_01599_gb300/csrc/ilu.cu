@@ -4,24 +4,20 @@
 //
 // Setup: the host derives, from the pattern alone, the dependency level of
 // every row for the forward substitution (level(i) = 1 + max level(k) over the
-// stored k < i in row i) and for the backward one (over the stored j > i); rows
-// are grouped by level.  The numeric factorization then runs level by level on
-// the device, one warp per row: for each stored (i, k), k < i, in ascending k,
-// l_ik = a_ik / u_kk, and every stored (i, j), j > k, subtracts l_ik u_kj when
-// (k, j) is stored (binary search in row k, which an earlier level finished).
-// Each substitution is one launch per level; inside a level every row is
-// independent: a thread per row, with rows longer than 32 stored entries in
-// the triangle taken by the whole warp (lanes stride over the row, shuffle
-// reduction), and rows longer than kLongRow by a whole CTA, so a power-law row
-// does not serialise one thread or one warp.  The launch sequence of both
-// substitutions is captured once into a CUDA graph on fixed operand buffers
-// (a 3D stencil has 3N - 2 levels per triangle, so per-launch overhead would
-// otherwise dominate).
+// stored k < i in row i) and for the backward one (over the stored j > i).  The
+// numeric factorization runs level by level on the device, one warp per row:
+// for each stored (i, k), k < i, in ascending k, l_ik = a_ik / u_kk, and every
+// stored (i, j), j > k, subtracts l_ik u_kj when (k, j) is stored (binary search
+// in row k, which an earlier level finished).  Both substitutions run in one
+// launch in which rows wait for the values they need (the flow path), or as one
+// kernel per level and row tier, captured once in a CUDA graph (the graph path).
 #include "common.cuh"
 
 #include <algorithm>
+#include <climits>
 #include <cstdlib>
 #include <cmath>
+#include <thread>
 
 namespace {
 
@@ -169,141 +165,301 @@ __global__ void k_ell_fill(long long cnt, const int *__restrict__ src,
     if (e < cnt) val[e] = src[e] >= 0 ? lu[src[e]] : 0.0;
 }
 __global__ void k_diag_fill(int n, const int *__restrict__ rows, const int *__restrict__ dpos,
-                            const double *__restrict__ lu, double *__restrict__ diag) {
+                            const double *__restrict__ lu, double *__restrict__ diag,
+                            double *__restrict__ rdiag, int *__restrict__ odd) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < n) diag[s] = lu[dpos[rows[s]]];
+    if (s >= n) return;
+    const double d = lu[dpos[rows[s]]];
+    diag[s] = d;
+    if (rdiag) {
+        rdiag[s] = 1.0 / d;
+        if (!(fabs(d) > 1e-280 && fabs(d) < 1e280)) *odd = 1;  // d and 1 / d in the normal range?
+    }
 }
 
-// ---- persistent substitution ---------------------------------------------------
-// Both substitutions in one cooperative launch (every CTA resident, one per
-// SM): each level is processed by the whole grid, then a grid barrier.  The
-// barrier is a counter and a generation word in global memory; a CTA that
-// waits longer than `polls` polls (kernel argument; default kBarSpins) sets
-// the error flag and leaves, so every wait is bounded, and every CTA then
-// leaves at its next barrier too.  Values of z written by other CTAs are read
-// at L2.
-constexpr unsigned kBarSpins = 1u << 20;  // polls of ~0.5 us: a wait gives up after ~0.5 s
+// ---- flow substitution ---------------------------------------------------------
+// Both substitutions in one cooperative launch without barriers between
+// levels.  CTA c owns a block of consecutive rows, in both triangles, and takes
+// its rows in level order as items: up to 32 rows of one level (a lane each),
+// or one long row (the warp).  A row's value is published as soon as it is
+// formed and a row waits for the very values it needs: those of the CTA's own
+// rows in shared memory, the others in device memory, where a value travels as
+// two 8-byte words that both carry the number of the application (so nothing
+// is reset between applications and no fence is needed).
+//
+// What bounds it: the longest chain of rows, one hop per level.  A hop through
+// shared memory takes 0.4 us (an FP64 FMA alone 0.1), one through device memory
+// 1.0 us and, with every CTA waiting on others, up to 2; the level barrier this
+// replaces took ~6 us and a kernel per level ~4 us.  Consecutive rows per CTA
+// keep most hops of a stencil inside a CTA.  One application (GB300; the graph
+// of level launches or the level barrier, whichever was faster, in brackets):
+// 96^3 convection-diffusion 0.71 ms (2.0), 30^3 0.13 (0.44), 180^3 (blocks too
+// large for shared memory) 3.8 (4.3), power-law rows n = 20,000 0.46 (1.1), n =
+// 1M 1.03 (3.4).
+//
+// Every wait ends: warps take a CTA's items in level order, so of the rows not
+// yet done in the whole grid those of the lowest level wait for nothing; and a
+// wait is bounded all the same (`polls` polls, or `limit` ns): then the kernel
+// sets the error flag and every warp leaves at its next poll.
+constexpr int kFlowWarps = 16;
+constexpr int kFlowMinRows = 2048;  // rows of a CTA below which fewer CTAs do (30^3 grid: 122 us
+                                    // with 2048, 140 with 1024, 170 with 512)
+constexpr int kFlowShort = 32;   // triangle entries above which a row gets a warp
+constexpr int kFlowFirst = 4;    // entries of each kind a row starts with
+constexpr int kFlowGroup = 8;    // further remote entries loaded together
+constexpr unsigned long long kNotReady = 0xffffffffffffffffull;  // a NaN that is never stored
 
-struct TriDev {
-    int nlev;
-    const int *meta;        // per level: off, n0, n1, w (4 ints)
-    const long long *eoff;  // per level: ELL base offset
-    const int *rows, *ecol;
-    const double *eval, *diag;
+struct FlowTri {
+    const int4 *items;      // {first slot, rows | long << 8, remote | local entries << 16, entries from ebase}
+    const int *iptr;        // per CTA: its items
+    const long long *ebase; // per CTA: its entries
+    const int *rows;        // slot -> row
+    const int *ecol;        // remote: column; local: row of the block; -1: none
+    const double *eval;
+    const double *diag, *rdiag;  // by slot (backward): pivot and its reciprocal
+};
+struct FlowArgs {
+    FlowTri L, U;
+    const int *bstart;      // per CTA: first row
+    const int *rp, *ci, *dpos;
+    const double *lu, *r;
+    double *z;
+    ulonglong2 *ty, *tz;    // published values of the two substitutions
+    unsigned seq, polls, look;  // polls of one wait (0: the clock decides); polls between looks
+    unsigned long long limit;
+    volatile int *err;      // host-visible
+    int *stop;              // the same for the grid
+    int cap;                // rows whose values shared memory holds
 };
 
-__device__ __forceinline__ bool grid_bar(unsigned *bar, int *err, unsigned polls) {
-    __syncthreads();
-    __shared__ int ok;
-    if (threadIdx.x == 0) {
-        volatile unsigned *gen = bar + 1;
-        const unsigned g = *gen;
-        __threadfence();
-        if (atomicAdd(bar, 1u) == gridDim.x - 1) {
-            bar[0] = 0u;
-            __threadfence();
-            atomicAdd(bar + 1, 1u);
-            ok = 1;
-        } else {
-            unsigned it = 0;
-            while (*gen == g && ++it < polls) {
-            }
-            ok = (*gen != g);
-            if (!ok) atomicExch(err, 1);
+__device__ __forceinline__ void flow_put(ulonglong2 *p, double v, unsigned seq) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const unsigned long long s = (unsigned long long)seq << 32;
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(s | (b & 0xffffffffu)),
+                 "l"(s | (b >> 32)) : "memory");
+}
+__device__ __forceinline__ bool flow_get(const ulonglong2 *p, unsigned seq, double &v) {
+    unsigned long long x, y;
+    asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "l"(p) : "memory");
+    v = __longlong_as_double((long long)((x & 0xffffffffu) | (y << 32)));
+    return (unsigned)(x >> 32) == seq && (unsigned)(y >> 32) == seq;
+}
+
+__device__ __forceinline__ void flow_fail(const FlowArgs &a) {
+    *reinterpret_cast<volatile int *>(a.stop) = 1;
+    *a.err = 1;
+}
+// A warp's patience with one wait: false once it has run out.  Between looks at
+// the clock and the grid's flag a poll costs one add.
+struct FlowWait {
+    unsigned it = 0;
+    unsigned long long t0 = 0;
+    __device__ __forceinline__ bool more(const FlowArgs &a) {
+        if (++it < a.look) return true;
+        if (a.polls == 0) {
+            unsigned long long now;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+            if (t0 == 0) t0 = now;
+            it = 0;
+            if (now - t0 <= a.limit && *reinterpret_cast<volatile int *>(a.stop) == 0) return true;
         }
-        __threadfence();
+        flow_fail(a);
+        return false;
     }
-    __syncthreads();
-    return ok;
+};
+
+// x / d with d's reciprocal (both in the normal range): one correction step, as
+// accurate as the division and a quarter of its latency.
+__device__ __forceinline__ double flow_quot(double x, double d, double rd) {
+    const double q = x * rd, c = fma(fma(-q, d, x), rd, q);
+    // an infinite x or quotient stays one (a NaN c: exponent and a fraction bit)
+    return ((unsigned)__double2hiint(c) & 0x7fffffffu) > 0x7ff00000u ? q : c;
+}
+
+__device__ __forceinline__ bool flow_ready(double x) {
+    return __double2hiint(x) != -1;  // kNotReady's high word; no value that is stored has it
+}
+
+// s + the sum of the item's m <= kFlowFirst local entries; false when a wait ran
+// out (warp-uniform, as all below).  The first entry is polled alone: a warp
+// that waits reads one word a poll and leaves the shared memory to the others.
+__device__ __forceinline__ bool flow_local(const FlowArgs &a, const volatile double *zs, int m,
+                                           const int (&c)[kFlowFirst], const double (&v)[kFlowFirst],
+                                           double &s) {
+    FlowWait w;
+    double x[kFlowFirst];
+    while (x[0] = zs[c[0]], !__all_sync(0xffffffffu, flow_ready(x[0])))
+        if (!w.more(a)) return false;
+    if (m > 1) {
+        for (;;) {
+            bool all = true;
+#pragma unroll
+            for (int q = 1; q < kFlowFirst; q++)
+                if (q < m) {
+                    x[q] = zs[c[q]];
+                    all = all && flow_ready(x[q]);
+                }
+            if (__all_sync(0xffffffffu, all)) break;
+            if (!w.more(a)) return false;
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < kFlowFirst; q++)
+        if (q < m) s = fma(v[q], x[q], s);
+    return true;
+}
+
+// The same for values in device memory (c < 0: none).
+template <int N>
+__device__ __forceinline__ bool flow_remote(const FlowArgs &a, const ulonglong2 *tag, const int (&c)[N],
+                                            const double (&v)[N], double &s) {
+    FlowWait w;
+    double x[N];
+    bool miss[N];
+#pragma unroll
+    for (int q = 0; q < N; q++) {
+        x[q] = 0.0;
+        miss[q] = c[q] >= 0;
+    }
+    for (;;) {
+        bool any = false;
+#pragma unroll
+        for (int q = 0; q < N; q++)
+            if (miss[q]) miss[q] = !flow_get(tag + c[q], a.seq, x[q]);
+#pragma unroll
+        for (int q = 0; q < N; q++) any = any || miss[q];
+        if (!__any_sync(0xffffffffu, any)) break;
+        if (!w.more(a)) return false;
+    }
+#pragma unroll
+    for (int q = 0; q < N; q++)
+        if (c[q] >= 0) s = fma(v[q], x[q], s);
+    return true;
 }
 
 template <bool FWD>
-__device__ void persist_level(const TriDev &t, int l, const int *__restrict__ rp,
-                              const int *__restrict__ ci, const int *__restrict__ dpos,
-                              const double *__restrict__ lu, const double *__restrict__ r,
-                              double *z, double *sh) {
-    const int off = t.meta[4 * l], c0 = t.meta[4 * l + 1], c1 = t.meta[4 * l + 2];
-    const int w = t.meta[4 * l + 3];
-    const int c2 = t.meta[4 * (l + 1)] - off - c0 - c1;
-    const int gt = blockIdx.x * blockDim.x + threadIdx.x, gs = gridDim.x * blockDim.x;
-    // ELL tier: a thread per row
-    const long long eo = t.eoff[l];
-    for (int slot = gt; slot < c0; slot += gs) {
-        const int i = t.rows[off + slot];
-        double s = 0.0;
-        for (int q = 0; q < w; q++) {
-            const long long e = eo + (long long)q * c0 + slot;
-            s = fma(__ldg(t.eval + e), __ldcg(z + __ldg(t.ecol + e)), s);
-        }
-        if (FWD) z[i] = __ldg(r + i) - s;
-        else z[i] = (__ldcg(z + i) - s) / __ldg(t.diag + off + slot);
-    }
-    // CSR tier: thread per row, warp for rows over 32 entries
-    const int lane = threadIdx.x & 31, wi = gt >> 5, nw = gs >> 5;
-    for (int base = wi * 32; base < c1; base += nw * 32) {  // warp-uniform
-        const int slot = base + lane;
-        int i = -1, ka = 0, kb = 0;
-        if (slot < c1) {
-            i = t.rows[off + c0 + slot];
-            const int d = dpos[i];
-            ka = FWD ? rp[i] : d + 1;
-            kb = FWD ? d : rp[i + 1];
-        }
-        const bool lng = kb - ka > 32;
-        double s = 0.0;
-        if (!lng)
-            for (int k = ka; k < kb; k++) s = fma(__ldg(lu + k), __ldcg(z + __ldg(ci + k)), s);
-        unsigned todo = __ballot_sync(0xffffffffu, lng);
-        while (todo) {
-            const int src = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const int la = __shfl_sync(0xffffffffu, ka, src);
-            const int lb = __shfl_sync(0xffffffffu, kb, src);
-            double v = 0.0;
-            for (int k = la + lane; k < lb; k += 32)
-                v = fma(__ldg(lu + k), __ldcg(z + __ldg(ci + k)), v);
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == src) s = v;
-        }
-        if (i >= 0) {
-            if (FWD) z[i] = __ldg(r + i) - s;
-            else z[i] = (__ldcg(z + i) - s) / lu[dpos[i]];
+__device__ __forceinline__ bool flow_item(const FlowArgs &a, const FlowTri &t, int4 it, long long ebase,
+                                          int r0, int nr, double *zs, bool held, int lane) {
+    const int cnt = it.y & 0xff, gw = it.z & 0xffff, lw = it.z >> 16;
+    ulonglong2 *tag = FWD ? a.ty : a.tz;
+    int row = -1;
+    double s = 0.0, b = 0.0, d = 1.0, rd = 1.0;
+    if (lane < cnt) {
+        row = __ldg(t.rows + it.x + lane);
+        if (FWD) {
+            b = __ldg(a.r + row);
+        } else {
+            flow_get(a.ty + row, a.seq, b);  // this CTA's, complete since its barrier
+            d = __ldg(t.diag + it.x + lane);
+            rd = __ldg(t.rdiag + it.x + lane);
         }
     }
-    // long rows: a CTA per row (the loop bound is uniform over the CTA)
-    for (int q = blockIdx.x; q < c2; q += gridDim.x) {
-        const int i = t.rows[off + c0 + c1 + q];
-        const int d = dpos[i];
-        const int ka = FWD ? rp[i] : d + 1, kb = FWD ? d : rp[i + 1];
-        double v = 0.0;
-        for (int k = ka + threadIdx.x; k < kb; k += blockDim.x)
-            v = fma(__ldg(lu + k), __ldcg(z + __ldg(ci + k)), v);
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) sh[threadIdx.x >> 5] = v;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double sum = 0.0;
-            for (int k = 0; k < (int)(blockDim.x >> 5); k++) sum += sh[k];
-            if (FWD) z[i] = __ldg(r + i) - sum;
-            else z[i] = (__ldcg(z + i) - sum) / lu[d];
+    int k0 = 0, k1 = gw, step = kFlowGroup;
+    const bool lng = it.y & 256;
+    const long long e = ebase + it.w + lane;
+    int cl[kFlowFirst];
+    double vl[kFlowFirst];
+    if (lng) {  // the lanes take the row's entries in turn
+        const int i = __shfl_sync(0xffffffffu, row, 0), dp = __ldg(a.dpos + i);
+        k0 = FWD ? __ldg(a.rp + i) : dp + 1;
+        k1 = FWD ? dp : __ldg(a.rp + i + 1);
+        step = 32 * kFlowGroup;
+    } else {
+        // the first entries of both kinds, on their way before the first wait
+        int c[kFlowFirst];
+        double v[kFlowFirst];
+#pragma unroll
+        for (int q = 0; q < kFlowFirst; q++) {
+            const bool in = q < gw && lane < cnt;
+            c[q] = in ? __ldg(t.ecol + e + q * cnt) : -1;
+            v[q] = in ? __ldg(t.eval + e + q * cnt) : 0.0;
         }
-        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kFlowFirst; q++) {
+            const bool in = q < lw && lane < cnt;
+            cl[q] = in ? __ldg(t.ecol + e + (gw + q) * cnt) : -1;
+            vl[q] = in ? __ldg(t.eval + e + (gw + q) * cnt) : 0.0;
+            if (cl[q] < 0) cl[q] = nr;  // zs[nr] is 0, and ready
+        }
+        if (gw > 0 && !flow_remote<kFlowFirst>(a, tag, c, v, s)) return false;
+        k0 = kFlowFirst;
+    }
+    for (int k = k0; k < k1; k += step) {  // warp-uniform: further remote entries
+        int c[kFlowGroup];
+        double v[kFlowGroup];
+#pragma unroll
+        for (int q = 0; q < kFlowGroup; q++) {
+            const int at = lng ? k + q * 32 + lane : k + q;
+            const bool in = at < k1 && (lng || lane < cnt);
+            const long long p = lng ? at : e + (long long)at * cnt;
+            c[q] = in ? __ldg((lng ? a.ci : t.ecol) + p) : -1;
+            v[q] = in ? __ldg((lng ? a.lu : t.eval) + p) : 0.0;
+        }
+        if (!flow_remote<kFlowGroup>(a, tag, c, v, s)) return false;
+    }
+    if (lng) {
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    }
+    for (int t0 = 0; t0 < lw; t0 += kFlowFirst) {
+        if (t0 > 0) {
+#pragma unroll
+            for (int q = 0; q < kFlowFirst; q++) {
+                const bool in = t0 + q < lw && lane < cnt;
+                cl[q] = in ? __ldg(t.ecol + e + (long long)(gw + t0 + q) * cnt) : -1;
+                vl[q] = in ? __ldg(t.eval + e + (long long)(gw + t0 + q) * cnt) : 0.0;
+                if (cl[q] < 0) cl[q] = nr;
+            }
+        }
+        if (!flow_local(a, zs, min(kFlowFirst, lw - t0), cl, vl, s)) return false;
+    }
+    if (row >= 0) {
+        s = b - s;  // one rounding at the size of b, however many entries
+        if (!FWD) s = flow_quot(s, d, rd);
+        if (!flow_ready(s)) s = nan("");
+        if (held) *reinterpret_cast<volatile double *>(zs + (row - r0)) = s;
+        flow_put(tag + row, s, a.seq);
+        if (!FWD) a.z[row] = s;
+    }
+    return true;
+}
+
+template <bool FWD>
+__device__ void flow_pass(const FlowArgs &a, const FlowTri &t, double *zs, bool held, int nr, int *ticket) {
+    const int lane = threadIdx.x & 31, r0 = a.bstart[blockIdx.x];
+    const int i0 = t.iptr[blockIdx.x], ni = t.iptr[blockIdx.x + 1] - i0;
+    const long long ebase = t.ebase[blockIdx.x];
+    auto take = [&]() {
+        int q = 0;
+        if (lane == 0) q = atomicAdd(ticket, 1);
+        return __shfl_sync(0xffffffffu, q, 0);
+    };
+    // the next item is known while this one waits for its values
+    int q = take();
+    int4 it = q < ni ? __ldg(t.items + i0 + q) : make_int4(0, 0, 0, 0);
+    while (q < ni) {
+        const int qn = take();
+        const int4 nx = qn < ni ? __ldg(t.items + i0 + qn) : make_int4(0, 0, 0, 0);
+        if (!flow_item<FWD>(a, t, it, ebase, r0, nr, zs, held, lane)) return;
+        q = qn;
+        it = nx;
     }
 }
 
-__global__ void __launch_bounds__(512, 1) k_ilu_persist(TriDev L, TriDev U, const int *rp,
-                                                     const int *ci, const int *dpos,
-                                                     const double *lu, const double *r,
-                                                     double *z, unsigned *bar, int *err,
-                                                     unsigned polls) {
-    __shared__ double sh[16];
-    for (int l = 0; l < L.nlev; l++) {
-        persist_level<true>(L, l, rp, ci, dpos, lu, r, z, sh);
-        if (!grid_bar(bar, err, polls)) return;
-    }
-    for (int l = 0; l < U.nlev; l++) {
-        persist_level<false>(U, l, rp, ci, dpos, lu, r, z, sh);
-        if (l + 1 < U.nlev && !grid_bar(bar, err, polls)) return;
+__global__ void __launch_bounds__(32 * kFlowWarps, 1) k_ilu_flow(const __grid_constant__ FlowArgs a) {
+    extern __shared__ double zs[];
+    __shared__ int ticket[2];
+    const int nr = a.bstart[blockIdx.x + 1] - a.bstart[blockIdx.x];
+    const bool held = nr <= a.cap;
+    if (threadIdx.x < 2) ticket[threadIdx.x] = 0;
+    for (int p = 0; p < 2; p++) {
+        if (held)
+            for (int i = threadIdx.x; i < nr; i += blockDim.x)
+                zs[i] = __longlong_as_double((long long)kNotReady);
+        if (held && threadIdx.x == 0) zs[nr] = 0.0;  // what the missing entries of an item read
+        __syncthreads();
+        if (p == 0) flow_pass<true>(a, a.L, zs, held, nr, &ticket[0]);
+        else flow_pass<false>(a, a.U, zs, held, nr, &ticket[1]);
+        __syncthreads();
     }
 }
 
@@ -371,6 +527,161 @@ void build_ell(const std::vector<int> &rows, const std::vector<int> &off,
         }
 }
 
+// Rows in level order, ascending inside a level.
+void level_order(const std::vector<int> &lev, int nlev, std::vector<int> &rows, std::vector<int> &off) {
+    const int n = (int)lev.size();
+    off.assign(nlev + 1, 0);
+    for (int i = 0; i < n; i++) off[lev[i] + 1]++;
+    for (int l = 0; l < nlev; l++) off[l + 1] += off[l];
+    rows.resize(n);
+    std::vector<int> at(off.begin(), off.end() - 1);
+    for (int i = 0; i < n; i++) rows[at[lev[i]]++] = i;
+}
+
+// The flow substitution's layout of one triangle (FlowTri): every block's rows
+// in level order, cut into items.  The entries of row i are positions
+// [beg(i), end(i)) of the CRS arrays; blocks of more than cap rows have no
+// local entries.
+struct FlowHost {
+    std::vector<int4> items;
+    std::vector<int> iptr, rows, ecol, esrc;
+    std::vector<long long> ebase;
+};
+// Blocks [c0, c1) appended to h (their rows go to rows[bstart[c]..]).
+template <typename Beg, typename End>
+void flow_blocks(const std::vector<int> &lev, const std::vector<int> &bstart, int c0, int c1, int cap,
+                 const int *ci, Beg beg, End end, int *rows, FlowHost &h) {
+    std::vector<int> lng, shrt, cnt, order;
+    for (int c = c0; c < c1; c++) {
+        const int r0 = bstart[c], r1 = bstart[c + 1], nr = r1 - r0;
+        const bool held = nr <= cap;
+        int lo = nr > 0 ? lev[r0] : 0, hi = lo;
+        for (int i = r0; i < r1; i++) {
+            lo = std::min(lo, lev[i]);
+            hi = std::max(hi, lev[i]);
+        }
+        order.resize(nr);
+        if (hi - lo < 4 * nr + 64) {  // counting sort by level
+            cnt.assign(hi - lo + 2, 0);
+            for (int i = r0; i < r1; i++) cnt[lev[i] - lo + 1]++;
+            for (int l = 0; l <= hi - lo; l++) cnt[l + 1] += cnt[l];
+            for (int i = r0; i < r1; i++) order[cnt[lev[i] - lo]++] = i;
+        } else {
+            for (int i = 0; i < nr; i++) order[i] = r0 + i;
+            std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return lev[x] < lev[y]; });
+        }
+        const size_t ebase = h.ecol.size();
+        for (int a = 0; a < nr;) {  // one level
+            int b = a, least = INT_MAX, most = 0;
+            shrt.clear();
+            lng.clear();
+            for (; b < nr && lev[order[b]] == lev[order[a]]; b++) {
+                const int len = end(order[b]) - beg(order[b]);
+                if (len > kFlowShort) {
+                    lng.push_back(order[b]);
+                } else {
+                    shrt.push_back(order[b]);
+                    least = std::min(least, len);
+                    most = std::max(most, len);
+                }
+            }
+            // long rows first: they take longest
+            for (size_t q = 0; q < lng.size(); q++) {
+                rows[r0 + a + q] = lng[q];
+                h.items.push_back(make_int4(r0 + a + (int)q, 1 | 256, 0, 0));
+            }
+            a += (int)lng.size();
+            // rows of about equal length share an item
+            if (most > least && shrt.size() > 32)
+                std::stable_sort(shrt.begin(), shrt.end(),
+                                 [&](int x, int y) { return end(x) - beg(x) < end(y) - beg(y); });
+            for (size_t q0 = 0; q0 < shrt.size(); q0 += 32) {
+                const int m = (int)std::min<size_t>(32, shrt.size() - q0);
+                int gw = 0, lw = 0;
+                for (int q = 0; q < m; q++) {
+                    const int i = shrt[q0 + q], kb = end(i);
+                    rows[r0 + a + q] = i;
+                    int l = 0;
+                    for (int k = beg(i); k < kb; k++) l += held && ci[k] >= r0 && ci[k] < r1;
+                    gw = std::max(gw, kb - beg(i) - l);
+                    lw = std::max(lw, l);
+                }
+                const size_t e = h.ecol.size();
+                h.ecol.resize(e + (size_t)(gw + lw) * m, -1);
+                h.esrc.resize(e + (size_t)(gw + lw) * m, -1);
+                int *ec = h.ecol.data() + e, *es = h.esrc.data() + e;
+                for (int q = 0; q < m; q++) {
+                    const int i = shrt[q0 + q], kb = end(i);
+                    int g = 0, l = gw;
+                    for (int k = beg(i); k < kb; k++) {
+                        const bool in = held && ci[k] >= r0 && ci[k] < r1;
+                        const int at = (in ? l++ : g++) * m + q;
+                        ec[at] = in ? ci[k] - r0 : ci[k];
+                        es[at] = k;
+                    }
+                }
+                h.items.push_back(make_int4(r0 + a, m, gw | lw << 16, (int)(e - ebase)));
+                a += m;
+            }
+        }
+        h.iptr.push_back((int)h.items.size());
+        h.ebase.push_back((long long)h.ecol.size());
+    }
+}
+// Every block, by several host threads when there are many rows; false when
+// memory ran out.
+template <typename Beg, typename End>
+bool flow_layout(const std::vector<int> &lev, const std::vector<int> &bstart, int cap, const int *ci,
+                 Beg beg, End end, FlowHost &h) {
+    const int n = (int)lev.size(), G = (int)bstart.size() - 1;
+    const int T = n < 100000 ? 1 : std::min({G, 8, std::max(1, (int)std::thread::hardware_concurrency())});
+    std::vector<FlowHost> part(T);
+    std::vector<char> ok(T, 0);
+    h.rows.resize(n);
+    auto work = [&](int t) {
+        try {
+            const int c0 = (int)((long long)G * t / T), c1 = (int)((long long)G * (t + 1) / T);
+            const size_t guess = (size_t)(bstart[c1] - bstart[c0]) * 4;
+            part[t].ecol.reserve(guess);
+            part[t].esrc.reserve(guess);
+            flow_blocks(lev, bstart, c0, c1, cap, ci, beg, end, h.rows.data(), part[t]);
+            ok[t] = 1;
+        } catch (...) {
+        }
+    };
+    std::vector<std::thread> pool;
+    for (int t = 1; t < T; t++) {
+        try {
+            pool.emplace_back(work, t);
+        } catch (...) {
+            work(t);
+        }
+    }
+    work(0);
+    for (auto &p : pool) p.join();
+    size_t ni = 0, ne = 0;
+    for (int t = 0; t < T; t++) {
+        if (!ok[t]) return false;
+        ni += part[t].items.size();
+        ne += part[t].ecol.size();
+    }
+    h.items.reserve(ni);
+    h.ecol.reserve(ne);
+    h.esrc.reserve(ne);
+    h.iptr.assign(1, 0);
+    h.ebase.assign(1, 0);
+    for (const FlowHost &p : part) {
+        const int i0 = (int)h.items.size();
+        const long long e0 = (long long)h.ecol.size();
+        for (int v : p.iptr) h.iptr.push_back(i0 + v);
+        for (long long v : p.ebase) h.ebase.push_back(e0 + v);
+        h.items.insert(h.items.end(), p.items.begin(), p.items.end());
+        h.ecol.insert(h.ecol.end(), p.ecol.begin(), p.ecol.end());
+        h.esrc.insert(h.esrc.end(), p.esrc.begin(), p.esrc.end());
+    }
+    return true;
+}
+
 // Launch one substitution's levels on stream s (also used inside the capture).
 template <bool FWD>
 void launch_levels(const xb_plan *p, const int *d_rows, const std::vector<int> &off,
@@ -401,28 +712,17 @@ namespace xb {
 
 void ilu_free(xb_plan *p) {
     IluData &u = p->ilu;
-    cudaFree(u.d_lu);
-    cudaFree(u.d_dpos);
-    cudaFree(u.d_lrows);
-    cudaFree(u.d_urows);
-    cudaFree(u.d_flag);
-    cudaFree(u.d_in);
-    cudaFree(u.d_out);
-    cudaFree(u.d_lecol);
-    cudaFree(u.d_uecol);
-    cudaFree(u.d_leval);
-    cudaFree(u.d_ueval);
-    cudaFree(u.d_lesrc);
-    cudaFree(u.d_uesrc);
-    cudaFree(u.d_udiag);
+    for (void *d : {(void *)u.d_lu, (void *)u.d_dpos, (void *)u.d_flag, (void *)u.d_in, (void *)u.d_out,
+                    (void *)u.d_bstart, (void *)u.d_ty, (void *)u.d_tz, (void *)u.d_stop,
+                    (void *)u.d_lrows, (void *)u.d_urows, (void *)u.d_lecol, (void *)u.d_uecol,
+                    (void *)u.d_leval, (void *)u.d_ueval, (void *)u.d_udiag})
+        cudaFree(d);
+    for (IluData::Flow *f : {&u.fl, &u.fu})
+        for (void *d : {(void *)f->d_items, (void *)f->d_iptr, (void *)f->d_ebase, (void *)f->d_rows,
+                        (void *)f->d_ecol, (void *)f->d_eval, (void *)f->d_diag, (void *)f->d_rdiag})
+            cudaFree(d);
     if (u.exec) cudaGraphExecDestroy(u.exec);
     if (u.graph) cudaGraphDestroy(u.graph);
-    cudaFree(u.d_lmeta);
-    cudaFree(u.d_umeta);
-    cudaFree(u.d_leo);
-    cudaFree(u.d_ueo);
-    cudaFree(u.d_bar);
-    cudaFree(u.d_err);
     u = IluData();
 }
 
@@ -454,6 +754,108 @@ int ilu_levels(int n, const int *rp, const int *ci, std::vector<int> &dpos, std:
     return XB_OK;
 }
 
+namespace {
+
+int upload(int **d, const std::vector<int> &h, cudaStream_t s) {
+    XB_CUDA(cudaMalloc(d, std::max<size_t>(1, h.size()) * 4));
+    if (!h.empty()) XB_CUDA(cudaMemcpyAsync(*d, h.data(), h.size() * 4, cudaMemcpyHostToDevice, s));
+    return XB_OK;
+}
+
+// ELL values of a layout's entries from the factors.
+int fill_entries(double **val, const std::vector<int> &src, const double *lu, cudaStream_t s) {
+    int *d_src = nullptr;
+    XB_CUDA(cudaMalloc(val, std::max<size_t>(1, src.size()) * sizeof(double)));
+    XB_TRY(upload(&d_src, src, s));
+    if (!src.empty()) {
+        k_ell_fill<<<(unsigned)((src.size() + 255) / 256), 256, 0, s>>>((long long)src.size(), d_src, lu, *val);
+        XB_LAUNCHED("k_ell_fill");
+    }
+    cudaFree(d_src);  // waits for the kernel
+    return XB_OK;
+}
+
+int upload_flow(IluData::Flow &f, const FlowHost &h, const double *lu, cudaStream_t s) {
+    static_assert(sizeof(int4) == 16 && sizeof(long long) == 8, "layout");
+    XB_CUDA(cudaMalloc(&f.d_items, std::max<size_t>(1, h.items.size()) * sizeof(int4)));
+    XB_CUDA(cudaMemcpyAsync(f.d_items, h.items.data(), h.items.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
+    XB_CUDA(cudaMalloc(&f.d_ebase, h.ebase.size() * sizeof(long long)));
+    XB_CUDA(cudaMemcpyAsync(f.d_ebase, h.ebase.data(), h.ebase.size() * sizeof(long long),
+                            cudaMemcpyHostToDevice, s));
+    XB_TRY(upload(&f.d_iptr, h.iptr, s));
+    XB_TRY(upload(&f.d_rows, h.rows, s));
+    XB_TRY(upload(&f.d_ecol, h.ecol, s));
+    return fill_entries(&f.d_eval, h.esrc, lu, s);
+}
+
+int rows_host(xb_plan *p, std::vector<int> &ci) {
+    ci.resize(p->nnz);
+    if (p->nnz > 0) XB_CUDA(cudaMemcpy(ci.data(), p->col, (size_t)p->nnz * 4, cudaMemcpyDeviceToHost));
+    return XB_OK;
+}
+
+// The level launches of both substitutions (path 0), captured once: built when
+// that path is first taken.
+int ensure_graph(xb_plan *p, cudaStream_t s) {
+    IluData &u = p->ilu;
+    if (u.exec) return XB_OK;
+    const int n = p->n;
+    const std::vector<int> &rp = p->h_rowptr;
+    std::vector<int> ci, dpos, lev, ulev;
+    int nl = 0, nu = 0;
+    XB_TRY(rows_host(p, ci));
+    XB_TRY(ilu_levels(n, rp.data(), ci.data(), dpos, lev, ulev, &nl, &nu));
+    std::vector<int> llen(n), ulen(n);
+    for (int i = 0; i < n; i++) {
+        llen[i] = dpos[i] - rp[i];
+        ulen[i] = rp[i + 1] - dpos[i] - 1;
+    }
+    std::vector<int> lrows, urows, loff, uoff, ln0, ln1, un0, un1, lw, uw, lecol, lesrc, uecol, uesrc;
+    std::vector<long long> leoff, ueoff;
+    group_levels(lev, llen, nl, lrows, loff, ln0, ln1);
+    group_levels(ulev, ulen, nu, urows, uoff, un0, un1);
+    build_ell(lrows, loff, ln0, ci, [&](int i) { return rp[i]; }, [&](int i) { return dpos[i]; }, lw,
+              leoff, lecol, lesrc);
+    build_ell(urows, uoff, un0, ci, [&](int i) { return dpos[i] + 1; },
+              [&](int i) { return rp[i + 1]; }, uw, ueoff, uecol, uesrc);
+    for (int **d : {&u.d_lrows, &u.d_urows, &u.d_lecol, &u.d_uecol}) {
+        cudaFree(*d);
+        *d = nullptr;
+    }
+    for (double **d : {&u.d_leval, &u.d_ueval, &u.d_udiag, &u.d_out}) {
+        cudaFree(*d);
+        *d = nullptr;
+    }
+    XB_TRY(upload(&u.d_lrows, lrows, s));
+    XB_TRY(upload(&u.d_urows, urows, s));
+    XB_TRY(upload(&u.d_lecol, lecol, s));
+    XB_TRY(upload(&u.d_uecol, uecol, s));
+    XB_TRY(fill_entries(&u.d_leval, lesrc, u.d_lu, s));
+    XB_TRY(fill_entries(&u.d_ueval, uesrc, u.d_lu, s));
+    XB_CUDA(cudaMalloc(&u.d_udiag, std::max<size_t>(1, (size_t)n) * sizeof(double)));
+    XB_CUDA(cudaMalloc(&u.d_out, std::max<size_t>(1, (size_t)n) * sizeof(double)));
+    k_diag_fill<<<(n + 255) / 256, 256, 0, s>>>(n, u.d_urows, u.d_dpos, u.d_lu, u.d_udiag, nullptr,
+                                                nullptr);
+    XB_LAUNCHED("k_diag_fill");
+    cudaStream_t cs = nullptr;
+    XB_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
+    cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        launch_levels<true>(p, u.d_lrows, loff, ln0, ln1, lw, leoff, u.d_lecol, u.d_leval, u.d_udiag,
+                            u.d_in, u.d_out, cs);
+        launch_levels<false>(p, u.d_urows, uoff, un0, un1, uw, ueoff, u.d_uecol, u.d_ueval, u.d_udiag,
+                             u.d_out, u.d_out, cs);
+        e = cudaStreamEndCapture(cs, &u.graph);
+    }
+    cudaStreamDestroy(cs);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&u.exec, u.graph, 0);
+    if (e != cudaSuccess) return cuda_error(e, "ILU(0): capture of the substitutions");
+    XB_CUDA(cudaStreamSynchronize(s));
+    return XB_OK;
+}
+
+}  // namespace
+
 int ensure_ilu(xb_plan *p, cudaStream_t s) {
     if (!p->subs.empty())
         return set_error(XB_EINVAL, "ILU(0): not available for a plan split into row blocks");
@@ -463,180 +865,145 @@ int ensure_ilu(xb_plan *p, cudaStream_t s) {
     ilu_free(p);  // a build that failed half-way left nothing usable
     const int n = p->n, nnz = p->nnz;
     const std::vector<int> &rp = p->h_rowptr;
-    std::vector<int> ci(nnz);
-    if (nnz > 0) XB_CUDA(cudaMemcpy(ci.data(), p->col, (size_t)nnz * 4, cudaMemcpyDeviceToHost));
-    std::vector<int> dpos, lev, ulev;
+    std::vector<int> ci, dpos, lev, ulev, lorder, loff;
     int nl = 0, nu = 0;
+    XB_TRY(rows_host(p, ci));
     XB_TRY(ilu_levels(n, rp.data(), ci.data(), dpos, lev, ulev, &nl, &nu));
-    std::vector<int> llen(n), ulen(n);
-    for (int i = 0; i < n; i++) {
-        llen[i] = dpos[i] - rp[i];
-        ulen[i] = rp[i + 1] - dpos[i] - 1;
-    }
-    std::vector<int> lrows, urows;
-    group_levels(lev, llen, nl, lrows, u.loff, u.ln0, u.ln1);
-    group_levels(ulev, ulen, nu, urows, u.uoff, u.un0, u.un1);
-    std::vector<int> lecol, lesrc, uecol, uesrc;
-    build_ell(lrows, u.loff, u.ln0, ci, [&](int i) { return rp[i]; },
-              [&](int i) { return dpos[i]; }, u.lw, u.leoff, lecol, lesrc);
-    build_ell(urows, u.uoff, u.un0, ci, [&](int i) { return dpos[i] + 1; },
-              [&](int i) { return rp[i + 1]; }, u.uw, u.ueoff, uecol, uesrc);
-    auto up = [&](int **d, const std::vector<int> &h) -> int {
-        XB_CUDA(cudaMalloc(d, std::max<size_t>(1, h.size()) * 4));
-        if (!h.empty())
-            XB_CUDA(cudaMemcpyAsync(*d, h.data(), h.size() * 4, cudaMemcpyHostToDevice, s));
-        return XB_OK;
-    };
-    XB_TRY(up(&u.d_dpos, dpos));
-    XB_TRY(up(&u.d_lrows, lrows));
-    XB_TRY(up(&u.d_urows, urows));
-    XB_TRY(up(&u.d_lecol, lecol));
-    XB_TRY(up(&u.d_lesrc, lesrc));
-    XB_TRY(up(&u.d_uecol, uecol));
-    XB_TRY(up(&u.d_uesrc, uesrc));
-    XB_CUDA(cudaMalloc(&u.d_leval, std::max<size_t>(1, lecol.size()) * sizeof(double)));
-    XB_CUDA(cudaMalloc(&u.d_ueval, std::max<size_t>(1, uecol.size()) * sizeof(double)));
-    XB_CUDA(cudaMalloc(&u.d_udiag, std::max<size_t>(1, (size_t)n) * sizeof(double)));
+    level_order(lev, nl, lorder, loff);
+    // factors, level by level
+    int *d_order = nullptr;
+    XB_TRY(upload(&u.d_dpos, dpos, s));
+    XB_TRY(upload(&d_order, lorder, s));
     XB_CUDA(cudaMalloc(&u.d_lu, std::max<size_t>(1, (size_t)nnz) * sizeof(double)));
-    XB_CUDA(cudaMalloc(&u.d_flag, sizeof(int)));
+    XB_CUDA(cudaMalloc(&u.d_flag, 2 * sizeof(int)));  // zero pivot; pivot out of the flow path's range
     XB_CUDA(cudaMalloc(&u.d_in, std::max<size_t>(1, (size_t)n) * sizeof(double)));
-    XB_CUDA(cudaMalloc(&u.d_out, std::max<size_t>(1, (size_t)n) * sizeof(double)));
-    XB_CUDA(cudaMemsetAsync(u.d_flag, 0, sizeof(int), s));
+    XB_CUDA(cudaMemsetAsync(u.d_flag, 0, 2 * sizeof(int), s));
     if (nnz > 0)
         XB_CUDA(cudaMemcpyAsync(u.d_lu, p->val, (size_t)nnz * sizeof(double),
                                 cudaMemcpyDeviceToDevice, s));
     for (int l = 0; l < nl; l++) {
-        const int cnt = u.loff[l + 1] - u.loff[l];
+        const int cnt = loff[l + 1] - loff[l];
         if (cnt == 0) continue;
         const int wpb = 8;  // warps per CTA
         k_ilu_factor<<<(cnt + wpb - 1) / wpb, 32 * wpb, 0, s>>>(
-            cnt, u.d_lrows + u.loff[l], p->rowptr, p->col, u.d_dpos, u.d_lu, u.d_flag);
+            cnt, d_order + loff[l], p->rowptr, p->col, u.d_dpos, u.d_lu, u.d_flag);
     }
     XB_LAUNCHED("k_ilu_factor");
-    if (!lecol.empty())
-        k_ell_fill<<<(unsigned)((lecol.size() + 255) / 256), 256, 0, s>>>(
-            (long long)lecol.size(), u.d_lesrc, u.d_lu, u.d_leval);
-    if (!uecol.empty())
-        k_ell_fill<<<(unsigned)((uecol.size() + 255) / 256), 256, 0, s>>>(
-            (long long)uecol.size(), u.d_uesrc, u.d_lu, u.d_ueval);
-    if (n > 0)
-        k_diag_fill<<<(n + 255) / 256, 256, 0, s>>>(n, u.d_urows, u.d_dpos, u.d_lu, u.d_udiag);
-    XB_LAUNCHED("k_ell_fill");
-    int flag = 0;
-    XB_CUDA(cudaMemcpyAsync(&flag, u.d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
-    XB_CUDA(cudaStreamSynchronize(s));
-    u.built = true;
-    u.status = flag ? XB_EBREAKDOWN : XB_OK;
-    if (flag) return set_error(XB_EBREAKDOWN, "ILU(0): zero pivot");
-    // capture both substitutions (d_in -> d_out) on a private stream
-    cudaStream_t cs = nullptr;
-    XB_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-    cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-        launch_levels<true>(p, u.d_lrows, u.loff, u.ln0, u.ln1, u.lw, u.leoff, u.d_lecol,
-                            u.d_leval, u.d_udiag, u.d_in, u.d_out, cs);
-        launch_levels<false>(p, u.d_urows, u.uoff, u.un0, u.un1, u.uw, u.ueoff, u.d_uecol,
-                             u.d_ueval, u.d_udiag, u.d_out, u.d_out, cs);
-        e = cudaStreamEndCapture(cs, &u.graph);
-    }
-    cudaStreamDestroy(cs);
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&u.exec, u.graph, 0);
-    if (e != cudaSuccess) {
-        u.built = false;
-        return cuda_error(e, "ILU(0): capture of the substitutions");
-    }
-    // level tables for the persistent substitution
-    auto meta = [](const std::vector<int> &off, const std::vector<int> &n0,
-                   const std::vector<int> &n1, const std::vector<int> &w) {
-        const int nl = (int)n0.size();
-        std::vector<int> m(4 * (nl + 1), 0);
-        for (int l = 0; l < nl; l++) {
-            m[4 * l] = off[l];
-            m[4 * l + 1] = n0[l];
-            m[4 * l + 2] = n1[l];
-            m[4 * l + 3] = w[l];
-        }
-        m[4 * nl] = off[nl];
-        return m;
-    };
-    XB_TRY(up(&u.d_lmeta, meta(u.loff, u.ln0, u.ln1, u.lw)));
-    XB_TRY(up(&u.d_umeta, meta(u.uoff, u.un0, u.un1, u.uw)));
-    XB_CUDA(cudaMalloc(&u.d_leo, u.leoff.size() * sizeof(long long)));
-    XB_CUDA(cudaMalloc(&u.d_ueo, u.ueoff.size() * sizeof(long long)));
-    XB_CUDA(cudaMemcpyAsync(u.d_leo, u.leoff.data(), u.leoff.size() * sizeof(long long),
-                            cudaMemcpyHostToDevice, s));
-    XB_CUDA(cudaMemcpyAsync(u.d_ueo, u.ueoff.data(), u.ueoff.size() * sizeof(long long),
-                            cudaMemcpyHostToDevice, s));
-    XB_CUDA(cudaMalloc(&u.d_bar, 2 * sizeof(unsigned)));
-    XB_CUDA(cudaMalloc(&u.d_err, sizeof(int)));
-    XB_CUDA(cudaMemsetAsync(u.d_err, 0, sizeof(int), s));
-    int dev = 0, coop = 0, per = 0;
+    int dev = 0, coop = 0, smem = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-    if (coop && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ilu_persist, 512, 0) ==
-                    cudaSuccess &&
-        per >= 1)
-        u.pgrid = num_sms();
-    cudaGetLastError();
+    cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (coop && n > 0) {  // the flow layout, while the factorization runs
+        const int cap = (smem - 1024) / 8 - 1;
+        const int G = std::max(1, std::min(num_sms(), (n + kFlowMinRows - 1) / kFlowMinRows));
+        std::vector<int> bstart(G + 1, n);
+        bstart[0] = 0;
+        const double total = (double)nnz + 4.0 * n;  // blocks of about equal work
+        for (int i = 0, c = 0; i < n && c + 1 < G; i++)
+            while (c + 1 < G && (double)rp[i] + 4.0 * i >= total * (c + 1) / G) bstart[++c] = i;
+        for (int c = 1; c <= G; c++) u.maxrows = std::max(u.maxrows, bstart[c] - bstart[c - 1]);
+        u.cap = std::min(u.maxrows, cap);
+        FlowHost hl, hu;
+        if (!flow_layout(lev, bstart, cap, ci.data(), [&](int i) { return rp[i]; },
+                         [&](int i) { return dpos[i]; }, hl) ||
+            !flow_layout(ulev, bstart, cap, ci.data(), [&](int i) { return dpos[i] + 1; },
+                         [&](int i) { return rp[i + 1]; }, hu)) {
+            cudaStreamSynchronize(s);
+            cudaFree(d_order);
+            return set_error(XB_ENOMEM, "ILU(0): host memory for the substitutions' layout");
+        }
+        XB_TRY(upload(&u.d_bstart, bstart, s));
+        XB_TRY(upload_flow(u.fl, hl, u.d_lu, s));
+        XB_TRY(upload_flow(u.fu, hu, u.d_lu, s));
+        XB_CUDA(cudaMalloc(&u.fu.d_diag, (size_t)n * sizeof(double)));
+        XB_CUDA(cudaMalloc(&u.fu.d_rdiag, (size_t)n * sizeof(double)));
+        k_diag_fill<<<(n + 255) / 256, 256, 0, s>>>(n, u.fu.d_rows, u.d_dpos, u.d_lu, u.fu.d_diag,
+                                                    u.fu.d_rdiag, u.d_flag + 1);
+        XB_LAUNCHED("k_diag_fill");
+        XB_CUDA(cudaMalloc(&u.d_ty, (size_t)n * 16));
+        XB_CUDA(cudaMalloc(&u.d_tz, (size_t)n * 16));
+        XB_CUDA(cudaMalloc(&u.d_stop, sizeof(int)));
+        XB_CUDA(cudaMemsetAsync(u.d_ty, 0, (size_t)n * 16, s));
+        XB_CUDA(cudaMemsetAsync(u.d_tz, 0, (size_t)n * 16, s));
+        XB_CUDA(cudaMemsetAsync(u.d_stop, 0, sizeof(int), s));
+        XB_CUDA(cudaFuncSetAttribute(k_ilu_flow, cudaFuncAttributeMaxDynamicSharedMemorySize, smem - 1024));
+        u.grid = G;
+        u.limit_ns = 2000000000ull + 2000ull * (nl + nu);
+    }
+    int flag[2] = {0, 0};
+    XB_CUDA(cudaMemcpyAsync(flag, u.d_flag, sizeof flag, cudaMemcpyDeviceToHost, s));
     XB_CUDA(cudaStreamSynchronize(s));
+    cudaFree(d_order);
+    u.built = true;
+    u.status = flag[0] ? XB_EBREAKDOWN : XB_OK;
+    if (flag[1]) u.grid = 0;  // the graph path divides
+    if (flag[0]) return set_error(XB_EBREAKDOWN, "ILU(0): zero pivot");
     return XB_OK;
 }
 
-// Which substitution to run: the persistent launch pays one grid barrier per
-// level, the captured graph one kernel per non-empty row tier of a level
-// (measured: ~6 us per barrier, ~4 us per graph kernel), so the persistent
-// launch wins when levels hold several tiers (power-law rows) and the graph
-// when every level is one ELL kernel (stencils).  XB_ILU_MODE=0/1 forces one.
-int ilu_mode(const xb_plan *p, const IluData &u) {
+// Which substitution to run: the flow launch, faster on every pattern measured
+// (k_ilu_flow), or (0) the captured graph of level launches, where there is no
+// cooperative launch or a pivot's reciprocal leaves the normal range.
+// XB_ILU_MODE=0/1 forces one.
+int ilu_mode(const xb_plan *p) {
     static const int env = [] {
         const char *e = std::getenv("XB_ILU_MODE");
         return e ? std::atoi(e) : -1;
     }();
+    if (p->ilu.grid == 0) return 0;
     if (p->ilu_mode >= 0) return p->ilu_mode;
-    if (env >= 0) return env;
-    long long levels = (long long)u.ln0.size() + (long long)u.un0.size(), kernels = 0;
-    auto tiers = [](const std::vector<int> &off, const std::vector<int> &n0,
-                    const std::vector<int> &n1) {
-        long long k = 0;
-        for (size_t l = 0; l < n0.size(); l++)
-            k += (n0[l] > 0) + (n1[l] > 0) + (off[l + 1] - off[l] > n0[l] + n1[l]);
-        return k;
-    };
-    kernels = tiers(u.loff, u.ln0, u.ln1) + tiers(u.uoff, u.un0, u.un1);
-    return 4 * kernels > 6 * levels ? 1 : 0;
+    return env >= 0 ? env : 1;
 }
 
 int ilu_check(xb_plan *p) {
-    IluData &u = p->ilu;
-    if (!u.built || !u.d_err) return XB_OK;
-    int err = 0;
-    XB_CUDA(cudaMemcpy(&err, u.d_err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (err) {
-        cudaMemset(u.d_err, 0, sizeof(int));
-        return set_error(XB_ETIMEOUT, "ILU(0): a level barrier wait ran out");
-    }
-    return XB_OK;
+    volatile int *err = reinterpret_cast<volatile int *>(p->h_pin + 61);
+    if (!*err) return XB_OK;
+    *err = 0;
+    if (p->ilu.d_stop) XB_CUDA(cudaMemset(p->ilu.d_stop, 0, sizeof(int)));
+    return set_error(XB_ETIMEOUT, "ILU(0): a wait for another row's value ran out");
 }
 
 int ilu_apply(xb_plan *p, const double *r, double *z, cudaStream_t s) {
     IluData &u = p->ilu;
     XB_TRY(ensure_ilu(p, s));
     if (p->n == 0) return XB_OK;
-    if (u.pgrid > 0 && ilu_mode(p, u) == 1) {
-        TriDev L{(int)u.ln0.size(), u.d_lmeta, u.d_leo, u.d_lrows, u.d_lecol, u.d_leval, u.d_udiag};
-        TriDev U{(int)u.un0.size(), u.d_umeta, u.d_ueo, u.d_urows, u.d_uecol, u.d_ueval, u.d_udiag};
-        const int *rp = p->rowptr, *ci = p->col, *dp = u.d_dpos;
-        const double *lu = u.d_lu;
-        unsigned *bar = u.d_bar;
-        int *err = u.d_err;
-        unsigned polls = p->ilu_polls > 0 ? (unsigned)p->ilu_polls : kBarSpins;
-        void *args[] = {&L, &U, (void *)&rp, (void *)&ci, (void *)&dp, (void *)&lu, (void *)&r,
-                        (void *)&z, (void *)&bar, (void *)&err, (void *)&polls};
-        XB_CUDA(cudaMemsetAsync(u.d_bar, 0, 2 * sizeof(unsigned), s));
-        XB_CUDA(cudaLaunchCooperativeKernel((const void *)k_ilu_persist, u.pgrid, 512, args, 0, s));
+    const size_t bytes = (size_t)p->n * sizeof(double);
+    if (ilu_mode(p) == 1) {
+        const uintptr_t ra = (uintptr_t)r, za = (uintptr_t)z;
+        if (ra < za + bytes && za < ra + bytes) {  // overlapping operands: rows of r are read late
+            XB_CUDA(cudaMemcpyAsync(u.d_in, r, bytes, cudaMemcpyDeviceToDevice, s));
+            r = u.d_in;
+        }
+        auto tri = [](const IluData::Flow &f) {
+            return FlowTri{reinterpret_cast<const int4 *>(f.d_items), f.d_iptr, f.d_ebase, f.d_rows,
+                           f.d_ecol, f.d_eval, f.d_diag, f.d_rdiag};
+        };
+        FlowArgs a{};
+        a.L = tri(u.fl);
+        a.U = tri(u.fu);
+        a.bstart = u.d_bstart;
+        a.rp = p->rowptr;
+        a.ci = p->col;
+        a.dpos = u.d_dpos;
+        a.lu = u.d_lu;
+        a.r = r;
+        a.z = z;
+        a.ty = reinterpret_cast<ulonglong2 *>(u.d_ty);
+        a.tz = reinterpret_cast<ulonglong2 *>(u.d_tz);
+        if (++u.seq == 0) u.seq = 1;
+        a.seq = u.seq;
+        a.polls = (unsigned)p->ilu_polls;
+        a.look = a.polls ? a.polls : 64u;
+        a.limit = u.limit_ns;
+        a.err = reinterpret_cast<volatile int *>(p->h_pin + 61);
+        a.stop = u.d_stop;
+        a.cap = u.cap;
+        void *args[] = {&a};
+        XB_CUDA(cudaLaunchCooperativeKernel((const void *)k_ilu_flow, u.grid, 32 * kFlowWarps, args,
+                                            (size_t)(u.cap + 1) * sizeof(double), s));
         return XB_OK;
     }
-    const size_t bytes = (size_t)p->n * sizeof(double);
+    XB_TRY(ensure_graph(p, s));
     XB_CUDA(cudaMemcpyAsync(u.d_in, r, bytes, cudaMemcpyDeviceToDevice, s));
     XB_CUDA(cudaGraphLaunch(u.exec, s));
     XB_CUDA(cudaMemcpyAsync(z, u.d_out, bytes, cudaMemcpyDeviceToDevice, s));

@@ -230,6 +230,7 @@ struct xb_plan {
     void *d_work = nullptr;
     size_t work_bytes = 0;
     double *h_pin = nullptr;             // pinned host mirror of a few scalars
+    unsigned long long gs_tag = 0;       // orthogonalisations launched
     // tuned choice
     int variant = XB_VAR_NNZ, block = 256, ipt = 8;
     float tuned_ms = 0.f;

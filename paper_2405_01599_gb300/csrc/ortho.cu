@@ -31,6 +31,7 @@ struct GsArgs {
     unsigned *hdr;        // [0] exchange number, [1] a wait ran out
     ulonglong2 *slots;    // 2 x kGsVals x kGsMaxClusters
     int *err;             // host-visible: a wait ran out
+    unsigned long long *late, tag;  // host-visible words: 4 tag + GM_STOP after step tag
 };
 
 // ---- values that carry their exchange number ------------------------------------
@@ -623,6 +624,11 @@ __device__ void scalar_warp(Ctx<VB, KB> &c, unsigned seq, bool raw) {
         hn = sqrt(nn);
         rr = hypot(t, hn);
     }
+    // one word tells the host: no copy in the stream, no fence
+    auto tell = [&](int stop) {
+        if (stop) st.misc[xb::GM_STOP] = (double)stop;
+        *reinterpret_cast<volatile unsigned long long *>(a.late + (a.tag & 1)) = 4 * a.tag + stop;
+    };
     const double q = (lane == 0 ? t : lane == 1 ? hn : 1.0) / (lane < 2 ? rr : hn);
     const double cs = __shfl_sync(0xffffffffu, q, 0), sn = __shfl_sync(0xffffffffu, q, 1);
     const double inv = __shfl_sync(0xffffffffu, q, 2);
@@ -631,7 +637,7 @@ __device__ void scalar_warp(Ctx<VB, KB> &c, unsigned seq, bool raw) {
     if (rr == 0.0) {  // A v_j lies in span(v_0..v_{j-1}) with a zero pivot: singular
         a.col[j] = t;
         a.col[j + 1] = hn;
-        st.misc[xb::GM_STOP] = 2.0;
+        tell(2);
         return;
     }
     st.cs[j] = cs;
@@ -644,14 +650,14 @@ __device__ void scalar_warp(Ctx<VB, KB> &c, unsigned seq, bool raw) {
     st.misc[xb::GM_RES] = res;
     st.misc[xb::GM_K] = (double)(j + 1);
     if (hn <= 1e-14 * sqrt(len2 + hn * hn)) {  // happy breakdown: the Krylov space is invariant
-        st.misc[xb::GM_STOP] = 1.0;
         st.sc[j + 1] = 0.0;
         st.scf[j + 1] = 0.0f;
+        tell(1);
         return;
     }
     st.sc[j + 1] = inv;
     st.scf[j + 1] = (float)inv;
-    if (res <= tau) st.misc[xb::GM_STOP] = 1.0;
+    tell(res <= tau ? 1 : 0);
 }
 
 // What bounds it and why this form.  At small n the time of an
@@ -976,6 +982,8 @@ int gs_run(xb_plan *p, GsArgs<VB> &a, bool seen, cudaStream_t s) {
     a.hdr = p->d_ticket + 64;
     a.slots = reinterpret_cast<ulonglong2 *>(p->d_ticket + 128);
     a.err = reinterpret_cast<int *>(p->h_pin + 60);
+    a.late = reinterpret_cast<unsigned long long *>(p->h_pin + 40);
+    a.tag = ++p->gs_tag;
     if (a.method == XB_ORTHO_BCGS) return plan_launch<VB, 4, 0>(a, s);
     if (a.method != XB_ORTHO_MGS) return plan_launch<VB, 8, 0>(a, s);
     if constexpr (sizeof(VB) == 8) {

@@ -147,3 +147,26 @@ def test_mixed_inner_solve(env, name):
     r = b - oracle.spmv(A, x.cpu().numpy())
     assert info["status"] == 0 and info["fallback"] == 0, info
     assert np.linalg.norm(r) <= 1e-10 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("check_every", [1, 2, 5, 100])
+def test_late_look(env, check_every):
+    """The host sees a cycle's end one check late and only in the word of the
+    step that ended it: the counts are those of the steps taken."""
+    xb, dev = env
+    import torch
+    A = gen.convdiff3d(N=20, dims=(23, 21, 20))
+    b = oracle.spmv(A, np.ones(A["n"]))
+    plan = xb.Plan.from_host(A, dev)
+    infos = []
+    for every in (1, check_every):
+        for prec in (xb.PREC_FP64, xb.PREC_MIXED):
+            x = torch.zeros(A["n"], dtype=torch.float64, device=dev)
+            infos.append(plan.gmres(torch.tensor(b, device=dev), x, m=17, tol=1e-9, precision=prec,
+                                    check_every=every, small_n=0))
+            assert infos[-1]["status"] == 0
+    for i, j in ((0, 2), (1, 3)):
+        for k in ("iters", "inner_iters", "restarts", "outer"):
+            assert infos[i][k] == infos[j][k], k
+    # one SpMV per step and per residual, none for the step that did nothing
+    assert infos[0]["spmv_calls"] == infos[0]["iters"] + infos[0]["restarts"] + 1

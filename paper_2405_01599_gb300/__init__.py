@@ -188,19 +188,41 @@ def _check(code, ok=(XB_OK,)):
     return code
 
 
+_raw_stream = None
+
+
+def _current_stream():
+    """Handle of torch's current stream on the current device, as an int (a
+    Stream object per call costs 2 us, as much as a launch)."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        get, dev = (getattr(torch._C, k, None) for k in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+        if get is not None and dev is not None:
+            torch.cuda.current_stream()  # initialises CUDA
+            _raw_stream = lambda: get(dev())
+        else:
+            _raw_stream = lambda: torch.cuda.current_stream().cuda_stream
+    return _raw_stream()
+
+
 def _stream(stream=None):
-    import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    return stream.cuda_stream if stream is not None else _current_stream()
 
 
 def _ptr(t):
-    return C.c_void_p(t.data_ptr()) if t is not None and t.numel() > 0 else C.c_void_p(0)
+    return t.data_ptr() if t is not None and t.numel() > 0 else None
+
+
+_Tensor = None
 
 
 def _need(t, dtype, name):
-    import torch
-    if not isinstance(t, torch.Tensor) or not t.is_cuda:
+    global _Tensor
+    if _Tensor is None:
+        import torch
+        _Tensor = torch.Tensor
+    if not isinstance(t, _Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype or not t.is_contiguous():
         raise TypeError(f"{name} must be a contiguous {dtype} tensor (got {t.dtype})")
@@ -337,6 +359,7 @@ class Plan:
         self.nnz = col.numel()
         self.sym_upper = bool(sym_upper)
         self._keep = (rowptr, col, val)
+        self._f64 = torch.float64
         h = C.c_void_p()
         if wide:
             self._csr = Csr64(self.n, self.nnz, _ptr(rowptr), _ptr(col), _ptr(val), int(sym_upper))
@@ -367,9 +390,8 @@ class Plan:
 
     # ---- SpMV ----
     def _vec(self, x, y):
-        import torch
-        _need(x, torch.float64, "x")
-        _need(y, torch.float64, "y")
+        _need(x, self._f64, "x")
+        _need(y, self._f64, "y")
         if x.numel() != self.n or y.numel() != self.n:
             raise ValueError("vector length != n")
 

@@ -30,6 +30,12 @@
 // buffers alternate, and a buffer is rewritten only after a cluster barrier
 // that follows every read of it.
 //
+// Gram-Schmidt.  Both methods take the basis in blocks of four, one exchange
+// each (64 x 64 Poisson, GMRES(30): MGS with an exchange per vector 17.3 us a
+// step, in corrected blocks 14.4, BCGS 12.6; eight at once would add as many FP64
+// sums as it saves exchanges).  The inner products that correct MGS's blocks are
+// taken with ||w||^2 and stand in H's unused lower triangle.
+//
 // Reductions.  One, or four at once, sums over the cluster: each warp
 // reduces its lanes' partials with shuffles (four sums in a transposed tree:
 // 6 adds rather than 20), and lanes store the warp's sums into the same slot
@@ -66,7 +72,7 @@ constexpr int kBT = 32 * kW;
 constexpr unsigned kFull = 0xffffffffu;
 
 struct ResArgs {
-    int n, rpc, lmax, m, m_max, maxiter, bcgs;
+    int n, rpc, lmax, m, m_max, maxiter;
     double tol, theta;
     unsigned long long budget_ns;
     const int *rowptr, *col;
@@ -77,7 +83,7 @@ struct ResArgs {
 
 // Byte offsets of the dynamic shared memory regions (doubles first).
 struct ResLayout {
-    size_t V, W, ev, bs, ms, H, cs, sn, g, y, ea, p2, mb, total;
+    size_t V, W, ev, bs, ms, H, cs, sn, g, y, ea, mb, total;
 };
 
 __host__ __device__ inline ResLayout res_layout(int rpp, int lmax, int mmax, int P) {
@@ -99,8 +105,6 @@ __host__ __device__ inline ResLayout res_layout(int rpp, int lmax, int mmax, int
     L.g = take((size_t)(mmax + 1) * 8);
     L.y = take((size_t)mmax * 8);
     L.ea = take((size_t)lmax * rpp * 4);
-    // R <= 4: each thread's part of (v_{i-1}, v_i), formed once per basis vector
-    L.p2 = take(rpp <= 4 * 128 ? (size_t)(mmax + 1) * 128 * 8 : 0);
     L.mb = take(2 * 8 + 4);  // two mbarriers, the abort flag
     L.total = o;
     return L;
@@ -237,7 +241,7 @@ struct Red {
     double *bs, *ms;       // barrier / mbarrier slots: 2 phases x 4 sums x P
     unsigned mb;           // shared address of the two mbarriers
     volatile int *abort;   // set when an mbarrier wait gave up
-    int slot, bph, mk, K;  // this warp's slot, phases, sums per mbarrier exchange
+    int slot, bph, mk;     // this warp's slot, phases
 };
 
 // Barrier-completed sum of one value (also publishes the caller's earlier
@@ -273,15 +277,7 @@ __device__ __forceinline__ void bget4(double (&v)[4], Red<NCL> &R) {
     R.bph ^= 1;
 }
 
-// mbarrier-completed sums (R.K values: 1 for MGS, 4 for BCGS).
-template <int NCL>
-__device__ __forceinline__ void mput1(double v, const Red<NCL> &R) {
-    v = warp_sum1(v);
-    const int lane = threadIdx.x & 31, p = R.mk & 1;
-    if (lane < NCL)
-        st_async(map_rank(smem_addr(R.ms + p * 4 * R.P + R.slot), (unsigned)lane), v,
-                 map_rank(R.mb + 8 * p, (unsigned)lane));
-}
+// mbarrier-completed sums of four values.
 template <int NCL>
 __device__ __forceinline__ void mput4(const double (&v)[4], const Red<NCL> &R) {
     const double k = warp_sum4(v);
@@ -309,7 +305,7 @@ __device__ __forceinline__ const double *mwait(Red<NCL> &R) {
     }
     // re-arm only a completed phase (after a timeout the exchange is lost and
     // every later wait returns at once)
-    if (threadIdx.x == 0 && done) mb_arm(a, (unsigned)(R.K * R.P * 8));
+    if (threadIdx.x == 0 && done) mb_arm(a, (unsigned)(4 * R.P * 8));
     R.mk++;
     return R.ms + p * 4 * R.P;
 }
@@ -341,7 +337,7 @@ __device__ __forceinline__ void rows_spmv(const double *__restrict__ ev, const i
     }
 }
 
-template <int R, int NCL>
+template <int R, int NCL, bool BCGS>
 __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int rpp = kBT * R;
@@ -356,7 +352,6 @@ __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
     double *g = reinterpret_cast<double *>(smem + L.g);
     double *yv = reinterpret_cast<double *>(smem + L.y);
     int *ea = reinterpret_cast<int *>(smem + L.ea);
-    double *P2 = reinterpret_cast<double *>(smem + L.p2);  // R <= 4 only
     const unsigned rank = cluster_rank();
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     Red<NCL> Rd;
@@ -367,14 +362,13 @@ __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
     Rd.slot = (int)rank * kW + warp;
     Rd.bph = 0;
     Rd.mk = 0;
-    Rd.K = A.bcgs ? 4 : 1;
     if (t == 0) {
         *Rd.abort = 0;
         mb_init(Rd.mb);
         mb_init(Rd.mb + 8);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        mb_arm(Rd.mb, (unsigned)(Rd.K * Rd.P * 8));
-        mb_arm(Rd.mb + 8, (unsigned)(Rd.K * Rd.P * 8));
+        mb_arm(Rd.mb, (unsigned)(4 * Rd.P * 8));
+        mb_arm(Rd.mb + 8, (unsigned)(4 * Rd.P * 8));
     }
     const bool lead = rank == 0 && t == 0;
     const unsigned long long ts = gtimer(), deadline = ts + A.budget_ns;
@@ -482,6 +476,9 @@ __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
             const double tol_g = tau * bnorm;  // |g_{j+1}| <= tau ||b||
             double gj = beta;                  // g_j of the least-squares right-hand side
             int k = 0;
+            // where (v_i, v_k), k in i's block of 4 before i, stand: column
+            // mmax - 1 - i of H from row mmax + 1 - i on, which is unused
+            auto gram = [&](int i) { return mmax * ldh - i * (ldh + 1); };
             for (int j = 0; j < m; j++) {
                 iters++;
                 rows_spmv<R>(ev, ea, len, rpp, wbuf[wb], w);
@@ -505,110 +502,79 @@ __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
                     }
                 };
                 double *wn = W + (wb ^ 1) * rpp;
-                double last[4];
-                int nlast, i_last;
-                if (A.bcgs) {
-                    // blocks of 4: one exchange per block takes the block's
-                    // dots after the previous block's projection
-                    double c4[4] = {0.0, 0.0, 0.0, 0.0};
-                    int u0 = 0, nu = 0;
-                    for (int d0 = 0; d0 <= j; d0 += 4) {
-                        const int nd = min(4, j + 1 - d0);
-                        double a4[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-                        for (int r = 0; r < R; r++) {
-                            const int l = r * kBT + t;
-#pragma unroll
-                            for (int q = 0; q < 4; q++)
-                                if (q < nu) w[r] = fma(-c4[q], V[(u0 + q) * rpp + l], w[r]);
-#pragma unroll
-                            for (int q = 0; q < 4; q++)
-                                if (q < nd) a4[q] = fma(w[r], V[(d0 + q) * rpp + l], a4[q]);
-                        }
-                        mput4(a4, Rd);
-#pragma unroll
-                        for (int q = 0; q < 4; q++)
-                            if (q < nu) take(u0 + q, c4[q]);
-                        slots_sum4<NCL>(mwait(Rd), a4);
-#pragma unroll
-                        for (int q = 0; q < 4; q++) c4[q] = a4[q];
-                        u0 = d0;
-                        nu = nd;
-                    }
+                // blocks of 4: one exchange per block takes the block's dots
+                // after the previous block's projection.  BCGS uses them as they
+                // are; for MGS they are corrected by the block's own inner
+                // products, (w - sum_{k<i} h_k v_k, v_i) = (w, v_i) -
+                // sum_{k<i} h_k (v_k, v_i), which is the same method with a
+                // quarter of the exchanges
+                double c4[4] = {0.0, 0.0, 0.0, 0.0};
+                int u0 = 0, nu = 0;
+                for (int d0 = 0; d0 <= j; d0 += 4) {
+                    const int nd = min(4, j + 1 - d0);
+                    double a4[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
                     for (int r = 0; r < R; r++) {
                         const int l = r * kBT + t;
 #pragma unroll
                         for (int q = 0; q < 4; q++)
                             if (q < nu) w[r] = fma(-c4[q], V[(u0 + q) * rpp + l], w[r]);
+#pragma unroll
+                        for (int q = 0; q < 4; q++)
+                            if (q < nd) a4[q] = fma(w[r], V[(d0 + q) * rpp + l], a4[q]);
                     }
+                    mput4(a4, Rd);
 #pragma unroll
-                    for (int q = 0; q < 4; q++) last[q] = c4[q];
-                    nlast = nu;
-                    i_last = u0;
-                } else {
-                    // fused MGS: pass i applies the projection on v_{i-1} and
-                    // takes (w, v_i)
-                    double hprev = 0.0;
-                    if constexpr (R <= 4) {
-                        // the thread's part of (w - h_{i-1} v_{i-1}, v_i) as
-                        // (w, v_i) - h_{i-1} (v_{i-1}, v_i): the first part is
-                        // formed while the previous exchange is in flight,
-                        // the second once when v_i was written, so one FMA
-                        // separates h_{i-1} from the next send (measured
-                        // faster than the direct form at 2 and 4 rows per
-                        // thread; at 8 the window's work would outgrow the
-                        // exchange, and the direct form below serves it)
-                        double p1 = 0.0, p2 = 0.0;
-#pragma unroll
-                        for (int r = 0; r < R; r++) p1 = fma(w[r], V[r * kBT + t], p1);
-                        for (int i = 0; i <= j; i++) {
-                            mput1(i == 0 ? p1 : fma(-hprev, p2, p1), Rd);
-                            if (i > 0) {
-#pragma unroll
-                                for (int r = 0; r < R; r++)
-                                    w[r] = fma(-hprev, V[(i - 1) * rpp + r * kBT + t], w[r]);
-                            }
-                            if (i < j) {
-                                p1 = 0.0;
-#pragma unroll
-                                for (int r = 0; r < R; r++)
-                                    p1 = fma(w[r], V[(i + 1) * rpp + r * kBT + t], p1);
-                                p2 = P2[(i + 1) * kBT + t];
-                            }
-                            if (i > 0) take(i - 1, hprev);
-                            hprev = slots_sum1<NCL>(mwait(Rd));
-                        }
+                    for (int q = 0; q < 4; q++)
+                        if (q < nu) take(u0 + q, c4[q]);
+                    if constexpr (BCGS) {
+                        slots_sum4<NCL>(mwait(Rd), c4);
                     } else {
-                        for (int i = 0; i <= j; i++) {
-                            double a = 0.0;
+                        double gr[4][3];
 #pragma unroll
-                            for (int r = 0; r < R; r++) {
-                                const int l = r * kBT + t;
-                                if (i > 0) w[r] = fma(-hprev, V[(i - 1) * rpp + l], w[r]);
-                                a = fma(w[r], V[i * rpp + l], a);
-                            }
-                            mput1(a, Rd);
-                            if (i > 0) take(i - 1, hprev);
-                            hprev = slots_sum1<NCL>(mwait(Rd));
-                        }
+                        for (int q = 1; q < 4; q++)
+#pragma unroll
+                            for (int k = 0; k < q; k++)
+                                gr[q][k] = q < nd ? H[gram(d0 + q) + k] : 0.0;
+                        slots_sum4<NCL>(mwait(Rd), c4);
+#pragma unroll
+                        for (int k = 0; k < 3; k++)
+#pragma unroll
+                            for (int q = k + 1; q < 4; q++)
+                                if (q < nd) c4[q] = fma(-c4[k], gr[q][k], c4[q]);
                     }
-#pragma unroll
-                    for (int r = 0; r < R; r++) w[r] = fma(-hprev, V[j * rpp + r * kBT + t], w[r]);
-                    last[0] = hprev;
-                    nlast = 1;
-                    i_last = j;
+                    u0 = d0;
+                    nu = nd;
                 }
-                wb ^= 1;
-                double a = 0.0;
 #pragma unroll
                 for (int r = 0; r < R; r++) {
-                    wn[r * kBT + t] = w[r];  // published by the norm's barrier
-                    a = fma(w[r], w[r], a);
+                    const int l = r * kBT + t;
+#pragma unroll
+                    for (int q = 0; q < 4; q++)
+                        if (q < nu) w[r] = fma(-c4[q], V[(u0 + q) * rpp + l], w[r]);
                 }
-                bput1(a, Rd);
-                for (int q = 0; q < nlast; q++) take(i_last + q, last[q]);
-                const double hn2 = bget1(Rd);
+                wb ^= 1;
+                // ||w||^2 and, for MGS, w's products with the basis vectors it
+                // will share a block with
+                const int ng = BCGS || j + 1 >= m ? 0 : (j + 1) & 3, g0 = j + 1 - ng;
+                double n4[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+                for (int r = 0; r < R; r++) {
+                    const int l = r * kBT + t;
+                    wn[l] = w[r];  // published by the norm's barrier
+                    n4[0] = fma(w[r], w[r], n4[0]);
+#pragma unroll
+                    for (int q = 0; q < 3; q++)
+                        if (q < ng) n4[1 + q] = fma(w[r], V[(g0 + q) * rpp + l], n4[1 + q]);
+                }
+                if (ng > 0) bput4(n4, Rd);
+                else bput1(n4[0], Rd);
+#pragma unroll
+                for (int q = 0; q < 4; q++)
+                    if (q < nu) take(u0 + q, c4[q]);
+                if (ng > 0) bget4(n4, Rd);
+                else n4[0] = bget1(Rd);
+                const double hn2 = n4[0];
                 // the new rotation, from values every thread holds alike
                 // (|h| <= ||A|| sqrt(m): no overflow in tt^2 + hn^2)
                 int flag = 0;
@@ -624,6 +590,7 @@ __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
                         H[j * ldh + j + 1] = rr2 * irr;  // the diagonal, until the restart
                         g[j] = c * gj;
                     }
+                    if (!BCGS && t < ng) H[gram(j + 1) + t] = (t == 0 ? n4[1] : t == 1 ? n4[2] : n4[3]) * ihn;
                     gj = -s * gj;
                     if (hn2 <= 1e-28 * (len2 + hn2)) flag = 1;  // hn <= 1e-14 |column|
                     else if (fabs(gj) <= tol_g) flag = 3;
@@ -645,15 +612,6 @@ __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
                 double *Vn = V + (j + 1) * rpp;
 #pragma unroll
                 for (int r = 0; r < R; r++) Vn[r * kBT + t] = w[r] * sc;
-                if constexpr (R <= 4) {
-                    if (!A.bcgs) {  // MGS: (v_j, v_{j+1}), this thread's part
-                        double pv = 0.0;
-#pragma unroll
-                        for (int r = 0; r < R; r++)
-                            pv = fma(V[j * rpp + r * kBT + t], w[r] * sc, pv);
-                        P2[(j + 1) * kBT + t] = pv;
-                    }
-                }
                 if (flag == 3) {
                     claimed = 1;
                     break;
@@ -744,23 +702,23 @@ __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
 
 typedef void (*ResKernel)(const ResArgs);
 
-template <int R>
+template <int R, bool BCGS>
 ResKernel res_kernel_r(int ncl) {
     switch (ncl) {
-        case 2: return k_gmres_resident<R, 2>;
-        case 4: return k_gmres_resident<R, 4>;
-        case 8: return k_gmres_resident<R, 8>;
-        case 16: return k_gmres_resident<R, 16>;
+        case 2: return k_gmres_resident<R, 2, BCGS>;
+        case 4: return k_gmres_resident<R, 4, BCGS>;
+        case 8: return k_gmres_resident<R, 8, BCGS>;
+        case 16: return k_gmres_resident<R, 16, BCGS>;
         default: return nullptr;
     }
 }
 
-ResKernel res_kernel(int R, int ncl) {
+ResKernel res_kernel(int R, int ncl, bool bcgs) {
     switch (R) {
-        case 1: return res_kernel_r<1>(ncl);
-        case 2: return res_kernel_r<2>(ncl);
-        case 4: return res_kernel_r<4>(ncl);
-        case 8: return res_kernel_r<8>(ncl);
+        case 1: return bcgs ? res_kernel_r<1, true>(ncl) : res_kernel_r<1, false>(ncl);
+        case 2: return bcgs ? res_kernel_r<2, true>(ncl) : res_kernel_r<2, false>(ncl);
+        case 4: return bcgs ? res_kernel_r<4, true>(ncl) : res_kernel_r<4, false>(ncl);
+        case 8: return bcgs ? res_kernel_r<8, true>(ncl) : res_kernel_r<8, false>(ncl);
         default: return nullptr;
     }
 }
@@ -815,7 +773,7 @@ int resident_gmres(xb_plan *p, const double *b, double *x, const xb_options &o, 
         const int rpc = (p->n + ncl - 1) / ncl;
         int R = 1;
         while (R * kBT < rpc) R *= 2;
-        ResKernel kf = res_kernel(R, ncl);
+        ResKernel kf = res_kernel(R, ncl, o.ortho == XB_ORTHO_BCGS);
         if (!kf) continue;
         const ResLayout L = res_layout(kBT * R, lmax, mmax, ncl * kW);
         if (L.total > (size_t)optin) continue;
@@ -852,7 +810,6 @@ int resident_gmres(xb_plan *p, const double *b, double *x, const xb_options &o, 
     a.m = o.m;
     a.m_max = mmax;
     a.maxiter = o.maxiter;
-    a.bcgs = o.ortho == XB_ORTHO_BCGS ? 1 : 0;
     a.tol = o.tol;
     a.theta = o.dafrt ? o.dafrt_theta : 0.0;
     a.budget_ns = (unsigned long long)(std::min(o.maxtime_s, 3600.0) * 1e9);
@@ -884,7 +841,7 @@ int resident_gmres(xb_plan *p, const double *b, double *x, const xb_options &o, 
     inf.restarts = r.restarts;
     inf.m_final = r.m;
     inf.res_true = r.res_true;
-    inf.ortho_used = a.bcgs ? XB_ORTHO_BCGS : XB_ORTHO_MGS;
+    inf.ortho_used = o.ortho == XB_ORTHO_BCGS ? XB_ORTHO_BCGS : XB_ORTHO_MGS;
     inf.persistent = 2;
     // algorithmic bytes, counted as for the multi-launch step: per Arnoldi
     // step one SpMV and the Gram-Schmidt passes at the cycle's mean basis

@@ -3,7 +3,7 @@
 //
 // The launch is a grid of 8-CTA thread-block clusters, fed by two atomic
 // queues (each ordered largest first):
-//   - a system with n >= kLargeN is solved by a whole cluster: every CTA
+//   - a large system (split_systems) is solved by a whole cluster: every CTA
 //     owns a slice of the rows, dot products are combined across the cluster
 //     through distributed shared memory (every CTA sums the 8 partials in rank
 //     order, so all CTAs hold identical values), and hardware cluster
@@ -17,10 +17,10 @@
 // that rank 0 decides and broadcasts through a reduction), so all CTAs of a
 // cluster reach the same barriers in the same order.
 //
-// The solver is restarted GMRES(m) with modified Gram-Schmidt (fused: each
-// pass applies the previous projection and takes the next inner product) or
-// blocked classical Gram-Schmidt with block length 4 (one pass and one
-// four-value reduction per block),
+// The solver is restarted GMRES(m) with modified Gram-Schmidt or blocked
+// classical Gram-Schmidt, both over blocks of 4 basis vectors (one pass, which
+// applies the previous block's projection, and one four-value reduction per
+// block; for MGS the block's dots are corrected by its own inner products),
 // Givens least squares, the true-residual check at every restart (fault
 // convergence narrows the implicit threshold), and, when enabled, the
 // MM-ratio restart rule of Eq. (1) / Fig. 2 / Sec. 4.3 (m grows by 5, up to
@@ -40,7 +40,7 @@ namespace cg = cooperative_groups;
 namespace {
 constexpr int kCl = 8;          // CTAs per cluster
 constexpr int kBT = 512;        // threads per CTA
-constexpr int kLargeN = 30000;  // systems this large are solved by a whole cluster
+constexpr int kTeamRow = 64;    // mode 1: rows longer than this are summed by a whole warp
 constexpr int kCtaRow = 1024;   // mode 1: rows longer than this are summed by the whole CTA
 }  // namespace
 
@@ -76,11 +76,16 @@ __device__ __forceinline__ unsigned long long gtimer() {
     return t;
 }
 
+constexpr int kNW = kBT / 32;
+
 struct Smem {
-    double sh[40];
-    double slot[2];  // this CTA's partial of the current cluster reduction
-    double sh4[4][kBT / 32], slot4[2][4], tot4[4];  // the same for 4 sums at once
+    double sh[40];                                   // cta_sum (long rows)
+    double part[2][4][kNW], slot[2][4], tot[2][4];   // sums of up to 4 values, two phases
     double g[XB_BATCH_MAX_M + 1], cs[XB_BATCH_MAX_M], sn[XB_BATCH_MAX_M], yv[XB_BATCH_MAX_M];
+    double hc[XB_BATCH_MAX_M + 2];                   // the step's Hessenberg column, unrotated
+    double hn[XB_BATCH_MAX_M + 1], sc[XB_BATCH_MAX_M + 1];  // norms of the stored basis vectors, 1 / them
+    double sg[(XB_BATCH_MAX_M + 1) * 4];             // sc_i^2 (V_i, V_k), k in i's block of 4 before i
+    double tt, len2;
     unsigned long long t_start;
     int q;
     int flag;
@@ -108,59 +113,69 @@ struct Part {
     int r0, r1, coop, phase;
 };
 
-// Sum over all cooperating CTAs (one cluster barrier), identical everywhere.
-// The two partial slots alternate, so a slot is rewritten only after every
-// CTA has passed the barrier of the reduction that follows its last read.
-__device__ double coop_sum(double v, Smem &S, Part &P) {
-    const double t = cta_sum(v, S);
-    if (!P.coop) return t;
-    cg::cluster_group cl = cg::this_cluster();
-    if (threadIdx.x == 0) S.slot[P.phase] = t;
-    cl.sync();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int r = 0; r < kCl; r++) tot += cl.map_shared_rank(S.slot, r)[P.phase];
-        S.sh[34] = tot;
+// Sums of NV <= 4 values over all cooperating CTAs, in a fixed order.  Every
+// warp adds its lanes' values (four in a transposed tree: 6 adds instead of 20;
+// an FP64 add holds a quarter of the SM for ~80 cycles whatever it adds), warp 0
+// the warps' sums and, for a cluster, the 8 CTAs' after one cluster barrier.
+// `while_w2` runs in warp 2 beside warp 0's sums, `fin` in warp 0 with value
+// lane >> 3 of the total in every lane; then the CTA meets.  Slots of two phases
+// alternate, so a slot is rewritten only after every CTA has passed the barrier
+// of the sum that follows its last read.  The cluster barrier (or the CTA's)
+// also orders the vectors written before it.
+template <int NV, typename W2, typename Fin>
+__device__ __forceinline__ void sums(const double (&v)[NV], Smem &S, Part &P, W2 while_w2, Fin fin) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, ph = P.phase;
+    double k;
+    if constexpr (NV == 4) {
+        const bool h16 = lane & 16, h8 = lane & 8;
+        double k0 = h16 ? v[2] : v[0], k1 = h16 ? v[3] : v[1];
+        const double s0 = h16 ? v[0] : v[2], s1 = h16 ? v[1] : v[3];
+        k0 += __shfl_xor_sync(0xffffffffu, s0, 16);
+        k1 += __shfl_xor_sync(0xffffffffu, s1, 16);
+        k = h8 ? k1 : k0;
+        k += __shfl_xor_sync(0xffffffffu, h8 ? k0 : k1, 8);
+    } else {
+        k = v[0];
+        k += __shfl_xor_sync(0xffffffffu, k, 16);
+        k += __shfl_xor_sync(0xffffffffu, k, 8);
     }
-    __syncthreads();
-    const double tot = S.sh[34];
-    __syncthreads();
-    P.phase ^= 1;
-    return tot;
-}
-
-// Four sums at once over all cooperating CTAs (one CTA barrier pair and one
-// cluster barrier for the four), identical everywhere, in a fixed order.
-__device__ void coop_sum4(double (&v)[4], Smem &S, Part &P) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-    for (int q = 0; q < 4; q++)
-        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+    for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+    if ((lane & 7) == 0 && (lane >> 3) < NV) S.part[ph][lane >> 3][w] = k;
     __syncthreads();
-    if (lane == 0)
+    const int q = lane >> 3, r = lane & 7;
+    double a = 0.0;
+    if (w == 0) {
+        if (q < NV) a = S.part[ph][q][r] + S.part[ph][q][r + 8];
 #pragma unroll
-        for (int q = 0; q < 4; q++) S.sh4[q][w] = v[q];
-    __syncthreads();
-    if (threadIdx.x < 4) {
-        double a = 0.0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); k++) a += S.sh4[threadIdx.x][k];
-        if (P.coop) S.slot4[P.phase][threadIdx.x] = a;
-        else S.tot4[threadIdx.x] = a;
+        for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (P.coop && r == 0) S.slot[ph][q] = a;
+    } else if (w == 2) {
+        while_w2();
     }
     if (P.coop) {
         cg::cluster_group cl = cg::this_cluster();
         cl.sync();
-        if (threadIdx.x < 4) {
-            double tot = 0.0;
-            for (int r = 0; r < kCl; r++) tot += cl.map_shared_rank(&S.slot4[0][0], r)[P.phase * 4 + threadIdx.x];
-            S.tot4[threadIdx.x] = tot;
+        if (w == 0) {
+            a = cl.map_shared_rank(&S.slot[0][0], r)[ph * 4 + q];
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
         }
-        P.phase ^= 1;
+    }
+    if (w == 0) {
+        fin(a);
+        if (r == 0) S.tot[ph][q] = a;
     }
     __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 4; q++) v[q] = S.tot4[q];
-    __syncthreads();
+    P.phase ^= 1;
+}
+
+// The plain sum of one value, the same in every thread.
+__device__ double coop_sum(double v, Smem &S, Part &P) {
+    const double v1[1] = {v};
+    const int ph = P.phase;
+    sums<1>(v1, S, P, [] {}, [](double &) {});
+    return S.tot[ph][0];
 }
 
 // Make every cooperating CTA's writes to the shared vectors visible to all.
@@ -170,11 +185,11 @@ __device__ __forceinline__ void coop_barrier(const Part &P) {
 }
 
 // y[r0:r1] = alpha*A[r0:r1,:]*x (+ beta*y).  x is written by the other CTAs
-// of the cluster during the launch, so it is read at L2 (ld.global.cg), the
-// coherence point, never through the SM-local read-only path.
+// of the cluster during the launch: ordinary loads, ordered by the barrier
+// (release / acquire) that follows the writes, never the read-only path.
 //   mode 0: one thread per row;
-//   mode 1: rows in warp-sized blocks, one thread per row, except that rows
-//           longer than 32 non-zeros are taken by the whole warp in turn
+//   mode 1: rows in warp-sized blocks, 8 lanes per row, except that rows
+//           longer than kTeamRow non-zeros are taken by the whole warp in turn
 //           (lanes stride over the row, shuffle reduction), and rows longer
 //           than kCtaRow (the system's list, ascending) by the whole CTA
 //           after the blocks, so a power-law row of thousands of entries
@@ -191,13 +206,58 @@ __device__ __forceinline__ double row_dot(const int *__restrict__ col,
                   c3 = __ldg(col + k + 3 * step);
         const double v0 = __ldg(val + k), v1 = __ldg(val + k + step), v2 = __ldg(val + k + 2 * step),
                      v3 = __ldg(val + k + 3 * step);
-        s0 = fma(v0, __ldcg(x + c0), s0);
-        s1 = fma(v1, __ldcg(x + c1), s1);
-        s2 = fma(v2, __ldcg(x + c2), s2);
-        s3 = fma(v3, __ldcg(x + c3), s3);
+        s0 = fma(v0, x[c0], s0);
+        s1 = fma(v1, x[c1], s1);
+        s2 = fma(v2, x[c2], s2);
+        s3 = fma(v3, x[c3], s3);
     }
-    for (; k < kb; k += step) s0 = fma(__ldg(val + k), __ldcg(x + __ldg(col + k)), s0);
+    for (; k < kb; k += step) s0 = fma(__ldg(val + k), x[__ldg(col + k)], s0);
     return (s0 + s1) + (s2 + s3);
+}
+
+// The products of a warp's 32 rows (lane l's row is entries [ka, kb), l's
+// result its sum): teams of 8 lanes take 4 rows at a time, 8 times, so a warp's
+// loads of col and val cover whole sectors and only the gathers of x take a
+// cache line per lane.  The 8 partial sums of a lane meet in a transposed tree,
+// 7 adds for the 32 rows, after which lane l holds row l.
+__device__ __forceinline__ double team_dots(const int *__restrict__ col,
+                                            const double *__restrict__ val, const double *x,
+                                            int ka, int kb) {
+    const int lane = threadIdx.x & 31, t = lane & 7, q8 = lane & 24;
+    double s[8];
+    int k[8], e[8];
+#pragma unroll
+    for (int g = 0; g < 8; g++) {
+        k[g] = __shfl_sync(0xffffffffu, ka, q8 + g) + t;
+        e[g] = __shfl_sync(0xffffffffu, kb, q8 + g);
+        s[g] = 0.0;
+    }
+    const int len = __reduce_max_sync(0xffffffffu, kb - ka);
+    for (int it = 0; it < len; it += 8) {
+        int c[8];
+        double v[8], xv[8];
+#pragma unroll
+        for (int g = 0; g < 8; g++) {
+            c[g] = k[g] < e[g] ? __ldg(col + k[g]) : -1;
+            v[g] = k[g] < e[g] ? __ldg(val + k[g]) : 0.0;
+            k[g] += 8;
+        }
+#pragma unroll
+        for (int g = 0; g < 8; g++) xv[g] = c[g] >= 0 ? x[c[g]] : 0.0;
+#pragma unroll
+        for (int g = 0; g < 8; g++)
+            if (c[g] >= 0) s[g] = fma(v[g], xv[g], s[g]);
+    }
+#pragma unroll
+    for (int h = 4; h > 0; h >>= 1) {
+        const bool up = t & h;
+#pragma unroll
+        for (int g = 0; g < h; g++) {
+            const double mine = up ? s[g + h] : s[g], other = up ? s[g] : s[g + h];
+            s[g] = mine + __shfl_xor_sync(0xffffffffu, other, h);
+        }
+    }
+    return s[0];
 }
 
 __device__ void part_spmv(const xb_batch_dev &D, const Part &P, Smem &S, double alpha,
@@ -218,8 +278,8 @@ __device__ void part_spmv(const xb_batch_dev &D, const Part &P, Smem &S, double 
                 kb = __ldg(rp + r + 1);
             }
             const bool cta = kb - ka > kCtaRow;
-            const bool lng = kb - ka > 32 && !cta;
-            double s = (lng || cta) ? 0.0 : row_dot(D.col, D.val, x, ka, kb, 1);
+            const bool lng = kb - ka > kTeamRow && !cta;
+            double s = team_dots(D.col, D.val, x, ka, lng || cta ? ka : kb);
             unsigned todo = __ballot_sync(0xffffffffu, lng);
             while (todo) {
                 const int src = __ffs(todo) - 1;
@@ -255,53 +315,11 @@ __device__ void part_spmv(const xb_batch_dev &D, const Part &P, Smem &S, double 
     __syncthreads();
 }
 
-// One fused MGS pass over rows [r0, r1) of this CTA (four rows per thread in
-// flight): OP 0 returns (w, vn); OP 1 applies w -= c vp and returns (w, vn);
-// OP 2 applies w -= c vp and returns (w, w).
-template <int OP>
-__device__ __forceinline__ double mgs_rows(double *__restrict__ w, const double *__restrict__ vp,
-                                           const double *__restrict__ vn, double c, int r0,
-                                           int r1) {
-    const int S = blockDim.x;
-    double a0 = 0.0, a1 = 0.0;
-    int e = r0 + threadIdx.x;
-    for (; e + 3 * S < r1; e += 4 * S) {
-        double x[4], p[4], q[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) x[u] = w[e + u * S];
-        if (OP != 0) {
-#pragma unroll
-            for (int u = 0; u < 4; u++) p[u] = vp[e + u * S];
-        }
-        if (OP != 2) {
-#pragma unroll
-            for (int u = 0; u < 4; u++) q[u] = vn[e + u * S];
-        }
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            if (OP != 0) x[u] = fma(-c, p[u], x[u]);
-            const double o = OP == 2 ? x[u] : q[u];
-            if (u & 1) a1 = fma(x[u], o, a1);
-            else a0 = fma(x[u], o, a0);
-            if (OP != 0) w[e + u * S] = x[u];
-        }
-    }
-    for (; e < r1; e += S) {
-        double xe = w[e];
-        if (OP != 0) {
-            xe = fma(-c, vp[e], xe);
-            w[e] = xe;
-        }
-        a0 = fma(xe, OP == 2 ? xe : vn[e], a0);
-    }
-    return a0 + a1;
-}
-
 // One block Gram-Schmidt pass over rows [r0, r1): w -= sum_{q < nu} c[q] V_{u0+q}
-// (nu <= 4), then the nd <= 4 dots (w, V_{d0+q}) into a[] (or (w, w) into a[0]
-// when nd == 0).  Two rows per thread, every load of both issued before their
-// arithmetic (the pass is latency-bound on one SM).
-template <int R>
+// (nu <= 4), then the nd <= 4 dots (w, V_{d0+q}) into a[] or, with NORM, (w, w)
+// into a[0] and the nd <= 3 dots into a[1..].  Two rows per thread, every load
+// of both issued before their arithmetic (the pass is latency-bound on one SM).
+template <int R, bool NORM>
 __device__ __forceinline__ void bgs_row(double *__restrict__ w, const double *__restrict__ V,
                                         int64_t ld, int u0, int nu, const double (&c)[4], int d0,
                                         int nd, int e0, int B, double (&a)[4]) {
@@ -322,16 +340,14 @@ __device__ __forceinline__ void bgs_row(double *__restrict__ w, const double *__
         for (int q = 0; q < 4; q++)
             if (q < nu) x[r] = fma(-c[q], pu[r][q], x[r]);
         if (nu > 0) w[e0 + r * B] = x[r];
-        if (nd == 0) {
-            a[0] = fma(x[r], x[r], a[0]);
-        } else {
+        if (NORM) a[0] = fma(x[r], x[r], a[0]);
 #pragma unroll
-            for (int q = 0; q < 4; q++)
-                if (q < nd) a[q] = fma(x[r], pd[r][q], a[q]);
-        }
+        for (int q = 0; q < (NORM ? 3 : 4); q++)
+            if (q < nd) a[NORM ? q + 1 : q] = fma(x[r], pd[r][q], a[NORM ? q + 1 : q]);
     }
 }
 
+template <bool NORM>
 __device__ __forceinline__ void bgs_rows(double *__restrict__ w, const double *__restrict__ V,
                                          int64_t ld, int u0, int nu, const double (&c)[4], int d0,
                                          int nd, int r0, int r1, double (&a)[4]) {
@@ -339,8 +355,8 @@ __device__ __forceinline__ void bgs_rows(double *__restrict__ w, const double *_
     for (int q = 0; q < 4; q++) a[q] = 0.0;
     const int B = blockDim.x;
     int e = r0 + threadIdx.x;
-    for (; e + B < r1; e += 2 * B) bgs_row<2>(w, V, ld, u0, nu, c, d0, nd, e, B, a);
-    if (e < r1) bgs_row<1>(w, V, ld, u0, nu, c, d0, nd, e, B, a);
+    for (; e + B < r1; e += 2 * B) bgs_row<2, NORM>(w, V, ld, u0, nu, c, d0, nd, e, B, a);
+    if (e < r1) bgs_row<1, NORM>(w, V, ld, u0, nu, c, d0, nd, e, B, a);
 }
 
 __device__ void solve_one(const xb_batch_dev &D, Part &P, Smem &S, double tol, int maxiter,
@@ -397,108 +413,172 @@ __device__ void solve_one(const xb_batch_dev &D, Part &P, Smem &S, double tol, i
                     K = 0;
                 }
             }
-            const double ib = 1.0 / beta;
-            for (int i = r0 + threadIdx.x; i < r1; i += blockDim.x) V[i] *= ib;
-            for (int i = threadIdx.x; i <= m; i += blockDim.x) S.g[i] = 0.0;
+            // the basis is stored unnormalised: v_i = sc_i V_i
+            if (threadIdx.x == 0) {
+                S.hn[0] = beta;
+                S.sc[0] = 1.0 / beta;
+            }
             __syncthreads();
-            if (threadIdx.x == 0) S.g[0] = beta;
+            double gj = beta;  // warp 0: entry j of the least-squares right-hand side
+            const double tol_g = tau * bnorm;
+            const int lane = threadIdx.x & 31;
             int k = 0;
             for (int j = 0; j < m; j++) {
                 iters++;
                 double *w = V + (size_t)(j + 1) * ld;
-                coop_barrier(P);  // v_j complete
-                part_spmv(D, P, S, 1.0, V + (size_t)j * ld, 0.0, w);
-                double len2 = 0.0, hn;
-                if (bcgs) {
-                    // BCGS, block length 4: one pass per block applies the previous
-                    // block's projection and takes the dots with this block
-                    double c[4] = {0.0, 0.0, 0.0, 0.0}, a4[4];
-                    int u0 = 0, nu = 0;
-                    for (int d0 = 0; d0 <= j; d0 += 4) {
-                        const int nd = min(4, j + 1 - d0);
-                        bgs_rows(w, V, ld, u0, nu, c, d0, nd, r0, r1, a4);
-                        coop_sum4(a4, S, P);
+                // v_j is complete: the norm's sum (or the residual's) ordered it
+                part_spmv(D, P, S, S.sc[j], V + (size_t)j * ld, 0.0, w);
+                // warp 2 keeps tt, the column's newest entry rotated by the earlier
+                // rotations, and the sum of squares, a block behind
+                double tt = 0.0, len2 = 0.0;
+                int u0 = 0, nu = 0;
+                auto take = [&]() {
+                    for (int q = 0; q < nu; q++) {
+                        const double h = S.hc[u0 + q];
+                        len2 = fma(h, h, len2);
+                        tt = u0 + q == 0 ? h : fma(-S.sn[u0 + q - 1], tt, S.cs[u0 + q - 1] * h);
+                    }
+                };
+                // blocks of 4: one pass and one exchange each.  The dots of a block
+                // are taken with the same w; for MGS they are corrected by the
+                // block's own inner products: (w - sum_{k<i} c_k V_k, V_i) =
+                // (w, V_i) - sum_{k<i} c_k (V_k, V_i), the same method with a quarter
+                // of the exchanges
+                double c[4] = {0.0, 0.0, 0.0, 0.0}, a4[4];
+                for (int d0 = 0; d0 <= j; d0 += 4) {
+                    const int nd = min(4, j + 1 - d0);
+                    bgs_rows<false>(w, V, ld, u0, nu, c, d0, nd, r0, r1, a4);
+                    const int ph = P.phase;
+                    sums<4>(a4, S, P, take, [&](double &t) {
+                        const int q = lane >> 3;
+                        const bool in = q < nd;
+                        const double sq = in ? S.sc[d0 + q] : 0.0;
+                        t = (t * sq) * sq;
+                        if (!bcgs) {
 #pragma unroll
-                        for (int q = 0; q < 4; q++) {
-                            if (q < nd) {
-                                if (threadIdx.x == 0) H[(size_t)j * (m_max + 1) + d0 + q] = a4[q];
-                                len2 += a4[q] * a4[q];
-                                c[q] = a4[q];
+                            for (int i = 0; i < 3; i++) {
+                                const double ci = __shfl_sync(0xffffffffu, t, 8 * i);
+                                if (in && q > i) t = fma(-ci, S.sg[(d0 + q) * 4 + i], t);
                             }
                         }
-                        u0 = d0;
-                        nu = nd;
-                    }
-                    bgs_rows(w, V, ld, u0, nu, c, 0, 0, r0, r1, a4);
-                    hn = sqrt(coop_sum(a4[0], S, P));
-                } else {
-                    // fused MGS: pass i applies the projection on v_{i-1}, takes (w, v_i)
-                    double hprev = 0.0;
-                    for (int i = 0; i <= j; i++) {
-                        const double *vi = V + (size_t)i * ld;
-                        a = i == 0 ? mgs_rows<0>(w, nullptr, vi, 0.0, r0, r1)
-                                   : mgs_rows<1>(w, vi - ld, vi, hprev, r0, r1);
-                        const double h = coop_sum(a, S, P);
-                        if (threadIdx.x == 0) H[(size_t)j * (m_max + 1) + i] = h;
-                        len2 += h * h;
-                        hprev = h;
-                    }
-                    a = mgs_rows<2>(w, V + (size_t)j * ld, nullptr, hprev, r0, r1);
-                    hn = sqrt(coop_sum(a, S, P));
+                        if (in && (lane & 7) == 0) S.hc[d0 + q] = t * S.hn[d0 + q];
+                    });
+#pragma unroll
+                    for (int q = 0; q < 4; q++) c[q] = S.tot[ph][q];
+                    u0 = d0;
+                    nu = nd;
                 }
-                if (threadIdx.x == 0) {
-                    double *col = H + (size_t)j * (m_max + 1);
-                    col[j + 1] = hn;
-                    for (int i = 0; i < j; i++) {
-                        const double c0 = col[i], c1 = col[i + 1];
-                        col[i] = S.cs[i] * c0 + S.sn[i] * c1;
-                        col[i + 1] = -S.sn[i] * c0 + S.cs[i] * c1;
+                // the last projection, ||w||^2 and, for MGS, w's products with the
+                // basis vectors it will share a block with
+                const int ng = bcgs || j + 1 >= m ? 0 : (j + 1) & 3, g0 = j + 1 - ng;
+                bgs_rows<true>(w, V, ld, u0, nu, c, g0, ng, r0, r1, a4);
+                sums<4>(a4, S, P,
+                        [&]() {
+                            take();
+                            if (lane == 0) {
+                                S.tt = tt;
+                                S.len2 = len2;
+                            }
+                            double *col = H + (size_t)j * (m_max + 1);
+                            for (int i = lane; i <= j; i += 32) col[i] = S.hc[i];
+                        },
+                        [&](double &) {});
+                // the new rotation (warp 0): both reciprocal roots in one sequence;
+                // hypot where the square leaves the range in which it is exact enough
+                if (threadIdx.x < 32) {
+                    const double *tot = S.tot[P.phase ^ 1];
+                    const double t0 = S.tt, hn2 = tot[0], rr2 = fma(t0, t0, hn2);
+                    const double root = rsqrt(lane == 0 ? hn2 : rr2);
+                    const double ihn = hn2 > 0.0 ? __shfl_sync(0xffffffffu, root, 0) : 0.0;
+                    const double irr = __shfl_sync(0xffffffffu, root, 1);
+                    const double hnj = hn2 * ihn;
+                    double rr = rr2 * irr, c1 = t0 * irr, s1 = hnj * irr;
+                    if (!(rr2 > 1e-280 && rr2 < 1e300)) {
+                        rr = hypot(t0, hnj);
+                        c1 = t0 / rr;
+                        s1 = hnj / rr;
                     }
-                    const double c0 = col[j];
-                    const double rr = hypot(c0, hn);
                     int flag = 0;
                     if (rr == 0.0) {
                         flag = 2;
                     } else {
-                        S.cs[j] = c0 / rr;
-                        S.sn[j] = hn / rr;
-                        col[j] = rr;
-                        col[j + 1] = 0.0;
-                        S.g[j + 1] = -S.sn[j] * S.g[j];
-                        S.g[j] = S.cs[j] * S.g[j];
-                        if (hn <= 1e-14 * sqrt(len2 + hn * hn)) flag = 1;
-                        else if (fabs(S.g[j + 1]) / bnorm <= tau) flag = 3;
+                        if (lane == 0) {
+                            S.cs[j] = c1;
+                            S.sn[j] = s1;
+                            S.g[j] = c1 * gj;
+                            H[(size_t)j * (m_max + 1) + j + 1] = rr;  // the diagonal, until the restart
+                            S.hn[j + 1] = hnj;
+                            S.sc[j + 1] = ihn;
+                        }
+                        if (lane < ng) S.sg[(j + 1) * 4 + lane] = (tot[1 + lane] * ihn) * ihn;
+                        gj = -s1 * gj;
+                        if (hn2 <= 1e-28 * (S.len2 + hn2)) flag = 1;  // hn <= 1e-14 |column|
+                        else if (fabs(gj) <= tol_g) flag = 3;
                     }
-                    S.flag = flag;
+                    if (lane == 0) S.flag = flag;
                 }
                 __syncthreads();
                 const int flag = S.flag;
-                __syncthreads();
                 if (flag == 2) {
                     k = j;
                     status = XB_EBREAKDOWN;
                     break;
                 }
                 k = j + 1;
-                if (flag == 1) {
-                    claimed = 1;
-                    break;
-                }
-                const double ih = 1.0 / hn;
-                for (int e = r0 + threadIdx.x; e < r1; e += blockDim.x) w[e] *= ih;
-                if (flag == 3) {
+                if (flag != 0) {
                     claimed = 1;
                     break;
                 }
                 if (iters >= maxiter) break;
             }
             if (status == XB_EBREAKDOWN) break;
-            // R y = g (every cooperating CTA holds the same R and g), x += V y
-            if (threadIdx.x == 0) {
+            // R y = g by columns on warp 0 (lane c holds g_c and 1 / R_cc; every
+            // cooperating CTA holds the same R and g), then x += sum y_i sc_i V_i
+            if (threadIdx.x < 32) {
+                constexpr int QM = (XB_BATCH_MAX_M + 31) / 32;
+                const int ldh = m_max + 1;
+                // lane c rotates column c's entries with G_0..G_{c-1} (the arithmetic
+                // of the steps' running value) and moves its diagonal into place
+#pragma unroll
+                for (int q = 0; q < QM; q++) {
+                    const int cc = lane + 32 * q;
+                    if (cc < k) {
+                        double *col = H + (size_t)cc * ldh;
+                        double tr = col[0];
+                        for (int i = 1; i <= cc; i++) {
+                            const double hi = col[i], cg_ = S.cs[i - 1], sg_ = S.sn[i - 1];
+                            col[i - 1] = fma(cg_, tr, sg_ * hi);
+                            tr = fma(-sg_, tr, cg_ * hi);
+                        }
+                        col[cc] = col[cc + 1];
+                    }
+                }
+                __syncwarp();
+                double gl[QM], dl[QM], hv[QM];
+#pragma unroll
+                for (int q = 0; q < QM; q++) {
+                    const int cc = lane + 32 * q;
+                    gl[q] = cc < k ? S.g[cc] : 0.0;
+                    dl[q] = cc < k ? 1.0 / H[(size_t)cc * ldh + cc] : 0.0;
+                    hv[q] = k > 0 && cc < k - 1 ? H[(size_t)(k - 1) * ldh + cc] : 0.0;
+                }
                 for (int i = k - 1; i >= 0; i--) {
-                    double s = S.g[i];
-                    for (int c = i + 1; c < k; c++) s -= H[(size_t)c * (m_max + 1) + i] * S.yv[c];
-                    S.yv[i] = s / H[(size_t)i * (m_max + 1) + i];
+                    const int qi = i >> 5, li = i & 31;
+                    double gs = gl[0], ds = dl[0];
+#pragma unroll
+                    for (int q = 1; q < QM; q++)
+                        if (qi == q) {
+                            gs = gl[q];
+                            ds = dl[q];
+                        }
+                    const double yi = __shfl_sync(0xffffffffu, gs, li) * __shfl_sync(0xffffffffu, ds, li);
+                    if (lane == 0) S.yv[i] = yi * S.sc[i];
+#pragma unroll
+                    for (int q = 0; q < QM; q++) {
+                        const int cc = lane + 32 * q;
+                        if (32 * q < i && cc < i) gl[q] = fma(-hv[q], yi, gl[q]);
+                        hv[q] = cc < i - 1 ? H[(size_t)(i - 1) * ldh + cc] : 0.0;  // the next column
+                    }
                 }
             }
             __syncthreads();
@@ -596,6 +676,76 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kBT, 1)
         phase1();
         phase2();
     }
+}
+
+// Whole clusters of the kernel that fit on the GPU at once.
+int resident_clusters() {
+    cudaLaunchConfig_t lc;
+    std::memset(&lc, 0, sizeof lc);
+    lc.gridDim = dim3(kCl, 1, 1);
+    lc.blockDim = dim3(kBT, 1, 1);
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, (void *)k_batch_gmres, &lc) != cudaSuccess || clusters < 1) {
+        cudaGetLastError();
+        clusters = xb::num_sms() / kCl;
+    }
+    return std::max(1, clusters);
+}
+
+// Estimated time of an Arnoldi step, in us, at the cycle's mean basis size m / 2:
+// 2 + m / 8 sums at 2 us (3 us across a cluster), and n m + 2 nnz FP64 terms (4 nnz
+// for mode 1's uneven rows) at 0.4 ns a CTA, with a fifth lost to the split over a
+// cluster's 8.  Fitted to 48 systems of 1000 to 57,000 rows at m = 30 (one CTA 28 to
+// 1300 us, a cluster 18 to 200 us a step).
+double step_us(const xb_batch_dev &d, bool cluster) {
+    const double sums = 2.0 + d.m / 8.0,
+                 terms = 4e-4 * ((double)d.m * d.n + (d.mode == 1 ? 4.0 : 2.0) * d.nnz);
+    return cluster ? 3.0 * sums + 1.2 * terms / kCl : 2.0 * sums + terms;
+}
+
+// Decides which systems a whole cluster solves and returns the order of the
+// queues: the cluster's systems first, each part largest first, so that the long
+// solves start in the first wave.  A cluster solves a system sooner but at up to 8
+// times the SM time, so the k largest go to clusters with the k whose estimated
+// end is first: no earlier than the longest cluster solve, than the longest
+// single-CTA one, and than all the work spread over the resident CTAs (equal
+// step counts assumed).  Few systems thus all go to clusters, many small ones
+// to a CTA each.  The environment variable XB_BATCH_COOP_MIN_N sets a number of
+// rows from which on a cluster takes a system instead.
+std::vector<int> split_systems(std::vector<xb_batch_dev> &h, int clusters) {
+    const int count = (int)h.size();
+    std::vector<int> order(count);
+    std::iota(order.begin(), order.end(), 0);
+    const char *env = std::getenv("XB_BATCH_COOP_MIN_N");
+    if (env) {
+        const long coop_min = std::max(1L, std::atol(env));
+        for (xb_batch_dev &d : h) d.coop = d.n >= coop_min ? 1 : 0;
+        std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+            if (h[a].coop != h[b].coop) return h[a].coop > h[b].coop;
+            return step_us(h[a], false) > step_us(h[b], false);
+        });
+        return order;
+    }
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int a, int b) { return step_us(h[a], false) > step_us(h[b], false); });
+    double spread = 0.0;  // SM time of all systems with the first k in clusters
+    for (const xb_batch_dev &d : h) spread += step_us(d, false);
+    double best = 0.0, longest = 0.0;
+    int take = 0;
+    for (int k = 0; k <= count; k++) {
+        const double alone = k < count ? step_us(h[order[k]], false) : 0.0;
+        const double end = std::max({longest, alone, spread / (kCl * clusters)});
+        if (k == 0 || end < best) {
+            best = end;
+            take = k;
+        }
+        if (k == count) break;
+        const double c = step_us(h[order[k]], true);
+        longest = std::max(longest, c);
+        spread += kCl * c - alone;
+    }
+    for (int k = 0; k < count; k++) h[order[k]].coop = k < take ? 1 : 0;
+    return order;
 }
 
 }  // namespace
@@ -716,10 +866,6 @@ int xb_batch_create(int32_t count, const xb_batch_sys *sys, const xb_options *op
         return xb::set_error(XB_EINVAL, "batch_create: orthogonalisation must be MGS, BCGS or AUTO");
     std::vector<xb_batch_dev> h(count);
     size_t ws = 0;
-    // systems with n >= coop_min are solved by a whole cluster (environment
-    // variable XB_BATCH_COOP_MIN_N overrides the default)
-    long coop_min = kLargeN;
-    if (const char *env = std::getenv("XB_BATCH_COOP_MIN_N")) coop_min = std::max(1L, std::atol(env));
     for (int i = 0; i < count; i++) {
         const xb_batch_sys &q = sys[i];
         if (q.n < 0 || q.nnz < 0 || q.m < 1 || q.m > XB_BATCH_MAX_M || (q.mode != 0 && q.mode != 1) ||
@@ -733,15 +879,17 @@ int xb_batch_create(int32_t count, const xb_batch_sys *sys, const xb_options *op
         d.m_max = o.dafrt ? std::max(q.m, std::min(o.m_max, XB_BATCH_MAX_M)) : q.m;
         d.mode = q.mode;
         d.zero_x = q.zero_x;
-        d.coop = q.n >= coop_min ? 1 : 0;
         d.ld = ((int64_t)q.n + 31) / 32 * 32;
         d.rowptr = q.rowptr;
         d.col = q.col;
         d.val = q.val;
         d.b = q.b;
         d.x = q.x;
-        ws += (size_t)(d.m_max + 1) * d.ld + (size_t)(d.coop ? kCl : 1) * (d.m_max + 1) * d.m_max + 32;
     }
+    const int clusters = resident_clusters();
+    const std::vector<int> order = split_systems(h, clusters);
+    for (const xb_batch_dev &d : h)
+        ws += (size_t)(d.m_max + 1) * d.ld + (size_t)(d.coop ? kCl : 1) * (d.m_max + 1) * d.m_max + 32;
     // mode 1: each system's rows longer than kCtaRow (summed by a whole CTA),
     // from a host copy of its row pointer
     std::vector<int> lr_all, rp_h;
@@ -786,14 +934,6 @@ int xb_batch_create(int32_t count, const xb_batch_sys *sys, const xb_options *op
         h[i].H = bt->d_ws + off;
         off += (size_t)(h[i].coop ? kCl : 1) * (h[i].m_max + 1) * h[i].m_max + 32;
     }
-    // the cluster systems first, then the single-CTA ones, each part
-    // largest first: the long solves start in the first wave
-    std::vector<int> order(count);
-    std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-        if (h[a].coop != h[b].coop) return h[a].coop > h[b].coop;
-        return (int64_t)h[a].nnz + h[a].n > (int64_t)h[b].nnz + h[b].n;
-    });
     int nbig = 0;
     for (int i = 0; i < count; i++) nbig += h[i].coop ? 1 : 0;
     e = cudaMalloc(&bt->d_sys, std::max(count, 1) * sizeof(xb_batch_dev));
@@ -805,30 +945,14 @@ int xb_batch_create(int32_t count, const xb_batch_sys *sys, const xb_options *op
     if (e == cudaSuccess && count > 0)
         e = cudaMemcpy(bt->d_order, order.data(), count * sizeof(int), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return fail(xb::cuda_error(e, "batch_create"));
-    // persistent grid: as many whole clusters as can be co-resident
-    cudaLaunchConfig_t lc;
-    std::memset(&lc, 0, sizeof lc);
-    lc.gridDim = dim3(kCl, 1, 1);
-    lc.blockDim = dim3(kBT, 1, 1);
-    int clusters = 0;
-    e = cudaOccupancyMaxActiveClusters(&clusters, (void *)k_batch_gmres, &lc);
-    if (e != cudaSuccess || clusters < 1) {
-        cudaGetLastError();
-        clusters = std::max(1, xb::num_sms() / kCl);
-    }
-    bt->grid = kCl * std::max(1, clusters);
+    bt->grid = kCl * clusters;  // persistent: as many whole clusters as can be co-resident
     // clusters that take the single-CTA systems from the start: their share
-    // of the work, with nnz + m n (one step's SpMV and Gram-Schmidt) as the
-    // per-system weight; none without cluster systems to balance against
+    // of the work; none without cluster systems to balance against
     double w_big = 0.0, w_small = 0.0;
-    for (int i = 0; i < count; i++) {
-        const double wi = (double)h[i].nnz + (double)h[i].m * h[i].n;
-        (h[i].coop ? w_big : w_small) += wi;
-    }
-    const int ncl = std::max(1, clusters);
+    for (const xb_batch_dev &d : h) (d.coop ? w_big : w_small) += d.coop ? kCl * step_us(d, true) : step_us(d, false);
     int nsmall_cl = 0;
     if (nbig > 0 && w_small > 0.0)
-        nsmall_cl = std::min(ncl - 1, (int)std::lround(ncl * w_small / (w_big + w_small)));
+        nsmall_cl = std::min(clusters - 1, (int)std::lround(clusters * w_small / (w_big + w_small)));
     const unsigned long long budget = (unsigned long long)(std::min(o.maxtime_s, 3600.0) * 1e9);
     const double theta = o.dafrt ? o.dafrt_theta : 0.0;  // theta 0: the rule never fires
     // orthogonalisation: MGS or BCGS (block length 4); the accuracy policy's

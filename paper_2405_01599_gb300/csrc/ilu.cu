@@ -181,7 +181,8 @@ __global__ void k_diag_fill(int n, const int *__restrict__ rows, const int *__re
 // Both substitutions in one cooperative launch without barriers between
 // levels.  CTA c owns a block of consecutive rows, in both triangles, and takes
 // its rows in level order as items: up to 32 rows of one level (a lane each),
-// or one long row (the warp).  A row's value is published as soon as it is
+// or fewer rows with 2 to 32 lanes each, so that no lane has more than four
+// entries, or one longer row (the warp).  A row's value is published as soon as it is
 // formed and a row waits for the very values it needs: those of the CTA's own
 // rows in shared memory, the others in device memory, where a value travels as
 // two 8-byte words that both carry the number of the application (so nothing
@@ -193,9 +194,16 @@ __global__ void k_diag_fill(int n, const int *__restrict__ rows, const int *__re
 // replaces took ~6 us and a kernel per level ~4 us.  Consecutive rows per CTA
 // keep most hops of a stencil inside a CTA.  One application (GB300; the graph
 // of level launches or the level barrier, whichever was faster, in brackets):
-// 96^3 convection-diffusion 0.71 ms (2.0), 30^3 0.13 (0.44), 180^3 (blocks too
-// large for shared memory) 3.8 (4.3), power-law rows n = 20,000 0.46 (1.1), n =
-// 1M 1.03 (3.4).
+// 96^3 convection-diffusion 0.67 ms (2.0), 30^3 0.11 (0.44), 180^3 (blocks too
+// large for shared memory) 2.6 (4.3), power-law rows n = 20,000 0.16 (1.1), n =
+// 1M 0.50 (3.4).
+//
+// Four entries a lane: an item is one round of loads and waits.  With a lane for
+// a row of up to 32 entries (up to 5 rounds of ~2 us, and the rows of a power law's
+// late levels are long) n = 1M took 1.04 ms, n = 20,000 0.46; with 2 / 3 / 6 entries
+// a lane n = 1M takes 0.76 / 0.54 / 0.49, n = 20,000 0.23 / 0.18 / 0.19.  The lanes'
+// sums meet in a tree: against exact arithmetic 4.5e-17 of ||z||, one by one 4.6e-17
+// (power law, n = 200,000).
 //
 // Every wait ends: warps take a CTA's items in level order, so of the rows not
 // yet done in the whole grid those of the lowest level wait for nothing; and a
@@ -204,13 +212,13 @@ __global__ void k_diag_fill(int n, const int *__restrict__ rows, const int *__re
 constexpr int kFlowWarps = 16;
 constexpr int kFlowMinRows = 2048;  // rows of a CTA below which fewer CTAs do (30^3 grid: 122 us
                                     // with 2048, 140 with 1024, 170 with 512)
-constexpr int kFlowShort = 32;   // triangle entries above which a row gets a warp
-constexpr int kFlowFirst = 4;    // entries of each kind a row starts with
-constexpr int kFlowGroup = 8;    // further remote entries loaded together
+constexpr int kFlowFirst = 4;    // entries of each kind a lane has: all on their way at once
+constexpr int kFlowGroup = 8;    // entries a lane loads together in such a row
 constexpr unsigned long long kNotReady = 0xffffffffffffffffull;  // a NaN that is never stored
 
 struct FlowTri {
-    const int4 *items;      // {first slot, rows | long << 8, remote | local entries << 16, entries from ebase}
+    const int4 *items;      // {first slot, rows | long << 8 | log2(lanes of a row) << 9,
+                            //  a lane's remote | local entries << 16, entries from ebase}
     const int *iptr;        // per CTA: its items
     const long long *ebase; // per CTA: its entries
     const int *rows;        // slot -> row
@@ -280,39 +288,38 @@ __device__ __forceinline__ bool flow_ready(double x) {
     return __double2hiint(x) != -1;  // kNotReady's high word; no value that is stored has it
 }
 
-// s + the sum of the item's m <= kFlowFirst local entries; false when a wait ran
-// out (warp-uniform, as all below).  The first entry is polled alone: a warp
+// s + the sum of M local entries a lane; false when a wait ran out (warp-uniform,
+// as all below).  The first entry is polled alone: a warp
 // that waits reads one word a poll and leaves the shared memory to the others.
-__device__ __forceinline__ bool flow_local(const FlowArgs &a, const volatile double *zs, int m,
+template <int M>
+__device__ __forceinline__ bool flow_local(const FlowArgs &a, const volatile double *zs,
                                            const int (&c)[kFlowFirst], const double (&v)[kFlowFirst],
                                            double &s) {
     FlowWait w;
-    double x[kFlowFirst];
+    double x[M];
     while (x[0] = zs[c[0]], !__all_sync(0xffffffffu, flow_ready(x[0])))
         if (!w.more(a)) return false;
-    if (m > 1) {
+    if constexpr (M > 1) {
         for (;;) {
             bool all = true;
 #pragma unroll
-            for (int q = 1; q < kFlowFirst; q++)
-                if (q < m) {
-                    x[q] = zs[c[q]];
-                    all = all && flow_ready(x[q]);
-                }
+            for (int q = 1; q < M; q++) {
+                x[q] = zs[c[q]];
+                all = all && flow_ready(x[q]);
+            }
             if (__all_sync(0xffffffffu, all)) break;
             if (!w.more(a)) return false;
         }
     }
 #pragma unroll
-    for (int q = 0; q < kFlowFirst; q++)
-        if (q < m) s = fma(v[q], x[q], s);
+    for (int q = 0; q < M; q++) s = fma(v[q], x[q], s);
     return true;
 }
 
-// The same for values in device memory (c < 0: none).
-template <int N>
-__device__ __forceinline__ bool flow_remote(const FlowArgs &a, const ulonglong2 *tag, const int (&c)[N],
-                                            const double (&v)[N], double &s) {
+// The same for the first N values in device memory (c < 0: none).
+template <int N, int C>
+__device__ __forceinline__ bool flow_remote(const FlowArgs &a, const ulonglong2 *tag, const int (&c)[C],
+                                            const double (&v)[C], double &s) {
     FlowWait w;
     double x[N];
     bool miss[N];
@@ -340,34 +347,40 @@ __device__ __forceinline__ bool flow_remote(const FlowArgs &a, const ulonglong2 
 template <bool FWD>
 __device__ __forceinline__ bool flow_item(const FlowArgs &a, const FlowTri &t, int4 it, long long ebase,
                                           int r0, int nr, double *zs, bool held, int lane) {
-    const int cnt = it.y & 0xff, gw = it.z & 0xffff, lw = it.z >> 16;
+    const int team = it.y >> 9 & 7, cnt = (it.y & 0xff) << team, gw = it.z & 0xffff, lw = it.z >> 16;
     ulonglong2 *tag = FWD ? a.ty : a.tz;
     int row = -1;
     double s = 0.0, b = 0.0, d = 1.0, rd = 1.0;
-    if (lane < cnt) {
-        row = __ldg(t.rows + it.x + lane);
+    if (lane < cnt && (lane & ((1 << team) - 1)) == 0) {  // the row's first lane ends it
+        const int at = it.x + (lane >> team);
+        row = __ldg(t.rows + at);
         if (FWD) {
             b = __ldg(a.r + row);
         } else {
             flow_get(a.ty + row, a.seq, b);  // this CTA's, complete since its barrier
-            d = __ldg(t.diag + it.x + lane);
-            rd = __ldg(t.rdiag + it.x + lane);
+            d = __ldg(t.diag + at);
+            rd = __ldg(t.rdiag + at);
         }
     }
-    int k0 = 0, k1 = gw, step = kFlowGroup;
-    const bool lng = it.y & 256;
-    const long long e = ebase + it.w + lane;
-    int cl[kFlowFirst];
-    double vl[kFlowFirst];
-    if (lng) {  // the lanes take the row's entries in turn
+    if (it.y & 256) {  // the lanes take the row's entries in turn
         const int i = __shfl_sync(0xffffffffu, row, 0), dp = __ldg(a.dpos + i);
-        k0 = FWD ? __ldg(a.rp + i) : dp + 1;
-        k1 = FWD ? dp : __ldg(a.rp + i + 1);
-        step = 32 * kFlowGroup;
+        const int k1 = FWD ? dp : __ldg(a.rp + i + 1);
+        for (int k = FWD ? __ldg(a.rp + i) : dp + 1; k < k1; k += 32 * kFlowGroup) {
+            int c[kFlowGroup];
+            double v[kFlowGroup];
+#pragma unroll
+            for (int q = 0; q < kFlowGroup; q++) {
+                const int at = k + q * 32 + lane;
+                c[q] = at < k1 ? __ldg(a.ci + at) : -1;
+                v[q] = at < k1 ? __ldg(a.lu + at) : 0.0;
+            }
+            if (!flow_remote<kFlowGroup>(a, tag, c, v, s)) return false;
+        }
     } else {
-        // the first entries of both kinds, on their way before the first wait
-        int c[kFlowFirst];
-        double v[kFlowFirst];
+        // the entries of both kinds, on their way before the first wait
+        const long long e = ebase + it.w + lane;
+        int c[kFlowFirst], cl[kFlowFirst];
+        double v[kFlowFirst], vl[kFlowFirst];
 #pragma unroll
         for (int q = 0; q < kFlowFirst; q++) {
             const bool in = q < gw && lane < cnt;
@@ -381,37 +394,17 @@ __device__ __forceinline__ bool flow_item(const FlowArgs &a, const FlowTri &t, i
             vl[q] = in ? __ldg(t.eval + e + (gw + q) * cnt) : 0.0;
             if (cl[q] < 0) cl[q] = nr;  // zs[nr] is 0, and ready
         }
-        if (gw > 0 && !flow_remote<kFlowFirst>(a, tag, c, v, s)) return false;
-        k0 = kFlowFirst;
+        // the code for just as many: a poll's instructions are part of the hop
+        if (gw > 0 && !(gw == 1   ? flow_remote<1>(a, tag, c, v, s)
+                        : gw == 2 ? flow_remote<2>(a, tag, c, v, s)
+                                  : flow_remote<kFlowFirst>(a, tag, c, v, s)))
+            return false;
+        if (lw > 0 && !(lw == 1   ? flow_local<1>(a, zs, cl, vl, s)
+                        : lw == 2 ? flow_local<2>(a, zs, cl, vl, s)
+                                  : flow_local<kFlowFirst>(a, zs, cl, vl, s)))
+            return false;
     }
-    for (int k = k0; k < k1; k += step) {  // warp-uniform: further remote entries
-        int c[kFlowGroup];
-        double v[kFlowGroup];
-#pragma unroll
-        for (int q = 0; q < kFlowGroup; q++) {
-            const int at = lng ? k + q * 32 + lane : k + q;
-            const bool in = at < k1 && (lng || lane < cnt);
-            const long long p = lng ? at : e + (long long)at * cnt;
-            c[q] = in ? __ldg((lng ? a.ci : t.ecol) + p) : -1;
-            v[q] = in ? __ldg((lng ? a.lu : t.eval) + p) : 0.0;
-        }
-        if (!flow_remote<kFlowGroup>(a, tag, c, v, s)) return false;
-    }
-    if (lng) {
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    }
-    for (int t0 = 0; t0 < lw; t0 += kFlowFirst) {
-        if (t0 > 0) {
-#pragma unroll
-            for (int q = 0; q < kFlowFirst; q++) {
-                const bool in = t0 + q < lw && lane < cnt;
-                cl[q] = in ? __ldg(t.ecol + e + (long long)(gw + t0 + q) * cnt) : -1;
-                vl[q] = in ? __ldg(t.eval + e + (long long)(gw + t0 + q) * cnt) : 0.0;
-                if (cl[q] < 0) cl[q] = nr;
-            }
-        }
-        if (!flow_local(a, zs, min(kFlowFirst, lw - t0), cl, vl, s)) return false;
-    }
+    for (int o = 1 << team >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (row >= 0) {
         s = b - s;  // one rounding at the size of b, however many entries
         if (!FWD) s = flow_quot(s, d, rd);
@@ -551,7 +544,7 @@ struct FlowHost {
 template <typename Beg, typename End>
 void flow_blocks(const std::vector<int> &lev, const std::vector<int> &bstart, int c0, int c1, int cap,
                  const int *ci, Beg beg, End end, int *rows, FlowHost &h) {
-    std::vector<int> lng, shrt, cnt, order;
+    std::vector<int> team[7], cnt, order;  // a level's rows by log2 of their lanes; 6: long
     for (int c = c0; c < c1; c++) {
         const int r0 = bstart[c], r1 = bstart[c + 1], nr = r1 - r0;
         const bool held = nr <= cap;
@@ -571,57 +564,58 @@ void flow_blocks(const std::vector<int> &lev, const std::vector<int> &bstart, in
             std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return lev[x] < lev[y]; });
         }
         const size_t ebase = h.ecol.size();
+        // rows of an item with a lane each: where the values of a block leave the L1
+        // less than the lines that 16 warps have on their way, or every value comes
+        // from device memory, smaller items wait less (96^3 grid, 5,800 rows a block,
+        // items of 32 / 16 / 8: 661 / 663 / 696 us; 150^3, 22,000 rows 1377 / 1404 /
+        // 1552; 160^3, 27,000 rows 2483 / 1868 / 1828; 100 x 200 x 200 1749 / 1588 /
+        // 1943; 180^3, not held 3986 / 2743 / 2516)
+        const int rows1 = !held ? 8 : nr > 24000 ? 16 : 32;
         for (int a = 0; a < nr;) {  // one level
-            int b = a, least = INT_MAX, most = 0;
-            shrt.clear();
-            lng.clear();
+            int b = a;
+            for (std::vector<int> &v : team) v.clear();
             for (; b < nr && lev[order[b]] == lev[order[a]]; b++) {
                 const int len = end(order[b]) - beg(order[b]);
-                if (len > kFlowShort) {
-                    lng.push_back(order[b]);
-                } else {
-                    shrt.push_back(order[b]);
-                    least = std::min(least, len);
-                    most = std::max(most, len);
-                }
+                int g = 0;
+                while (g < 6 && len > kFlowFirst << g) g++;
+                team[g].push_back(order[b]);
             }
             // long rows first: they take longest
-            for (size_t q = 0; q < lng.size(); q++) {
-                rows[r0 + a + q] = lng[q];
-                h.items.push_back(make_int4(r0 + a + (int)q, 1 | 256, 0, 0));
+            for (int i : team[6]) {
+                rows[r0 + a] = i;
+                h.items.push_back(make_int4(r0 + a++, 1 | 256 | 5 << 9, 0, 0));
             }
-            a += (int)lng.size();
-            // rows of about equal length share an item
-            if (most > least && shrt.size() > 32)
-                std::stable_sort(shrt.begin(), shrt.end(),
-                                 [&](int x, int y) { return end(x) - beg(x) < end(y) - beg(y); });
-            for (size_t q0 = 0; q0 < shrt.size(); q0 += 32) {
-                const int m = (int)std::min<size_t>(32, shrt.size() - q0);
-                int gw = 0, lw = 0;
-                for (int q = 0; q < m; q++) {
-                    const int i = shrt[q0 + q], kb = end(i);
-                    rows[r0 + a + q] = i;
-                    int l = 0;
-                    for (int k = beg(i); k < kb; k++) l += held && ci[k] >= r0 && ci[k] < r1;
-                    gw = std::max(gw, kb - beg(i) - l);
-                    lw = std::max(lw, l);
-                }
-                const size_t e = h.ecol.size();
-                h.ecol.resize(e + (size_t)(gw + lw) * m, -1);
-                h.esrc.resize(e + (size_t)(gw + lw) * m, -1);
-                int *ec = h.ecol.data() + e, *es = h.esrc.data() + e;
-                for (int q = 0; q < m; q++) {
-                    const int i = shrt[q0 + q], kb = end(i);
-                    int g = 0, l = gw;
-                    for (int k = beg(i); k < kb; k++) {
-                        const bool in = held && ci[k] >= r0 && ci[k] < r1;
-                        const int at = (in ? l++ : g++) * m + q;
-                        ec[at] = in ? ci[k] - r0 : ci[k];
-                        es[at] = k;
+            for (int g = 5; g >= 0; g--) {
+                const std::vector<int> &set = team[g];
+                const int T = 1 << g, most = g > 0 ? 32 >> g : rows1;
+                for (size_t q0 = 0; q0 < set.size(); q0 += most) {
+                    const int m = (int)std::min<size_t>(most, set.size() - q0), wide = m << g;
+                    int gw = 0, lw = 0;
+                    for (int q = 0; q < m; q++) {
+                        const int i = set[q0 + q], kb = end(i);
+                        rows[r0 + a + q] = i;
+                        int l = 0;
+                        for (int k = beg(i); k < kb; k++) l += held && ci[k] >= r0 && ci[k] < r1;
+                        gw = std::max(gw, (kb - beg(i) - l + T - 1) >> g);
+                        lw = std::max(lw, (l + T - 1) >> g);
                     }
+                    const size_t e = h.ecol.size();
+                    h.ecol.resize(e + (size_t)(gw + lw) * wide, -1);
+                    h.esrc.resize(e + (size_t)(gw + lw) * wide, -1);
+                    int *ec = h.ecol.data() + e, *es = h.esrc.data() + e;
+                    for (int q = 0; q < m; q++) {
+                        const int i = set[q0 + q], kb = end(i);
+                        int gn = 0, ln = gw << g;  // row q's entry x: lane x mod T of its T, turn x / T
+                        for (int k = beg(i); k < kb; k++) {
+                            const bool in = held && ci[k] >= r0 && ci[k] < r1;
+                            const int x = in ? ln++ : gn++, at = (x >> g) * wide + (q << g) + (x & (T - 1));
+                            ec[at] = in ? ci[k] - r0 : ci[k];
+                            es[at] = k;
+                        }
+                    }
+                    h.items.push_back(make_int4(r0 + a, m | g << 9, gw | lw << 16, (int)(e - ebase)));
+                    a += m;
                 }
-                h.items.push_back(make_int4(r0 + a, m, gw | lw << 16, (int)(e - ebase)));
-                a += m;
             }
         }
         h.iptr.push_back((int)h.items.size());

@@ -40,8 +40,7 @@ namespace cg = cooperative_groups;
 namespace {
 constexpr int kCl = 8;          // CTAs per cluster
 constexpr int kBT = 512;        // threads per CTA
-constexpr int kTeamRow = 64;    // mode 1: rows longer than this are summed by a whole warp
-constexpr int kCtaRow = 1024;   // mode 1: rows longer than this are summed by the whole CTA
+constexpr int kTile = 256;      // mode 1: entries a warp sums at a time, 8 a lane
 }  // namespace
 
 struct xb_batch_dev {
@@ -52,8 +51,12 @@ struct xb_batch_dev {
     double *x;
     double *V;  // (m_max+1) * ld basis
     double *H;  // per cooperating CTA: (m_max+1) * m_max Hessenberg (column-major)
-    const int *lrows;  // mode 1: the rows longer than kCtaRow, ascending
-    int nl;
+    // mode 1: tiles of kTile entries of each CTA's part of the rows; part c has
+    // tiles tptr[c] .. tptr[c + 1]
+    int tptr[kCl + 1];
+    const int *trow;  // row of a tile's first entry
+    int *tinfo;       // row that a tile ends but does not start; -2: none, -1: ends no row
+    double2 *tsum;    // sums of that row's entries in the tile, and of the entries after the last end
 };
 
 struct xb_batch {
@@ -62,7 +65,7 @@ struct xb_batch {
     xb_batch_info *d_info = nullptr;
     int *d_order = nullptr, *d_queue = nullptr;
     double *d_ws = nullptr;
-    int *d_lrows = nullptr;
+    void *d_tiles = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     int grid = 0;
@@ -79,7 +82,6 @@ __device__ __forceinline__ unsigned long long gtimer() {
 constexpr int kNW = kBT / 32;
 
 struct Smem {
-    double sh[40];                                   // cta_sum (long rows)
     double part[2][4][kNW], slot[2][4], tot[2][4];   // sums of up to 4 values, two phases
     double g[XB_BATCH_MAX_M + 1], cs[XB_BATCH_MAX_M], sn[XB_BATCH_MAX_M], yv[XB_BATCH_MAX_M];
     double hc[XB_BATCH_MAX_M + 2];                   // the step's Hessenberg column, unrotated
@@ -90,22 +92,6 @@ struct Smem {
     int q;
     int flag;
 };
-
-// Sum over the CTA, result returned to every thread.
-__device__ double cta_sum(double v, Smem &S) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if (lane == 0) S.sh[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        v = lane < (int)(blockDim.x >> 5) ? S.sh[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) S.sh[32] = v;
-    }
-    __syncthreads();
-    return S.sh[32];
-}
 
 // The solve's view of the work: rows [r0, r1) of this CTA, and whether the
 // CTAs of the cluster cooperate on this system.
@@ -184,131 +170,163 @@ __device__ __forceinline__ void coop_barrier(const Part &P) {
     else __syncthreads();
 }
 
-// y[r0:r1] = alpha*A[r0:r1,:]*x (+ beta*y).  x is written by the other CTAs
+// y[r0:r1] = alpha*A[r0:r1,:]*x (+ beta*y), beta 0 or 1.  x is written by the other CTAs
 // of the cluster during the launch: ordinary loads, ordered by the barrier
 // (release / acquire) that follows the writes, never the read-only path.
 //   mode 0: one thread per row;
-//   mode 1: rows in warp-sized blocks, 8 lanes per row, except that rows
-//           longer than kTeamRow non-zeros are taken by the whole warp in turn
-//           (lanes stride over the row, shuffle reduction), and rows longer
-//           than kCtaRow (the system's list, ascending) by the whole CTA
-//           after the blocks, so a power-law row of thousands of entries
-//           neither serialises one thread nor one warp.
-// Every row's sum has one fixed order (its stride and four interleaved
-// partial sums), so results do not depend on scheduling.
+//   mode 1: part_tiles.
+// Every row's sum has one fixed order, so results do not depend on scheduling.
 __device__ __forceinline__ double row_dot(const int *__restrict__ col,
                                           const double *__restrict__ val, const double *x,
-                                          int ka, int kb, int step) {
+                                          int ka, int kb) {
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
     int k = ka;
-    for (; k + 3 * step < kb; k += 4 * step) {  // four gathers in flight
-        const int c0 = __ldg(col + k), c1 = __ldg(col + k + step), c2 = __ldg(col + k + 2 * step),
-                  c3 = __ldg(col + k + 3 * step);
-        const double v0 = __ldg(val + k), v1 = __ldg(val + k + step), v2 = __ldg(val + k + 2 * step),
-                     v3 = __ldg(val + k + 3 * step);
+    for (; k + 3 < kb; k += 4) {  // four gathers in flight
+        const int c0 = __ldg(col + k), c1 = __ldg(col + k + 1), c2 = __ldg(col + k + 2), c3 = __ldg(col + k + 3);
+        const double v0 = __ldg(val + k), v1 = __ldg(val + k + 1), v2 = __ldg(val + k + 2), v3 = __ldg(val + k + 3);
         s0 = fma(v0, x[c0], s0);
         s1 = fma(v1, x[c1], s1);
         s2 = fma(v2, x[c2], s2);
         s3 = fma(v3, x[c3], s3);
     }
-    for (; k < kb; k += step) s0 = fma(__ldg(val + k), x[__ldg(col + k)], s0);
+    for (; k < kb; k++) s0 = fma(__ldg(val + k), x[__ldg(col + k)], s0);
     return (s0 + s1) + (s2 + s3);
 }
 
-// The products of a warp's 32 rows (lane l's row is entries [ka, kb), l's
-// result its sum): teams of 8 lanes take 4 rows at a time, 8 times, so a warp's
-// loads of col and val cover whole sectors and only the gathers of x take a
-// cache line per lane.  The 8 partial sums of a lane meet in a transposed tree,
-// 7 adds for the 32 rows, after which lane l holds row l.
-__device__ __forceinline__ double team_dots(const int *__restrict__ col,
-                                            const double *__restrict__ val, const double *x,
-                                            int ka, int kb) {
-    const int lane = threadIdx.x & 31, t = lane & 7, q8 = lane & 24;
-    double s[8];
-    int k[8], e[8];
-#pragma unroll
-    for (int g = 0; g < 8; g++) {
-        k[g] = __shfl_sync(0xffffffffu, ka, q8 + g) + t;
-        e[g] = __shfl_sync(0xffffffffu, kb, q8 + g);
-        s[g] = 0.0;
+// A warp's shared memory in mode 1: the tile's values and gathered x, 8 entries
+// and a gap for each lane (no bank conflicts), and the marks of row ends.
+struct TileBuf {
+    double2 vx[kTile + kTile / 8];
+    unsigned char end[kTile];
+};
+
+// Mode 1: the CTA's entries in tiles of 256, whatever their rows.  A power law's
+// rows differ by orders of magnitude, and an FP64 instruction holds a quarter of
+// the SM for ~64 cycles however few lanes need it, so a lane sums 8 consecutive
+// entries (8 FMAs for 256 of them), a segmented scan, ended by a vote, carries the
+// sums of rows over lanes, and rows that leave their tile are completed after the
+// CTA has met.  Loads of col and val cover whole sectors; the next tile's are on
+// their way during the sums.  n = 40,900, 522,000 non-zeros, GMRES(30) on 8 CTAs:
+// 133 us a step, 203 with a lane for a row of up to 32 entries and a warp for
+// longer ones, 193 with 8 lanes for a row.
+__device__ void part_tiles(const xb_batch_dev &D, const Part &P, int part, TileBuf *buf, double alpha,
+                           const double *x, double beta, double *y) {
+    const int *__restrict__ rp = D.rowptr;
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    TileBuf &B = buf[threadIdx.x >> 5];
+    const int t0 = D.tptr[part], t1 = D.tptr[part + 1];
+    if (t0 == t1) {
+        if (beta == 0.0)
+            for (int r = P.r0 + threadIdx.x; r < P.r1; r += blockDim.x) y[r] = 0.0;
+        return;
     }
-    const int len = __reduce_max_sync(0xffffffffu, kb - ka);
-    for (int it = 0; it < len; it += 8) {
-        int c[8];
-        double v[8], xv[8];
+    const int e0 = __ldg(rp + P.r0), e1 = __ldg(rp + P.r1);
+    int c[8];
+    double v[8];
+    auto load = [&](int t) {
+        const unsigned at = (unsigned)e0 + (unsigned)(t - t0) * kTile + lane;
 #pragma unroll
-        for (int g = 0; g < 8; g++) {
-            c[g] = k[g] < e[g] ? __ldg(col + k[g]) : -1;
-            v[g] = k[g] < e[g] ? __ldg(val + k[g]) : 0.0;
-            k[g] += 8;
+        for (int i = 0; i < 8; i++) {
+            const bool in = t < t1 && at + 32 * i < (unsigned)e1;
+            c[i] = in ? __ldg(D.col + at + 32 * i) : -1;
+            v[i] = in ? __ldg(D.val + at + 32 * i) : 0.0;
+        }
+    };
+    int t = t0 + (threadIdx.x >> 5);
+    load(t);
+    for (; t < t1; t += nw) {
+        const int tb = e0 + (t - t0) * kTile, te = e1 - tb > kTile ? tb + kTile : e1;
+        const int ra = t == t0 ? P.r0 : __ldg(D.trow + t), rb = t + 1 < t1 ? __ldg(D.trow + t + 1) + 1 : P.r1;
+        double xv[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) xv[i] = c[i] >= 0 ? x[c[i]] : 0.0;
+        reinterpret_cast<uint2 *>(B.end)[lane] = make_uint2(0, 0);
+        __syncwarp();
+        // the first 32 rows' bounds stay in registers
+        const int fs = ra + lane < rb ? __ldg(rp + ra + lane) : 0, fe = ra + lane < rb ? __ldg(rp + ra + lane + 1) : 0;
+        for (int q = ra; q < rb; q += 32) {
+            const int r = q + lane;
+            const int a = q == ra ? fs : r < rb ? __ldg(rp + r) : 0, b = q == ra ? fe : r < rb ? __ldg(rp + r + 1) : 0;
+            if (b > a && b > tb && b <= te) B.end[b - 1 - tb] = 1;
         }
 #pragma unroll
-        for (int g = 0; g < 8; g++) xv[g] = c[g] >= 0 ? x[c[g]] : 0.0;
+        for (int i = 0; i < 8; i++) B.vx[(32 * i + lane) / 8 * 9 + (lane & 7)] = make_double2(v[i], xv[i]);
+        __syncwarp();
+        load(t + nw);
+        // the lane's entries; sums of rows that end go to their last entry's place
+        const uint2 m = reinterpret_cast<const uint2 *>(B.end)[lane];
+        double s = 0.0, f = 0.0;
+        int first = -1;
 #pragma unroll
-        for (int g = 0; g < 8; g++)
-            if (c[g] >= 0) s[g] = fma(v[g], xv[g], s[g]);
-    }
-#pragma unroll
-    for (int h = 4; h > 0; h >>= 1) {
-        const bool up = t & h;
-#pragma unroll
-        for (int g = 0; g < h; g++) {
-            const double mine = up ? s[g + h] : s[g], other = up ? s[g] : s[g + h];
-            s[g] = mine + __shfl_xor_sync(0xffffffffu, other, h);
+        for (int i = 0; i < 8; i++) {
+            double2 &z = B.vx[lane * 9 + i];
+            s = fma(z.x, z.y, s);
+            if (((i < 4 ? m.x : m.y) >> 8 * (i & 3)) & 1u) {
+                if (first < 0) {
+                    first = i;
+                    f = s;
+                } else {
+                    z.x = s;
+                }
+                s = 0.0;
+            }
         }
+        // the sums that lanes hand on: inclusive, back to the last lane in which a row ends
+        bool stop = first >= 0;
+        const bool any = __any_sync(0xffffffffu, stop);
+        for (int o = 1; o < 32; o <<= 1) {
+            const bool need = !stop && lane >= o;
+            if (!__any_sync(0xffffffffu, need)) break;
+            const double us = __shfl_up_sync(0xffffffffu, s, o);
+            const bool ub = __shfl_up_sync(0xffffffffu, (int)stop, o);
+            if (need) {
+                s += us;
+                stop = ub;
+            }
+        }
+        const double in = __shfl_up_sync(0xffffffffu, s, 1);
+        if (first >= 0) B.vx[lane * 9 + first].x = lane > 0 ? f + in : f;
+        __syncwarp();
+        for (int q = ra; q < rb; q += 32) {
+            const int r = q + lane;
+            const int a = q == ra ? fs : r < rb ? __ldg(rp + r) : 0, b = q == ra ? fe : r < rb ? __ldg(rp + r + 1) : 0;
+            if (b > a && b > tb && b <= te) {
+                const int e = b - 1 - tb;
+                const double w = B.vx[e / 8 * 9 + (e & 7)].x;
+                if (a < tb) D.tsum[t].x = w;
+                else y[r] = beta == 0.0 ? alpha * w : fma(alpha, w, beta * y[r]);
+            } else if (r < rb && a == b && beta == 0.0) {
+                y[r] = 0.0;
+            }
+        }
+        if (lane == 31) D.tsum[t].y = s;
+        if (lane == 0) D.tinfo[t] = !any ? -1 : fs < tb ? ra : -2;
+        __syncwarp();
     }
-    return s[0];
+    __syncthreads();
+    for (int q = t0 + threadIdx.x; q < t1; q += blockDim.x) {
+        const int r = D.tinfo[q];
+        if (r < 0) continue;
+        double w = 0.0;
+        for (int z = q - 1; z >= t0; z--) {
+            w += D.tsum[z].y;
+            if (D.tinfo[z] != -1) break;
+        }
+        w += D.tsum[q].x;
+        y[r] = beta == 0.0 ? alpha * w : fma(alpha, w, beta * y[r]);
+    }
 }
 
-__device__ void part_spmv(const xb_batch_dev &D, const Part &P, Smem &S, double alpha,
+__device__ void part_spmv(const xb_batch_dev &D, const Part &P, TileBuf *buf, int part, double alpha,
                           const double *x, double beta, double *y) {
-    const int *__restrict__ rp = D.rowptr;
     if (D.mode == 0) {
+        const int *__restrict__ rp = D.rowptr;
         for (int r = P.r0 + threadIdx.x; r < P.r1; r += blockDim.x) {
-            const double s = row_dot(D.col, D.val, x, __ldg(rp + r), __ldg(rp + r + 1), 1);
+            const double s = row_dot(D.col, D.val, x, __ldg(rp + r), __ldg(rp + r + 1));
             y[r] = beta == 0.0 ? alpha * s : fma(alpha, s, beta * y[r]);
         }
     } else {
-        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-        for (int base = P.r0 + 32 * w; base < P.r1; base += 32 * nw) {  // warp-uniform
-            const int r = base + lane;
-            int ka = 0, kb = 0;
-            if (r < P.r1) {
-                ka = __ldg(rp + r);
-                kb = __ldg(rp + r + 1);
-            }
-            const bool cta = kb - ka > kCtaRow;
-            const bool lng = kb - ka > kTeamRow && !cta;
-            double s = team_dots(D.col, D.val, x, ka, lng || cta ? ka : kb);
-            unsigned todo = __ballot_sync(0xffffffffu, lng);
-            while (todo) {
-                const int src = __ffs(todo) - 1;
-                todo &= todo - 1;
-                const int la = __shfl_sync(0xffffffffu, ka, src);
-                const int lb = __shfl_sync(0xffffffffu, kb, src);
-                double t = row_dot(D.col, D.val, x, la + lane, lb, 32);
-                for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-                if (lane == src) s = t;
-            }
-            if (r < P.r1 && !cta) y[r] = beta == 0.0 ? alpha * s : fma(alpha, s, beta * y[r]);
-        }
-        if (D.nl > 0) {
-            // the CTA's long rows: first list entry >= r0 (binary search), up to r1
-            int lo = 0, hi = D.nl;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (__ldg(D.lrows + mid) < P.r0) lo = mid + 1;
-                else hi = mid;
-            }
-            for (int q = lo; q < D.nl; q++) {  // CTA-uniform
-                const int r = __ldg(D.lrows + q);
-                if (r >= P.r1) break;
-                const int ka = __ldg(rp + r), kb = __ldg(rp + r + 1);
-                const double t = cta_sum(row_dot(D.col, D.val, x, ka + (int)threadIdx.x, kb,
-                                                 (int)blockDim.x), S);
-                if (threadIdx.x == 0) y[r] = beta == 0.0 ? alpha * t : fma(alpha, t, beta * y[r]);
-            }
-        }
+        part_tiles(D, P, part, buf, alpha, x, beta, y);
     }
     // rows were stored by other threads than the ones that read them next,
     // so the CTA meets before anyone reads y
@@ -359,7 +377,7 @@ __device__ __forceinline__ void bgs_rows(double *__restrict__ w, const double *_
     if (e < r1) bgs_row<1, NORM>(w, V, ld, u0, nu, c, d0, nd, e, B, a);
 }
 
-__device__ void solve_one(const xb_batch_dev &D, Part &P, Smem &S, double tol, int maxiter,
+__device__ void solve_one(const xb_batch_dev &D, Part &P, Smem &S, TileBuf *buf, double tol, int maxiter,
                           unsigned long long deadline, int rank, double theta, int bcgs,
                           xb_batch_info *out) {
     const unsigned long long ts = gtimer();
@@ -383,7 +401,7 @@ __device__ void solve_one(const xb_batch_dev &D, Part &P, Smem &S, double tol, i
             coop_barrier(P);  // x complete before A x
             for (int i = r0 + threadIdx.x; i < r1; i += blockDim.x) V[i] = D.b[i];
             __syncthreads();  // the SpMV reads V_0 rows through other threads
-            part_spmv(D, P, S, -1.0, D.x, 1.0, V);
+            part_spmv(D, P, buf, rank, -1.0, D.x, 1.0, V);
             a = 0.0;
             for (int i = r0 + threadIdx.x; i < r1; i += blockDim.x) a = fma(V[i], V[i], a);
             const double beta = sqrt(coop_sum(a, S, P));
@@ -427,7 +445,7 @@ __device__ void solve_one(const xb_batch_dev &D, Part &P, Smem &S, double tol, i
                 iters++;
                 double *w = V + (size_t)(j + 1) * ld;
                 // v_j is complete: the norm's sum (or the residual's) ordered it
-                part_spmv(D, P, S, S.sc[j], V + (size_t)j * ld, 0.0, w);
+                part_spmv(D, P, buf, rank, S.sc[j], V + (size_t)j * ld, 0.0, w);
                 // warp 2 keeps tt, the column's newest entry rotated by the earlier
                 // rotations, and the sum of squares, a block behind
                 double tt = 0.0, len2 = 0.0;
@@ -626,6 +644,8 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kBT, 1)
                   int *__restrict__ queue, double tol, int maxiter, unsigned long long budget_ns,
                   double theta, int bcgs) {
     __shared__ Smem S;
+    extern __shared__ __align__(16) unsigned char dyn[];
+    TileBuf *buf = reinterpret_cast<TileBuf *>(dyn);
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     if (threadIdx.x == 0) S.t_start = gtimer();
@@ -653,7 +673,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kBT, 1)
             const xb_batch_dev D = sys[order[q]];
             const int per = (D.n + kCl - 1) / kCl;
             Part P{min(D.n, rank * per), min(D.n, (rank + 1) * per), 1, 0};
-            solve_one(D, P, S, tol, maxiter, deadline, rank, theta, bcgs, out + order[q]);
+            solve_one(D, P, S, buf, tol, maxiter, deadline, rank, theta, bcgs, out + order[q]);
         }
     };
     auto phase2 = [&]() {
@@ -665,7 +685,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kBT, 1)
             if (q >= count) return;  // CTA-uniform
             const xb_batch_dev D = sys[order[q]];
             Part P{0, D.n, 0, 0};
-            solve_one(D, P, S, tol, maxiter, deadline, 0, theta, bcgs, out + order[q]);
+            solve_one(D, P, S, buf, tol, maxiter, deadline, 0, theta, bcgs, out + order[q]);
         }
     };
     if (small_first) {
@@ -678,12 +698,33 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kBT, 1)
     }
 }
 
+constexpr int kDyn = (int)sizeof(TileBuf) * (kBT / 32);
+
+// Mode 1's tiles of a system whose host row pointer is rp: tptr and, appended to
+// trow, the tiles' rows.
+void cut_tiles(xb_batch_dev &d, const int *rp, std::vector<int> &trow) {
+    const int parts = d.coop ? kCl : 1, per = (d.n + parts - 1) / parts;
+    const size_t base = trow.size();
+    for (int c = 0; c < kCl; c++) {
+        d.tptr[c] = (int)(trow.size() - base);
+        if (c >= parts) continue;
+        int r = std::min(d.n, c * per);
+        const int r1 = std::min(d.n, (c + 1) * per);
+        for (int64_t e = rp[r]; e < rp[r1]; e += kTile) {
+            while (rp[r + 1] <= e) r++;
+            trow.push_back(r);
+        }
+    }
+    d.tptr[kCl] = (int)(trow.size() - base);
+}
+
 // Whole clusters of the kernel that fit on the GPU at once.
 int resident_clusters() {
     cudaLaunchConfig_t lc;
     std::memset(&lc, 0, sizeof lc);
     lc.gridDim = dim3(kCl, 1, 1);
     lc.blockDim = dim3(kBT, 1, 1);
+    lc.dynamicSmemBytes = kDyn;
     int clusters = 0;
     if (cudaOccupancyMaxActiveClusters(&clusters, (void *)k_batch_gmres, &lc) != cudaSuccess || clusters < 1) {
         cudaGetLastError();
@@ -693,14 +734,14 @@ int resident_clusters() {
 }
 
 // Estimated time of an Arnoldi step, in us, at the cycle's mean basis size m / 2:
-// 2 + m / 8 sums at 2 us (3 us across a cluster), and n m + 2 nnz FP64 terms (4 nnz
-// for mode 1's uneven rows) at 0.4 ns a CTA, with a fifth lost to the split over a
-// cluster's 8.  Fitted to 48 systems of 1000 to 57,000 rows at m = 30 (one CTA 28 to
-// 1300 us, a cluster 18 to 200 us a step).
+// 2 + m / 8 sums at 2 us (3.3 us across a cluster), and n m + nnz FP64 terms (1.5
+// nnz in mode 1) at 0.4 ns a CTA, with a seventh lost to the split over a cluster's
+// 8.  Fitted to 48 systems of 1000 to 57,000 rows at m = 30 (one CTA 28 to 825 us,
+// a cluster 18 to 133 us a step), within a fifth.
 double step_us(const xb_batch_dev &d, bool cluster) {
     const double sums = 2.0 + d.m / 8.0,
-                 terms = 4e-4 * ((double)d.m * d.n + (d.mode == 1 ? 4.0 : 2.0) * d.nnz);
-    return cluster ? 3.0 * sums + 1.2 * terms / kCl : 2.0 * sums + terms;
+                 terms = 4e-4 * ((double)d.m * d.n + (d.mode == 1 ? 1.5 : 1.0) * d.nnz);
+    return cluster ? 3.3 * sums + 1.15 * terms / kCl : 2.0 * sums + terms;
 }
 
 // Decides which systems a whole cluster solves and returns the order of the
@@ -735,7 +776,7 @@ std::vector<int> split_systems(std::vector<xb_batch_dev> &h, int clusters) {
     for (int k = 0; k <= count; k++) {
         const double alone = k < count ? step_us(h[order[k]], false) : 0.0;
         const double end = std::max({longest, alone, spread / (kCl * clusters)});
-        if (k == 0 || end < best) {
+        if (k == 0 || end <= best) {  // a tie: the shorter solves
             best = end;
             take = k;
         }
@@ -782,12 +823,21 @@ int batch_single(xb_plan *p, const double *b, double *x, const xb_options &o, in
     const size_t nv = (size_t)(d.m_max + 1) * d.ld;
     const size_t nh = (size_t)(d.coop ? kCl : 1) * (d.m_max + 1) * d.m_max + 32;
     const size_t meta = 4096;  // descriptor, result, order, queue
-    // mode 1: the rows longer than kCtaRow, from the plan's host row pointer
-    std::vector<int> lr;
-    if (mode == 1 && p->nnz > kCtaRow && (int)p->h_rowptr.size() == p->n + 1)
-        for (int r = 0; r < p->n; r++)
-            if (p->h_rowptr[r + 1] - p->h_rowptr[r] > kCtaRow) lr.push_back(r);
-    XB_TRY(ensure_work(p, (nv + nh) * sizeof(double) + meta + lr.size() * sizeof(int)));
+    // mode 1: the tiles, from the plan's host row pointer
+    std::vector<int> trow;
+    std::memset(d.tptr, 0, sizeof d.tptr);
+    if (mode == 1) {
+        std::vector<int> rp_h;
+        const int *rp = p->h_rowptr.data();
+        if ((int)p->h_rowptr.size() != p->n + 1) {
+            rp_h.resize((size_t)p->n + 1);
+            XB_CUDA(cudaMemcpy(rp_h.data(), p->rowptr, rp_h.size() * sizeof(int), cudaMemcpyDeviceToHost));
+            rp = rp_h.data();
+        }
+        cut_tiles(d, rp, trow);
+    }
+    const size_t nt = trow.size();
+    XB_TRY(ensure_work(p, (nv + nh) * sizeof(double) + meta + nt * (sizeof(double2) + 2 * sizeof(int))));
     char *w = static_cast<char *>(p->d_work);
     d.V = reinterpret_cast<double *>(w);
     d.H = d.V + nv;
@@ -797,13 +847,11 @@ int batch_single(xb_plan *p, const double *b, double *x, const xb_options &o, in
     int *d_order = reinterpret_cast<int *>(m0 + 2048);
     int *d_queue = d_order + 1;
     static_assert(sizeof(xb_batch_dev) <= 1024 && sizeof(xb_batch_info) <= 1024, "meta layout");
-    d.nl = (int)lr.size();
-    d.lrows = nullptr;
-    if (!lr.empty()) {
-        int *d_lr = reinterpret_cast<int *>(m0 + meta);
-        XB_CUDA(cudaMemcpyAsync(d_lr, lr.data(), lr.size() * sizeof(int), cudaMemcpyHostToDevice, s));
-        d.lrows = d_lr;
-    }
+    d.tsum = reinterpret_cast<double2 *>(m0 + meta);
+    d.tinfo = reinterpret_cast<int *>(d.tsum + nt);
+    d.trow = d.tinfo + nt;
+    if (nt > 0)
+        XB_CUDA(cudaMemcpyAsync(d.tinfo + nt, trow.data(), nt * sizeof(int), cudaMemcpyHostToDevice, s));
     const int zero = 0;
     XB_CUDA(cudaMemcpyAsync(d_sys, &d, sizeof d, cudaMemcpyHostToDevice, s));
     XB_CUDA(cudaMemcpyAsync(d_order, &zero, sizeof zero, cudaMemcpyHostToDevice, s));
@@ -811,7 +859,8 @@ int batch_single(xb_plan *p, const double *b, double *x, const xb_options &o, in
     const unsigned long long budget = (unsigned long long)(std::min(o.maxtime_s, 3600.0) * 1e9);
     const double theta = o.dafrt ? o.dafrt_theta : 0.0;
     const int bcgs = o.ortho == XB_ORTHO_BCGS ? 1 : 0;
-    k_batch_gmres<<<kCl, kBT, 0, s>>>(d_sys, d_info, d_order, 1, 1, 0, d_queue, o.tol, o.maxiter,
+    XB_CUDA(cudaFuncSetAttribute(k_batch_gmres, cudaFuncAttributeMaxDynamicSharedMemorySize, kDyn));
+    k_batch_gmres<<<kCl, kBT, kDyn, s>>>(d_sys, d_info, d_order, 1, 1, 0, d_queue, o.tol, o.maxiter,
                                       budget, theta, bcgs);
     XB_LAUNCHED("k_batch_gmres (single system)");
     xb_batch_info r;
@@ -848,7 +897,7 @@ int xb_batch_destroy(xb_batch *bt) {
     cudaFree(bt->d_order);
     cudaFree(bt->d_queue);
     cudaFree(bt->d_ws);
-    cudaFree(bt->d_lrows);
+    cudaFree(bt->d_tiles);
     delete bt;
     return XB_OK;
 }
@@ -886,26 +935,27 @@ int xb_batch_create(int32_t count, const xb_batch_sys *sys, const xb_options *op
         d.b = q.b;
         d.x = q.x;
     }
+    cudaError_t e = cudaFuncSetAttribute(k_batch_gmres, cudaFuncAttributeMaxDynamicSharedMemorySize, kDyn);
+    if (e != cudaSuccess) return xb::cuda_error(e, "batch_create: shared memory");
     const int clusters = resident_clusters();
     const std::vector<int> order = split_systems(h, clusters);
     for (const xb_batch_dev &d : h)
         ws += (size_t)(d.m_max + 1) * d.ld + (size_t)(d.coop ? kCl : 1) * (d.m_max + 1) * d.m_max + 32;
-    // mode 1: each system's rows longer than kCtaRow (summed by a whole CTA),
-    // from a host copy of its row pointer
-    std::vector<int> lr_all, rp_h;
-    std::vector<size_t> lr_off(count, 0);
+    // mode 1: each system's tiles, from a host copy of its row pointer
+    std::vector<int> trow, rp_h;
+    std::vector<size_t> toff(count, 0);
     for (int i = 0; i < count; i++) {
-        h[i].lrows = nullptr;
-        h[i].nl = 0;
-        if (h[i].mode != 1 || h[i].n < 1 || h[i].nnz <= kCtaRow) continue;
+        std::memset(h[i].tptr, 0, sizeof h[i].tptr);
+        h[i].trow = nullptr;
+        h[i].tinfo = nullptr;
+        h[i].tsum = nullptr;
+        toff[i] = trow.size();
+        if (h[i].mode != 1 || h[i].n < 1 || h[i].nnz < 1) continue;
         rp_h.resize((size_t)h[i].n + 1);
-        cudaError_t e = cudaMemcpy(rp_h.data(), h[i].rowptr, rp_h.size() * sizeof(int),
+        e = cudaMemcpy(rp_h.data(), h[i].rowptr, rp_h.size() * sizeof(int),
                                    cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return xb::cuda_error(e, "batch_create: read rowptr");
-        lr_off[i] = lr_all.size();
-        for (int r = 0; r < h[i].n; r++)
-            if (rp_h[r + 1] - rp_h[r] > kCtaRow) lr_all.push_back(r);
-        h[i].nl = (int)(lr_all.size() - lr_off[i]);
+        cut_tiles(h[i], rp_h.data(), trow);
     }
     xb_batch *bt = new xb_batch();
     bt->count = count;
@@ -913,19 +963,27 @@ int xb_batch_create(int32_t count, const xb_batch_sys *sys, const xb_options *op
         xb_batch_destroy(bt);
         return code;
     };
-    cudaError_t e = cudaMalloc(&bt->d_ws, std::max<size_t>(ws, 1) * sizeof(double));
+    e = cudaMalloc(&bt->d_ws, std::max<size_t>(ws, 1) * sizeof(double));
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(xb::set_error(XB_ENOMEM, "batch_create: %zu bytes of workspace", ws * 8));
     }
-    if (!lr_all.empty()) {
-        e = cudaMalloc(&bt->d_lrows, lr_all.size() * sizeof(int));
-        if (e == cudaSuccess)
-            e = cudaMemcpy(bt->d_lrows, lr_all.data(), lr_all.size() * sizeof(int),
-                           cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) return fail(xb::cuda_error(e, "batch_create: long-row lists"));
-        for (int i = 0; i < count; i++)
-            if (h[i].nl > 0) h[i].lrows = bt->d_lrows + lr_off[i];
+    const size_t nt = trow.size();
+    if (nt > 0) {
+        e = cudaMalloc(&bt->d_tiles, nt * (sizeof(double2) + 2 * sizeof(int)));
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return fail(xb::set_error(XB_ENOMEM, "batch_create: tiles"));
+        }
+        double2 *ts = static_cast<double2 *>(bt->d_tiles);
+        int *ti = reinterpret_cast<int *>(ts + nt);
+        e = cudaMemcpy(ti + nt, trow.data(), nt * sizeof(int), cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) return fail(xb::cuda_error(e, "batch_create: tiles"));
+        for (int i = 0; i < count; i++) {
+            h[i].tsum = ts + toff[i];
+            h[i].tinfo = ti + toff[i];
+            h[i].trow = ti + nt + toff[i];
+        }
     }
     size_t off = 0;
     for (int i = 0; i < count; i++) {
@@ -971,7 +1029,7 @@ int xb_batch_create(int32_t count, const xb_batch_sys *sys, const xb_options *op
         return fail(xb::cuda_error(e, "batch_create: begin capture"));
     }
     cudaMemsetAsync(bt->d_queue, 0, 2 * sizeof(int), cs);
-    k_batch_gmres<<<bt->grid, kBT, 0, cs>>>(bt->d_sys, bt->d_info, bt->d_order, count, nbig,
+    k_batch_gmres<<<bt->grid, kBT, kDyn, cs>>>(bt->d_sys, bt->d_info, bt->d_order, count, nbig,
                                              nsmall_cl, bt->d_queue,
                                              o.tol, o.maxiter, budget, theta, bcgs);
     cudaError_t el = cudaGetLastError();

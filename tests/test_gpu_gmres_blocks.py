@@ -5,9 +5,9 @@ one-at-a-time GMRES: x after a full cycle and three steps of the next.
 Sizes: restart lengths around the blocks of 4 and the 32 lanes of the
 triangular solve; 1 to 2049 rows, so that CTAs and lanes stand empty; MGS
 (corrected blocks) and BCGS; every cluster size; batched in one CTA, in
-a cluster and by the default rule, there with rows at the edges of the 64 and
-1024 entries at which mode 1 changes its form.  A batched system of one row at
-values near the ends of the FP64 range converges as at 1.
+a cluster and by the default rule, there with rows of up to 1025 entries, which
+mode 1's tiles of 256 cut, and rows without entries.  A batched system of one row
+at values near the ends of the FP64 range converges as at 1.
 
 Tolerance: A = I + E with ||E|| <= 0.45, so cond(A) <= 2.7.  Each of the m + 3
 steps carries a few eps cond^2 into x: 32 (m + 3) 2.7^2 eps, eps = 1.1e-16,
@@ -44,10 +44,15 @@ def _matrix(n, seed, long=()):
         for c in rng.permutation(n)[:k]:
             if len(r) < k:
                 r.setdefault(int(c), rng.uniform(-1e-4, 1e-4))
+    b = rng.standard_normal(n)
+    if long:  # rows without entries (and b = 0 there), alone and several at a time
+        for i in [0, 1, 2, n - 1] + list(range(300, 340)) + list(range(400, n, 97)):
+            rows[i] = {}
+            b[i] = 0.0
     rp = np.cumsum([0] + [len(r) for r in rows]).astype(np.int32)
     col = np.concatenate([np.array(sorted(r), np.int32) for r in rows])
     val = np.concatenate([np.array([r[c] for c in sorted(r)]) for r in rows])
-    return dict(n=n, rowptr=rp, col=col, val=val), rng.standard_normal(n)
+    return dict(n=n, rowptr=rp, col=col, val=val), b
 
 
 def _close(x, xo, m):

@@ -40,6 +40,7 @@ namespace cg = cooperative_groups;
 namespace {
 constexpr int kCl = 8;          // CTAs per cluster
 constexpr int kBT = 512;        // threads per CTA
+constexpr int kLargeN = 30000;  // systems this large are always solved by a whole cluster
 constexpr int kTile = 256;      // mode 1: entries a warp sums at a time, 8 a lane
 }  // namespace
 
@@ -171,9 +172,11 @@ __device__ __forceinline__ void coop_barrier(const Part &P) {
 }
 
 // y[r0:r1] = alpha*A[r0:r1,:]*x (+ beta*y), beta 0 or 1.  x is written by the other CTAs
-// of the cluster during the launch: ordinary loads, ordered by the barrier
-// (release / acquire) that follows the writes, never the read-only path.
-//   mode 0: one thread per row;
+// of the cluster during the launch and ordered by the barrier (release / acquire)
+// that follows: never the read-only path.
+//   mode 0: one thread per row, x read at L2 (ld.global.cg), which leaves the L1
+//           to the rows' entries (512 systems, power-law rows among them: 15.0 s,
+//           16.0 through the L1; 48 systems 21.6 and 21.4 ms);
 //   mode 1: part_tiles.
 // Every row's sum has one fixed order, so results do not depend on scheduling.
 __device__ __forceinline__ double row_dot(const int *__restrict__ col,
@@ -184,12 +187,12 @@ __device__ __forceinline__ double row_dot(const int *__restrict__ col,
     for (; k + 3 < kb; k += 4) {  // four gathers in flight
         const int c0 = __ldg(col + k), c1 = __ldg(col + k + 1), c2 = __ldg(col + k + 2), c3 = __ldg(col + k + 3);
         const double v0 = __ldg(val + k), v1 = __ldg(val + k + 1), v2 = __ldg(val + k + 2), v3 = __ldg(val + k + 3);
-        s0 = fma(v0, x[c0], s0);
-        s1 = fma(v1, x[c1], s1);
-        s2 = fma(v2, x[c2], s2);
-        s3 = fma(v3, x[c3], s3);
+        s0 = fma(v0, __ldcg(x + c0), s0);
+        s1 = fma(v1, __ldcg(x + c1), s1);
+        s2 = fma(v2, __ldcg(x + c2), s2);
+        s3 = fma(v3, __ldcg(x + c3), s3);
     }
-    for (; k < kb; k++) s0 = fma(__ldg(val + k), x[__ldg(col + k)], s0);
+    for (; k < kb; k++) s0 = fma(__ldg(val + k), __ldcg(x + __ldg(col + k)), s0);
     return (s0 + s1) + (s2 + s3);
 }
 
@@ -719,12 +722,12 @@ void cut_tiles(xb_batch_dev &d, const int *rp, std::vector<int> &trow) {
 }
 
 // Whole clusters of the kernel that fit on the GPU at once.
-int resident_clusters() {
+int resident_clusters(size_t dyn) {
     cudaLaunchConfig_t lc;
     std::memset(&lc, 0, sizeof lc);
     lc.gridDim = dim3(kCl, 1, 1);
     lc.blockDim = dim3(kBT, 1, 1);
-    lc.dynamicSmemBytes = kDyn;
+    lc.dynamicSmemBytes = dyn;
     int clusters = 0;
     if (cudaOccupancyMaxActiveClusters(&clusters, (void *)k_batch_gmres, &lc) != cudaSuccess || clusters < 1) {
         cudaGetLastError();
@@ -747,36 +750,39 @@ double step_us(const xb_batch_dev &d, bool cluster) {
 // Decides which systems a whole cluster solves and returns the order of the
 // queues: the cluster's systems first, each part largest first, so that the long
 // solves start in the first wave.  A cluster solves a system sooner but at up to 8
-// times the SM time, so the k largest go to clusters with the k whose estimated
-// end is first: no earlier than the longest cluster solve, than the longest
-// single-CTA one, and than all the work spread over the resident CTAs (equal
-// step counts assumed).  Few systems thus all go to clusters, many small ones
-// to a CTA each.  The environment variable XB_BATCH_COOP_MIN_N sets a number of
-// rows from which on a cluster takes a system instead.
+// times the SM time.  From kLargeN rows on it takes a system always: step counts
+// and row lengths are unknown, and a long solve on one CTA can outlast all others
+// (512 systems, some of which run 3000 steps: 24.2 s without this, 15.0 with it).
+// Of the others the k largest follow, for the k whose estimated end is first: no
+// earlier than the longest cluster solve, than the longest single-CTA one, and than
+// all the work spread over the resident CTAs, at equal step counts.  Few systems
+// thus all go to clusters, many small ones to a CTA each.  The environment variable
+// XB_BATCH_COOP_MIN_N sets the number of rows and leaves the estimate out.
 std::vector<int> split_systems(std::vector<xb_batch_dev> &h, int clusters) {
     const int count = (int)h.size();
+    const char *env = std::getenv("XB_BATCH_COOP_MIN_N");
+    const long coop_min = env ? std::max(1L, std::atol(env)) : kLargeN;
+    for (xb_batch_dev &d : h) d.coop = d.n >= coop_min ? 1 : 0;
     std::vector<int> order(count);
     std::iota(order.begin(), order.end(), 0);
-    const char *env = std::getenv("XB_BATCH_COOP_MIN_N");
-    if (env) {
-        const long coop_min = std::max(1L, std::atol(env));
-        for (xb_batch_dev &d : h) d.coop = d.n >= coop_min ? 1 : 0;
-        std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-            if (h[a].coop != h[b].coop) return h[a].coop > h[b].coop;
-            return step_us(h[a], false) > step_us(h[b], false);
-        });
-        return order;
-    }
-    std::stable_sort(order.begin(), order.end(),
-                     [&](int a, int b) { return step_us(h[a], false) > step_us(h[b], false); });
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+        if (h[a].coop != h[b].coop) return h[a].coop > h[b].coop;
+        return step_us(h[a], false) > step_us(h[b], false);
+    });
+    if (env) return order;
     double spread = 0.0;  // SM time of all systems with the first k in clusters
-    for (const xb_batch_dev &d : h) spread += step_us(d, false);
     double best = 0.0, longest = 0.0;
-    int take = 0;
-    for (int k = 0; k <= count; k++) {
+    int first = 0, take = 0;
+    for (const xb_batch_dev &d : h) {
+        const double c = step_us(d, true);
+        spread += d.coop ? kCl * c : step_us(d, false);
+        if (d.coop) longest = std::max(longest, c);
+        first += d.coop;
+    }
+    for (int k = first; k <= count; k++) {
         const double alone = k < count ? step_us(h[order[k]], false) : 0.0;
         const double end = std::max({longest, alone, spread / (kCl * clusters)});
-        if (k == 0 || end <= best) {  // a tie: the shorter solves
+        if (k == first || end <= best) {  // a tie: the shorter solves
             best = end;
             take = k;
         }
@@ -785,7 +791,7 @@ std::vector<int> split_systems(std::vector<xb_batch_dev> &h, int clusters) {
         longest = std::max(longest, c);
         spread += kCl * c - alone;
     }
-    for (int k = 0; k < count; k++) h[order[k]].coop = k < take ? 1 : 0;
+    for (int k = first; k < take; k++) h[order[k]].coop = 1;
     return order;
 }
 
@@ -860,7 +866,7 @@ int batch_single(xb_plan *p, const double *b, double *x, const xb_options &o, in
     const double theta = o.dafrt ? o.dafrt_theta : 0.0;
     const int bcgs = o.ortho == XB_ORTHO_BCGS ? 1 : 0;
     XB_CUDA(cudaFuncSetAttribute(k_batch_gmres, cudaFuncAttributeMaxDynamicSharedMemorySize, kDyn));
-    k_batch_gmres<<<kCl, kBT, kDyn, s>>>(d_sys, d_info, d_order, 1, 1, 0, d_queue, o.tol, o.maxiter,
+    k_batch_gmres<<<kCl, kBT, mode == 1 ? kDyn : 0, s>>>(d_sys, d_info, d_order, 1, 1, 0, d_queue, o.tol, o.maxiter,
                                       budget, theta, bcgs);
     XB_LAUNCHED("k_batch_gmres (single system)");
     xb_batch_info r;
@@ -937,7 +943,9 @@ int xb_batch_create(int32_t count, const xb_batch_sys *sys, const xb_options *op
     }
     cudaError_t e = cudaFuncSetAttribute(k_batch_gmres, cudaFuncAttributeMaxDynamicSharedMemorySize, kDyn);
     if (e != cudaSuccess) return xb::cuda_error(e, "batch_create: shared memory");
-    const int clusters = resident_clusters();
+    // without mode 1 its tiles' shared memory is left to the L1
+    const size_t dyn = std::any_of(h.begin(), h.end(), [](const xb_batch_dev &d) { return d.mode == 1; }) ? kDyn : 0;
+    const int clusters = resident_clusters(dyn);
     const std::vector<int> order = split_systems(h, clusters);
     for (const xb_batch_dev &d : h)
         ws += (size_t)(d.m_max + 1) * d.ld + (size_t)(d.coop ? kCl : 1) * (d.m_max + 1) * d.m_max + 32;
@@ -1029,7 +1037,7 @@ int xb_batch_create(int32_t count, const xb_batch_sys *sys, const xb_options *op
         return fail(xb::cuda_error(e, "batch_create: begin capture"));
     }
     cudaMemsetAsync(bt->d_queue, 0, 2 * sizeof(int), cs);
-    k_batch_gmres<<<bt->grid, kBT, kDyn, cs>>>(bt->d_sys, bt->d_info, bt->d_order, count, nbig,
+    k_batch_gmres<<<bt->grid, kBT, dyn, cs>>>(bt->d_sys, bt->d_info, bt->d_order, count, nbig,
                                              nsmall_cl, bt->d_queue,
                                              o.tol, o.maxiter, budget, theta, bcgs);
     cudaError_t el = cudaGetLastError();

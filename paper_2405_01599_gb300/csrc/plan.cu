@@ -87,9 +87,12 @@ std::vector<int> tile_rows(int n, const int *rp, int block, int ipt) {
     int r = 0;
     while (r < n) {
         const int64_t k0 = rp[r];
-        int r1 = r + 1;
-        if ((int64_t)rp[r + 1] - k0 <= T)
-            while (r1 < n && r1 - r < block && (int64_t)rp[r1 + 1] - k0 <= T) r1++;
+        // the last row within T entries, block rows at most, one row at least: looked
+        // up, not walked to (a plan's first SpMV pays for this)
+        const int most = std::min<int64_t>(n, (int64_t)r + block);
+        int r1 = most;
+        if ((int64_t)rp[most] - k0 > T)
+            r1 = std::max(r + 1, (int)(std::upper_bound(rp + r, rp + most, k0 + T) - rp) - 1);
         rows.push_back(r1);
         r = r1;
     }

@@ -968,9 +968,9 @@ def batch(xb, torch, dev, args, cpu):
     systems, plans, shapes = [], [], []
     t_ml = t_ex = 0.0
     # the batched kernel's two in-CTA SpMV forms: thread per row (the U1
-    # counterpart) and warp-sized row blocks with warp- and CTA-wide long rows
-    # (the counterpart of the nnz-balanced U2 and U3); a tuned system takes
-    # the form of the family its tuner chose
+    # counterpart) and tiles of 256 entries (the counterpart of the
+    # nnz-balanced U2 and U3); a tuned system takes the form of the family its
+    # tuner chose
     mode_of = lambda v: 1 if v in (xb.VAR_NNZ, xb.VAR_SEGSCAN) else 0
     for sp in specs:
         A = gen.from_spec(sp)

@@ -667,9 +667,11 @@ int xb_tune_mlp(xb_plan *plan, const xb_csr *A, xb_mlp *model, xb_choice *out, i
  * the same algorithm as gmres_solve.  One persistent kernel (captured once in
  * a CUDA graph, replayed by xb_batch_run) holds as many CTAs as fit on the
  * GPU, in 8-CTA clusters; work comes from two atomic queues.  A system with
- * n >= 30000 (XB_BATCH_COOP_MIN_N in the environment overrides the
- * threshold) is solved by a whole cluster, its dot products combined through
- * distributed shared memory; these are taken first, largest first.  Once
+ * n >= 30000 is solved by a whole cluster, its dot products combined through
+ * distributed shared memory, and so are the largest others when an estimate of
+ * the launch's end says that it pays (XB_BATCH_COOP_MIN_N in the environment
+ * sets the rows and leaves the estimate out); these are taken first, largest
+ * first.  Once
  * they are all taken, every CTA pulls the smaller systems (largest first)
  * one at a time as soon as it is free, with no inter-CTA synchronisation.  opt: tol, maxiter (per
  * system), maxtime_s (whole launch; checked at every restart), dafrt /
@@ -677,10 +679,8 @@ int xb_tune_mlp(xb_plan *plan, const xb_csr *A, xb_mlp *model, xb_choice *out, i
  * (XB_ORTHO_MGS, XB_ORTHO_BCGS, or XB_ORTHO_AUTO: BCGS for tol > 1e-10,
  * else MGS; others are rejected).  Per system:
  * m in [1, XB_BATCH_MAX_M] and the SpMV mode inside the CTA (0: thread per
- * row; 1: thread per row in warp-sized row blocks, rows longer than 32
- * non-zeros taken by the whole warp, rows longer than 1024 by the whole CTA
- * after the blocks -- xb_batch_create reads each mode-1 system's row pointer
- * once to list them), as chosen by a tuner; zero_x = 1 makes the kernel
+ * row; 1: tiles of 256 non-zeros whatever their rows -- xb_batch_create reads
+ * each mode-1 system's row pointer once to cut them), as chosen by a tuner; zero_x = 1 makes the kernel
  * start from x = 0 (so a replay repeats the same solve). */
 #define XB_BATCH_MAX_M 128
 typedef struct xb_batch_sys {

@@ -735,12 +735,11 @@ int gmres_solve(xb_plan *p, const double *b, double *x, const xb_options *opt, x
                                   return r;
                               }
                               // else the batched kernel's single-system path (thread
-                              // per row, or warp-sized row blocks when rows are long),
+                              // per row, or tiles of non-zeros when rows are long),
                               // whose cluster streams the basis from L2: only while a
                               // step's work (about nnz + m n) stays small does it beat
-                              // the multi-launch step (measured: n = 4096 stencil 57
-                              // vs 148 us per step; n = 20,000 power-law rows 592 vs
-                              // 168 us on one CTA)
+                              // the multi-launch step (n = 4096 stencil: 23 vs 35 us
+                              // per step)
                               if ((double)p->nnz + (double)o.m * p->n <= 32.0 * o.small_n) {
                                   const int mode = p->max_row > 32 ? 1 : 0;
                                   r = xb::batch_single(p, b, x, o, mode, inf, &by, s);

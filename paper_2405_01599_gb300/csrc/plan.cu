@@ -795,11 +795,17 @@ using namespace xb;
 namespace xb {
 // Reduction scratch, pinned host mirror and timing events of a plan.
 int plan_scratch(xb_plan *p, cudaStream_t s) {
-    cudaError_t e = cudaMalloc(&p->d_part, (size_t)kRedSlots * kRedValues * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&p->d_ticket, gs_scratch_bytes());
-    if (e == cudaSuccess) e = cudaMalloc(&p->d_scal, (size_t)kScalars * sizeof(double));
-    if (e == cudaSuccess) e = cudaMemsetAsync(p->d_ticket, 0, gs_scratch_bytes(), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(p->d_scal, 0, (size_t)kScalars * sizeof(double), s);
+    // one allocation: the counters and the exchange, then the scalars (both zero at
+    // the start), then the partials
+    const size_t nt = (gs_scratch_bytes() + 255) / 256 * 256, ns = (size_t)kScalars * sizeof(double);
+    char *base = nullptr;
+    cudaError_t e = cudaMalloc(&base, nt + ns + (size_t)kRedSlots * kRedValues * sizeof(double));
+    if (e == cudaSuccess) {
+        p->d_ticket = reinterpret_cast<unsigned *>(base);
+        p->d_scal = reinterpret_cast<double *>(base + nt);
+        p->d_part = reinterpret_cast<double *>(base + nt + ns);
+        e = cudaMemsetAsync(base, 0, nt + ns, s);
+    }
     if (e == cudaSuccess) e = cudaMallocHost(&p->h_pin, 64 * sizeof(double));
     if (e == cudaSuccess) std::memset(p->h_pin, 0, 64 * sizeof(double));
     if (e == cudaSuccess) e = cudaEventCreate(&p->ev[0]);
@@ -982,9 +988,7 @@ int xb_plan_destroy(xb_plan *p) {
         cudaFree(t.d_val32);
     }
     cudaFree(p->d_empty);
-    cudaFree(p->d_part);
-    cudaFree(p->d_ticket);
-    cudaFree(p->d_scal);
+    cudaFree(p->d_ticket);  // with d_scal and d_part
     cudaFree(p->d_work);
     xb::ilu_free(p);
     if (p->h_pin) cudaFreeHost(p->h_pin);

@@ -194,14 +194,14 @@ __global__ void k_diag_fill(int n, const int *__restrict__ rows, const int *__re
 // replaces took ~6 us and a kernel per level ~4 us.  Consecutive rows per CTA
 // keep most hops of a stencil inside a CTA.  One application (GB300; the graph
 // of level launches or the level barrier, whichever was faster, in brackets):
-// 96^3 convection-diffusion 0.67 ms (2.0), 30^3 0.11 (0.44), 180^3 (blocks too
-// large for shared memory) 2.6 (4.3), power-law rows n = 20,000 0.16 (1.1), n =
-// 1M 0.50 (3.4).
+// 96^3 convection-diffusion 0.62-0.65 ms (2.0), 64^3 0.26, 30^3 0.11 (0.44), 180^3
+// (blocks too large for shared memory) 2.6 (4.3), power-law rows n = 20,000 0.09
+// (1.1), n = 1M 0.50 (3.4).
 //
 // Four entries a lane: an item is one round of loads and waits.  With a lane for
 // a row of up to 32 entries (up to 5 rounds of ~2 us, and the rows of a power law's
-// late levels are long) n = 1M took 1.04 ms, n = 20,000 0.46; with 2 / 3 / 6 entries
-// a lane n = 1M takes 0.76 / 0.54 / 0.49, n = 20,000 0.23 / 0.18 / 0.19.  The lanes'
+// late levels are long) n = 1M took 1.04 ms, n = 20,000 0.46 and 0.16 with four (2048
+// rows a block); with 2 / 3 / 6 entries a lane 0.76 / 0.54 / 0.49 and 0.23 / 0.18 / 0.19.  The lanes'
 // sums meet in a tree: against exact arithmetic 4.5e-17 of ||z||, one by one 4.6e-17
 // (power law, n = 200,000).
 //
@@ -210,8 +210,6 @@ __global__ void k_diag_fill(int n, const int *__restrict__ rows, const int *__re
 // wait is bounded all the same (`polls` polls, or `limit` ns): then the kernel
 // sets the error flag and every warp leaves at its next poll.
 constexpr int kFlowWarps = 16;
-constexpr int kFlowMinRows = 2048;  // rows of a CTA below which fewer CTAs do (30^3 grid: 122 us
-                                    // with 2048, 140 with 1024, 170 with 512)
 constexpr int kFlowFirst = 4;    // entries of each kind a lane has: all on their way at once
 constexpr int kFlowGroup = 8;    // entries a lane loads together in such a row
 constexpr unsigned long long kNotReady = 0xffffffffffffffffull;  // a NaN that is never stored
@@ -529,6 +527,30 @@ void level_order(const std::vector<int> &lev, int nlev, std::vector<int> &rows, 
     rows.resize(n);
     std::vector<int> at(off.begin(), off.end() - 1);
     for (int i = 0; i < n; i++) rows[at[lev[i]]++] = i;
+}
+
+// Rows of a CTA below which fewer CTAs do.  Where a block of R = 17 sqrt(n) rows
+// (16384 at most) is half as long again as nine of ten entries (of up to 4096 rows)
+// reach from the diagonal, such blocks keep more hops inside a CTA, until its 16
+// warps become the bound: grids of 30^3 / 48^3 / 64^3 / 96^3 take 112 / 219 / 321 / 664
+// us with 2048 rows or n / 152, 108 / 190 / 313 / 664 with 4096, 116 / 194 / 264 / 672
+// with 8192, 145 / - / 280 / 611 with 16384, - / - / 454 / 855 with 24576; 1000^2 1490 /
+// - / 1470 / 1396 / 1651.  A block that holds hardly one plane gains nothing (140 x
+// 100 x 60: 583 us with n / 152, 621 with 15,600).  Where entries reach far, a block's
+// rows wait for other blocks anyway, and more warps help: power-law rows n = 20,000
+// 156 us with 2048, 118 with 1024, 88 with 256, n = 200,000 178 / 147 / 147.
+int flow_min_rows(int n, const int *rp, const int *ci) {
+    const int R = (int)std::min(16384.0, 17.0 * std::sqrt((double)n)), step = std::max(1, n / 4096);
+    long long near = 0, reach = 0, all = 0;
+    for (int i = 0; i < n; i += step)
+        for (int k = rp[i]; k < rp[i + 1]; k++) {
+            const int d = std::abs(ci[k] - i);
+            if (d == 0) continue;
+            all++;
+            near += 2 * d <= R;
+            reach += 3 * d <= 2 * R;
+        }
+    return 10 * reach >= 9 * all ? std::max(256, R) : 2 * near >= all ? 2048 : 256;
 }
 
 // The flow substitution's layout of one triangle (FlowTri): every block's rows
@@ -889,7 +911,8 @@ int ensure_ilu(xb_plan *p, cudaStream_t s) {
     cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (coop && n > 0) {  // the flow layout, while the factorization runs
         const int cap = (smem - 1024) / 8 - 1;
-        const int G = std::max(1, std::min(num_sms(), (n + kFlowMinRows - 1) / kFlowMinRows));
+        const int least = flow_min_rows(n, rp.data(), ci.data());
+        const int G = std::max(1, std::min(num_sms(), (n + least - 1) / least));
         std::vector<int> bstart(G + 1, n);
         bstart[0] = 0;
         const double total = (double)nnz + 4.0 * n;  // blocks of about equal work

@@ -538,8 +538,10 @@ void level_order(const std::vector<int> &lev, int nlev, std::vector<int> &rows, 
 // - / 1470 / 1396 / 1651.  A block that holds hardly one plane gains nothing (140 x
 // 100 x 60: 583 us with n / 152, 621 with 15,600).  Where entries reach far, a block's
 // rows wait for other blocks anyway, and more warps help: power-law rows n = 20,000
-// 156 us with 2048, 118 with 1024, 88 with 256, n = 200,000 178 / 147 / 147.
-int flow_min_rows(int n, const int *rp, const int *ci) {
+// 156 us with 2048, 118 with 1024, 88 with 256, n = 200,000 178 / 147 / 147.  Large
+// blocks are for long chains (a level gives a CTA 64 rows at most), small ones for
+// wide levels (64 rows and more): else 2048.
+int flow_min_rows(int n, int levels, const int *rp, const int *ci) {
     const int R = (int)std::min(16384.0, 17.0 * std::sqrt((double)n)), step = std::max(1, n / 4096);
     long long near = 0, reach = 0, all = 0;
     for (int i = 0; i < n; i += step)
@@ -550,7 +552,8 @@ int flow_min_rows(int n, const int *rp, const int *ci) {
             near += 2 * d <= R;
             reach += 3 * d <= 2 * R;
         }
-    return 10 * reach >= 9 * all ? std::max(256, R) : 2 * near >= all ? 2048 : 256;
+    if (10 * reach >= 9 * all) return 64LL * levels >= R ? std::max(256, R) : 2048;
+    return 2 * near < all && 64LL * levels <= n ? 256 : 2048;
 }
 
 // The flow substitution's layout of one triangle (FlowTri): every block's rows
@@ -911,7 +914,7 @@ int ensure_ilu(xb_plan *p, cudaStream_t s) {
     cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (coop && n > 0) {  // the flow layout, while the factorization runs
         const int cap = (smem - 1024) / 8 - 1;
-        const int least = flow_min_rows(n, rp.data(), ci.data());
+        const int least = flow_min_rows(n, std::max(nl, nu), rp.data(), ci.data());
         const int G = std::max(1, std::min(num_sms(), (n + least - 1) / least));
         std::vector<int> bstart(G + 1, n);
         bstart[0] = 0;

@@ -452,6 +452,12 @@ int xb_mgs(xb_plan *plan, int32_t n, int32_t k, const double *V, int64_t ld, dou
  * h: device, k+1 doubles; 1 <= k <= 512; XB_ORTHO_AUTO is rejected. */
 int xb_orth(xb_plan *plan, int32_t n, int32_t k, const double *V, int64_t ld, double *w,
             double *h, int32_t ortho, void *stream);
+/* Controls of the plan's orthogonalisations (xb_orth, xb_mgs, the Arnoldi steps
+ * of the solvers), for tests and diagnosis.  XB_ORTH_NUMBER: the number after
+ * which the exchanges between CTAs are counted on (0 .. 2^32 - 1).  XB_EINVAL
+ * for another control or a value outside its range. */
+#define XB_ORTH_NUMBER 0
+int xb_orth_config(xb_plan *plan, int32_t what, int64_t value);
 
 /* ---- restarted Lanczos eigensolver (OpenATI_EIGENSOLVE, Sec. 2.2 / 4.3) ---
  * The nev largest eigenvalues of a symmetric A (general storage holding both

@@ -23,6 +23,7 @@ VAR_SYM_PART, VAR_SYM_WAGG, VAR_BCSR = 6, 7, 8
 VARIANT_NAMES = {0: "row", 1: "nnz", 2: "segscan", 3: "sym_atomic", 4: "sym_tile", 5: "sell",
                  6: "sym_part", 7: "sym_wagg", 8: "bcsr"}
 ORTHO_MGS, ORTHO_CGS, ORTHO_DGKS, ORTHO_BCGS, ORTHO_AUTO = 0, 1, 2, 3, 4
+ORTH_NUMBER = 0
 POLICY_NONE, POLICY_TIME, POLICY_ACCURACY, POLICY_MEMORY, POLICY_STABLE = 0, 1, 2, 3, 4
 PRECOND_NONE, PRECOND_ILU0 = 0, 1
 EIG_LR, EIG_LM = 0, 1
@@ -127,6 +128,7 @@ def lib():
         "xb_axpy": (i32, [i32, f64, vp, vp, vp]),
         "xb_mgs": (i32, [vp, i32, i32, vp, C.c_int64, vp, vp, vp]),
         "xb_orth": (i32, [vp, i32, i32, vp, C.c_int64, vp, vp, i32, vp]),
+        "xb_orth_config": (i32, [vp, i32, C.c_int64]),
         "xb_lanczos": (i32, [vp, i32, i32, i32, f64, f64, i32, i32, vp, P(f64), vp, P(f64),
                              P(i32), P(f64), vp]),
         "xb_arnoldi": (i32, [vp, i32, i32, i32, f64, f64, i32, i32, i32, i32, vp, P(f64), P(f64),
@@ -570,6 +572,11 @@ class Plan:
         lu = torch.empty(self.nnz, dtype=torch.float64, device=self._keep[2].device)
         _check(lib().xb_ilu0_factors(self._h, _ptr(lu), _stream(stream)))
         return lu
+
+    def orth_config(self, what, value):
+        """Sets a control of the orthogonalisations (ORTH_NUMBER: the number
+        after which their exchanges are counted on)."""
+        _check(lib().xb_orth_config(self._h, int(what), int(value)))
 
     def orth(self, V, w, ortho, stream=None):
         """Orthogonalise w against the k rows of V with ORTHO_MGS / CGS / DGKS /

@@ -231,6 +231,8 @@ struct xb_plan {
     size_t work_bytes = 0;
     double *h_pin = nullptr;             // pinned host mirror of a few scalars
     unsigned long long gs_tag = 0;       // orthogonalisations launched
+    unsigned gs_number = 0;              // the newest one's last exchange number
+    bool gs_recount = false;             // the number was set back: slots may hold what comes
     // tuned choice
     int variant = XB_VAR_NNZ, block = 256, ipt = 8;
     float tuned_ms = 0.f;

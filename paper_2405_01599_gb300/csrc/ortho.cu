@@ -18,6 +18,8 @@ constexpr int kGsMaxClusters = 96;   // clusters one exchange has room for
 constexpr int kGsVals = 64;          // values of one exchange
 constexpr int kGsMaxK = 512;         // basis rows
 constexpr int kGsMaxStages = 8;
+constexpr int kGsSlotsAt = 128;      // words of d_ticket before the grid's exchange slots
+constexpr size_t kGsSlotBytes = sizeof(ulonglong2) * 2 * kGsVals * kGsMaxClusters;
 constexpr long long kGsWait = 4000000000LL;  // cycles (~2 s) after which a wait gives up
 
 template <typename VB>
@@ -28,7 +30,8 @@ struct GsArgs {
     xb::GmDev st;         // misc null: a plain sweep (unit scales, never stopped)
     double *col;          // column j: h_0..h_j, then ||w||
     int j, method, cs, stages;
-    unsigned *hdr;        // [0] exchange number, [1] a wait ran out
+    unsigned base;        // this launch's exchanges have the numbers base + 1, base + 2, ..
+    unsigned *stop;       // a wait of the grid ran out
     ulonglong2 *slots;    // 2 x kGsVals x kGsMaxClusters
     int *err;             // host-visible: a wait ran out
     unsigned long long *late, tag;  // host-visible words: 4 tag + GM_STOP after step tag
@@ -37,7 +40,8 @@ struct GsArgs {
 // ---- values that carry their exchange number ------------------------------------
 // A double travels as two 8-byte words, each with the number of its exchange:
 // a reader that sees the number in both has the whole value, whatever order
-// the words arrive in, and no fence or flag is needed.
+// the words arrive in, and no fence or flag is needed.  A slot that was never
+// written has number 0, which no exchange has (gs_numbers).
 __device__ __forceinline__ void pack(double v, unsigned seq, unsigned long long &x,
                                      unsigned long long &y) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
@@ -139,11 +143,11 @@ __device__ __forceinline__ void bulk_copy(unsigned dst, const void *src, unsigne
 struct Patience {
     unsigned it = 0;
     long long t0 = 0;
-    __device__ __forceinline__ bool expired(const unsigned *hdr) {
+    __device__ __forceinline__ bool expired(const unsigned *stop) {
         if (++it & 255u) return false;
         const long long now = clock64();
         if (t0 == 0) t0 = now;
-        return now - t0 > kGsWait || *reinterpret_cast<const volatile unsigned *>(hdr + 1) != 0u;
+        return now - t0 > kGsWait || *reinterpret_cast<const volatile unsigned *>(stop) != 0u;
     }
 };
 
@@ -197,7 +201,6 @@ struct GsShared {
     VB cf[kGsMaxK];                               // CGS, DGKS: one for the CTA
     VB cfw[gs_threads<VB>() / 32][KB];            // block methods: one for each warp
     int abort;
-    unsigned base;
 };
 
 // The CTA's state: everything the roles share.
@@ -225,7 +228,7 @@ struct Ctx {
 template <typename VB, int KB>
 __device__ __forceinline__ void give_up(Ctx<VB, KB> &c) {
     *reinterpret_cast<volatile int *>(&c.S->abort) = 1;
-    *reinterpret_cast<volatile unsigned *>(c.a->hdr + 1) = 1u;
+    *reinterpret_cast<volatile unsigned *>(c.a->stop) = 1u;
     *reinterpret_cast<volatile int *>(c.a->err) = 1;
     c.fine = false;
 }
@@ -235,7 +238,7 @@ __device__ __forceinline__ bool wait_bar(Ctx<VB, KB> &c, unsigned bar, unsigned 
     Patience w;
     while (!mbar_done(bar, parity)) {
         if (*reinterpret_cast<volatile int *>(&c.S->abort)) return false;
-        if (w.expired(c.a->hdr)) {
+        if (w.expired(c.a->stop)) {
             give_up(c);
             return false;
         }
@@ -492,7 +495,7 @@ __device__ __forceinline__ double cluster_sum(Ctx<VB, KB> &c, int q, unsigned se
                 all = all && got[s];
             }
         if (__all_sync(0xffffffffu, all)) break;
-        if (__any_sync(0xffffffffu, w.expired(c.a->hdr))) {
+        if (__any_sync(0xffffffffu, w.expired(c.a->stop))) {
             give_up(c);
             break;
         }
@@ -530,7 +533,7 @@ __device__ __forceinline__ double grid_sum(Ctx<VB, KB> &c, int q, unsigned seq) 
                 all = all && got[s];
             }
         if (__all_sync(0xffffffffu, all)) break;
-        if (__any_sync(0xffffffffu, w.expired(c.a->hdr))) {
+        if (__any_sync(0xffffffffu, w.expired(c.a->stop))) {
             give_up(c);
             break;
         }
@@ -572,7 +575,7 @@ __device__ __forceinline__ double totals(Ctx<VB, KB> &c, int q0, int nv, unsigne
             if (got) r = v;
         }
         if (__all_sync(0xffffffffu, got)) break;
-        if (__any_sync(0xffffffffu, w.expired(c.a->hdr))) {
+        if (__any_sync(0xffffffffu, w.expired(c.a->stop))) {
             give_up(c);
             break;
         }
@@ -608,7 +611,6 @@ __device__ void scalar_warp(Ctx<VB, KB> &c, unsigned seq, bool raw) {
         }
     }
     const double nn = grid_sum(c, 0, seq);
-    if (lane == 0) a.hdr[0] = seq;
     if (!c.fine) return;
     if (raw) {
         if (lane == 0) a.col[j + 1] = sqrt(nn);
@@ -713,7 +715,6 @@ __global__ void __launch_bounds__(gs_threads<VB>() + 64, 1) k_gs(const __grid_co
         reinterpret_cast<ulonglong2 *>(dyn)[i] = make_ulonglong2(0, 0);
     if (tid == 0) {
         S.abort = 0;
-        S.base = *reinterpret_cast<volatile unsigned *>(a.hdr);
         for (int s = 0; s < a.stages; s++) {
             mbar_init(sptr(&S.full[s]), 1);
             mbar_init(sptr(&S.empty[s]), NW);
@@ -721,7 +722,7 @@ __global__ void __launch_bounds__(gs_threads<VB>() + 64, 1) k_gs(const __grid_co
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     cluster_sync();
-    unsigned seq = S.base;
+    unsigned seq = a.base;
     const bool blocks = a.method == XB_ORTHO_MGS || a.method == XB_ORTHO_BCGS;
     const int nb = (k + KB - 1) / KB, rounds = a.method == XB_ORTHO_DGKS ? 2 : 1;
     const int groups = (k + kGsVals - 1) / kGsVals;
@@ -755,11 +756,8 @@ __global__ void __launch_bounds__(gs_threads<VB>() + 64, 1) k_gs(const __grid_co
     } else if (c.wv > NW) {
         if (blockIdx.x == 0) {
             bar_sync(2, NT + 32);
-            if (*reinterpret_cast<volatile int *>(&S.abort)) {
-                if (c.lane == 0) a.hdr[0] = seq + 1024u;
-            } else {
+            if (!*reinterpret_cast<volatile int *>(&S.abort))
                 scalar_warp(c, seq + (blocks ? nb : rounds * groups) + 1, raw);
-            }
         }
     } else {
         VB *wg = a.w + c0;
@@ -937,8 +935,22 @@ int launch(GsArgs<VB> &a, int clusters, size_t smem, cudaStream_t s) {
     return XB_OK;
 }
 
+// The numbers of a launch of `used` exchanges, after those of the launch before.
+// They never pass 0: before they would, the grid's slots, in which a number may
+// have stood since the last time round, are cleared and the count begins again
+// (a launch clears its CTAs' slots itself).
+int gs_numbers(xb_plan *p, unsigned used, unsigned *base, cudaStream_t s) {
+    const bool pass = p->gs_number > 0xffffffffu - used;
+    if (pass || p->gs_recount) XB_CUDA(cudaMemsetAsync(p->d_ticket + kGsSlotsAt, 0, kGsSlotBytes, s));
+    if (pass) p->gs_number = 0;
+    p->gs_recount = false;
+    *base = p->gs_number;
+    p->gs_number += used;
+    return XB_OK;
+}
+
 template <typename VB, int KB, int GRAM>
-int plan_launch(GsArgs<VB> &a, cudaStream_t s) {
+int plan_launch(xb_plan *p, GsArgs<VB> &a, cudaStream_t s) {
     struct Limits {
         cudaError_t e;
         int nc[9];
@@ -974,41 +986,46 @@ int plan_launch(GsArgs<VB> &a, cudaStream_t s) {
     const bool sm = fixed + 3 * stage + wb <= (size_t)xb::kGsDynMax;
     a.stages = (int)std::min<size_t>(kGsMaxStages, (xb::kGsDynMax - fixed - (sm ? wb : 0)) / stage);
     const size_t smem = fixed + a.stages * stage + (sm ? wb : 0);
+    const int k = a.j + 1;
+    const bool blocks = a.method == XB_ORTHO_MGS || a.method == XB_ORTHO_BCGS;
+    const int sums = blocks ? (k + KB - 1) / KB
+                            : (a.method == XB_ORTHO_DGKS ? 2 : 1) * ((k + kGsVals - 1) / kGsVals);
+    XB_TRY(gs_numbers(p, (unsigned)sums + 1, &a.base, s));
     return sm ? launch<VB, KB, GRAM, true>(a, nc, smem, s) : launch<VB, KB, GRAM, false>(a, nc, smem, s);
 }
 
 template <typename VB>
 int gs_run(xb_plan *p, GsArgs<VB> &a, bool seen, cudaStream_t s) {
-    a.hdr = p->d_ticket + 64;
-    a.slots = reinterpret_cast<ulonglong2 *>(p->d_ticket + 128);
+    a.stop = p->d_ticket + 64;
+    a.slots = reinterpret_cast<ulonglong2 *>(p->d_ticket + kGsSlotsAt);
     a.err = reinterpret_cast<int *>(p->h_pin + 60);
     a.late = reinterpret_cast<unsigned long long *>(p->h_pin + 40);
     a.tag = ++p->gs_tag;
-    if (a.method == XB_ORTHO_BCGS) return plan_launch<VB, 4, 0>(a, s);
-    if (a.method != XB_ORTHO_MGS) return plan_launch<VB, 8, 0>(a, s);
+    if (a.method == XB_ORTHO_BCGS) return plan_launch<VB, 4, 0>(p, a, s);
+    if (a.method != XB_ORTHO_MGS) return plan_launch<VB, 8, 0>(p, a, s);
     if constexpr (sizeof(VB) == 8) {
         if (!seen) {
             // n = 262,144 (16 rows): blocks of 4 / 2 59.9 / 61.5 us; n = 1M (20
             // rows) 162 / 151 us: beyond, the rows' own products cost more FP64
             // time than the exchanges they save
-            if (a.n < 600000) return plan_launch<VB, 4, 2>(a, s);
-            return plan_launch<VB, 2, 2>(a, s);
+            if (a.n < 600000) return plan_launch<VB, 4, 2>(p, a, s);
+            return plan_launch<VB, 2, 2>(p, a, s);
         }
     }
-    return plan_launch<VB, 8, 1>(a, s);
+    return plan_launch<VB, 8, 1>(p, a, s);
 }
 
 }  // namespace
 
 namespace xb {
 
-size_t gs_scratch_bytes() { return 128 * sizeof(unsigned) + sizeof(ulonglong2) * 2 * kGsVals * kGsMaxClusters; }
+size_t gs_scratch_bytes() { return kGsSlotsAt * sizeof(unsigned) + kGsSlotBytes; }
 
 int gs_check(xb_plan *p) {
     volatile int *err = reinterpret_cast<volatile int *>(p->h_pin + 60);
     if (!*err) return XB_OK;
     *err = 0;
-    XB_CUDA(cudaMemset(p->d_ticket + 64, 0, gs_scratch_bytes() - 64 * sizeof(unsigned)));
+    XB_CUDA(cudaMemset(p->d_ticket + 64, 0, sizeof(unsigned)));
     return set_error(XB_ETIMEOUT, "orthogonalisation: a grid exchange ran out of time");
 }
 
@@ -1045,3 +1062,12 @@ int ortho_sweep(xb_plan *p, int64_t n, int k, const double *V, int64_t ld, doubl
 }
 
 }  // namespace xb
+
+extern "C" int xb_orth_config(xb_plan *p, int32_t what, int64_t value) {
+    if (p && what == XB_ORTH_NUMBER && value >= 0 && value <= 0xffffffffLL) {
+        p->gs_recount = p->gs_recount || (unsigned)value < p->gs_number;
+        p->gs_number = (unsigned)value;
+        return XB_OK;
+    }
+    return xb::set_error(XB_EINVAL, "orth_config: plan %p control %d value %lld", (void *)p, what, (long long)value);
+}

@@ -454,9 +454,14 @@ int xb_orth(xb_plan *plan, int32_t n, int32_t k, const double *V, int64_t ld, do
             double *h, int32_t ortho, void *stream);
 /* Controls of the plan's orthogonalisations (xb_orth, xb_mgs, the Arnoldi steps
  * of the solvers), for tests and diagnosis.  XB_ORTH_NUMBER: the number after
- * which the exchanges between CTAs are counted on (0 .. 2^32 - 1).  XB_EINVAL
- * for another control or a value outside its range. */
+ * which the exchanges between CTAs are counted on (0 .. 2^32 - 1).
+ * XB_ORTH_POLLS: how many times a warp polls in one wait before it gives up
+ * (0 .. 2^31 - 1; 0 = default: about 2 s); then every warp leaves at its next
+ * look at the flag, and the call reports XB_ETIMEOUT (w, h and a solver's x are
+ * not usable; the next call is).  XB_EINVAL for another control or a value
+ * outside its range. */
 #define XB_ORTH_NUMBER 0
+#define XB_ORTH_POLLS 1
 int xb_orth_config(xb_plan *plan, int32_t what, int64_t value);
 
 /* ---- restarted Lanczos eigensolver (OpenATI_EIGENSOLVE, Sec. 2.2 / 4.3) ---

@@ -84,7 +84,7 @@ int xb_mgs(xb_plan *p, int32_t n, int32_t k, const double *V, int64_t ld, double
     cudaStream_t s = (cudaStream_t)stream;
     XB_TRY(xb::ortho_sweep(p, n, k, V, ld, w, h, XB_ORTHO_MGS, s));
     XB_CUDA(cudaStreamSynchronize(s));
-    return xb::gs_check(p);
+    return xb::gs_check(p, s);
 }
 
 int xb_orth(xb_plan *p, int32_t n, int32_t k, const double *V, int64_t ld, double *w, double *h,
@@ -95,7 +95,7 @@ int xb_orth(xb_plan *p, int32_t n, int32_t k, const double *V, int64_t ld, doubl
     cudaStream_t s = (cudaStream_t)stream;
     XB_TRY(xb::ortho_sweep(p, n, k, V, ld, w, h, ortho, s));
     XB_CUDA(cudaStreamSynchronize(s));
-    return xb::gs_check(p);
+    return xb::gs_check(p, s);
 }
 
 }  // extern "C"

@@ -280,7 +280,7 @@ int xb_lanczos(xb_plan *p, int32_t nev, int32_t m, int32_t m_max, double theta, 
         XB_CUDA(cudaMemcpyAsync(H.data(), st.H, H.size() * sizeof(double), cudaMemcpyDeviceToHost,
                                 s));
         XB_CUDA(cudaStreamSynchronize(s));
-        XB_TRY(xb::gs_check(p));
+        XB_TRY(xb::gs_check(p, s));
         for (int j = k; j < m; j++)
             for (int i = 0; i <= j + 1; i++)
                 T[(size_t)i * (M + 1) + j] = H[(size_t)j * (M + 1) + i];
@@ -498,7 +498,7 @@ int xb_arnoldi(xb_plan *p, int32_t nev, int32_t m, int32_t m_max, double theta, 
         XB_CUDA(cudaMemcpyAsync(H.data(), st.H, H.size() * sizeof(double), cudaMemcpyDeviceToHost,
                                 s));
         XB_CUDA(cudaStreamSynchronize(s));
-        XB_TRY(xb::gs_check(p));
+        XB_TRY(xb::gs_check(p, s));
         for (int j = k; j < m; j++)
             for (int i = 0; i <= j + 1; i++)
                 T[(size_t)i * (M + 1) + j] = H[(size_t)j * (M + 1) + i];

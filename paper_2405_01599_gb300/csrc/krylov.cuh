@@ -52,8 +52,8 @@ int gm_ortho_step(xb_plan *p, GmDev st, int64_t n, const VB *V, int64_t ld, VB *
 // w against the k rows of V (unit scales); h: k coefficients, then ||w||.
 int ortho_sweep(xb_plan *p, int64_t n, int k, const double *V, int64_t ld, double *w, double *h,
                 int ortho, cudaStream_t s);
-// XB_ETIMEOUT if a grid exchange of an earlier, finished launch ran out of time.
-int gs_check(xb_plan *p);
+// XB_ETIMEOUT if a wait of an earlier, finished launch (on stream s) ran out.
+int gs_check(xb_plan *p, cudaStream_t s);
 // Algorithmic vector passes (multiples of n elements read + written) of one
 // orthogonalisation of step j.
 double ortho_passes(int ortho, int j);

@@ -32,6 +32,7 @@ struct GsArgs {
     int j, method, cs, stages;
     unsigned base;        // this launch's exchanges have the numbers base + 1, base + 2, ..
     unsigned *stop;       // a wait of the grid ran out
+    unsigned polls, look; // polls of one wait (0: the clock decides); polls between looks
     ulonglong2 *slots;    // 2 x kGsVals x kGsMaxClusters
     int *err;             // host-visible: a wait ran out
     unsigned long long *late, tag;  // host-visible words: 4 tag + GM_STOP after step tag
@@ -138,16 +139,20 @@ __device__ __forceinline__ void bulk_copy(unsigned dst, const void *src, unsigne
                  : "memory");
 }
 
-// A bounded wait: expired() is true once the wait has lasted kGsWait cycles or
-// another wait of the grid has run out.
+// A bounded wait: expired() is true once the wait has lasted kGsWait cycles, or
+// as many polls as the caller allows, or another wait of the grid has run out.
+// Between looks at the clock and the grid's flag a poll costs one add.
 struct Patience {
     unsigned it = 0;
     long long t0 = 0;
-    __device__ __forceinline__ bool expired(const unsigned *stop) {
-        if (++it & 255u) return false;
+    template <typename VB>
+    __device__ __forceinline__ bool expired(const GsArgs<VB> &a) {
+        if (++it < a.look) return false;
+        if (a.polls != 0) return true;
+        it = 0;
         const long long now = clock64();
         if (t0 == 0) t0 = now;
-        return now - t0 > kGsWait || *reinterpret_cast<const volatile unsigned *>(stop) != 0u;
+        return now - t0 > kGsWait || *reinterpret_cast<const volatile unsigned *>(a.stop) != 0u;
     }
 };
 
@@ -233,17 +238,21 @@ __device__ __forceinline__ void give_up(Ctx<VB, KB> &c) {
     c.fine = false;
 }
 
+// The whole warp waits and goes on, or gives up, together: what follows a wait
+// has shuffles and votes in it.
 template <typename VB, int KB>
 __device__ __forceinline__ bool wait_bar(Ctx<VB, KB> &c, unsigned bar, unsigned parity) {
     Patience w;
-    while (!mbar_done(bar, parity)) {
-        if (*reinterpret_cast<volatile int *>(&c.S->abort)) return false;
-        if (w.expired(c.a->stop)) {
+    bool ok = true;
+    while (ok && !mbar_done(bar, parity)) {
+        if (*reinterpret_cast<volatile int *>(&c.S->abort)) {
+            ok = false;
+        } else if (w.expired(*c.a)) {
             give_up(c);
-            return false;
+            ok = false;
         }
     }
-    return true;
+    return __all_sync(0xffffffffu, ok);
 }
 
 // ---- producer ---------------------------------------------------------------------
@@ -273,16 +282,16 @@ __device__ __forceinline__ void produce(Ctx<VB, KB> &c, int t, int row0, int nr,
     c.next();
 }
 
-// Waits for the copies that are in flight (a sweep that is given up must not
-// leave any behind).
+// Waits for the copies that are in flight.  The consumers of a sweep that is
+// given up may leave them behind, at any time until the end, and a CTA must not
+// end before its copies; a sweep that is not has waited for them all.
 template <typename VB, int KB>
 __device__ void drain(Ctx<VB, KB> &c) {
     for (int i = 0; i < c.a->stages; i++) {
         const int ph = i < c.st ? c.ph : c.ph - 1;  // the stage's last use
         if (ph < 0) continue;
-        Patience w;
-        while (!mbar_done(sptr(&c.S->full[i]), ph & 1))
-            if (++w.it > (1u << 22)) break;
+        for (unsigned it = 0; it < (1u << 22) && !mbar_done(sptr(&c.S->full[i]), ph & 1); it++) {
+        }
     }
 }
 
@@ -495,7 +504,7 @@ __device__ __forceinline__ double cluster_sum(Ctx<VB, KB> &c, int q, unsigned se
                 all = all && got[s];
             }
         if (__all_sync(0xffffffffu, all)) break;
-        if (__any_sync(0xffffffffu, w.expired(c.a->stop))) {
+        if (__any_sync(0xffffffffu, w.expired(*c.a))) {
             give_up(c);
             break;
         }
@@ -533,7 +542,7 @@ __device__ __forceinline__ double grid_sum(Ctx<VB, KB> &c, int q, unsigned seq) 
                 all = all && got[s];
             }
         if (__all_sync(0xffffffffu, all)) break;
-        if (__any_sync(0xffffffffu, w.expired(c.a->stop))) {
+        if (__any_sync(0xffffffffu, w.expired(*c.a))) {
             give_up(c);
             break;
         }
@@ -575,7 +584,7 @@ __device__ __forceinline__ double totals(Ctx<VB, KB> &c, int q0, int nv, unsigne
             if (got) r = v;
         }
         if (__all_sync(0xffffffffu, got)) break;
-        if (__any_sync(0xffffffffu, w.expired(c.a->stop))) {
+        if (__any_sync(0xffffffffu, w.expired(*c.a))) {
             give_up(c);
             break;
         }
@@ -752,7 +761,7 @@ __global__ void __launch_bounds__(gs_threads<VB>() + 64, 1) k_gs(const __grid_co
                     }
                 }
         }
-        if (!c.fine) drain(c);
+        drain(c);
     } else if (c.wv > NW) {
         if (blockIdx.x == 0) {
             bar_sync(2, NT + 32);
@@ -997,6 +1006,8 @@ int plan_launch(xb_plan *p, GsArgs<VB> &a, cudaStream_t s) {
 template <typename VB>
 int gs_run(xb_plan *p, GsArgs<VB> &a, bool seen, cudaStream_t s) {
     a.stop = p->d_ticket + 64;
+    a.polls = p->gs_polls;
+    a.look = a.polls ? a.polls : 256u;
     a.slots = reinterpret_cast<ulonglong2 *>(p->d_ticket + kGsSlotsAt);
     a.err = reinterpret_cast<int *>(p->h_pin + 60);
     a.late = reinterpret_cast<unsigned long long *>(p->h_pin + 40);
@@ -1021,11 +1032,12 @@ namespace xb {
 
 size_t gs_scratch_bytes() { return kGsSlotsAt * sizeof(unsigned) + kGsSlotBytes; }
 
-int gs_check(xb_plan *p) {
+int gs_check(xb_plan *p, cudaStream_t s) {
     volatile int *err = reinterpret_cast<volatile int *>(p->h_pin + 60);
     if (!*err) return XB_OK;
     *err = 0;
-    XB_CUDA(cudaMemset(p->d_ticket + 64, 0, sizeof(unsigned)));
+    XB_CUDA(cudaMemsetAsync(p->d_ticket + 64, 0, sizeof(unsigned), s));
+    XB_CUDA(cudaStreamSynchronize(s));  // the next launch may be on another stream
     return set_error(XB_ETIMEOUT, "orthogonalisation: a grid exchange ran out of time");
 }
 
@@ -1067,6 +1079,10 @@ extern "C" int xb_orth_config(xb_plan *p, int32_t what, int64_t value) {
     if (p && what == XB_ORTH_NUMBER && value >= 0 && value <= 0xffffffffLL) {
         p->gs_recount = p->gs_recount || (unsigned)value < p->gs_number;
         p->gs_number = (unsigned)value;
+        return XB_OK;
+    }
+    if (p && what == XB_ORTH_POLLS && value >= 0 && value <= 0x7fffffffLL) {
+        p->gs_polls = (unsigned)value;
         return XB_OK;
     }
     return xb::set_error(XB_EINVAL, "orth_config: plan %p control %d value %lld", (void *)p, what, (long long)value);

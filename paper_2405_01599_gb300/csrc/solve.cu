@@ -30,7 +30,7 @@ double secs_since(clk::time_point t0) {
 int peek(xb_plan *p, const double *dev, int cnt, cudaStream_t s) {
     XB_CUDA(cudaMemcpyAsync(p->h_pin, dev, cnt * sizeof(double), cudaMemcpyDeviceToHost, s));
     XB_CUDA(cudaStreamSynchronize(s));
-    return xb::gs_check(p);
+    return xb::gs_check(p, s);
 }
 
 // The stop flag of the orthogonalisation launched as number tag, which its

@@ -9,6 +9,7 @@
 // summed over the grid with one exchange per block of rows instead of one
 // launch per row.
 #include "krylov.cuh"
+#include "perdevice.cuh"
 
 #include <algorithm>
 
@@ -908,7 +909,7 @@ __global__ void __launch_bounds__(gs_threads<VB>() + 64, 1) k_gs(const __grid_co
 
 // Largest number of clusters of cs CTAs, one CTA per SM, that the GPU holds.
 template <typename K>
-int max_clusters(K kernel, int threads, int cs) {
+int max_clusters(K kernel, int threads, int cs, int *clusters) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cs);
     cfg.blockDim = dim3(threads);
@@ -920,9 +921,9 @@ int max_clusters(K kernel, int threads, int cs) {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int nc = 0;
-    if (cudaOccupancyMaxActiveClusters(&nc, kernel, &cfg) != cudaSuccess) nc = 0;
-    cudaGetLastError();
-    return std::min(nc, kGsMaxClusters);
+    XB_CUDA(cudaOccupancyMaxActiveClusters(&nc, kernel, &cfg));
+    *clusters = std::min(nc, kGsMaxClusters);
+    return XB_OK;
 }
 
 template <typename VB, int KB, int GRAM, bool SM>
@@ -961,20 +962,21 @@ int gs_numbers(xb_plan *p, unsigned used, unsigned *base, cudaStream_t s) {
 template <typename VB, int KB, int GRAM>
 int plan_launch(xb_plan *p, GsArgs<VB> &a, cudaStream_t s) {
     struct Limits {
-        cudaError_t e;
         int nc[9];
     };
-    static const Limits lim = [] {
-        Limits l{};
-        l.e = cudaFuncSetAttribute(k_gs<VB, KB, GRAM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   xb::kGsDynMax);
-        if (l.e == cudaSuccess)
-            l.e = cudaFuncSetAttribute(k_gs<VB, KB, GRAM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       xb::kGsDynMax);
-        for (int cs : {2, 4, 8}) l.nc[cs] = max_clusters(k_gs<VB, KB, GRAM, true>, gs_threads<VB>() + 64, cs);
-        return l;
-    }();
-    if (lim.e != cudaSuccess) return xb::cuda_error(lim.e, "orthogonalisation: shared memory");
+    static xb::PerDevice<Limits> limits;
+    Limits lim;
+    int dev = 0;
+    XB_CUDA(cudaGetDevice(&dev));
+    XB_TRY(limits.get(dev, [](Limits &l) {
+        XB_CUDA(cudaFuncSetAttribute(k_gs<VB, KB, GRAM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     xb::kGsDynMax));
+        XB_CUDA(cudaFuncSetAttribute(k_gs<VB, KB, GRAM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     xb::kGsDynMax));
+        for (int cs : {2, 4, 8})
+            XB_TRY(max_clusters(k_gs<VB, KB, GRAM, true>, gs_threads<VB>() + 64, cs, &l.nc[cs]));
+        return (int)XB_OK;
+    }, &lim));
     // Larger clusters make the exchange cheaper (3.1 / 3.5 / 4.6 us with 8 / 4 / 2
     // CTAs) but leave SMs out (120 / 144 / 152 of 152 hold a CTA).  DGKS against 20
     // rows, clusters of 2 / 4 / 8: n = 27,000 32.0 / 30.7 / 30.6 us; against 16

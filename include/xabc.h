@@ -17,6 +17,15 @@
  *     that stream.
  *   - Return value: XB_OK (0) or a negative XB_E* code.  The message of the
  *     last error on the calling host thread is returned by xb_last_error().
+ *   - Some launches hold their SMs together, one CTA on each: an
+ *     orthogonalisation (xb_orth, xb_mgs, and every step of the multi-launch
+ *     GMRES and of the eigensolvers; up to every SM from about 40,000 rows on)
+ *     and an ILU(0) substitution (up to every SM).  Such a launch starts when
+ *     all its SMs are free, so beside work on other streams it waits for that
+ *     work's CTAs to end, and the calls' results do not depend on it.  A kernel
+ *     that stays on an SM until such a call is over must be left its SM:
+ *     xb_orth_config with XB_ORTH_CTAS, and xb_ilu0_config with mode 0 (a launch
+ *     per dependency level, which needs no SMs together).
  *   - A plan (xb_plan) owns library workspace in device memory, created by
  *     xb_plan_create and released by xb_plan_destroy.  A plan may be used by
  *     one host thread / one stream at a time.
@@ -458,10 +467,12 @@ int xb_orth(xb_plan *plan, int32_t n, int32_t k, const double *V, int64_t ld, do
  * XB_ORTH_POLLS: how many times a warp polls in one wait before it gives up
  * (0 .. 2^31 - 1; 0 = default: about 2 s); then every warp leaves at its next
  * look at the flag, and the call reports XB_ETIMEOUT (w, h and a solver's x are
- * not usable; the next call is).  XB_EINVAL for another control or a value
- * outside its range. */
+ * not usable; the next call is).  XB_ORTH_CTAS: the most CTAs, one per SM, that
+ * one may hold (0 = default: as many as fit and n fills; else at least 2).
+ * XB_EINVAL for another control or a value outside its range. */
 #define XB_ORTH_NUMBER 0
 #define XB_ORTH_POLLS 1
+#define XB_ORTH_CTAS 2
 int xb_orth_config(xb_plan *plan, int32_t what, int64_t value);
 
 /* ---- restarted Lanczos eigensolver (OpenATI_EIGENSOLVE, Sec. 2.2 / 4.3) ---

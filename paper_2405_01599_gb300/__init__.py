@@ -23,7 +23,7 @@ VAR_SYM_PART, VAR_SYM_WAGG, VAR_BCSR = 6, 7, 8
 VARIANT_NAMES = {0: "row", 1: "nnz", 2: "segscan", 3: "sym_atomic", 4: "sym_tile", 5: "sell",
                  6: "sym_part", 7: "sym_wagg", 8: "bcsr"}
 ORTHO_MGS, ORTHO_CGS, ORTHO_DGKS, ORTHO_BCGS, ORTHO_AUTO = 0, 1, 2, 3, 4
-ORTH_NUMBER, ORTH_POLLS = 0, 1
+ORTH_NUMBER, ORTH_POLLS, ORTH_CTAS = 0, 1, 2
 POLICY_NONE, POLICY_TIME, POLICY_ACCURACY, POLICY_MEMORY, POLICY_STABLE = 0, 1, 2, 3, 4
 PRECOND_NONE, PRECOND_ILU0 = 0, 1
 EIG_LR, EIG_LM = 0, 1
@@ -576,7 +576,7 @@ class Plan:
     def orth_config(self, what, value):
         """Sets a control of the orthogonalisations (ORTH_NUMBER: the number
         after which their exchanges are counted on; ORTH_POLLS: polls of one
-        wait, 0 for the default)."""
+        wait, 0 for the default; ORTH_CTAS: the SMs one may hold, 0 for all)."""
         _check(lib().xb_orth_config(self._h, int(what), int(value)))
 
     def orth(self, V, w, ortho, stream=None):

@@ -231,6 +231,7 @@ struct xb_plan {
     size_t work_bytes = 0;
     double *h_pin = nullptr;             // pinned host mirror of a few scalars
     unsigned long long gs_tag = 0;       // orthogonalisations launched
+    int gs_ctas = 0;                     // CTAs one may hold (0: as many as fit)
     unsigned gs_polls = 0;               // polls of one of their waits (0: default)
     unsigned gs_number = 0;              // the newest one's last exchange number
     bool gs_recount = false;             // the number was set back: slots may hold what comes

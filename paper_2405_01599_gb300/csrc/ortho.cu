@@ -983,12 +983,15 @@ int plan_launch(xb_plan *p, GsArgs<VB> &a, cudaStream_t s) {
     // rows, n = 262,144 53.7 / 54.9 / 60.9 us (BCGS 44.5 / 42.0 / 44.7); n = 1M
     // 191 / 201 / 237 us.
     a.cs = a.n < 150000 ? 8 : (a.n < 400000 ? 4 : 2);
+    if (p->gs_ctas)
+        while (a.cs > 2 && a.cs > p->gs_ctas) a.cs /= 2;
     if (lim.nc[a.cs] < 1) return xb::set_error(XB_ECUDA, "orthogonalisation: no cluster of %d fits", a.cs);
     // a CTA has at least an element per thread (n = 9,600, MGS against 20 rows:
     // 33.0 us with 256 elements a CTA, 42.9 with 1024)
     const int64_t per = gs_threads<VB>();
     const int64_t want = (a.n + per * a.cs - 1) / (per * a.cs);
-    const int nc = (int)std::max<int64_t>(1, std::min<int64_t>(lim.nc[a.cs], want));
+    const int most = p->gs_ctas ? std::min(lim.nc[a.cs], p->gs_ctas / a.cs) : lim.nc[a.cs];
+    const int nc = (int)std::max<int64_t>(1, std::min<int64_t>(most, want));
     const int64_t G = (int64_t)nc * a.cs;
     a.chunk = ((a.n + G - 1) / G + 3) / 4 * 4;
     // w in shared memory when three stages fit beside it
@@ -1085,6 +1088,10 @@ extern "C" int xb_orth_config(xb_plan *p, int32_t what, int64_t value) {
     }
     if (p && what == XB_ORTH_POLLS && value >= 0 && value <= 0x7fffffffLL) {
         p->gs_polls = (unsigned)value;
+        return XB_OK;
+    }
+    if (p && what == XB_ORTH_CTAS && (value == 0 || (value >= 2 && value <= 0x7fffffffLL))) {
+        p->gs_ctas = (int)value;
         return XB_OK;
     }
     return xb::set_error(XB_EINVAL, "orth_config: plan %p control %d value %lld", (void *)p, what, (long long)value);

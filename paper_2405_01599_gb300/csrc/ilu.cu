@@ -255,20 +255,23 @@ __device__ __forceinline__ void flow_fail(const FlowArgs &a) {
     *reinterpret_cast<volatile int *>(a.stop) = 1;
     *a.err = 1;
 }
-// A warp's patience with one wait: false once it has run out.  Between looks at
-// the clock and the grid's flag a poll costs one add.
+// A warp's patience with one wait: false once it has run out, for all lanes (a
+// vote at the look: what follows a wait has shuffles and votes in it).  Between
+// looks at the clock and the grid's flag a poll costs one add.
 struct FlowWait {
     unsigned it = 0;
     unsigned long long t0 = 0;
     __device__ __forceinline__ bool more(const FlowArgs &a) {
         if (++it < a.look) return true;
+        bool out = true;
         if (a.polls == 0) {
             unsigned long long now;
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
             if (t0 == 0) t0 = now;
             it = 0;
-            if (now - t0 <= a.limit && *reinterpret_cast<volatile int *>(a.stop) == 0) return true;
+            out = now - t0 > a.limit || *reinterpret_cast<volatile int *>(a.stop) != 0;
         }
+        if (!__any_sync(0xffffffffu, out)) return true;
         flow_fail(a);
         return false;
     }

@@ -296,7 +296,7 @@ int batch_single(xb_plan *p, const double *b, double *x, const xb_options &o, in
 int resident_gmres(xb_plan *p, const double *b, double *x, const xb_options &o, xb_info &inf,
                    double *alg_bytes, cudaStream_t s, bool *ran);
 double ilu_apply_bytes(const xb_plan *p);
-int ilu_check(xb_plan *p);  // XB_ETIMEOUT if a substitution's barrier wait ran out
+int ilu_check(xb_plan *p, cudaStream_t s);  // XB_ETIMEOUT if a wait of a finished substitution ran out
 void ilu_free(xb_plan *p);
 bool variant_fits(const xb_plan *p, int variant);
 // Consecutive row blocks of a 64-bit row pointer, each holding at most

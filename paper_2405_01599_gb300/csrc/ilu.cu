@@ -978,11 +978,14 @@ int ilu_mode(const xb_plan *p) {
     return env >= 0 ? env : 1;
 }
 
-int ilu_check(xb_plan *p) {
+int ilu_check(xb_plan *p, cudaStream_t s) {
     volatile int *err = reinterpret_cast<volatile int *>(p->h_pin + 61);
     if (!*err) return XB_OK;
     *err = 0;
-    if (p->ilu.d_stop) XB_CUDA(cudaMemset(p->ilu.d_stop, 0, sizeof(int)));
+    if (p->ilu.d_stop) {
+        XB_CUDA(cudaMemsetAsync(p->ilu.d_stop, 0, sizeof(int), s));
+        XB_CUDA(cudaStreamSynchronize(s));  // the next application may be on another stream
+    }
     return set_error(XB_ETIMEOUT, "ILU(0): a wait for another row's value ran out");
 }
 
@@ -1057,7 +1060,7 @@ int xb_ilu0_apply(xb_plan *p, const double *r, double *z, void *stream) {
     cudaStream_t s = (cudaStream_t)stream;
     XB_TRY(xb::ilu_apply(p, r, z, s));
     XB_CUDA(cudaStreamSynchronize(s));
-    return xb::ilu_check(p);
+    return xb::ilu_check(p, s);
 }
 
 int xb_ilu0_config(xb_plan *p, int32_t mode, int32_t barrier_polls) {

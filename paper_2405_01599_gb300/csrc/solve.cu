@@ -163,7 +163,7 @@ int gmres_fp64(xb_plan *p, const double *b, double *x, const xb_options &o, xb_i
         XB_TRY(xb::gm_cycle_init(p, st, n, V, tau, s));
         ac.bytes += 8.0 * n;
         XB_TRY(peek(p, st.misc, xb::GM_NMISC, s));
-        if (prec) XB_TRY(xb::ilu_check(p));  // a preconditioner wait ran out: stop here
+        if (prec) XB_TRY(xb::ilu_check(p, s));  // a preconditioner wait ran out: stop here
         res_true = p->h_pin[xb::GM_RES];
         if (res_true <= o.tol) {
             status = XB_OK;
@@ -468,7 +468,7 @@ int bicgstab_run(xb_plan *p, const double *b, double *x, const xb_options &o, xb
         XB_TRY(xb::vnrm2(p, n, r, sc + xb::BI_N + 1, s));
         ac.bytes += 8.0 * n;
         XB_TRY(peek(p, sc + xb::BI_N + 1, 1, s));
-        if (prec) XB_TRY(xb::ilu_check(p));  // a preconditioner wait ran out: stop here
+        if (prec) XB_TRY(xb::ilu_check(p, s));  // a preconditioner wait ran out: stop here
         res_true = p->h_pin[0] / bnorm;
         if (res_true <= o.tol) {
             status = XB_OK;
@@ -518,7 +518,7 @@ int bicgstab_run(xb_plan *p, const double *b, double *x, const xb_options &o, xb
             ac.spmv += 2;
             if (iters % check == 0 || iters >= o.maxiter) {
                 XB_TRY(peek(p, sc, xb::BI_N, s));
-                if (prec) XB_TRY(xb::ilu_check(p));
+                if (prec) XB_TRY(xb::ilu_check(p, s));
                 flag = (int)p->h_pin[xb::BI_FLAG];
                 res_rec = std::sqrt(p->h_pin[xb::BI_RNORM2]) / bnorm;
                 if (flag != 0) break;
@@ -683,7 +683,7 @@ int run_solver(xb_plan *p, const double *b, double *x, const xb_options *opt, xb
             cudaError_t e = cudaStreamSynchronize(s);
             if (e != cudaSuccess && st == XB_OK) st = xb::cuda_error(e, "solve");
             if (o.precond == XB_PRECOND_ILU0 && st != XB_ECUDA) {
-                const int ci = xb::ilu_check(p);
+                const int ci = xb::ilu_check(p, s);
                 if (ci != XB_OK) st = ci;
             }
         }

@@ -2,7 +2,7 @@
 has (a lane a row, a few lanes a row, the warp for a long row, values from
 shared memory and from other CTAs): with one poll a wait, a warp gives up as a
 whole, the application reports XB_ETIMEOUT (a bounded wait, no fault), and the
-next one returns what another plan does, bit for bit."""
+next one, on another stream too, returns what another plan does, bit for bit."""
 import numpy as np
 import pytest
 
@@ -37,10 +37,14 @@ def test_gives_up_and_recovers(make):
         p.ilu0_config(1)
         p.ilu0_setup()
     want = other.ilu0_apply(r, torch.empty_like(r))
-    for _ in range(5):
+    torch.cuda.synchronize()
+    streams = [torch.cuda.current_stream(), torch.cuda.Stream()]
+    for i in range(6):
         plan.ilu0_config(1, barrier_polls=1)
         with pytest.raises(xb.XbError) as e:
             plan.ilu0_apply(r, torch.empty_like(r))
         assert e.value.code == xb.XB_ETIMEOUT
         plan.ilu0_config(1, barrier_polls=0)
-        assert torch.equal(plan.ilu0_apply(r, torch.empty_like(r)), want)
+        got = plan.ilu0_apply(r, torch.empty_like(r), stream=streams[i % 2])
+        torch.cuda.synchronize()
+        assert torch.equal(got, want)

@@ -1259,6 +1259,8 @@ int launch_sym(xb_plan *p, int variant, const int *rp, const int *ci, const V *v
     const xb::TilePart *tp = xb::get_tiles(p, block, ipt, s, &err);
     if (!tp) return err;
     if (tp->ntiles == 0) return XB_OK;
+    if (ipt != 1 && ipt != 2 && ipt != 4 && ipt != 8 && ipt != 16)  // for rows of any length
+        return xb::set_error(XB_EINVAL, "sym tile: unsupported ipt %d", ipt);
     if (p->max_row <= kSymShort) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)tp->ntiles);

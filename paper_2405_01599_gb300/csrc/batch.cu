@@ -837,7 +837,8 @@ int batch_single(xb_plan *p, const double *b, double *x, const xb_options &o, in
         const int *rp = p->h_rowptr.data();
         if ((int)p->h_rowptr.size() != p->n + 1) {
             rp_h.resize((size_t)p->n + 1);
-            XB_CUDA(cudaMemcpy(rp_h.data(), p->rowptr, rp_h.size() * sizeof(int), cudaMemcpyDeviceToHost));
+            XB_CUDA(cudaMemcpyAsync(rp_h.data(), p->rowptr, rp_h.size() * sizeof(int), cudaMemcpyDeviceToHost, s));
+            XB_CUDA(cudaStreamSynchronize(s));
             rp = rp_h.data();
         }
         cut_tiles(d, rp, trow);
@@ -912,7 +913,9 @@ int xb_batch_create(int32_t count, const xb_batch_sys *sys, const xb_options *op
                     xb_batch **out) {
     if (count < 0 || (count > 0 && !sys) || !out) return xb::set_error(XB_EINVAL, "batch_create: bad argument");
     *out = nullptr;
-    (void)stream;
+    // the systems' arrays may still be on their way on the caller's stream, which
+    // the legacy default stream does not wait for
+    cudaStream_t s = (cudaStream_t)stream;
     xb_options o;
     if (opt) o = *opt;
     else xb_options_default(&o);
@@ -960,8 +963,8 @@ int xb_batch_create(int32_t count, const xb_batch_sys *sys, const xb_options *op
         toff[i] = trow.size();
         if (h[i].mode != 1 || h[i].n < 1 || h[i].nnz < 1) continue;
         rp_h.resize((size_t)h[i].n + 1);
-        e = cudaMemcpy(rp_h.data(), h[i].rowptr, rp_h.size() * sizeof(int),
-                                   cudaMemcpyDeviceToHost);
+        e = cudaMemcpyAsync(rp_h.data(), h[i].rowptr, rp_h.size() * sizeof(int), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return xb::cuda_error(e, "batch_create: read rowptr");
         cut_tiles(h[i], rp_h.data(), trow);
     }
@@ -985,7 +988,7 @@ int xb_batch_create(int32_t count, const xb_batch_sys *sys, const xb_options *op
         }
         double2 *ts = static_cast<double2 *>(bt->d_tiles);
         int *ti = reinterpret_cast<int *>(ts + nt);
-        e = cudaMemcpy(ti + nt, trow.data(), nt * sizeof(int), cudaMemcpyHostToDevice);
+        e = cudaMemcpyAsync(ti + nt, trow.data(), nt * sizeof(int), cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) return fail(xb::cuda_error(e, "batch_create: tiles"));
         for (int i = 0; i < count; i++) {
             h[i].tsum = ts + toff[i];
@@ -1007,9 +1010,10 @@ int xb_batch_create(int32_t count, const xb_batch_sys *sys, const xb_options *op
     if (e == cudaSuccess) e = cudaMalloc(&bt->d_order, std::max(count, 1) * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&bt->d_queue, 2 * sizeof(int));
     if (e == cudaSuccess && count > 0)
-        e = cudaMemcpy(bt->d_sys, h.data(), count * sizeof(xb_batch_dev), cudaMemcpyHostToDevice);
+        e = cudaMemcpyAsync(bt->d_sys, h.data(), count * sizeof(xb_batch_dev), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && count > 0)
-        e = cudaMemcpy(bt->d_order, order.data(), count * sizeof(int), cudaMemcpyHostToDevice);
+        e = cudaMemcpyAsync(bt->d_order, order.data(), count * sizeof(int), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // a run may be on another stream
     if (e != cudaSuccess) return fail(xb::cuda_error(e, "batch_create"));
     bt->grid = kCl * clusters;  // persistent: as many whole clusters as can be co-resident
     // clusters that take the single-CTA systems from the start: their share

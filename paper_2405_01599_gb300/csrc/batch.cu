@@ -20,8 +20,8 @@
 // The solver is restarted GMRES(m) with modified Gram-Schmidt or blocked
 // classical Gram-Schmidt, both over blocks of 4 basis vectors (one pass, which
 // applies the previous block's projection, and one four-value reduction per
-// block; for MGS the block's dots are corrected by its own inner products),
-// Givens least squares, the true-residual check at every restart (fault
+// block; for MGS the block's dots are corrected by its own inner products, or,
+// with many rows a CTA, taken a vector at a time), Givens least squares, the true-residual check at every restart (fault
 // convergence narrows the implicit threshold), and, when enabled, the
 // MM-ratio restart rule of Eq. (1) / Fig. 2 / Sec. 4.3 (m grows by 5, up to
 // m_max, when 5 consecutive restart residuals change by less than theta).
@@ -46,6 +46,7 @@ constexpr int kTile = 256;      // mode 1: entries a warp sums at a time, 8 a la
 
 struct xb_batch_dev {
     int n, nnz, m, m_max, mode, zero_x, coop;
+    int single;  // MGS a vector at a time (single_dots)
     int64_t ld;
     const int *rowptr, *col;
     const double *val, *b;
@@ -380,6 +381,37 @@ __device__ __forceinline__ void bgs_rows(double *__restrict__ w, const double *_
     if (e < r1) bgs_row<1, NORM>(w, V, ld, u0, nu, c, d0, nd, e, B, a);
 }
 
+// MGS a vector at a time over rows [r0, r1): OP 0 returns (w, vn); OP 1 applies
+// w -= c vp and returns (w, vn); OP 2 applies w -= c vp and returns (w, w).  Four
+// rows per thread in flight.
+template <int OP>
+__device__ __forceinline__ double mgs_rows(double *__restrict__ w, const double *__restrict__ vp,
+                                           const double *__restrict__ vn, double c, int r0, int r1) {
+    const int B = blockDim.x;
+    double a0 = 0.0, a1 = 0.0;
+    auto row = [&](int e, double x, double p, double q, double &a) {
+        if (OP != 0) {
+            x = fma(-c, p, x);
+            w[e] = x;
+        }
+        a = fma(x, OP == 2 ? x : q, a);
+    };
+    int e = r0 + threadIdx.x;
+    for (; e + 3 * B < r1; e += 4 * B) {
+        double x[4], p[4], q[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            x[u] = w[e + u * B];
+            p[u] = OP != 0 ? vp[e + u * B] : 0.0;
+            q[u] = OP != 2 ? vn[e + u * B] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) row(e + u * B, x[u], p[u], q[u], u & 1 ? a1 : a0);
+    }
+    for (; e < r1; e += B) row(e, w[e], OP != 0 ? vp[e] : 0.0, OP != 2 ? vn[e] : 0.0, a0);
+    return a0 + a1;
+}
+
 __device__ void solve_one(const xb_batch_dev &D, Part &P, Smem &S, TileBuf *buf, double tol, int maxiter,
                           unsigned long long deadline, int rank, double theta, int bcgs,
                           xb_batch_info *out) {
@@ -464,9 +496,28 @@ __device__ void solve_one(const xb_batch_dev &D, Part &P, Smem &S, TileBuf *buf,
                 // are taken with the same w; for MGS they are corrected by the
                 // block's own inner products: (w - sum_{k<i} c_k V_k, V_i) =
                 // (w, V_i) - sum_{k<i} c_k (V_k, V_i), the same method with a quarter
-                // of the exchanges
+                // of the exchanges.  Or (single_dots) MGS a vector at a time
                 double c[4] = {0.0, 0.0, 0.0, 0.0}, a4[4];
-                for (int d0 = 0; d0 <= j; d0 += 4) {
+                if (D.single) {
+                    double ci = 0.0;
+                    for (int i = 0; i <= j; i++) {
+                        const double *vi = V + (size_t)i * ld;
+                        double a1[1];
+                        if (i == 0) a1[0] = mgs_rows<0>(w, nullptr, vi, 0.0, r0, r1);
+                        else a1[0] = mgs_rows<1>(w, vi - ld, vi, ci, r0, r1);
+                        const int ph = P.phase;
+                        sums<1>(a1, S, P, take, [&](double &t) {
+                            const double sq = S.sc[i];
+                            t = (t * sq) * sq;
+                            if (lane == 0) S.hc[i] = t * S.hn[i];
+                        });
+                        ci = S.tot[ph][0];
+                        u0 = i;
+                        nu = 1;
+                    }
+                    c[0] = ci;
+                }
+                for (int d0 = D.single ? j + 1 : 0; d0 <= j; d0 += 4) {
                     const int nd = min(4, j + 1 - d0);
                     bgs_rows<false>(w, V, ld, u0, nu, c, d0, nd, r0, r1, a4);
                     const int ph = P.phase;
@@ -491,8 +542,13 @@ __device__ void solve_one(const xb_batch_dev &D, Part &P, Smem &S, TileBuf *buf,
                 }
                 // the last projection, ||w||^2 and, for MGS, w's products with the
                 // basis vectors it will share a block with
-                const int ng = bcgs || j + 1 >= m ? 0 : (j + 1) & 3, g0 = j + 1 - ng;
-                bgs_rows<true>(w, V, ld, u0, nu, c, g0, ng, r0, r1, a4);
+                const int ng = bcgs || D.single || j + 1 >= m ? 0 : (j + 1) & 3, g0 = j + 1 - ng;
+                if (D.single) {
+                    a4[0] = mgs_rows<2>(w, V + (size_t)j * ld, nullptr, c[0], r0, r1);
+                    a4[1] = a4[2] = a4[3] = 0.0;
+                } else {
+                    bgs_rows<true>(w, V, ld, u0, nu, c, g0, ng, r0, r1, a4);
+                }
                 sums<4>(a4, S, P,
                         [&]() {
                             take();
@@ -747,6 +803,20 @@ double step_us(const xb_batch_dev &d, bool cluster) {
     return cluster ? 3.3 * sums + 1.15 * terms / kCl : 2.0 * sums + terms;
 }
 
+// Whether MGS takes a system's basis a vector at a time, an exchange each, instead
+// of in corrected blocks of 4.  A block saves exchanges (2 us, 3.3 across a
+// cluster) but takes up to 3 more dots a step for its own products and has fewer
+// rows of the vectors on their way, so it loses where a CTA has many rows for the
+// cycle's length.  Us a step, blocks / singly, one CTA: n = 1600, m = 5, 10, 20:
+// 24.2 / 20.9, 25.5 / 24.4, 31.5 / 34.1; n = 6400, m = 20, 30, 50: 91 / 84, 113 / 110,
+// 153 / 161; n = 28,900, m = 10, 30, 100: 341 / 275, 481 / 433, 1044 / 1072.  A
+// cluster: n = 40,000, m = 10, 20, 30: 61.5 / 54.1, 79.4 / 81.1, 98 / 108; n =
+// 202,500, m = 5, 20, 60: 305 / 243, 359 / 318, 638 / 642.
+int single_dots(const xb_batch_dev &d, int bcgs) {
+    const double rows = d.coop ? (d.n + kCl - 1) / kCl : d.n;
+    return !bcgs && rows >= (d.coop ? 2.4 : 1.5) * d.m * (d.m + 100.0);
+}
+
 // Decides which systems a whole cluster solves and returns the order of the
 // queues: the cluster's systems first, each part largest first, so that the long
 // solves start in the first wave.  A cluster solves a system sooner but at up to 8
@@ -826,6 +896,8 @@ int batch_single(xb_plan *p, const double *b, double *x, const xb_options &o, in
     d.val = p->val;
     d.b = b;
     d.x = x;
+    const int bcgs = o.ortho == XB_ORTHO_BCGS ? 1 : 0;
+    d.single = single_dots(d, bcgs);
     const size_t nv = (size_t)(d.m_max + 1) * d.ld;
     const size_t nh = (size_t)(d.coop ? kCl : 1) * (d.m_max + 1) * d.m_max + 32;
     const size_t meta = 4096;  // descriptor, result, order, queue
@@ -865,7 +937,6 @@ int batch_single(xb_plan *p, const double *b, double *x, const xb_options &o, in
     XB_CUDA(cudaMemsetAsync(d_queue, 0, 2 * sizeof(int), s));
     const unsigned long long budget = (unsigned long long)(std::min(o.maxtime_s, 3600.0) * 1e9);
     const double theta = o.dafrt ? o.dafrt_theta : 0.0;
-    const int bcgs = o.ortho == XB_ORTHO_BCGS ? 1 : 0;
     XB_CUDA(cudaFuncSetAttribute(k_batch_gmres, cudaFuncAttributeMaxDynamicSharedMemorySize, kDyn));
     k_batch_gmres<<<kCl, kBT, mode == 1 ? kDyn : 0, s>>>(d_sys, d_info, d_order, 1, 1, 0, d_queue, o.tol, o.maxiter,
                                       budget, theta, bcgs);
@@ -996,8 +1067,14 @@ int xb_batch_create(int32_t count, const xb_batch_sys *sys, const xb_options *op
             h[i].trow = ti + nt + toff[i];
         }
     }
+    // orthogonalisation: MGS or BCGS (block length 4); the accuracy policy's
+    // choice for AUTO (no fault switch inside the launch)
+    const int ortho = o.ortho == XB_ORTHO_AUTO ? (o.tol <= 1e-10 ? XB_ORTHO_MGS : XB_ORTHO_BCGS)
+                                               : o.ortho;
+    const int bcgs = ortho == XB_ORTHO_BCGS ? 1 : 0;
     size_t off = 0;
     for (int i = 0; i < count; i++) {
+        h[i].single = single_dots(h[i], bcgs);
         h[i].V = bt->d_ws + off;
         off += (size_t)(h[i].m_max + 1) * h[i].ld;
         h[i].H = bt->d_ws + off;
@@ -1025,11 +1102,6 @@ int xb_batch_create(int32_t count, const xb_batch_sys *sys, const xb_options *op
         nsmall_cl = std::min(clusters - 1, (int)std::lround(clusters * w_small / (w_big + w_small)));
     const unsigned long long budget = (unsigned long long)(std::min(o.maxtime_s, 3600.0) * 1e9);
     const double theta = o.dafrt ? o.dafrt_theta : 0.0;  // theta 0: the rule never fires
-    // orthogonalisation: MGS or BCGS (block length 4); the accuracy policy's
-    // choice for AUTO (no fault switch inside the launch)
-    const int ortho = o.ortho == XB_ORTHO_AUTO ? (o.tol <= 1e-10 ? XB_ORTHO_MGS : XB_ORTHO_BCGS)
-                                               : o.ortho;
-    const int bcgs = ortho == XB_ORTHO_BCGS ? 1 : 0;
     // capture on a private stream (the caller's may be the legacy default
     // stream, which cannot be captured): reset the queue, one persistent launch
     cudaStream_t cs = nullptr;

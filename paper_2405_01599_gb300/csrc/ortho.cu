@@ -181,38 +181,40 @@ constexpr int gram_count(int kb, int gram) {
     return gram == 1 ? kb - 1 : (gram == 2 ? kb * (kb - 1) / 2 : 0);
 }
 
-// FP32 partial sums are kept per element of the tile (shorter chains).
-template <typename VB>
-constexpr int chains() { return sizeof(VB) == 4 ? 4 : 1; }
+// Chains of a thread's FP32 partial sums: 13 terms each at n = 2.1M, 7 for MGS (where
+// their errors enter the corrections too), then FP64 takes over.
+template <typename VB, int KB, int GRAM>
+constexpr int chains() { return sizeof(VB) == 4 ? (KB <= 4 && GRAM ? 8 : 4) : 1; }
 
-// Launch shape: two compute warps on each quarter of the SM (one waits or
-// loads while the other's FMAs hold the FP64 pipe; more would only add to the
-// sums over threads).
-template <typename VB>
-constexpr int gs_threads() { return 256; }
-template <typename VB, int KB>
-constexpr int gs_elems() { return sizeof(VB) == 4 ? (KB <= 4 ? 8 : 4) : (KB == 2 ? 4 : 2); }  // per thread and tile
-template <typename VB, int KB>
-constexpr int gs_tile() { return gs_threads<VB>() * gs_elems<VB, KB>(); }
-template <typename VB, int KB>
-constexpr int gs_pitch() { return gs_tile<VB, KB>() * (int)sizeof(VB) + 16; }
+// Launch shape: NT = 256 compute threads, two warps on each quarter of the SM
+// (one waits or loads while the other's FMAs hold the FP64 pipe; more would only
+// add to the sums over threads), or 512 where the passes are long and w comes
+// from device memory, whose latency eight warps do not hide.
+template <typename VB, int KB, int NT>
+constexpr int gs_elems() {  // per thread and tile
+    return sizeof(VB) == 4 ? (KB <= 4 ? 8 : 4) : (KB == 2 && NT == 256 ? 4 : 2);
+}
+template <typename VB, int KB, int NT>
+constexpr int gs_tile() { return NT * gs_elems<VB, KB, NT>(); }
+template <typename VB, int KB, int NT>
+constexpr int gs_pitch() { return gs_tile<VB, KB, NT>() * (int)sizeof(VB) + 16; }
 // Shared memory besides w and the stages: exchange slots.
-template <typename VB>
-constexpr int gs_xch_bytes() { return 2 * kGsVals * (gs_threads<VB>() / 32) * 16 + 2 * kGsVals * 16; }
+template <int NT>
+constexpr int gs_xch_bytes() { return 2 * kGsVals * (NT / 32) * 16 + 2 * kGsVals * 16; }
 
-template <typename VB, int KB>
+template <typename VB, int KB, int NT>
 struct GsShared {
     unsigned long long full[kGsMaxStages], empty[kGsMaxStages];
     double hcol[kGsMaxK + 1];
     VB cf[kGsMaxK];                               // CGS, DGKS: one for the CTA
-    VB cfw[gs_threads<VB>() / 32][KB];            // block methods: one for each warp
+    VB cfw[NT / 32][KB];            // block methods: one for each warp
     int abort;
 };
 
 // The CTA's state: everything the roles share.
-template <typename VB, int KB>
+template <typename VB, int KB, int NT>
 struct Ctx {
-    GsShared<VB, KB> *S;
+    GsShared<VB, KB, NT> *S;
     const GsArgs<VB> *a;
     const VB *Vc;          // basis, from the CTA's first element
     unsigned ring;         // stages
@@ -231,8 +233,8 @@ struct Ctx {
     }
 };
 
-template <typename VB, int KB>
-__device__ __forceinline__ void give_up(Ctx<VB, KB> &c) {
+template <typename VB, int KB, int NT>
+__device__ __forceinline__ void give_up(Ctx<VB, KB, NT> &c) {
     *reinterpret_cast<volatile int *>(&c.S->abort) = 1;
     *reinterpret_cast<volatile unsigned *>(c.a->stop) = 1u;
     *reinterpret_cast<volatile int *>(c.a->err) = 1;
@@ -241,8 +243,8 @@ __device__ __forceinline__ void give_up(Ctx<VB, KB> &c) {
 
 // The whole warp waits and goes on, or gives up, together: what follows a wait
 // has shuffles and votes in it.
-template <typename VB, int KB>
-__device__ __forceinline__ bool wait_bar(Ctx<VB, KB> &c, unsigned bar, unsigned parity) {
+template <typename VB, int KB, int NT>
+__device__ __forceinline__ bool wait_bar(Ctx<VB, KB, NT> &c, unsigned bar, unsigned parity) {
     Patience w;
     bool ok = true;
     while (ok && !mbar_done(bar, parity)) {
@@ -259,15 +261,15 @@ __device__ __forceinline__ bool wait_bar(Ctx<VB, KB> &c, unsigned bar, unsigned 
 // ---- producer ---------------------------------------------------------------------
 // One unit: rows row0 .. row0 + nr - 1 of tile t.  The copies take whole 16-byte
 // blocks: an end that lies inside one belongs to the same allocation.
-template <typename VB, int KB>
-__device__ __forceinline__ void produce(Ctx<VB, KB> &c, int t, int row0, int nr, uint64_t policy) {
+template <typename VB, int KB, int NT>
+__device__ __forceinline__ void produce(Ctx<VB, KB, NT> &c, int t, int row0, int nr, uint64_t policy) {
     if (!c.fine) return;
     const unsigned full = sptr(&c.S->full[c.st]);
     if (c.ph > 0 && !wait_bar(c, sptr(&c.S->empty[c.st]), (c.ph - 1) & 1)) {
         c.fine = false;
         return;
     }
-    constexpr int T = gs_tile<VB, KB>();
+    constexpr int T = gs_tile<VB, KB, NT>();
     const int cnt = min(T, c.len - t * T);
     uintptr_t lo = 0, hi = 0;
     if (c.lane < nr) {
@@ -279,15 +281,15 @@ __device__ __forceinline__ void produce(Ctx<VB, KB> &c, int t, int row0, int nr,
     if (c.lane == 0) mbar_expect(full, bytes);
     __syncwarp();
     if (c.lane < nr)
-        bulk_copy(c.ring + (c.st * KB + c.lane) * gs_pitch<VB, KB>(), (const void *)lo, (unsigned)(hi - lo), full, policy);
+        bulk_copy(c.ring + (c.st * KB + c.lane) * gs_pitch<VB, KB, NT>(), (const void *)lo, (unsigned)(hi - lo), full, policy);
     c.next();
 }
 
 // Waits for the copies that are in flight.  The consumers of a sweep that is
 // given up may leave them behind, at any time until the end, and a CTA must not
 // end before its copies; a sweep that is not has waited for them all.
-template <typename VB, int KB>
-__device__ void drain(Ctx<VB, KB> &c) {
+template <typename VB, int KB, int NT>
+__device__ void drain(Ctx<VB, KB, NT> &c) {
     for (int i = 0; i < c.a->stages; i++) {
         const int ph = i < c.st ? c.ph : c.ph - 1;  // the stage's last use
         if (ph < 0) continue;
@@ -297,54 +299,54 @@ __device__ void drain(Ctx<VB, KB> &c) {
 }
 
 // ---- consumers --------------------------------------------------------------------
-template <typename VB, int KB>
-__device__ __forceinline__ bool unit_wait(Ctx<VB, KB> &c) {
+template <typename VB, int KB, int NT>
+__device__ __forceinline__ bool unit_wait(Ctx<VB, KB, NT> &c) {
     if (!c.fine) return false;
     if (!wait_bar(c, sptr(&c.S->full[c.st]), c.ph & 1)) c.fine = false;
     return c.fine;
 }
-template <typename VB, int KB>
-__device__ __forceinline__ void unit_free(Ctx<VB, KB> &c) {
+template <typename VB, int KB, int NT>
+__device__ __forceinline__ void unit_free(Ctx<VB, KB, NT> &c) {
     __syncwarp();
     if (c.lane == 0) mbar_arrive(sptr(&c.S->empty[c.st]));
     c.next();
 }
 // Address of row r of the current unit (rows whose start is not 16-byte aligned
 // sit at their offset in the block; tiles are whole blocks).
-template <typename VB, int KB>
-__device__ __forceinline__ unsigned unit_row(const Ctx<VB, KB> &c, int first, int r) {
-    return c.ring + (c.st * KB + r) * gs_pitch<VB, KB>() + ((c.row0 + (unsigned)(first + r) * c.pitch) & 15u);
+template <typename VB, int KB, int NT>
+__device__ __forceinline__ unsigned unit_row(const Ctx<VB, KB, NT> &c, int first, int r) {
+    return c.ring + (c.st * KB + r) * gs_pitch<VB, KB, NT>() + ((c.row0 + (unsigned)(first + r) * c.pitch) & 15u);
 }
 // A thread's E values of a row of the unit: FP64 NT apart (a row may start at
 // any 8-byte offset), FP32 four together in one 16-byte load (the solvers' FP32
 // rows are aligned).
-template <typename VB, int E>
+template <typename VB, int E, int NT>
 constexpr int place(int tid, int i) {
-    return sizeof(VB) == 4 ? 4 * tid + i % 4 + i / 4 * 4 * gs_threads<VB>() : tid + i * gs_threads<VB>();
+    return sizeof(VB) == 4 ? 4 * tid + i % 4 + i / 4 * 4 * NT : tid + i * NT;
 }
-template <int E>
+template <int NT, int E>
 __device__ __forceinline__ void lds_row(unsigned a, double (&v)[E]) {
 #pragma unroll
     for (int i = 0; i < E; i++)
-        asm volatile("ld.shared::cta.f64 %0, [%1];" : "=d"(v[i]) : "r"(a + i * gs_threads<double>() * 8));
+        asm volatile("ld.shared::cta.f64 %0, [%1];" : "=d"(v[i]) : "r"(a + i * NT * 8));
 }
-template <int E>
+template <int NT, int E>
 __device__ __forceinline__ void lds_row(unsigned a, float (&v)[E]) {
     static_assert(E % 4 == 0, "16-byte loads");
 #pragma unroll
     for (int i = 0; i < E; i += 4)
         asm volatile("ld.shared::cta.v4.f32 {%0, %1, %2, %3}, [%4];"
                      : "=f"(v[i]), "=f"(v[i + 1]), "=f"(v[i + 2]), "=f"(v[i + 3])
-                     : "r"(a + i * gs_threads<float>() * 4));
+                     : "r"(a + i * NT * 4));
 }
 
 // One tile of a pass; FULL: every thread has all its elements.
-template <typename VB, int KB, int GRAM, bool GR, bool FIN, bool FULL, int NA, int E>
-__device__ __forceinline__ bool gs_tile_pass(Ctx<VB, KB> &c, int e0, VB (&x)[E], VB *dst, int u0, int nu,
-                                             const VB *cf, int d0, int nd, VB (&acc)[NA][chains<VB>()]) {
-    constexpr int AW = chains<VB>();
+template <typename VB, int KB, int NT, int GRAM, bool GR, bool FIN, bool FULL, int NA, int E>
+__device__ __forceinline__ bool gs_tile_pass(Ctx<VB, KB, NT> &c, int e0, VB (&x)[E], VB *dst, int u0, int nu,
+                                             const VB *cf, int d0, int nd, VB (&acc)[NA][chains<VB, KB, GRAM>()]) {
+    constexpr int AW = chains<VB, KB, GRAM>();
     const int tid = threadIdx.x;
-    const unsigned off = place<VB, E>(tid, 0) * (int)sizeof(VB);
+    const unsigned off = place<VB, E, NT>(tid, 0) * (int)sizeof(VB);
     for (int i0 = 0; i0 < nu; i0 += KB) {
         if (!unit_wait(c)) return false;
         const int nr = min(KB, nu - i0);
@@ -352,7 +354,7 @@ __device__ __forceinline__ bool gs_tile_pass(Ctx<VB, KB> &c, int e0, VB (&x)[E],
         for (int r = 0; r < KB; r++) {
             if (r < nr) {
                 VB v[E];
-                lds_row(unit_row(c, u0 + i0, r) + off, v);
+                lds_row<NT>(unit_row(c, u0 + i0, r) + off, v);
                 const VB cr = cf[i0 + r];
 #pragma unroll
                 for (int i = 0; i < E; i++) x[i] = fma(-cr, v[i], x[i]);
@@ -363,25 +365,25 @@ __device__ __forceinline__ bool gs_tile_pass(Ctx<VB, KB> &c, int e0, VB (&x)[E],
     if (dst) {
 #pragma unroll
         for (int i = 0; i < E; i++)
-            if (FULL || e0 + place<VB, E>(tid, i) < c.len) dst[e0 + place<VB, E>(tid, i)] = x[i];
+            if (FULL || e0 + place<VB, E, NT>(tid, i) < c.len) dst[e0 + place<VB, E, NT>(tid, i)] = x[i];
     }
     if constexpr (FIN) {
 #pragma unroll
         for (int i = 0; i < E; i++)
-            if (FULL || e0 + place<VB, E>(tid, i) < c.len) acc[0][i % AW] = fma(x[i], x[i], acc[0][i % AW]);
+            if (FULL || e0 + place<VB, E, NT>(tid, i) < c.len) acc[0][i % AW] = fma(x[i], x[i], acc[0][i % AW]);
     } else {
         if (!unit_wait(c)) return false;
         constexpr bool ALL = GR && GRAM == 2;  // all pairs: the rows are held together
         VB v[ALL ? KB : 1][E], vl[E];
-        if constexpr (GR && GRAM == 1) lds_row(unit_row(c, d0, nd - 1) + off, vl);
+        if constexpr (GR && GRAM == 1) lds_row<NT>(unit_row(c, d0, nd - 1) + off, vl);
 #pragma unroll
         for (int r = 0; r < KB; r++) {
             if (r >= nd) break;
             VB(&vr)[E] = v[ALL ? r : 0];
-            lds_row(unit_row(c, d0, r) + off, vr);
+            lds_row<NT>(unit_row(c, d0, r) + off, vr);
 #pragma unroll
             for (int i = 0; i < E; i++) {
-                if (!FULL && e0 + place<VB, E>(tid, i) >= c.len) continue;
+                if (!FULL && e0 + place<VB, E, NT>(tid, i) >= c.len) continue;
                 acc[r][i % AW] = fma(x[i], vr[i], acc[r][i % AW]);
                 if constexpr (GR && GRAM == 1) {
                     if (r < KB - 1 && r < nd - 1)
@@ -405,11 +407,11 @@ __device__ __forceinline__ bool gs_tile_pass(Ctx<VB, KB> &c, int e0, VB (&x)[E],
 // cf), store, then (FIN) the squared norm or the dots with the nd <= KB rows
 // from d0 and, with GR, the rows' own inner products: GRAM 2 all pairs, GRAM 1
 // the newest row (d0 + nd - 1) with the others.
-template <typename VB, int KB, int GRAM, bool GR, bool FIN, int NA>
-__device__ __forceinline__ void gs_pass(Ctx<VB, KB> &c, const VB *src, bool from_global, VB *dst, int u0,
+template <typename VB, int KB, int NT, int GRAM, bool GR, bool FIN, int NA>
+__device__ __forceinline__ void gs_pass(Ctx<VB, KB, NT> &c, const VB *src, bool from_global, VB *dst, int u0,
                                         int nu, const VB *cf, int d0, int nd, double (&out)[NA]) {
-    constexpr int E = gs_elems<VB, KB>(), T = gs_tile<VB, KB>();
-    constexpr int AW = chains<VB>();
+    constexpr int E = gs_elems<VB, KB, NT>(), T = gs_tile<VB, KB, NT>();
+    constexpr int AW = chains<VB, KB, GRAM>();
     const int tid = threadIdx.x;
     constexpr int D = sizeof(VB) == 8 ? 3 : 2;  // tiles of w on their way (global w)
     VB acc[NA][AW], xn[D][E];
@@ -425,7 +427,7 @@ __device__ __forceinline__ void gs_pass(Ctx<VB, KB> &c, const VB *src, bool from
         for (int d = 0; d < D; d++)
 #pragma unroll
             for (int i = 0; i < E; i++) {
-                const int e = e0 + d * step + place<VB, E>(tid, i);
+                const int e = e0 + d * step + place<VB, E, NT>(tid, i);
                 xn[d][i] = e >= 0 && e < c.len ? src[e] : VB(0);
             }
     }
@@ -435,7 +437,7 @@ __device__ __forceinline__ void gs_pass(Ctx<VB, KB> &c, const VB *src, bool from
 #pragma unroll
             for (int i = 0; i < E; i++) {
                 x[i] = xn[0][i];
-                const int e = e0 + D * step + place<VB, E>(tid, i);
+                const int e = e0 + D * step + place<VB, E, NT>(tid, i);
 #pragma unroll
                 for (int d = 0; d + 1 < D; d++) xn[d][i] = xn[d + 1][i];
                 xn[D - 1][i] = e >= 0 && e < c.len ? src[e] : VB(0);
@@ -443,19 +445,22 @@ __device__ __forceinline__ void gs_pass(Ctx<VB, KB> &c, const VB *src, bool from
         } else {
 #pragma unroll
             for (int i = 0; i < E; i++) {
-                const int e = e0 + place<VB, E>(tid, i);
+                const int e = e0 + place<VB, E, NT>(tid, i);
                 x[i] = e < c.len ? src[e] : VB(0);
             }
         }
         if (!(e0 + T <= c.len
-                  ? gs_tile_pass<VB, KB, GRAM, GR, FIN, true>(c, e0, x, dst, u0, nu, cf, d0, nd, acc)
-                  : gs_tile_pass<VB, KB, GRAM, GR, FIN, false>(c, e0, x, dst, u0, nu, cf, d0, nd, acc)))
+                  ? gs_tile_pass<VB, KB, NT, GRAM, GR, FIN, true>(c, e0, x, dst, u0, nu, cf, d0, nd, acc)
+                  : gs_tile_pass<VB, KB, NT, GRAM, GR, FIN, false>(c, e0, x, dst, u0, nu, cf, d0, nd, acc)))
             break;
     }
 #pragma unroll
     for (int i = 0; i < NA; i++) {
         out[i] = (double)acc[i][0];
-        if constexpr (AW == 4)
+        if constexpr (AW == 8)
+#pragma unroll
+            for (int q = 0; q < 4; q++) acc[i][q] += acc[i][q + 4];
+        if constexpr (AW >= 4)
             out[i] = ((double)acc[i][0] + (double)acc[i][1]) + ((double)acc[i][2] + (double)acc[i][3]);
     }
 }
@@ -468,9 +473,9 @@ __device__ __forceinline__ void gs_pass(Ctx<VB, KB> &c, const VB *src, bool from
 // CTA of their cluster.  All sums in a fixed order.
 
 // The warp's sums of NV values, as values q0.. of exchange seq.
-template <int NV, typename VB, int KB>
-__device__ __forceinline__ void publish(Ctx<VB, KB> &c, double (&v)[NV], int q0, unsigned seq) {
-    constexpr int NW = gs_threads<VB>() / 32;
+template <int NV, typename VB, int KB, int NT>
+__device__ __forceinline__ void publish(Ctx<VB, KB, NT> &c, double (&v)[NV], int q0, unsigned seq) {
+    constexpr int NW = NT / 32;
     warp_totals<NV>(v, c.lane);
     if (c.lane % (32 / NV) == 0) {
         const int q = q0 + c.lane / (32 / NV), cs = c.a->cs;
@@ -480,9 +485,9 @@ __device__ __forceinline__ void publish(Ctx<VB, KB> &c, double (&v)[NV], int q0,
 }
 
 // Sum of value q over the warps of the cluster (owner's warp).
-template <typename VB, int KB>
-__device__ __forceinline__ double cluster_sum(Ctx<VB, KB> &c, int q, unsigned seq) {
-    constexpr int NW = gs_threads<VB>() / 32;
+template <typename VB, int KB, int NT>
+__device__ __forceinline__ double cluster_sum(Ctx<VB, KB, NT> &c, int q, unsigned seq) {
+    constexpr int NW = NT / 32;
     const int cs = c.a->cs, cnt = cs * NW;
     const unsigned at = c.part + (((seq & 1) * kGsVals + (q / cs) * cs) * NW) * 16;
     constexpr int SL = 8 * NW / 32;
@@ -519,8 +524,8 @@ __device__ __forceinline__ double cluster_sum(Ctx<VB, KB> &c, int q, unsigned se
 }
 
 // Sum of value q over the clusters.
-template <typename VB, int KB>
-__device__ __forceinline__ double grid_sum(Ctx<VB, KB> &c, int q, unsigned seq) {
+template <typename VB, int KB, int NT>
+__device__ __forceinline__ double grid_sum(Ctx<VB, KB, NT> &c, int q, unsigned seq) {
     constexpr int SL = kGsMaxClusters / 32;
     const int nc = gridDim.x / c.a->cs;
     const ulonglong2 *at = c.a->slots + ((size_t)(seq & 1) * kGsVals + q) * kGsMaxClusters + c.lane;
@@ -557,9 +562,9 @@ __device__ __forceinline__ double grid_sum(Ctx<VB, KB> &c, int q, unsigned seq) 
 }
 
 // The owner's share of exchange seq over nv values.
-template <typename VB, int KB>
-__device__ __forceinline__ void relay(Ctx<VB, KB> &c, int nv, unsigned seq) {
-    constexpr int NW = gs_threads<VB>() / 32;
+template <typename VB, int KB, int NT>
+__device__ __forceinline__ void relay(Ctx<VB, KB, NT> &c, int nv, unsigned seq) {
+    constexpr int NW = NT / 32;
     const int cs = c.a->cs, ci = blockIdx.x / cs;
     for (int q = c.rank + cs * c.wv; q < nv; q += cs * NW) {
         const double s = cluster_sum(c, q, seq);
@@ -573,8 +578,8 @@ __device__ __forceinline__ void relay(Ctx<VB, KB> &c, int nv, unsigned seq) {
 }
 
 // Totals q0 .. q0 + 31 of exchange seq, one per lane (0 from nv on).
-template <typename VB, int KB>
-__device__ __forceinline__ double totals(Ctx<VB, KB> &c, int q0, int nv, unsigned seq) {
+template <typename VB, int KB, int NT>
+__device__ __forceinline__ double totals(Ctx<VB, KB, NT> &c, int q0, int nv, unsigned seq) {
     bool got = q0 + c.lane >= nv;
     double r = 0.0;
     Patience w;
@@ -598,8 +603,8 @@ __device__ __forceinline__ double totals(Ctx<VB, KB> &c, int q0, int nv, unsigne
 // over the clusters and ends the step.  The roots, and then the quotients, are
 // taken by different lanes in one instruction sequence each: an FP64 sequence
 // takes as long for one lane as for 32.
-template <typename VB, int KB>
-__device__ void scalar_warp(Ctx<VB, KB> &c, unsigned seq, bool raw) {
+template <typename VB, int KB, int NT>
+__device__ void scalar_warp(Ctx<VB, KB, NT> &c, unsigned seq, bool raw) {
     const GsArgs<VB> &a = *c.a;
     const xb::GmDev &st = a.st;
     const double *h = c.S->hcol;
@@ -690,22 +695,22 @@ __device__ void scalar_warp(Ctx<VB, KB> &c, unsigned seq, bool raw) {
 // DGKS against 40 rows of n = 2.1M 614 us (940; the FP64 pipe's floor 557); BCGS
 // against 30 rows of n = 16.8M 2.12 ms (2.28; floor 1.68); MGS against 12 rows
 // of n = 16.8M 953 us (1090); FP32 BCGS against 16 rows of n = 2.1M 58 us.
-template <typename VB, int KB, int GRAM, bool SM>
-__global__ void __launch_bounds__(gs_threads<VB>() + 64, 1) k_gs(const __grid_constant__ GsArgs<VB> a) {
+template <typename VB, int KB, int NT, int GRAM, bool SM>
+__global__ void __launch_bounds__(NT + 64, 1) k_gs(const __grid_constant__ GsArgs<VB> a) {
     if (a.st.misc && a.st.misc[xb::GM_STOP] != 0.0) return;
     if (cluster_size() != a.cs) {  // launched in another shape (a tool's replay): no peers to talk to
         if (threadIdx.x == 0) *reinterpret_cast<volatile int *>(a.err) = 1;
         return;
     }
     extern __shared__ __align__(16) unsigned char dyn[];
-    __shared__ GsShared<VB, KB> S;
-    constexpr int NG = gram_count(KB, GRAM), NT = gs_threads<VB>(), NW = NT / 32;
+    __shared__ GsShared<VB, KB, NT> S;
+    constexpr int NG = gram_count(KB, GRAM), NW = NT / 32;
     constexpr int NX = KB + NG <= 1 ? 1 : KB + NG <= 2 ? 2 : KB + NG <= 4 ? 4 : KB + NG <= 8 ? 8 : 16;
     const int tid = threadIdx.x;
     const bool raw = !a.st.misc || a.st.misc[xb::GM_RAW] != 0.0;
     const int k = a.j + 1;
     const int64_t c0 = blockIdx.x * a.chunk;
-    Ctx<VB, KB> c;
+    Ctx<VB, KB, NT> c;
     c.S = &S;
     c.a = &a;
     c.Vc = a.V + c0;
@@ -713,7 +718,7 @@ __global__ void __launch_bounds__(gs_threads<VB>() + 64, 1) k_gs(const __grid_co
     c.bc = c.part + 2 * kGsVals * NW * 16;
     c.ring = c.bc + 2 * kGsVals * 16;
     c.len = (int)max((int64_t)0, min(a.chunk, a.n - c0));
-    c.tiles = (c.len + gs_tile<VB, KB>() - 1) / gs_tile<VB, KB>();
+    c.tiles = (c.len + gs_tile<VB, KB, NT>() - 1) / gs_tile<VB, KB, NT>();
     c.rank = cluster_rank();
     c.lane = tid & 31;
     c.wv = tid >> 5;
@@ -721,7 +726,7 @@ __global__ void __launch_bounds__(gs_threads<VB>() + 64, 1) k_gs(const __grid_co
     c.pitch = (unsigned)(a.ld * sizeof(VB));
     c.st = c.ph = c.pass = 0;
     c.fine = true;
-    for (int i = tid; i < gs_xch_bytes<VB>() / 16; i += NT + 64)
+    for (int i = tid; i < gs_xch_bytes<NT>() / 16; i += NT + 64)
         reinterpret_cast<ulonglong2 *>(dyn)[i] = make_ulonglong2(0, 0);
     if (tid == 0) {
         S.abort = 0;
@@ -771,7 +776,7 @@ __global__ void __launch_bounds__(gs_threads<VB>() + 64, 1) k_gs(const __grid_co
         }
     } else {
         VB *wg = a.w + c0;
-        VB *wl = SM ? reinterpret_cast<VB *>(dyn + gs_xch_bytes<VB>() + (size_t)a.stages * KB * gs_pitch<VB, KB>())
+        VB *wl = SM ? reinterpret_cast<VB *>(dyn + gs_xch_bytes<NT>() + (size_t)a.stages * KB * gs_pitch<VB, KB, NT>())
                     : wg;
         const VB *src = wg;
         bool fg = true;                // w comes from global memory
@@ -802,7 +807,7 @@ __global__ void __launch_bounds__(gs_threads<VB>() + 64, 1) k_gs(const __grid_co
                     if (gr) {
                         double v[NX], o[KB + NG];
                         nv = KB + NG;
-                        gs_pass<VB, KB, GRAM, true, false>(c, src, fg, dst, u0, nu, cu, d0, nd, o);
+                        gs_pass<VB, KB, NT, GRAM, true, false>(c, src, fg, dst, u0, nu, cu, d0, nd, o);
 #pragma unroll
                         for (int i = 0; i < NX; i++) v[i] = i < KB + NG ? o[i] : 0.0;
                         publish<NX>(c, v, 0, seq);
@@ -810,7 +815,7 @@ __global__ void __launch_bounds__(gs_threads<VB>() + 64, 1) k_gs(const __grid_co
                 }
                 if (GRAM != 2 && !gr) {
                     double v[KB];
-                    gs_pass<VB, KB, GRAM, false, false>(c, src, fg, dst, u0, nu, cu, d0, nd, v);
+                    gs_pass<VB, KB, NT, GRAM, false, false>(c, src, fg, dst, u0, nu, cu, d0, nd, v);
                     publish<KB>(c, v, 0, seq);
                 }
                 relay(c, nv, seq);
@@ -859,14 +864,14 @@ __global__ void __launch_bounds__(gs_threads<VB>() + 64, 1) k_gs(const __grid_co
                 src = dst = wl;
                 fg = !SM;
             }
-        } else if constexpr (KB == 8 && GRAM == 0) {
+        } else if constexpr (GRAM == 0) {
             for (int r = 0; r < rounds && c.fine; r++)
                 for (int g0 = 0; g0 < k && c.fine; g0 += kGsVals) {
                     const int kg = min(kGsVals, k - g0);
                     seq++;
                     for (int d0 = g0; d0 < g0 + kg; d0 += KB) {
                         double v[KB];
-                        gs_pass<VB, KB, 0, false, false>(c, src, fg, dst, 0, r > 0 && d0 == 0 ? k : 0, cu, d0,
+                        gs_pass<VB, KB, NT, 0, false, false>(c, src, fg, dst, 0, r > 0 && d0 == 0 ? k : 0, cu, d0,
                                                          min(KB, k - d0), v);
                         publish<KB>(c, v, d0 - g0, seq);
                         src = wl;
@@ -892,7 +897,7 @@ __global__ void __launch_bounds__(gs_threads<VB>() + 64, 1) k_gs(const __grid_co
         if (blockIdx.x == 0) bar_arrive(2, NT + 32);
         if (c.fine) {
             double v[1];
-            gs_pass<VB, KB, 0, false, true>(c, src, fg, wg, u0, nu, cu, 0, 0, v);
+            gs_pass<VB, KB, NT, GRAM, false, true>(c, src, fg, wg, u0, nu, cu, 0, 0, v);
             publish<1>(c, v, 0, seq + 1);
             if (c.rank == 0 && c.wv == 0) {
                 const double s = cluster_sum(c, 0, seq + 1);
@@ -926,11 +931,11 @@ int max_clusters(K kernel, int threads, int cs, int *clusters) {
     return XB_OK;
 }
 
-template <typename VB, int KB, int GRAM, bool SM>
+template <typename VB, int KB, int NT, int GRAM, bool SM>
 int launch(GsArgs<VB> &a, int clusters, size_t smem, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(clusters * a.cs));
-    cfg.blockDim = dim3(gs_threads<VB>() + 64);
+    cfg.blockDim = dim3(NT + 64);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[2];
@@ -941,7 +946,7 @@ int launch(GsArgs<VB> &a, int clusters, size_t smem, cudaStream_t s) {
     at[1].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    XB_CUDA(cudaLaunchKernelEx(&cfg, k_gs<VB, KB, GRAM, SM>, a));
+    XB_CUDA(cudaLaunchKernelEx(&cfg, k_gs<VB, KB, NT, GRAM, SM>, a));
     return XB_OK;
 }
 
@@ -959,7 +964,7 @@ int gs_numbers(xb_plan *p, unsigned used, unsigned *base, cudaStream_t s) {
     return XB_OK;
 }
 
-template <typename VB, int KB, int GRAM>
+template <typename VB, int KB, int GRAM, int NT = 256>
 int plan_launch(xb_plan *p, GsArgs<VB> &a, cudaStream_t s) {
     struct Limits {
         int nc[9];
@@ -969,12 +974,12 @@ int plan_launch(xb_plan *p, GsArgs<VB> &a, cudaStream_t s) {
     int dev = 0;
     XB_CUDA(cudaGetDevice(&dev));
     XB_TRY(limits.get(dev, [](Limits &l) {
-        XB_CUDA(cudaFuncSetAttribute(k_gs<VB, KB, GRAM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        XB_CUDA(cudaFuncSetAttribute(k_gs<VB, KB, NT, GRAM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      xb::kGsDynMax));
-        XB_CUDA(cudaFuncSetAttribute(k_gs<VB, KB, GRAM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        XB_CUDA(cudaFuncSetAttribute(k_gs<VB, KB, NT, GRAM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      xb::kGsDynMax));
         for (int cs : {2, 4, 8})
-            XB_TRY(max_clusters(k_gs<VB, KB, GRAM, true>, gs_threads<VB>() + 64, cs, &l.nc[cs]));
+            XB_TRY(max_clusters(k_gs<VB, KB, NT, GRAM, true>, NT + 64, cs, &l.nc[cs]));
         return (int)XB_OK;
     }, &lim));
     // Larger clusters make the exchange cheaper (3.1 / 3.5 / 4.6 us with 8 / 4 / 2
@@ -988,14 +993,14 @@ int plan_launch(xb_plan *p, GsArgs<VB> &a, cudaStream_t s) {
     if (lim.nc[a.cs] < 1) return xb::set_error(XB_ECUDA, "orthogonalisation: no cluster of %d fits", a.cs);
     // a CTA has at least an element per thread (n = 9,600, MGS against 20 rows:
     // 33.0 us with 256 elements a CTA, 42.9 with 1024)
-    const int64_t per = gs_threads<VB>();
+    const int64_t per = NT;
     const int64_t want = (a.n + per * a.cs - 1) / (per * a.cs);
     const int most = p->gs_ctas ? std::min(lim.nc[a.cs], p->gs_ctas / a.cs) : lim.nc[a.cs];
     const int nc = (int)std::max<int64_t>(1, std::min<int64_t>(most, want));
     const int64_t G = (int64_t)nc * a.cs;
     a.chunk = ((a.n + G - 1) / G + 3) / 4 * 4;
     // w in shared memory when three stages fit beside it
-    const size_t stage = (size_t)KB * gs_pitch<VB, KB>(), fixed = gs_xch_bytes<VB>();
+    const size_t stage = (size_t)KB * gs_pitch<VB, KB, NT>(), fixed = gs_xch_bytes<NT>();
     const size_t wb = (size_t)a.chunk * sizeof(VB);
     const bool sm = fixed + 3 * stage + wb <= (size_t)xb::kGsDynMax;
     a.stages = (int)std::min<size_t>(kGsMaxStages, (xb::kGsDynMax - fixed - (sm ? wb : 0)) / stage);
@@ -1005,7 +1010,7 @@ int plan_launch(xb_plan *p, GsArgs<VB> &a, cudaStream_t s) {
     const int sums = blocks ? (k + KB - 1) / KB
                             : (a.method == XB_ORTHO_DGKS ? 2 : 1) * ((k + kGsVals - 1) / kGsVals);
     XB_TRY(gs_numbers(p, (unsigned)sums + 1, &a.base, s));
-    return sm ? launch<VB, KB, GRAM, true>(a, nc, smem, s) : launch<VB, KB, GRAM, false>(a, nc, smem, s);
+    return sm ? launch<VB, KB, NT, GRAM, true>(a, nc, smem, s) : launch<VB, KB, NT, GRAM, false>(a, nc, smem, s);
 }
 
 template <typename VB>
@@ -1017,9 +1022,32 @@ int gs_run(xb_plan *p, GsArgs<VB> &a, bool seen, cudaStream_t s) {
     a.err = reinterpret_cast<int *>(p->h_pin + 60);
     a.late = reinterpret_cast<unsigned long long *>(p->h_pin + 40);
     a.tag = ++p->gs_tag;
+    // Rows of a block, and threads.  Long vectors want few rows: MGS pays for the
+    // products of its blocks (GMRES(10) of n = 8M, us a step: blocks of 8 510, of 4
+    // 474, of 2 422; n = 2.1M, GMRES(20): 191, 202, 197), and a unit of fewer rows
+    // than the block has leaves undone the copies that hide the latency (against 1
+    // row of n = 16.8M, blocks of 8 / 2: DGKS 484 / 285 us; 4 rows, 8 / 4: 680 / 604).
+    // Without products in the way 512 threads go with it (256 / 512: DGKS against 3,
+    // 9 rows 558 / 483, 1416 / 1329; BCGS against 5 513 / 387).  An FP32 basis of n =
+    // 2.1M / 16.8M, GMRES(10): MGS in 8 90 / 455, in 4 84 / 441; DGKS 108 / 574, 95 / 546
+    // (n = 1M, GMRES(30): MGS 74, 76).  MGS has one block size for a whole solve (st.gram).
+    const bool longv = a.n >= 3000000;
+    const int k = a.j + 1;
+    if constexpr (sizeof(VB) == 8) {
+        if (longv && (a.method != XB_ORTHO_MGS || k == 1)) {
+            // one row: every method takes one dot
+            if (k <= 2) return plan_launch<VB, 2, 0, 512>(p, a, s);
+            if (k <= 4 || a.method == XB_ORTHO_BCGS) return plan_launch<VB, 4, 0, 512>(p, a, s);
+            return plan_launch<VB, 8, 0, 512>(p, a, s);
+        }
+    } else {
+        if (a.n >= 1500000 && a.method != XB_ORTHO_BCGS)
+            return a.method == XB_ORTHO_MGS ? plan_launch<VB, 4, 1>(p, a, s) : plan_launch<VB, 4, 0>(p, a, s);
+    }
     if (a.method == XB_ORTHO_BCGS) return plan_launch<VB, 4, 0>(p, a, s);
     if (a.method != XB_ORTHO_MGS) return plan_launch<VB, 8, 0>(p, a, s);
     if constexpr (sizeof(VB) == 8) {
+        if (seen && longv) return plan_launch<VB, 2, 1>(p, a, s);
         if (!seen) {
             // n = 262,144 (16 rows): blocks of 4 / 2 59.9 / 61.5 us; n = 1M (20
             // rows) 162 / 151 us: beyond, the rows' own products cost more FP64

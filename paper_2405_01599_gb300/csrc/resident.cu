@@ -34,7 +34,8 @@
 // each (64 x 64 Poisson, GMRES(30): MGS with an exchange per vector 17.3 us a
 // step, in corrected blocks 14.4, BCGS 12.6; eight at once would add as many FP64
 // sums as it saves exchanges).  The inner products that correct MGS's blocks are
-// taken with ||w||^2 and stand in H's unused lower triangle.
+// taken with ||w||^2 and stand in H's unused lower triangle.  In short cycles MGS
+// takes a vector at a time (res_gs).
 //
 // Reductions.  One, or four at once, sums over the cluster: each warp
 // reduces its lanes' partials with shuffles (four sums in a transposed tree:
@@ -69,6 +70,8 @@ namespace {
 constexpr int kMaxRow = 64;  // longest row the ELL copy takes
 constexpr int kW = 4;        // warps per CTA: one per SM sub-partition
 constexpr int kBT = 32 * kW;
+// Gram-Schmidt: MGS and BCGS in blocks of four, MGS a vector at a time
+constexpr int kMgs4 = 0, kBcgs = 1, kMgs1 = 2;
 constexpr unsigned kFull = 0xffffffffu;
 
 struct ResArgs {
@@ -83,10 +86,10 @@ struct ResArgs {
 
 // Byte offsets of the dynamic shared memory regions (doubles first).
 struct ResLayout {
-    size_t V, W, ev, bs, ms, H, cs, sn, g, y, ea, mb, total;
+    size_t V, W, ev, bs, ms, H, cs, sn, g, y, ea, p2, mb, total;
 };
 
-__host__ __device__ inline ResLayout res_layout(int rpp, int lmax, int mmax, int P) {
+__host__ __device__ inline ResLayout res_layout(int rpp, int lmax, int mmax, int P, int gs) {
     ResLayout L;
     size_t o = 0;
     auto take = [&](size_t bytes) {
@@ -105,6 +108,8 @@ __host__ __device__ inline ResLayout res_layout(int rpp, int lmax, int mmax, int
     L.g = take((size_t)(mmax + 1) * 8);
     L.y = take((size_t)mmax * 8);
     L.ea = take((size_t)lmax * rpp * 4);
+    // kMgs1, R <= 4: each thread's part of (v_{i-1}, v_i), formed once per basis vector
+    L.p2 = take(gs == kMgs1 && rpp <= 4 * kBT ? (size_t)(mmax + 1) * kBT * 8 : 0);
     L.mb = take(2 * 8 + 4);  // two mbarriers, the abort flag
     L.total = o;
     return L;
@@ -241,7 +246,7 @@ struct Red {
     double *bs, *ms;       // barrier / mbarrier slots: 2 phases x 4 sums x P
     unsigned mb;           // shared address of the two mbarriers
     volatile int *abort;   // set when an mbarrier wait gave up
-    int slot, bph, mk;     // this warp's slot, phases
+    int slot, bph, mk, K;  // this warp's slot, phases, sums of an mbarrier exchange
 };
 
 // Barrier-completed sum of one value (also publishes the caller's earlier
@@ -277,7 +282,15 @@ __device__ __forceinline__ void bget4(double (&v)[4], Red<NCL> &R) {
     R.bph ^= 1;
 }
 
-// mbarrier-completed sums of four values.
+// mbarrier-completed sums (R.K values: 1 for kMgs1, else 4).
+template <int NCL>
+__device__ __forceinline__ void mput1(double v, const Red<NCL> &R) {
+    v = warp_sum1(v);
+    const int lane = threadIdx.x & 31, p = R.mk & 1;
+    if (lane < NCL)
+        st_async(map_rank(smem_addr(R.ms + p * 4 * R.P + R.slot), (unsigned)lane), v,
+                 map_rank(R.mb + 8 * p, (unsigned)lane));
+}
 template <int NCL>
 __device__ __forceinline__ void mput4(const double (&v)[4], const Red<NCL> &R) {
     const double k = warp_sum4(v);
@@ -305,7 +318,7 @@ __device__ __forceinline__ const double *mwait(Red<NCL> &R) {
     }
     // re-arm only a completed phase (after a timeout the exchange is lost and
     // every later wait returns at once)
-    if (threadIdx.x == 0 && done) mb_arm(a, (unsigned)(4 * R.P * 8));
+    if (threadIdx.x == 0 && done) mb_arm(a, (unsigned)(R.K * R.P * 8));
     R.mk++;
     return R.ms + p * 4 * R.P;
 }
@@ -337,12 +350,12 @@ __device__ __forceinline__ void rows_spmv(const double *__restrict__ ev, const i
     }
 }
 
-template <int R, int NCL, bool BCGS>
+template <int R, int NCL, int GS>
 __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int rpp = kBT * R;
     const int mmax = A.m_max, ldh = mmax + 1;
-    const ResLayout L = res_layout(rpp, A.lmax, mmax, 4 * NCL);
+    const ResLayout L = res_layout(rpp, A.lmax, mmax, 4 * NCL, GS);
     double *V = reinterpret_cast<double *>(smem + L.V);
     double *W = reinterpret_cast<double *>(smem + L.W);
     double *ev = reinterpret_cast<double *>(smem + L.ev);
@@ -352,6 +365,7 @@ __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
     double *g = reinterpret_cast<double *>(smem + L.g);
     double *yv = reinterpret_cast<double *>(smem + L.y);
     int *ea = reinterpret_cast<int *>(smem + L.ea);
+    double *P2 = reinterpret_cast<double *>(smem + L.p2);  // kMgs1, R <= 4
     const unsigned rank = cluster_rank();
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     Red<NCL> Rd;
@@ -362,13 +376,14 @@ __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
     Rd.slot = (int)rank * kW + warp;
     Rd.bph = 0;
     Rd.mk = 0;
+    Rd.K = GS == kMgs1 ? 1 : 4;
     if (t == 0) {
         *Rd.abort = 0;
         mb_init(Rd.mb);
         mb_init(Rd.mb + 8);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        mb_arm(Rd.mb, (unsigned)(4 * Rd.P * 8));
-        mb_arm(Rd.mb + 8, (unsigned)(4 * Rd.P * 8));
+        mb_arm(Rd.mb, (unsigned)(Rd.K * Rd.P * 8));
+        mb_arm(Rd.mb + 8, (unsigned)(Rd.K * Rd.P * 8));
     }
     const bool lead = rank == 0 && t == 0;
     const unsigned long long ts = gtimer(), deadline = ts + A.budget_ns;
@@ -510,7 +525,54 @@ __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
                 // quarter of the exchanges
                 double c4[4] = {0.0, 0.0, 0.0, 0.0};
                 int u0 = 0, nu = 0;
-                for (int d0 = 0; d0 <= j; d0 += 4) {
+                if constexpr (GS == kMgs1) {
+                    // pass i applies the projection on v_{i-1} and takes (w, v_i)
+                    double hprev = 0.0;
+                    if constexpr (R <= 4) {
+                        // the thread's part of (w - h_{i-1} v_{i-1}, v_i) as
+                        // (w, v_i) - h_{i-1} (v_{i-1}, v_i): the first part is
+                        // formed while the previous exchange is in flight, the
+                        // second once when v_i was written, so one FMA separates
+                        // h_{i-1} from the next send
+                        double p1 = 0.0, p2 = 0.0;
+#pragma unroll
+                        for (int r = 0; r < R; r++) p1 = fma(w[r], V[r * kBT + t], p1);
+                        for (int i = 0; i <= j; i++) {
+                            mput1(i == 0 ? p1 : fma(-hprev, p2, p1), Rd);
+                            if (i > 0) {
+#pragma unroll
+                                for (int r = 0; r < R; r++)
+                                    w[r] = fma(-hprev, V[(i - 1) * rpp + r * kBT + t], w[r]);
+                            }
+                            if (i < j) {
+                                p1 = 0.0;
+#pragma unroll
+                                for (int r = 0; r < R; r++)
+                                    p1 = fma(w[r], V[(i + 1) * rpp + r * kBT + t], p1);
+                                p2 = P2[(i + 1) * kBT + t];
+                            }
+                            if (i > 0) take(i - 1, hprev);
+                            hprev = slots_sum1<NCL>(mwait(Rd));
+                        }
+                    } else {
+                        for (int i = 0; i <= j; i++) {
+                            double a = 0.0;
+#pragma unroll
+                            for (int r = 0; r < R; r++) {
+                                const int l = r * kBT + t;
+                                if (i > 0) w[r] = fma(-hprev, V[(i - 1) * rpp + l], w[r]);
+                                a = fma(w[r], V[i * rpp + l], a);
+                            }
+                            mput1(a, Rd);
+                            if (i > 0) take(i - 1, hprev);
+                            hprev = slots_sum1<NCL>(mwait(Rd));
+                        }
+                    }
+                    c4[0] = hprev;
+                    u0 = j;
+                    nu = 1;
+                }
+                for (int d0 = 0; GS != kMgs1 && d0 <= j; d0 += 4) {
                     const int nd = min(4, j + 1 - d0);
                     double a4[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
@@ -527,7 +589,7 @@ __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
 #pragma unroll
                     for (int q = 0; q < 4; q++)
                         if (q < nu) take(u0 + q, c4[q]);
-                    if constexpr (BCGS) {
+                    if constexpr (GS == kBcgs) {
                         slots_sum4<NCL>(mwait(Rd), c4);
                     } else {
                         double gr[4][3];
@@ -556,7 +618,7 @@ __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
                 wb ^= 1;
                 // ||w||^2 and, for MGS, w's products with the basis vectors it
                 // will share a block with
-                const int ng = BCGS || j + 1 >= m ? 0 : (j + 1) & 3, g0 = j + 1 - ng;
+                const int ng = GS != kMgs4 || j + 1 >= m ? 0 : (j + 1) & 3, g0 = j + 1 - ng;
                 double n4[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
                 for (int r = 0; r < R; r++) {
@@ -590,7 +652,7 @@ __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
                         H[j * ldh + j + 1] = rr2 * irr;  // the diagonal, until the restart
                         g[j] = c * gj;
                     }
-                    if (!BCGS && t < ng) H[gram(j + 1) + t] = (t == 0 ? n4[1] : t == 1 ? n4[2] : n4[3]) * ihn;
+                    if (GS == kMgs4 && t < ng) H[gram(j + 1) + t] = (t == 0 ? n4[1] : t == 1 ? n4[2] : n4[3]) * ihn;
                     gj = -s * gj;
                     if (hn2 <= 1e-28 * (len2 + hn2)) flag = 1;  // hn <= 1e-14 |column|
                     else if (fabs(gj) <= tol_g) flag = 3;
@@ -612,6 +674,12 @@ __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
                 double *Vn = V + (j + 1) * rpp;
 #pragma unroll
                 for (int r = 0; r < R; r++) Vn[r * kBT + t] = w[r] * sc;
+                if constexpr (GS == kMgs1 && R <= 4) {
+                    double pv = 0.0;  // (v_j, v_{j+1}), this thread's part
+#pragma unroll
+                    for (int r = 0; r < R; r++) pv = fma(V[j * rpp + r * kBT + t], w[r] * sc, pv);
+                    P2[(j + 1) * kBT + t] = pv;
+                }
                 if (flag == 3) {
                     claimed = 1;
                     break;
@@ -702,25 +770,40 @@ __global__ void __launch_bounds__(kBT, 1) k_gmres_resident(const ResArgs A) {
 
 typedef void (*ResKernel)(const ResArgs);
 
-template <int R, bool BCGS>
+template <int R, int GS>
 ResKernel res_kernel_r(int ncl) {
     switch (ncl) {
-        case 2: return k_gmres_resident<R, 2, BCGS>;
-        case 4: return k_gmres_resident<R, 4, BCGS>;
-        case 8: return k_gmres_resident<R, 8, BCGS>;
-        case 16: return k_gmres_resident<R, 16, BCGS>;
+        case 2: return k_gmres_resident<R, 2, GS>;
+        case 4: return k_gmres_resident<R, 4, GS>;
+        case 8: return k_gmres_resident<R, 8, GS>;
+        case 16: return k_gmres_resident<R, 16, GS>;
         default: return nullptr;
     }
 }
 
-ResKernel res_kernel(int R, int ncl, bool bcgs) {
+template <int GS>
+ResKernel res_kernel_gs(int R, int ncl) {
     switch (R) {
-        case 1: return bcgs ? res_kernel_r<1, true>(ncl) : res_kernel_r<1, false>(ncl);
-        case 2: return bcgs ? res_kernel_r<2, true>(ncl) : res_kernel_r<2, false>(ncl);
-        case 4: return bcgs ? res_kernel_r<4, true>(ncl) : res_kernel_r<4, false>(ncl);
-        case 8: return bcgs ? res_kernel_r<8, true>(ncl) : res_kernel_r<8, false>(ncl);
+        case 1: return res_kernel_r<1, GS>(ncl);
+        case 2: return res_kernel_r<2, GS>(ncl);
+        case 4: return res_kernel_r<4, GS>(ncl);
+        case 8: return res_kernel_r<8, GS>(ncl);
         default: return nullptr;
     }
+}
+ResKernel res_kernel(int R, int ncl, int gs) {
+    return gs == kBcgs ? res_kernel_gs<kBcgs>(R, ncl) : gs == kMgs1 ? res_kernel_gs<kMgs1>(R, ncl)
+                                                                    : res_kernel_gs<kMgs4>(R, ncl);
+}
+
+// Short cycles of MGS take a vector at a time: a block's own products and four-value
+// sums cost more than the exchanges that blocks save (us a step, blocks / singly:
+// 1600 rows, one a thread, m = 5, 8: 9.0 / 9.0, 8.7 / 9.0; 4096, two a thread, m = 5, 10,
+// 20: 10.4 / 9.5, 10.2 / 10.1, 12.3 / 13.7; 8100, four a thread: m = 5, 10, 20: 12.5 /
+// 11.0, 12.7 / 12.1, 15.1 / 16.4).
+int res_gs(int ortho, int mmax, int R) {
+    if (ortho == XB_ORTHO_BCGS) return kBcgs;
+    return mmax <= (R == 1 ? 5 : R == 2 ? 10 : 13) ? kMgs1 : kMgs4;
 }
 
 }  // namespace
@@ -773,10 +856,14 @@ int resident_gmres(xb_plan *p, const double *b, double *x, const xb_options &o, 
         const int rpc = (p->n + ncl - 1) / ncl;
         int R = 1;
         while (R * kBT < rpc) R *= 2;
-        ResKernel kf = res_kernel(R, ncl, o.ortho == XB_ORTHO_BCGS);
-        if (!kf) continue;
-        const ResLayout L = res_layout(kBT * R, lmax, mmax, ncl * kW);
-        if (L.total > (size_t)optin) continue;
+        int gs = res_gs(o.ortho, mmax, R);
+        ResLayout L = res_layout(kBT * R, lmax, mmax, ncl * kW, gs);
+        if (gs == kMgs1 && L.total > (size_t)optin) {  // blocks need less shared memory
+            gs = kMgs4;
+            L = res_layout(kBT * R, lmax, mmax, ncl * kW, gs);
+        }
+        ResKernel kf = res_kernel(R, ncl, gs);
+        if (!kf || L.total > (size_t)optin) continue;
         XB_CUDA(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
         if (ncl > 8) XB_CUDA(cudaFuncSetAttribute(kf, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         cudaLaunchConfig_t cfg = {};

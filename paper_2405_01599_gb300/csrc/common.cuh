@@ -181,6 +181,8 @@ struct IluData {
     int grid = 0, maxrows = 0, cap = 0;
     unsigned seq = 0;                // number of the last application
     unsigned long long limit_ns = 0;
+    double bytes = 0.0;              // device memory of all of this
+    double flow_bytes = 0.0;         // read and written by one application on the flow path
     // graph path (built when first taken): inside a level rows are ordered by
     // tier, short rows (<= 8 entries in the triangle) first and stored again
     // level by level in ELL form, then rows of up to 512 entries (thread or warp
@@ -231,6 +233,8 @@ struct xb_plan {
     size_t work_bytes = 0;
     double *h_pin = nullptr;             // pinned host mirror of a few scalars
     unsigned long long gs_tag = 0;       // orthogonalisations launched
+    int gs_kb = 4;                       // the newest one's rows of a block, and whether
+    bool gs_held = true;                 // its CTAs held w
     int gs_ctas = 0;                     // CTAs one may hold (0: as many as fit)
     unsigned gs_polls = 0;               // polls of one of their waits (0: default)
     unsigned gs_number = 0;              // the newest one's last exchange number
@@ -316,7 +320,7 @@ double spmv_alg_bytes(const xb_plan *p, bool beta_nonzero, int val_bytes);
 // starts, BSS bitmask and warp rows, segment tables).
 double spmv_meta_bytes(const xb_plan *p, int variant, int block, int ipt);
 
-// ---- vector kernels (vec.cu) ------------------------------------------------
+// ---- vector kernels (krylov.cu) ------------------------------------------------
 // Deterministic reductions write their result to a device double.
 int vdot(xb_plan *p, int64_t n, const double *x, const double *y, double *out, cudaStream_t s);
 int vnrm2(xb_plan *p, int64_t n, const double *x, double *out, cudaStream_t s);

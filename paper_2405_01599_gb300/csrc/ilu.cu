@@ -778,36 +778,46 @@ int ilu_levels(int n, const int *rp, const int *ci, std::vector<int> &dpos, std:
 
 namespace {
 
-int upload(int **d, const std::vector<int> &h, cudaStream_t s) {
-    XB_CUDA(cudaMalloc(d, std::max<size_t>(1, h.size()) * 4));
+// Device memory that the preconditioner keeps.
+template <typename T>
+int keep(IluData &u, T **d, size_t bytes) {
+    XB_CUDA(cudaMalloc(d, std::max<size_t>(8, bytes)));
+    u.bytes += (double)bytes;
+    return XB_OK;
+}
+
+int upload(int **d, const std::vector<int> &h, cudaStream_t s, IluData *u = nullptr) {
+    if (u) XB_TRY(keep(*u, d, h.size() * 4));
+    else XB_CUDA(cudaMalloc(d, std::max<size_t>(1, h.size()) * 4));
     if (!h.empty()) XB_CUDA(cudaMemcpyAsync(*d, h.data(), h.size() * 4, cudaMemcpyHostToDevice, s));
     return XB_OK;
 }
 
 // ELL values of a layout's entries from the factors.
-int fill_entries(double **val, const std::vector<int> &src, const double *lu, cudaStream_t s) {
+int fill_entries(IluData &u, double **val, const std::vector<int> &src, cudaStream_t s) {
     int *d_src = nullptr;
-    XB_CUDA(cudaMalloc(val, std::max<size_t>(1, src.size()) * sizeof(double)));
+    XB_TRY(keep(u, val, src.size() * sizeof(double)));
     XB_TRY(upload(&d_src, src, s));
     if (!src.empty()) {
-        k_ell_fill<<<(unsigned)((src.size() + 255) / 256), 256, 0, s>>>((long long)src.size(), d_src, lu, *val);
+        k_ell_fill<<<(unsigned)((src.size() + 255) / 256), 256, 0, s>>>((long long)src.size(), d_src, u.d_lu, *val);
         XB_LAUNCHED("k_ell_fill");
     }
     cudaFree(d_src);  // waits for the kernel
     return XB_OK;
 }
 
-int upload_flow(IluData::Flow &f, const FlowHost &h, const double *lu, cudaStream_t s) {
+int upload_flow(IluData &u, IluData::Flow &f, const FlowHost &h, cudaStream_t s) {
     static_assert(sizeof(int4) == 16 && sizeof(long long) == 8, "layout");
-    XB_CUDA(cudaMalloc(&f.d_items, std::max<size_t>(1, h.items.size()) * sizeof(int4)));
+    XB_TRY(keep(u, &f.d_items, h.items.size() * sizeof(int4)));
     XB_CUDA(cudaMemcpyAsync(f.d_items, h.items.data(), h.items.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
-    XB_CUDA(cudaMalloc(&f.d_ebase, h.ebase.size() * sizeof(long long)));
+    XB_TRY(keep(u, &f.d_ebase, h.ebase.size() * sizeof(long long)));
     XB_CUDA(cudaMemcpyAsync(f.d_ebase, h.ebase.data(), h.ebase.size() * sizeof(long long),
                             cudaMemcpyHostToDevice, s));
-    XB_TRY(upload(&f.d_iptr, h.iptr, s));
-    XB_TRY(upload(&f.d_rows, h.rows, s));
-    XB_TRY(upload(&f.d_ecol, h.ecol, s));
-    return fill_entries(&f.d_eval, h.esrc, lu, s);
+    XB_TRY(upload(&f.d_iptr, h.iptr, s, &u));
+    XB_TRY(upload(&f.d_rows, h.rows, s, &u));
+    XB_TRY(upload(&f.d_ecol, h.ecol, s, &u));
+    u.flow_bytes += 16.0 * h.items.size() + 4.0 * h.rows.size() + 12.0 * h.ecol.size();
+    return fill_entries(u, &f.d_eval, h.esrc, s);
 }
 
 int rows_host(xb_plan *p, std::vector<int> &ci) {
@@ -848,14 +858,14 @@ int ensure_graph(xb_plan *p, cudaStream_t s) {
         cudaFree(*d);
         *d = nullptr;
     }
-    XB_TRY(upload(&u.d_lrows, lrows, s));
-    XB_TRY(upload(&u.d_urows, urows, s));
-    XB_TRY(upload(&u.d_lecol, lecol, s));
-    XB_TRY(upload(&u.d_uecol, uecol, s));
-    XB_TRY(fill_entries(&u.d_leval, lesrc, u.d_lu, s));
-    XB_TRY(fill_entries(&u.d_ueval, uesrc, u.d_lu, s));
-    XB_CUDA(cudaMalloc(&u.d_udiag, std::max<size_t>(1, (size_t)n) * sizeof(double)));
-    XB_CUDA(cudaMalloc(&u.d_out, std::max<size_t>(1, (size_t)n) * sizeof(double)));
+    XB_TRY(upload(&u.d_lrows, lrows, s, &u));
+    XB_TRY(upload(&u.d_urows, urows, s, &u));
+    XB_TRY(upload(&u.d_lecol, lecol, s, &u));
+    XB_TRY(upload(&u.d_uecol, uecol, s, &u));
+    XB_TRY(fill_entries(u, &u.d_leval, lesrc, s));
+    XB_TRY(fill_entries(u, &u.d_ueval, uesrc, s));
+    XB_TRY(keep(u, &u.d_udiag, (size_t)n * sizeof(double)));
+    XB_TRY(keep(u, &u.d_out, (size_t)n * sizeof(double)));
     k_diag_fill<<<(n + 255) / 256, 256, 0, s>>>(n, u.d_urows, u.d_dpos, u.d_lu, u.d_udiag, nullptr,
                                                 nullptr);
     XB_LAUNCHED("k_diag_fill");
@@ -894,11 +904,11 @@ int ensure_ilu(xb_plan *p, cudaStream_t s) {
     level_order(lev, nl, lorder, loff);
     // factors, level by level
     int *d_order = nullptr;
-    XB_TRY(upload(&u.d_dpos, dpos, s));
+    XB_TRY(upload(&u.d_dpos, dpos, s, &u));
     XB_TRY(upload(&d_order, lorder, s));
-    XB_CUDA(cudaMalloc(&u.d_lu, std::max<size_t>(1, (size_t)nnz) * sizeof(double)));
-    XB_CUDA(cudaMalloc(&u.d_flag, 2 * sizeof(int)));  // zero pivot; pivot out of the flow path's range
-    XB_CUDA(cudaMalloc(&u.d_in, std::max<size_t>(1, (size_t)n) * sizeof(double)));
+    XB_TRY(keep(u, &u.d_lu, (size_t)nnz * sizeof(double)));
+    XB_TRY(keep(u, &u.d_flag, 2 * sizeof(int)));  // zero pivot; pivot out of the flow path's range
+    XB_TRY(keep(u, &u.d_in, (size_t)n * sizeof(double)));
     XB_CUDA(cudaMemsetAsync(u.d_flag, 0, 2 * sizeof(int), s));
     if (nnz > 0)
         XB_CUDA(cudaMemcpyAsync(u.d_lu, p->val, (size_t)nnz * sizeof(double),
@@ -935,17 +945,24 @@ int ensure_ilu(xb_plan *p, cudaStream_t s) {
             cudaFree(d_order);
             return set_error(XB_ENOMEM, "ILU(0): host memory for the substitutions' layout");
         }
-        XB_TRY(upload(&u.d_bstart, bstart, s));
-        XB_TRY(upload_flow(u.fl, hl, u.d_lu, s));
-        XB_TRY(upload_flow(u.fu, hu, u.d_lu, s));
-        XB_CUDA(cudaMalloc(&u.fu.d_diag, (size_t)n * sizeof(double)));
-        XB_CUDA(cudaMalloc(&u.fu.d_rdiag, (size_t)n * sizeof(double)));
+        XB_TRY(upload(&u.d_bstart, bstart, s, &u));
+        XB_TRY(upload_flow(u, u.fl, hl, s));
+        XB_TRY(upload_flow(u, u.fu, hu, s));
+        // long rows come from the factors themselves, rows and all
+        long long stored = 0;
+        for (const FlowHost *h : {&hl, &hu})
+            stored += std::count_if(h->esrc.begin(), h->esrc.end(), [](int e) { return e >= 0; });
+        // r in, z out, the pivots and reciprocals, both triangles' published values
+        // out and the first one's in again
+        u.flow_bytes += 12.0 * ((double)nnz - n - stored) + (8.0 + 8.0 + 16.0 + 32.0 + 16.0) * n;
+        XB_TRY(keep(u, &u.fu.d_diag, (size_t)n * sizeof(double)));
+        XB_TRY(keep(u, &u.fu.d_rdiag, (size_t)n * sizeof(double)));
         k_diag_fill<<<(n + 255) / 256, 256, 0, s>>>(n, u.fu.d_rows, u.d_dpos, u.d_lu, u.fu.d_diag,
                                                     u.fu.d_rdiag, u.d_flag + 1);
         XB_LAUNCHED("k_diag_fill");
-        XB_CUDA(cudaMalloc(&u.d_ty, (size_t)n * 16));
-        XB_CUDA(cudaMalloc(&u.d_tz, (size_t)n * 16));
-        XB_CUDA(cudaMalloc(&u.d_stop, sizeof(int)));
+        XB_TRY(keep(u, &u.d_ty, (size_t)n * 16));
+        XB_TRY(keep(u, &u.d_tz, (size_t)n * 16));
+        XB_TRY(keep(u, &u.d_stop, sizeof(int)));
         XB_CUDA(cudaMemsetAsync(u.d_ty, 0, (size_t)n * 16, s));
         XB_CUDA(cudaMemsetAsync(u.d_tz, 0, (size_t)n * 16, s));
         XB_CUDA(cudaMemsetAsync(u.d_stop, 0, sizeof(int), s));
@@ -1037,7 +1054,8 @@ int ilu_apply(xb_plan *p, const double *r, double *z, cudaStream_t s) {
 }
 
 double ilu_apply_bytes(const xb_plan *p) {
-    // both triangles once (value + column), rowptr and diagonal positions
+    if (ilu_mode(p) == 1) return p->ilu.flow_bytes;
+    // the graph of level launches: both triangles once (value + column), rowptr and diagonal positions
     // twice, r read, z written by the forward pass, read and written by the
     // backward pass, and each row's level slot twice
     const double n = p->n, nnz = p->nnz;

@@ -505,14 +505,12 @@ int gm_cycle_init_f32(xb_plan *p, GmDev st, int64_t n, const float *r0, double t
     return XB_OK;
 }
 
-double ortho_passes(int ortho, int j) {
-    const int nb = (j + 1 + 3) / 4;
-    switch (ortho) {
-        case XB_ORTHO_CGS: return 2.0 * j + 5.0;
-        case XB_ORTHO_DGKS: return 3.0 * j + 8.0;
-        case XB_ORTHO_BCGS: return 2.0 * (j + 1) + 2.0 * nb + 1.0;
-        default: return 4.0 * j + 5.0;
-    }
+double ortho_passes(int ortho, int j, int kb, bool held) {
+    const int k = j + 1, nb = (k + kb - 1) / kb, rounds = ortho == XB_ORTHO_DGKS ? 2 : 1;
+    const double rows = 2.0 * rounds * k;
+    if (held) return rows + 2.0;
+    if (ortho == XB_ORTHO_MGS || ortho == XB_ORTHO_BCGS) return rows + 2.0 * nb + 1.0;
+    return rows + rounds * (nb + 1.0) + 1.0;
 }
 
 int ortho_choice(int ortho, double tol, bool faulted) {

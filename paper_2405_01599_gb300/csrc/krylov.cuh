@@ -21,7 +21,6 @@ struct GmDev {
 enum GmMisc {
     GM_BNORM = 0,   // ||b|| (relative-residual denominator)
     GM_RES = 1,     // |g_{k+1}| / ||b||
-    GM_COEF = 2,    // MGS coefficient for the pending axpy
     GM_LEN2 = 3,    // sum_i h_ij^2 of the current column
     GM_K = 4,       // Arnoldi steps completed in this cycle
     GM_STOP = 5,    // 0 running, 1 converged/happy breakdown, 2 singular
@@ -54,9 +53,11 @@ int ortho_sweep(xb_plan *p, int64_t n, int k, const double *V, int64_t ld, doubl
                 int ortho, cudaStream_t s);
 // XB_ETIMEOUT if a wait of an earlier, finished launch (on stream s) ran out.
 int gs_check(xb_plan *p, cudaStream_t s);
-// Algorithmic vector passes (multiples of n elements read + written) of one
-// orthogonalisation of step j.
-double ortho_passes(int ortho, int j);
+// Vector passes (multiples of n elements read + written) of one orthogonalisation
+// of step j in blocks of kb rows: every basis row for its dot and for its update, w
+// once in and once out where the CTAs hold it, else once in for every pass and out
+// for every update.  gm_ortho_step leaves kb and held in the plan.
+double ortho_passes(int ortho, int j, int kb, bool held);
 // The accuracy policy of Sec. 3.3.2: MGS for tol <= 1e-10, else BCGS; DGKS
 // once a fault convergence was seen.  Non-AUTO values pass through.
 int ortho_choice(int ortho, double tol, bool faulted);

@@ -1003,6 +1003,8 @@ int plan_launch(xb_plan *p, GsArgs<VB> &a, cudaStream_t s) {
     const size_t stage = (size_t)KB * gs_pitch<VB, KB, NT>(), fixed = gs_xch_bytes<NT>();
     const size_t wb = (size_t)a.chunk * sizeof(VB);
     const bool sm = fixed + 3 * stage + wb <= (size_t)xb::kGsDynMax;
+    p->gs_kb = KB;
+    p->gs_held = sm;
     a.stages = (int)std::min<size_t>(kGsMaxStages, (xb::kGsDynMax - fixed - (sm ? wb : 0)) / stage);
     const size_t smem = fixed + a.stages * stage + (sm ? wb : 0);
     const int k = a.j + 1;

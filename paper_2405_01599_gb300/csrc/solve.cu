@@ -137,6 +137,7 @@ int gmres_fp64(xb_plan *p, const double *b, double *x, const xb_options &o, xb_i
     if (prec) XB_TRY(xb::ensure_ilu(p, s));
     const double prec_b = prec ? xb::ilu_apply_bytes(p) : 0.0;
     const double spmv_b = xb::spmv_alg_bytes(p, false, 8);
+    std::vector<double> ortho_b(M);  // bytes of the cycle's orthogonalisations
 
     XB_TRY(xb::vnrm2(p, n, b, st.misc + xb::GM_BNORM, s));
     XB_TRY(peek(p, st.misc + xb::GM_BNORM, 1, s));
@@ -216,7 +217,8 @@ int gmres_fp64(xb_plan *p, const double *b, double *x, const xb_options &o, xb_i
             ac.spmv++;
             XB_TRY(xb::gm_ortho_step<double>(p, st, n, V, ld, V + (size_t)(j + 1) * ld, j, ortho,
                                              true, s));
-            ac.bytes += 8.0 * n * xb::ortho_passes(ortho, j);
+            ortho_b[j] = 8.0 * n * xb::ortho_passes(ortho, j, p->gs_kb, p->gs_held);
+            ac.bytes += ortho_b[j];
             launched++;
             const bool last = (j == m - 1) || (iters + launched >= iter_budget);
             if (last) break;
@@ -236,7 +238,7 @@ int gmres_fp64(xb_plan *p, const double *b, double *x, const xb_options &o, xb_i
         const int taken = (stop != 0.0) ? (stop == 2.0 ? k + 1 : k) : launched;
         // the step launched while the end was not yet seen did nothing
         for (; launched > std::min(m, (taken + check - 1) / check * check); launched--) {
-            ac.bytes -= spmv_b + 8.0 * n * xb::ortho_passes(ortho, launched - 1);
+            ac.bytes -= spmv_b + ortho_b[launched - 1];
             ac.spmv--;
         }
         iters += taken;
@@ -275,6 +277,7 @@ int gmres_f32_inner(xb_plan *p, const float *r32, float *d, float *V, int64_t ld
                     SpmvTimer &tm, int *steps, cudaStream_t s) {
     const int64_t n = p->n;
     const double spmv_b = xb::spmv_alg_bytes(p, false, 4);
+    std::vector<double> ortho_b(m);  // bytes of the cycle's orthogonalisations
     *steps = 0;
     XB_CUDA(cudaMemsetAsync(d, 0, n * sizeof(float), s));
     bool first = true;
@@ -314,7 +317,8 @@ int gmres_f32_inner(xb_plan *p, const float *r32, float *d, float *V, int64_t ld
             ac.spmv++;
             XB_TRY(xb::gm_ortho_step<float>(p, st, n, V, ld, V + (size_t)(j + 1) * ld, j, ortho,
                                             true, s));
-            ac.bytes += 4.0 * n * xb::ortho_passes(ortho, j);
+            ortho_b[j] = 4.0 * n * xb::ortho_passes(ortho, j, p->gs_kb, p->gs_held);
+            ac.bytes += ortho_b[j];
             launched++;
             const bool last = (j == m - 1) || (*steps + launched >= maxit);
             if (last) break;
@@ -328,7 +332,7 @@ int gmres_f32_inner(xb_plan *p, const float *r32, float *d, float *V, int64_t ld
         stop = p->h_pin[xb::GM_STOP];
         const int k = (int)p->h_pin[xb::GM_K];
         for (; stop != 0.0 && launched > std::min(m, (std::max(k, 1) + check - 1) / check * check); launched--) {
-            ac.bytes -= spmv_b + 4.0 * n * xb::ortho_passes(ortho, launched - 1);
+            ac.bytes -= spmv_b + ortho_b[launched - 1];
             ac.spmv--;
         }
         *steps += (stop != 0.0) ? k : launched;
@@ -697,7 +701,7 @@ int run_solver(xb_plan *p, const double *b, double *x, const xb_options *opt, xb
         inf.ipt_used = o.ipt > 0 ? o.ipt : p->ipt;
         inf.mem_bytes = ac.mem + xb::spmv_meta_bytes(p, inf.variant_used, inf.block_used, inf.ipt_used) +
                         (o.precision == XB_PREC_MIXED ? 4.0 * p->nnz64 : 0.0) +
-                        (o.precond == XB_PRECOND_ILU0 ? 8.0 * p->nnz64 + 12.0 * p->n : 0.0);
+                        (o.precond == XB_PRECOND_ILU0 ? p->ilu.bytes : 0.0);
         if (st == XB_EFAULT)
             xb::set_error(XB_EFAULT, "fault convergence: implicit residual met tol, "
                                      "||b-Ax||/||b|| = %.3e", inf.res_true);

@@ -850,7 +850,9 @@ __global__ void __launch_bounds__(NT + 64, 1) k_gs(const __grid_constant__ GsArg
 #pragma unroll
                     for (int i = 0; i < KB - 1; i++) {
                         const double ci = __shfl_sync(0xffffffffu, u, i);
-                        if (c.lane > i && c.lane < nd) {
+                        // (a row that w is orthogonal to takes nothing away, whatever its
+                        // products: they overflow sooner than one row's dot does)
+                        if (c.lane > i && c.lane < nd && ci != 0.0) {
                             t = fma(-ci, g[i], t);
                             u = s2 * t;
                         }

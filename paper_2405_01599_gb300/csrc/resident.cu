@@ -934,7 +934,7 @@ int resident_gmres(xb_plan *p, const double *b, double *x, const xb_options &o, 
     // step one SpMV and the Gram-Schmidt passes at the cycle's mean basis
     // size, plus a residual per restart
     const double jm = (r.m + 1) / 2.0, n = a.n;
-    *alg_bytes = r.iters * (spmv_alg_bytes(p, false, 8) + (4.0 * jm + 5.0) * 8.0 * n) +
+    *alg_bytes = r.iters * (spmv_alg_bytes(p, false, 8) + (2.0 * jm + 2.0) * 8.0 * n) +
                  (r.restarts + 1) * (spmv_alg_bytes(p, true, 8) + 16.0 * n);
     if (r.status == XB_EINVAL)
         return set_error(XB_EINVAL, "gmres: column index outside [0, n) in the matrix");

@@ -142,13 +142,14 @@ __device__ __forceinline__ void bulk_copy(unsigned dst, const void *src, unsigne
 
 // A bounded wait: expired() is true once the wait has lasted kGsWait cycles, or
 // as many polls as the caller allows, or another wait of the grid has run out.
-// Between looks at the clock and the grid's flag a poll costs one add.
+// Between looks at the clock and the grid's flag a poll costs one add (look: the
+// polls between them, in a register).
 struct Patience {
     unsigned it = 0;
     long long t0 = 0;
     template <typename VB>
-    __device__ __forceinline__ bool expired(const GsArgs<VB> &a) {
-        if (++it < a.look) return false;
+    __device__ __forceinline__ bool expired(const GsArgs<VB> &a, unsigned look) {
+        if (++it < look) return false;
         if (a.polls != 0) return true;
         it = 0;
         const long long now = clock64();
@@ -221,6 +222,7 @@ struct Ctx {
     unsigned part, bc;     // exchange slots: partial sums of the cluster, totals
     unsigned row0, pitch;  // low words of Vc and of a row's bytes (alignment)
     int len, tiles, rank, lane, wv;
+    unsigned look;
     int st, ph;            // ring position: stage, and times the ring went round
     int pass;              // odd passes take the tiles from the end: they start on the
                            // lines the previous one left in L2
@@ -241,21 +243,17 @@ __device__ __forceinline__ void give_up(Ctx<VB, KB, NT> &c) {
     c.fine = false;
 }
 
-// The whole warp waits and goes on, or gives up, together: what follows a wait
-// has shuffles and votes in it.
+// Waits for a stage.  A lane that gives up, or sees that another has, goes on with
+// what is there, beside the lanes that need not (the addresses stay those of the
+// stage): nothing branches on one lane's c.fine before a vote has made it the
+// warp's.
 template <typename VB, int KB, int NT>
-__device__ __forceinline__ bool wait_bar(Ctx<VB, KB, NT> &c, unsigned bar, unsigned parity) {
+__device__ __forceinline__ void wait_bar(Ctx<VB, KB, NT> &c, unsigned bar, unsigned parity) {
     Patience w;
-    bool ok = true;
-    while (ok && !mbar_done(bar, parity)) {
-        if (*reinterpret_cast<volatile int *>(&c.S->abort)) {
-            ok = false;
-        } else if (w.expired(*c.a)) {
-            give_up(c);
-            ok = false;
-        }
+    while (c.fine && !mbar_done(bar, parity)) {
+        if (*reinterpret_cast<volatile int *>(&c.S->abort)) c.fine = false;
+        else if (w.expired(*c.a, c.look)) give_up(c);
     }
-    return __all_sync(0xffffffffu, ok);
 }
 
 // ---- producer ---------------------------------------------------------------------
@@ -265,9 +263,12 @@ template <typename VB, int KB, int NT>
 __device__ __forceinline__ void produce(Ctx<VB, KB, NT> &c, int t, int row0, int nr, uint64_t policy) {
     if (!c.fine) return;
     const unsigned full = sptr(&c.S->full[c.st]);
-    if (c.ph > 0 && !wait_bar(c, sptr(&c.S->empty[c.st]), (c.ph - 1) & 1)) {
-        c.fine = false;
-        return;
+    if (c.ph > 0) {
+        // a consumer that gave up has said so before it freed a stage that may
+        // still be filling
+        wait_bar(c, sptr(&c.S->empty[c.st]), (c.ph - 1) & 1);
+        c.fine = __all_sync(0xffffffffu, c.fine && !*reinterpret_cast<volatile int *>(&c.S->abort));
+        if (!c.fine) return;
     }
     constexpr int T = gs_tile<VB, KB, NT>();
     const int cnt = min(T, c.len - t * T);
@@ -285,9 +286,8 @@ __device__ __forceinline__ void produce(Ctx<VB, KB, NT> &c, int t, int row0, int
     c.next();
 }
 
-// Waits for the copies that are in flight.  The consumers of a sweep that is
-// given up may leave them behind, at any time until the end, and a CTA must not
-// end before its copies; a sweep that is not has waited for them all.
+// Waits for the copies that are in flight: the consumers of a sweep that is given
+// up leave them behind, and a CTA must not end before its copies.
 template <typename VB, int KB, int NT>
 __device__ void drain(Ctx<VB, KB, NT> &c) {
     for (int i = 0; i < c.a->stages; i++) {
@@ -300,10 +300,8 @@ __device__ void drain(Ctx<VB, KB, NT> &c) {
 
 // ---- consumers --------------------------------------------------------------------
 template <typename VB, int KB, int NT>
-__device__ __forceinline__ bool unit_wait(Ctx<VB, KB, NT> &c) {
-    if (!c.fine) return false;
-    if (!wait_bar(c, sptr(&c.S->full[c.st]), c.ph & 1)) c.fine = false;
-    return c.fine;
+__device__ __forceinline__ void unit_wait(Ctx<VB, KB, NT> &c) {
+    wait_bar(c, sptr(&c.S->full[c.st]), c.ph & 1);
 }
 template <typename VB, int KB, int NT>
 __device__ __forceinline__ void unit_free(Ctx<VB, KB, NT> &c) {
@@ -342,13 +340,13 @@ __device__ __forceinline__ void lds_row(unsigned a, float (&v)[E]) {
 
 // One tile of a pass; FULL: every thread has all its elements.
 template <typename VB, int KB, int NT, int GRAM, bool GR, bool FIN, bool FULL, int NA, int E>
-__device__ __forceinline__ bool gs_tile_pass(Ctx<VB, KB, NT> &c, int e0, VB (&x)[E], VB *dst, int u0, int nu,
+__device__ __forceinline__ void gs_tile_pass(Ctx<VB, KB, NT> &c, int e0, VB (&x)[E], VB *dst, int u0, int nu,
                                              const VB *cf, int d0, int nd, VB (&acc)[NA][chains<VB, KB, GRAM>()]) {
     constexpr int AW = chains<VB, KB, GRAM>();
     const int tid = threadIdx.x;
     const unsigned off = place<VB, E, NT>(tid, 0) * (int)sizeof(VB);
     for (int i0 = 0; i0 < nu; i0 += KB) {
-        if (!unit_wait(c)) return false;
+        unit_wait(c);
         const int nr = min(KB, nu - i0);
 #pragma unroll
         for (int r = 0; r < KB; r++) {
@@ -372,7 +370,7 @@ __device__ __forceinline__ bool gs_tile_pass(Ctx<VB, KB, NT> &c, int e0, VB (&x)
         for (int i = 0; i < E; i++)
             if (FULL || e0 + place<VB, E, NT>(tid, i) < c.len) acc[0][i % AW] = fma(x[i], x[i], acc[0][i % AW]);
     } else {
-        if (!unit_wait(c)) return false;
+        unit_wait(c);
         constexpr bool ALL = GR && GRAM == 2;  // all pairs: the rows are held together
         VB v[ALL ? KB : 1][E], vl[E];
         if constexpr (GR && GRAM == 1) lds_row<NT>(unit_row(c, d0, nd - 1) + off, vl);
@@ -400,7 +398,6 @@ __device__ __forceinline__ bool gs_tile_pass(Ctx<VB, KB, NT> &c, int e0, VB (&x)
         }
         unit_free(c);
     }
-    return true;
 }
 
 // One pass over the CTA's part: w -= sum of the nu rows from u0 (coefficients
@@ -449,10 +446,8 @@ __device__ __forceinline__ void gs_pass(Ctx<VB, KB, NT> &c, const VB *src, bool 
                 x[i] = e < c.len ? src[e] : VB(0);
             }
         }
-        if (!(e0 + T <= c.len
-                  ? gs_tile_pass<VB, KB, NT, GRAM, GR, FIN, true>(c, e0, x, dst, u0, nu, cf, d0, nd, acc)
-                  : gs_tile_pass<VB, KB, NT, GRAM, GR, FIN, false>(c, e0, x, dst, u0, nu, cf, d0, nd, acc)))
-            break;
+        if (e0 + T <= c.len) gs_tile_pass<VB, KB, NT, GRAM, GR, FIN, true>(c, e0, x, dst, u0, nu, cf, d0, nd, acc);
+        else gs_tile_pass<VB, KB, NT, GRAM, GR, FIN, false>(c, e0, x, dst, u0, nu, cf, d0, nd, acc);
     }
 #pragma unroll
     for (int i = 0; i < NA; i++) {
@@ -510,7 +505,7 @@ __device__ __forceinline__ double cluster_sum(Ctx<VB, KB, NT> &c, int q, unsigne
                 all = all && got[s];
             }
         if (__all_sync(0xffffffffu, all)) break;
-        if (__any_sync(0xffffffffu, w.expired(*c.a))) {
+        if (__any_sync(0xffffffffu, w.expired(*c.a, c.look))) {
             give_up(c);
             break;
         }
@@ -548,7 +543,7 @@ __device__ __forceinline__ double grid_sum(Ctx<VB, KB, NT> &c, int q, unsigned s
                 all = all && got[s];
             }
         if (__all_sync(0xffffffffu, all)) break;
-        if (__any_sync(0xffffffffu, w.expired(*c.a))) {
+        if (__any_sync(0xffffffffu, w.expired(*c.a, c.look))) {
             give_up(c);
             break;
         }
@@ -590,7 +585,7 @@ __device__ __forceinline__ double totals(Ctx<VB, KB, NT> &c, int q0, int nv, uns
             if (got) r = v;
         }
         if (__all_sync(0xffffffffu, got)) break;
-        if (__any_sync(0xffffffffu, w.expired(*c.a))) {
+        if (__any_sync(0xffffffffu, w.expired(*c.a, c.look))) {
             give_up(c);
             break;
         }
@@ -724,6 +719,7 @@ __global__ void __launch_bounds__(NT + 64, 1) k_gs(const __grid_constant__ GsArg
     c.wv = tid >> 5;
     c.row0 = (unsigned)(uintptr_t)c.Vc;
     c.pitch = (unsigned)(a.ld * sizeof(VB));
+    c.look = a.look;
     c.st = c.ph = c.pass = 0;
     c.fine = true;
     for (int i = tid; i < gs_xch_bytes<NT>() / 16; i += NT + 64)
@@ -767,7 +763,6 @@ __global__ void __launch_bounds__(NT + 64, 1) k_gs(const __grid_constant__ GsArg
                     }
                 }
         }
-        drain(c);
     } else if (c.wv > NW) {
         if (blockIdx.x == 0) {
             bar_sync(2, NT + 32);
@@ -909,9 +904,11 @@ __global__ void __launch_bounds__(NT + 64, 1) k_gs(const __grid_constant__ GsArg
             }
         }
     }
-    // no CTA leaves while another of its cluster may write to its slots
+    // no CTA leaves while another of its cluster may write to its slots, or before
+    // its own copies
     __syncwarp();
     cluster_sync();
+    if (c.wv == NW && *reinterpret_cast<volatile int *>(&S.abort)) drain(c);
 }
 
 // Largest number of clusters of cs CTAs, one CTA per SM, that the GPU holds.

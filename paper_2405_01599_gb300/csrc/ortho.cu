@@ -178,6 +178,11 @@ __device__ __forceinline__ void warp_totals(double (&v)[NV], int lane) {
     for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
 }
 
+// GRAM: the rows' own products that a kernel takes, 0 none, 1 the newest row's, 2
+// all pairs of a block.  BCGS, CGS and DGKS take none: in FP64 one kernel has both
+// kinds of passes (apart, BCGS took 1.5% longer), in FP32 CGS and DGKS have their own
+// (together, BCGS took 0.4% longer).
+constexpr int kCgs = 3;
 constexpr int gram_count(int kb, int gram) {
     return gram == 1 ? kb - 1 : (gram == 2 ? kb * (kb - 1) / 2 : 0);
 }
@@ -185,7 +190,7 @@ constexpr int gram_count(int kb, int gram) {
 // Chains of a thread's FP32 partial sums: 13 terms each at n = 2.1M, 7 for MGS (where
 // their errors enter the corrections too), then FP64 takes over.
 template <typename VB, int KB, int GRAM>
-constexpr int chains() { return sizeof(VB) == 4 ? (KB <= 4 && GRAM ? 8 : 4) : 1; }
+constexpr int chains() { return sizeof(VB) == 4 ? (KB <= 4 && GRAM == 1 ? 8 : 4) : 1; }
 
 // Launch shape: NT = 256 compute threads, two warps on each quarter of the SM
 // (one waits or loads while the other's FMAs hold the FP64 pipe; more would only
@@ -734,7 +739,8 @@ __global__ void __launch_bounds__(NT + 64, 1) k_gs(const __grid_constant__ GsArg
     }
     cluster_sync();
     unsigned seq = a.base;
-    const bool blocks = a.method == XB_ORTHO_MGS || a.method == XB_ORTHO_BCGS;
+    constexpr bool either = GRAM == 0 && sizeof(VB) == 8;
+    const bool blocks = either ? a.method == XB_ORTHO_MGS || a.method == XB_ORTHO_BCGS : GRAM != kCgs;
     const int nb = (k + KB - 1) / KB, rounds = a.method == XB_ORTHO_DGKS ? 2 : 1;
     const int groups = (k + kGsVals - 1) / kGsVals;
     if (c.wv == NW) {  // producer: the units in the order the passes take them
@@ -864,7 +870,7 @@ __global__ void __launch_bounds__(NT + 64, 1) k_gs(const __grid_constant__ GsArg
                 src = dst = wl;
                 fg = !SM;
             }
-        } else if constexpr (GRAM == 0) {
+        } else if constexpr (either || GRAM == kCgs) {
             for (int r = 0; r < rounds && c.fine; r++)
                 for (int g0 = 0; g0 < k && c.fine; g0 += kGsVals) {
                     const int kg = min(kGsVals, k - g0);
@@ -1046,10 +1052,10 @@ int gs_run(xb_plan *p, GsArgs<VB> &a, bool seen, cudaStream_t s) {
         }
     } else {
         if (a.n >= 1500000 && a.method != XB_ORTHO_BCGS)
-            return a.method == XB_ORTHO_MGS ? plan_launch<VB, 4, 1>(p, a, s) : plan_launch<VB, 4, 0>(p, a, s);
+            return a.method == XB_ORTHO_MGS ? plan_launch<VB, 4, 1>(p, a, s) : plan_launch<VB, 4, kCgs>(p, a, s);
     }
     if (a.method == XB_ORTHO_BCGS) return plan_launch<VB, 4, 0>(p, a, s);
-    if (a.method != XB_ORTHO_MGS) return plan_launch<VB, 8, 0>(p, a, s);
+    if (a.method != XB_ORTHO_MGS) return plan_launch<VB, 8, sizeof(VB) == 8 ? 0 : kCgs>(p, a, s);
     if constexpr (sizeof(VB) == 8) {
         if (seen && longv) return plan_launch<VB, 2, 1>(p, a, s);
         if (!seen) {

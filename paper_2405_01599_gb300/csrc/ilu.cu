@@ -567,6 +567,7 @@ struct FlowHost {
     std::vector<int4> items;
     std::vector<int> iptr, rows, ecol, esrc;
     std::vector<long long> ebase;
+    long long longs = 0;  // entries of the rows that the warp takes from the factors
 };
 // Blocks [c0, c1) appended to h (their rows go to rows[bstart[c]..]).
 template <typename Beg, typename End>
@@ -610,6 +611,7 @@ void flow_blocks(const std::vector<int> &lev, const std::vector<int> &bstart, in
             }
             // long rows first: they take longest
             for (int i : team[6]) {
+                h.longs += end(i) - beg(i);
                 rows[r0 + a] = i;
                 h.items.push_back(make_int4(r0 + a++, 1 | 256 | 5 << 9, 0, 0));
             }
@@ -686,6 +688,7 @@ bool flow_layout(const std::vector<int> &lev, const std::vector<int> &bstart, in
         if (!ok[t]) return false;
         ni += part[t].items.size();
         ne += part[t].ecol.size();
+        h.longs += part[t].longs;
     }
     h.items.reserve(ni);
     h.ecol.reserve(ne);
@@ -948,13 +951,9 @@ int ensure_ilu(xb_plan *p, cudaStream_t s) {
         XB_TRY(upload(&u.d_bstart, bstart, s, &u));
         XB_TRY(upload_flow(u, u.fl, hl, s));
         XB_TRY(upload_flow(u, u.fu, hu, s));
-        // long rows come from the factors themselves, rows and all
-        long long stored = 0;
-        for (const FlowHost *h : {&hl, &hu})
-            stored += std::count_if(h->esrc.begin(), h->esrc.end(), [](int e) { return e >= 0; });
         // r in, z out, the pivots and reciprocals, both triangles' published values
         // out and the first one's in again
-        u.flow_bytes += 12.0 * ((double)nnz - n - stored) + (8.0 + 8.0 + 16.0 + 32.0 + 16.0) * n;
+        u.flow_bytes += 12.0 * (hl.longs + hu.longs) + (8.0 + 8.0 + 16.0 + 32.0 + 16.0) * n;
         XB_TRY(keep(u, &u.fu.d_diag, (size_t)n * sizeof(double)));
         XB_TRY(keep(u, &u.fu.d_rdiag, (size_t)n * sizeof(double)));
         k_diag_fill<<<(n + 255) / 256, 256, 0, s>>>(n, u.fu.d_rows, u.d_dpos, u.d_lu, u.fu.d_diag,

@@ -18,6 +18,9 @@ Run on a GPU:  python -m paper_2405_01599_gb300.tuner --make-data 750 --seed 100
 After an SpMV kernel changes, re-time the saved sweeps (the GMRES(m) timings
 are kept) and retrain:
                python -m paper_2405_01599_gb300.tuner --resweep D1.npz D2.npz ...
+or retrain only the heads that choose the SpMV, which leaves the choice of m,
+whose timings are the old ones, as it is:
+               python -m paper_2405_01599_gb300.tuner --train D.npz --spmv-heads-of M.bin --model M.bin
 """
 from __future__ import annotations
 
@@ -304,6 +307,28 @@ def train_model(D, epochs=400, batch=128, lr=3e-3, seed=0, dev="cuda"):
     return model, loss
 
 
+def retrain_spmv(model, D, steps=10000, lr=3e-3, dev="cuda"):
+    """Train the model's SpMV heads (variant, CTA size, ipt) on D by full-batch
+    Adam; the layers below them and the head for m stay as they are."""
+    import torch
+    X = torch.tensor(D["feat"].astype(np.float32), device=dev)
+    lab = labels_of(D)
+    lab[:, 3] = -1  # no loss for m
+    lab = torch.tensor(lab, device=dev)
+    d_in, h1, h2, heads = model.dims
+    w3 = h1 * d_in + h1 + h2 * h1 + h2
+    o, spmv = sum(heads), sum(heads[:3])
+    kept = np.ones(model.param_count(), bool)
+    kept[w3:w3 + spmv * h2] = False
+    kept[w3 + o * h2:w3 + o * h2 + spmv] = False
+    old = model.get_params()
+    for t in range(1, steps + 1):
+        loss, g = model.loss_grad(X, lab)
+        model.adam(t, lr=lr)
+        model.set_params(np.where(kept, old, model.get_params()))
+    return model, loss
+
+
 def evaluate(model, D, dev="cuda"):
     """Regret of the learned choice vs the exhaustive optimum and gain over the
     fixed default (no tuning), per matrix, for SpMV time and GMRES time."""
@@ -359,6 +384,8 @@ def main():
     ap.add_argument("--out", default=None)
     ap.add_argument("--train", nargs="*", default=None, help="dataset(s) to concatenate")
     ap.add_argument("--model", default=None)
+    ap.add_argument("--spmv-heads-of", default=None,
+                    help="with --train: start from this model and train its SpMV heads only")
     ap.add_argument("--evaluate", default=None)
     ap.add_argument("--evaluate-data", default=None,
                     help="saved held-out sweep (.npz) for --evaluate instead of --make-data")
@@ -393,7 +420,11 @@ def main():
                 p_["m_full"] = np.zeros(len(p_["feat"]), np.int32)
         Dt = {k: np.concatenate([p_[k] for p_ in parts]) for k in parts[0]}
         print(f"[tuner train] {n_records(Dt)} timing records from {len(Dt['feat'])} matrices")
-        model, loss = train_model(Dt, epochs=a.epochs)
+        if a.spmv_heads_of:
+            import paper_2405_01599_gb300 as xb
+            model, loss = retrain_spmv(xb.Mlp.load(a.spmv_heads_of), Dt)
+        else:
+            model, loss = train_model(Dt, epochs=a.epochs)
         print(f"[tuner train] {len(Dt['feat'])} samples, final loss {loss:.4f}")
         if a.model:
             model.save(a.model)

@@ -848,19 +848,24 @@ __global__ void __launch_bounds__(NT + 64, 1) k_gs(const __grid_constant__ GsArg
                 }
                 double u = s2 * t;
                 if constexpr (GRAM != 0) {
+                    // a row that w is orthogonal to takes nothing away, whatever its
+                    // products: they overflow sooner than one row's dot does.  Looked at
+                    // only where a total is not finite (in every block it cost 0.25 us), and
+                    // not in GMRES, whose rows' norms are finite squares
+                    auto correct = [&](bool look) {
 #pragma unroll
-                    for (int i = 0; i < KB - 1; i++) {
-                        const double ci = __shfl_sync(0xffffffffu, u, i);
-                        // a row that w is orthogonal to takes nothing away, whatever its
-                        // products: they overflow sooner than one row's dot does.  Not in
-                        // GMRES, whose rows' norms are finite squares (and where the look
-                        // costs 1.2 us a step of GMRES(30), n = 262,144)
-                        const bool takes = GRAM == 1 || __double_as_longlong(ci) << 1 != 0;
-                        if (c.lane > i && c.lane < nd && takes) {
-                            t = fma(-ci, g[i], t);
-                            u = s2 * t;
+                        for (int i = 0; i < KB - 1; i++) {
+                            const double ci = __shfl_sync(0xffffffffu, u, i);
+                            if (c.lane > i && c.lane < nd && !(look && ci == 0.0)) {
+                                t = fma(-ci, g[i], t);
+                                u = s2 * t;
+                            }
                         }
-                    }
+                    };
+                    if (GRAM == 2 && __any_sync(0xffffffffu, (__double2hiint(tot) & 0x7ff00000) == 0x7ff00000))
+                        correct(true);
+                    else
+                        correct(false);
                 }
                 if (c.lane < KB) S.cfw[c.wv][c.lane] = (VB)u;
                 if (c.wv == 0 && c.lane < nd) S.hcol[d0 + c.lane] = s1 * t;

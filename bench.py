@@ -959,8 +959,8 @@ def batch(xb, torch, dev, args, cpu):
     default vs the exhaustive run-time tuner (each system's SpMV candidates
     timed, Sec. 3.1; m fixed at 30) vs the learned tuner (SpMV choice and m).
     Throughput of a launch: algorithmic bytes and flops summed over the
-    systems' Arnoldi steps (one SpMV plus the MGS passes of the step at the
-    cycle's mean basis size) over the launch time."""
+    systems' Arnoldi steps (one SpMV, and each row of the cycle's mean basis twice
+    and w in and out) over the launch time."""
     import oracle
     from paper_2405_01599_gb300 import gen, tuner
     specs = gen.batch_specs(512, seed=5)
@@ -1012,7 +1012,7 @@ def batch(xb, torch, dev, args, cpu):
         for (n, nnz), q in zip(shapes, r):
             jm = (q["m"] + 1) / 2.0  # mean basis size of a cycle's step
             steps = q["iters"]
-            by += steps * ((12 * nnz + 4 * (n + 1) + 16 * n) + (4 * jm + 5) * 8 * n)
+            by += steps * ((12 * nnz + 4 * (n + 1) + 16 * n) + (2 * jm + 2) * 8 * n)
             fl += steps * (2 * nnz + 4 * n * (jm + 1))
         return {"GBs": by / (t_ms * 1e-3) / 1e9, "GFLOPs": fl / (t_ms * 1e-3) / 1e9,
                 "alg_GB": by / 1e9, "arnoldi_steps": int(sum(q["iters"] for q in r))}

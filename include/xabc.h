@@ -19,13 +19,13 @@
  *     last error on the calling host thread is returned by xb_last_error().
  *   - Some launches hold their SMs together, one CTA on each: an
  *     orthogonalisation (xb_orth, xb_mgs, and every step of the multi-launch
- *     GMRES and of the eigensolvers; up to every SM from about 40,000 rows on)
- *     and an ILU(0) substitution (up to every SM).  Such a launch starts when
- *     all its SMs are free, so beside work on other streams it waits for that
- *     work's CTAs to end, and the calls' results do not depend on it.  A kernel
- *     that stays on an SM until such a call is over must be left its SM:
- *     xb_orth_config with XB_ORTH_CTAS, and xb_ilu0_config with mode 0 (a launch
- *     per dependency level, which needs no SMs together).
+ *     GMRES and of the eigensolvers; 120 SMs from 30,000 rows on, every SM from
+ *     400,000 on) and an ILU(0) substitution (up to every SM).  Such a launch
+ *     starts when all its SMs are free, so beside work on other streams it waits
+ *     for that work's CTAs to end; results do not depend on it.  A kernel that
+ *     stays on an SM until such a call is over must be left its SM: xb_orth_config
+ *     with XB_ORTH_CTAS, and xb_ilu0_config with mode 0 (a launch per dependency
+ *     level, which needs no SMs together).
  *   - A plan (xb_plan) owns library workspace in device memory, created by
  *     xb_plan_create and released by xb_plan_destroy.  A plan may be used by
  *     one host thread / one stream at a time.
@@ -405,8 +405,11 @@ int xb_spmv_f32(xb_plan *plan, int32_t variant, float alpha, const float *x, flo
  * after every claimed convergence: the fault-convergence test of Sec. 3.1 and
  * 3.3.2, which narrows the implicit threshold and continues when the claim
  * was false), or with XB_ENOCONV at maxiter / maxtime_s, or XB_EBREAKDOWN.
- * b == 0 gives x = 0.  The host synchronises `stream` every
- * opt->check_every steps to read the residual. */
+ * b == 0 gives x = 0.  Every opt->check_every steps the host reads the residual:
+ * BiCGStab and preconditioned GMRES wait for the step, GMRES without a
+ * preconditioner looks at it after it has launched the next step (a word that
+ * the step writes to pinned memory; a step launched after a cycle's end does
+ * nothing). */
 
 /* Restarted GMRES(m) (Sec. 2.2, Sec. 4.3): Arnoldi with the
  * orthogonalisation opt->ortho -- MGS, CGS, DGKS (CGS run twice) or BCGS
@@ -451,7 +454,11 @@ int xb_dot(xb_plan *plan, int32_t n, const double *x, const double *y, double *o
 int xb_axpy(int32_t n, double a, const double *x, double *y, void *stream); /* y += a x */
 /* One modified Gram-Schmidt sweep (Sec. 3.2.2, MGS): for i = 0..k-1,
  * h[i] = (w, V_i); w -= h[i] V_i, with V row-major k x ld (ld >= n), then
- * h[k] = ||w||.  h: device, k+1 doubles. */
+ * h[k] = ||w||.  h: device, k+1 doubles.  Taken in blocks of 2 or 4 rows whose
+ * dots are corrected by the rows' own inner products: the same method, but an h[i]
+ * carries the rounding error of ||w|| as it was at the block's start (w = 1e8 V_0 +
+ * u, ||u|| = 1: w is off by as much as one row at a time, 1e-8, but meets the
+ * block's later rows to 1e-9 and not to 1e-17). */
 int xb_mgs(xb_plan *plan, int32_t n, int32_t k, const double *V, int64_t ld, double *w,
            double *h, void *stream);
 /* Orthogonalise w against the k rows of V (row-major k x ld, ld >= n, rows

@@ -563,8 +563,8 @@ class Plan:
         return z
 
     def ilu0_config(self, mode=-1, barrier_polls=0):
-        """ILU(0) substitution path (-1 automatic, 0 graph, 1 persistent) and
-        the persistent path's barrier poll limit (0 = default)."""
+        """ILU(0) substitution path (-1 automatic, 0 graph, 1 flow) and the polls
+        of one wait of the flow path (0 = default)."""
         _check(lib().xb_ilu0_config(self._h, int(mode), int(barrier_polls)))
 
     def ilu0_factors(self, stream=None):
@@ -769,7 +769,7 @@ class Mlp:
 class Batch:
     """Many independent systems solved by GMRES(m) in one persistent,
     graph-captured launch (xb_batch_*).  systems: list of dicts with device
-    tensors rowptr, col, val, b, x and ints m, mode (0 thread/row, 1 warp/row).
+    tensors rowptr, col, val, b, x and ints m, mode (0 thread/row, 1 tiles of 256 entries).
     """
 
     def __init__(self, systems, stream=None, zero_x=True, **opts):

@@ -796,7 +796,9 @@ int resident_clusters(size_t dyn) {
 // 2 + m / 8 sums at 2 us (3.3 us across a cluster), and n m + nnz FP64 terms (1.5
 // nnz in mode 1) at 0.4 ns a CTA, with a seventh lost to the split over a cluster's
 // 8.  Fitted to 48 systems of 1000 to 57,000 rows at m = 30 (one CTA 28 to 825 us,
-// a cluster 18 to 133 us a step), within a fifth.
+// a cluster 18 to 133 us a step), within a fifth.  At m = 10 it is a third too low for
+// both, at m = 100 a sixth too high; the split of five mixes of 20 to 300 systems is
+// within 14% of the best fixed number of rows at m = 10, 30 and 100.
 double step_us(const xb_batch_dev &d, bool cluster) {
     const double sums = 2.0 + d.m / 8.0,
                  terms = 4e-4 * ((double)d.m * d.n + (d.mode == 1 ? 1.5 : 1.0) * d.nnz);

@@ -287,7 +287,8 @@ __device__ __forceinline__ void produce(Ctx<VB, KB, NT> &c, int t, int row0, int
     if (c.lane == 0) mbar_expect(full, bytes);
     __syncwarp();
     if (c.lane < nr)
-        bulk_copy(c.ring + (c.st * KB + c.lane) * gs_pitch<VB, KB, NT>(), (const void *)lo, (unsigned)(hi - lo), full, policy);
+        bulk_copy(c.ring + (c.st * KB + c.lane) * gs_pitch<VB, KB, NT>(), (const void *)lo,
+                  (unsigned)(hi - lo), full, policy);
     c.next();
 }
 
@@ -682,11 +683,15 @@ __device__ void scalar_warp(Ctx<VB, KB, NT> &c, unsigned seq, bool raw) {
 // the FP64 pipe (two FMAs per basis element) or, for the FP32 basis, HBM.  So:
 // one launch; few warps (a sum over the threads of an SM costs FP64 time in
 // proportion to their number); w read once and written once; and an exchange
-// per block of KB rows.  For MGS that is exact, not an approximation:
+// per block of KB rows.  For MGS that is the same method in exact arithmetic:
 //   (w - sum_{k<i} c_k V_k, V_i) = (w, V_i) - sum_{k<i} c_k (V_k, V_i),
 // with k over the earlier rows of the block, so the dots of a block are all
 // taken with the same w and corrected by the rows' own inner products.  In
-// GMRES (GRAM 1) those are kept from the step in which a row was the newest
+// rounding, c_i carries eps ||w|| of the block's first w, not of what the earlier
+// rows left: as much as w's own updates carry into the result, so the loss against
+// the rows as a whole is MGS's (w = 1e4 V_0 + u: ||w'|| off by 1.4e-12, 0.9e-12 one at
+// a time; against the block's later rows 1e-13, 1e-17 one at a time).  In
+// GMRES (GRAM 1) the products are kept from the step in which a row was the newest
 // (at most KB - 1 more dots a step); a sweep against rows it has not seen
 // (GRAM 2) takes them in the same pass.
 //
@@ -1050,7 +1055,7 @@ int gs_run(xb_plan *p, GsArgs<VB> &a, bool seen, cudaStream_t s) {
     const int k = a.j + 1;
     if constexpr (sizeof(VB) == 8) {
         if (longv && (a.method != XB_ORTHO_MGS || k == 1)) {
-            // one row: every method takes one dot
+            // (MGS against one row has no products)
             if (k <= 2) return plan_launch<VB, 2, 0, 512>(p, a, s);
             if (k <= 4 || a.method == XB_ORTHO_BCGS) return plan_launch<VB, 4, 0, 512>(p, a, s);
             return plan_launch<VB, 8, 0, 512>(p, a, s);

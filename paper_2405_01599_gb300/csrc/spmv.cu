@@ -827,8 +827,11 @@ __global__ void __launch_bounds__(512) k_sym_tile(const int *__restrict__ rowptr
 // and only the in-tile transpose sums are in shared memory.  The scaling of y
 // runs beside the first loads (programmatic launch).  Bound: the FP64 pipe (a
 // product and an FMA per stored entry).  128^3 Laplacian, upper storage (n =
-// 2.1M): staged kernel after its scaling 83 us, this pair 41 us.  Longer rows
-// stay with the staged kernel, whose rows are walked in shared memory.
+// 2.1M): staged kernel after its scaling 83 us, this pair 53 us (45 the kernel
+// alone).  Rows of up to 9 / 21 / 29 entries within 1,000 columns, n = 1M (256 x
+// 8): staged 74 / 175 / 243 us, this 62 / 147 / 204; within 60 columns, 29 entries 309
+// / 253; anywhere 166 / 154; n = 20,000, 14 and 29 entries: 13.3 / 8.1, 17.9 / 10.5.
+// Longer rows stay with the staged kernel, whose rows are walked in shared memory.
 // ---------------------------------------------------------------------------
 constexpr int kSymShort = 32, kSymGroup = 4;
 template <typename V, bool A1>
